@@ -69,7 +69,7 @@ struct bop_ctx {
   int maxlev[BOP_MAX_K + 2];  // largest |C_k| per level, then the largest adjacency
   bool built = false, energized = false, weighted = false;
   // buffers
-  DBuf pos, cell_of, cell_count, cell_start, cell_fill, cell_atoms, deg, row_ptr, col, img, flag, bond_scan,
+  DBuf pos, cell_of, cell_count, cell_start, cell_fill, cell_atoms, cell_slot, deg, row_ptr, col, img, flag, bond_scan,
       bond_of_edge, bond_atoms, bond_img, bond_d, H64, H32, frac;
   DBuf hkeys, hvals, skeys, sslot, scount;
   DBuf level_end, atom_nsite, atom_nadj, max_level, site_off, adj_base, site_atom, site_img, adj_off, adj, lvcnt;
@@ -100,9 +100,11 @@ struct bop_ctx {
   DBuf psi_off, psis, lsum;
   DBuf fev;  // two device doubles of the distributed Fermi solve
   DBuf gs32;  // FP32 copy of gsig for the starting point of a cold Fermi solve
-  DBuf cw_misc, cw_keys, cw_epack;  // warp cluster builder: max degree / failure flags, site keys per
-                                    // atom, packed neighbour edges
-  int cw_maxdeg = -1;  // largest degree of the centres, read back with the neighbour list's status
+  // grid cluster builder: structure maxima / failure flag, site records and
+  // counts per atom, packed neighbour edges and rows; capacity tier
+  DBuf cw_misc, cw_keys, cw_cnt, cw_epack, cw_eoff, cw_rows;
+  int grid_max[5] = {0, 0, 0, 0, 0};
+  int cw_tier = 0;
   long long psi_tot = 0;
   bool psi_valid = false;
   size_t store_budget = (size_t)-1;
@@ -388,98 +390,119 @@ int geometry(bop_ctx* c, const double* cell, const int* pbc, Geometry* g) {
   return BOP_OK;
 }
 
-// Warp-per-atom builder (clusters of at most cluster_warp_max_sites()
-// sites, atoms of at most 32 neighbours); *done = false when it does not
-// apply, and the block builder below runs instead.
-int build_clusters_warp(bop_ctx* c, cudaStream_t s, bool* done) {
+// Grid builder (rows of at most 32 neighbours, a table that fits shared
+// memory); *done = false when it does not apply, and the block builder below
+// runs instead.  Capacities by tier: a cluster that outgrows one tier sends
+// the structure, and the context's later ones, to the next.
+int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
   *done = false;
   const int n = c->nc, K = c->K;  // clusters of the centres
-  if (n == 0 || (c->cl_maxs && c->cl_maxs > cluster_warp_max_sites())) return BOP_OK;
-  if (K > 5 && !(c->m.r_path > 0)) return BOP_OK;  // bcc has 1,105 sites within 6 hops
-  int misc[4] = {0, 0, 0, 0};
-  CKS(ensure(c, c->cw_misc, 4 * sizeof(int)));
-  if (c->cw_maxdeg < 0) {  // not read with the neighbour list
-    CK(cudaMemsetAsync(c->cw_misc.p, 0, 4 * sizeof(int), s));
-    launch_max_degree(n, P<long long>(c->row_ptr), P<int>(c->cw_misc), s);
-    Readback rb(c, s);
-    CKS(rb.add(misc, c->cw_misc.p, 4 * sizeof(int)));
-    CKS(rb.sync());
-    c->cw_maxdeg = misc[0];
-  }
-  const int max_deg = c->cw_maxdeg;
-  c->cw_maxdeg = -1;
-  CK(cudaMemsetAsync(P<int>(c->cw_misc) + 1, 0, 3 * sizeof(int), s));
-  if (max_deg > 32) return BOP_OK;
-  int* wfail = P<int>(c->cw_misc) + 1;
+  static const int CAP[4][2] = {{512, 256}, {1536, 512}, {4096, 1024}, {8192, 2048}};
+  GridPlan plan;
+  if (n == 0 || c->n >= (1 << 24) || c->grid_max[0] > 32 || !grid_plan(c->g, K, c->grid_max, &plan)) return BOP_OK;
   CKS(ensure(c, c->level_end, sizeof(int) * (size_t)n * (K + 1)));
   CKS(ensure(c, c->atom_nsite, sizeof(int) * (n + 1)));
   CKS(ensure(c, c->atom_nadj, sizeof(int) * (n + 1)));
-  CK(cudaMemsetAsync(c->atom_nsite.p, 0, sizeof(int) * (n + 1), s));
-  CK(cudaMemsetAsync(c->atom_nadj.p, 0, sizeof(int) * (n + 1), s));
   CKS(ensure(c, c->max_level, sizeof(int) * (K + 2)));
   CKS(ensure(c, c->site_off, sizeof(long long) * (n + 1)));
   CKS(ensure(c, c->adj_base, sizeof(long long) * (n + 1)));
-  CKS(ensure(c, c->cw_keys, sizeof(unsigned long long) * (size_t)n * cluster_warp_max_sites()));
   CKS(ensure(c, c->cw_epack, sizeof(int2) * (size_t)(c->E > 0 ? c->E : 1)));
-  launch_pack_edges(c->E, P<int>(c->col), P<signed char>(c->img), P<int2>(c->cw_epack), s);
-  CK(cudaMemsetAsync(c->max_level.p, 0, sizeof(int) * (K + 2), s));
+  CKS(ensure(c, c->cw_eoff, sizeof(int2) * (size_t)(c->E > 0 ? c->E : 1)));
+  CKS(ensure(c, c->cw_rows, sizeof(int2) * (size_t)c->n));
+  if (launch_pack_edges(c->n, plan, c->g, P<long long>(c->row_ptr), P<int>(c->col), P<signed char>(c->img),
+                        P<int>(c->bond_of_edge), P<int>(c->cell_of), P<int>(c->cell_slot), P<int2>(c->cw_epack),
+                        P<int2>(c->cw_eoff), P<int2>(c->cw_rows), s))
+    return fail(c, BOP_ERR_CUDA, "edge packing launch failed");
   PathCut pc;
   pc.pos = P<double>(c->pos);
   for (int q = 0; q < 9; q++) pc.cell[q] = c->g.cell[q];
   pc.r2 = c->m.r_path > 0 ? c->m.r_path * c->m.r_path : 0.0;
-  ClusterOut out{};
-  out.level_end = P<int>(c->level_end);
-  out.atom_nsite = P<int>(c->atom_nsite);
-  out.atom_nadj = P<int>(c->atom_nadj);
-  out.max_level = P<int>(c->max_level);
-  {
-    Region R0(c, PK_CLUSTER, 1, s);
-    if (launch_cluster_warp(0, n, K, max_deg, P<long long>(c->row_ptr), P<int2>(c->cw_epack),
-                            P<int>(c->bond_of_edge), pc, P<unsigned long long>(c->cw_keys), out, wfail,
-                            P<unsigned>(c->status), s))
-      return fail(c, BOP_ERR_CUDA, "cluster pass 0 launch failed");
+  const int first = c->m.r_path > 0 || K <= 4 ? 0 : (K <= 6 ? 1 : 2);
+  for (int tier = c->cw_tier > first ? c->cw_tier : first; tier < 4; tier++) {
+    CK(cudaMemsetAsync(c->atom_nsite.p, 0, sizeof(int) * (n + 1), s));
+    CK(cudaMemsetAsync(c->atom_nadj.p, 0, sizeof(int) * (n + 1), s));
+    CK(cudaMemsetAsync(c->max_level.p, 0, sizeof(int) * (K + 2), s));
+    CK(cudaMemsetAsync(c->cw_misc.p, 0, sizeof(int), s));
+    GridArgs a;
+    a.n = n;
+    a.K = K;
+    a.origin = plan.origin;
+    a.tsize = plan.tsize;
+    a.lpr_shift = c->grid_max[0] <= 16 ? 4 : 5;
+    a.maxs = CAP[tier][0];
+    a.newcap = CAP[tier][1];
+    a.sites = a.maxs;
+    a.mx = plan.mx;
+    a.my = plan.my;
+    a.mz = plan.mz;
+    a.ncode = (2 * a.mx + 1) * (2 * a.my + 1) * (2 * a.mz + 1);
+    a.qbits = 0;
+    while ((1 << a.qbits) < a.newcap) a.qbits++;
+    if ((unsigned long long)c->n * a.ncode >= 1ull << (32 - a.qbits)) return BOP_OK;  // 32-bit sort keys
+    CKS(ensure(c, c->cw_keys, sizeof(unsigned long long) * (size_t)n * a.maxs));
+    CKS(ensure(c, c->cw_cnt, (size_t)n * a.maxs));
+    a.rows = P<int2>(c->cw_rows);
+    a.epack = P<int2>(c->cw_epack);
+    a.eoff = P<int2>(c->cw_eoff);
+    a.slot = P<int>(c->cell_slot);
+    a.recs = P<unsigned long long>(c->cw_keys);
+    a.counts = P<unsigned char>(c->cw_cnt);
+    a.fail = P<int>(c->cw_misc);
+    a.status = P<unsigned>(c->status);
+    ClusterOut out{};
+    out.level_end = P<int>(c->level_end);
+    out.atom_nsite = P<int>(c->atom_nsite);
+    out.atom_nadj = P<int>(c->atom_nadj);
+    out.max_level = P<int>(c->max_level);
+    {
+      Region R0(c, PK_CLUSTER, 1, s);
+      const int r = launch_cluster_grid(0, a, pc, out, s);
+      if (r == -2) return BOP_OK;  // the table and the tier's records do not fit
+      if (r) return fail(c, BOP_ERR_CUDA, "cluster pass 0 launch failed");
+    }
+    // the sizes and the flag of pass 0 in one synchronisation (the scans run
+    // before it is known whether pass 0 succeeded; they are discarded if not)
+    CKS(exclusive_scan(c, P<int>(c->atom_nsite), P<long long>(c->site_off), n + 1, s));
+    CKS(exclusive_scan(c, P<int>(c->atom_nadj), P<long long>(c->adj_base), n + 1, s));
+    long long tot[2];
+    int failed = 0;
+    {
+      Readback rb(c, s);
+      CKS(rb.add(&tot[0], P<long long>(c->site_off) + n, sizeof(long long)));
+      CKS(rb.add(&tot[1], P<long long>(c->adj_base) + n, sizeof(long long)));
+      CKS(rb.add(c->maxlev, c->max_level.p, sizeof(int) * (K + 2)));
+      CKS(rb.add(&failed, c->cw_misc.p, sizeof(int)));
+      CKS(rb.finish());  // synchronises
+    }
+    if (failed) continue;
+    c->cw_tier = tier;
+    c->nsite = tot[0];
+    c->nadj = tot[1];
+    CKS(ensure(c, c->site_atom, sizeof(int) * c->nsite));
+    CKS(ensure(c, c->site_img, 3 * c->nsite));
+    CKS(ensure(c, c->adj_off, sizeof(long long) * (c->nsite + 1)));
+    CKS(ensure(c, c->adj, sizeof(int2) * c->nadj));
+    CKS(ensure(c, c->lvcnt, sizeof(unsigned long long) * c->nsite));
+    out.site_off = P<long long>(c->site_off);
+    out.adj_base = P<long long>(c->adj_base);
+    out.site_atom = P<int>(c->site_atom);
+    out.site_img = P<signed char>(c->site_img);
+    out.adj_off = P<long long>(c->adj_off);
+    out.adj = P<int2>(c->adj);
+    out.lvcnt = P<unsigned long long>(c->lvcnt);
+    CKS(ensure(c, c->nprod, sizeof(unsigned long long)));
+    CK(cudaMemsetAsync(c->nprod.p, 0, sizeof(unsigned long long), s));
+    out.n_products = P<unsigned long long>(c->nprod);
+    a.sites = c->maxlev[K];
+    {
+      Region R1(c, PK_CLUSTER, 1, s);
+      if (launch_cluster_grid(1, a, pc, out, s)) return fail(c, BOP_ERR_CUDA, "cluster pass 1 launch failed");
+    }
+    CK(cudaMemcpyAsync(P<long long>(c->adj_off) + c->nsite, P<long long>(c->adj_base) + n, sizeof(long long),
+                       cudaMemcpyDeviceToDevice, s));
+    *done = true;  // the status of pass 1 is read with the structure's last readback
+    return BOP_OK;
   }
-  // the sizes and the flags of pass 0 in one synchronisation (the scans run
-  // before it is known whether pass 0 succeeded; they are discarded if not)
-  CKS(exclusive_scan(c, P<int>(c->atom_nsite), P<long long>(c->site_off), n + 1, s));
-  CKS(exclusive_scan(c, P<int>(c->atom_nadj), P<long long>(c->adj_base), n + 1, s));
-  long long tot[2];
-  {
-    Readback rb(c, s);
-    CKS(rb.add(&tot[0], P<long long>(c->site_off) + n, sizeof(long long)));
-    CKS(rb.add(&tot[1], P<long long>(c->adj_base) + n, sizeof(long long)));
-    CKS(rb.add(c->maxlev, c->max_level.p, sizeof(int) * (K + 2)));
-    CKS(rb.add(misc, c->cw_misc.p, 4 * sizeof(int)));
-    CKS(rb.finish());  // synchronises
-  }
-  if (misc[1] != 0) return BOP_OK;  // too large for the warp builder
-  c->nsite = tot[0];
-  c->nadj = tot[1];
-  CKS(ensure(c, c->site_atom, sizeof(int) * c->nsite));
-  CKS(ensure(c, c->site_img, 3 * c->nsite));
-  CKS(ensure(c, c->adj_off, sizeof(long long) * (c->nsite + 1)));
-  CKS(ensure(c, c->adj, sizeof(int2) * c->nadj));
-  CKS(ensure(c, c->lvcnt, sizeof(unsigned long long) * c->nsite));
-  out.site_off = P<long long>(c->site_off);
-  out.adj_base = P<long long>(c->adj_base);
-  out.site_atom = P<int>(c->site_atom);
-  out.site_img = P<signed char>(c->site_img);
-  out.adj_off = P<long long>(c->adj_off);
-  out.adj = P<int2>(c->adj);
-  out.lvcnt = P<unsigned long long>(c->lvcnt);
-  CKS(ensure(c, c->nprod, sizeof(unsigned long long)));
-  CK(cudaMemsetAsync(c->nprod.p, 0, sizeof(unsigned long long), s));
-  out.n_products = P<unsigned long long>(c->nprod);
-  {
-    Region R1(c, PK_CLUSTER, 1, s);
-    if (launch_cluster_warp(1, n, K, max_deg, P<long long>(c->row_ptr), P<int2>(c->cw_epack),
-                            P<int>(c->bond_of_edge), pc, P<unsigned long long>(c->cw_keys), out, wfail,
-                            P<unsigned>(c->status), s))
-      return fail(c, BOP_ERR_CUDA, "cluster pass 1 launch failed");
-  }
-  CK(cudaMemcpyAsync(P<long long>(c->adj_off) + c->nsite, P<long long>(c->adj_base) + n, sizeof(long long),
-                     cudaMemcpyDeviceToDevice, s));
-  *done = true;  // the status of pass 1 is read with the structure's last readback
   return BOP_OK;
 }
 
@@ -487,7 +510,7 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
   const int n = c->nc, K = c->K;  // clusters of the centres
   {
     bool done = false;
-    CKS(build_clusters_warp(c, s, &done));
+    CKS(build_clusters_grid(c, s, &done));
     if (done) return BOP_OK;
   }
   int grid = n < 1216 ? n : 1216;
@@ -1394,7 +1417,7 @@ int bop_create(bop_ctx** out, const bop_model* model) {
 
 int bop_destroy(bop_ctx* c) {
   if (!c) return BOP_OK;
-  DBuf* bufs[] = {&c->pos, &c->cell_of, &c->cell_count, &c->cell_start, &c->cell_fill, &c->cell_atoms, &c->deg,
+  DBuf* bufs[] = {&c->pos, &c->cell_of, &c->cell_count, &c->cell_start, &c->cell_fill, &c->cell_atoms, &c->cell_slot, &c->deg,
                   &c->row_ptr, &c->col, &c->img, &c->flag, &c->bond_scan, &c->bond_of_edge, &c->bond_atoms,
                   &c->bond_img, &c->bond_d, &c->H64, &c->H32, &c->frac, &c->hkeys, &c->hvals, &c->skeys,
                   &c->sslot, &c->scount, &c->level_end, &c->atom_nsite, &c->atom_nadj, &c->max_level,
@@ -1407,7 +1430,7 @@ int bop_destroy(bop_ctx* c) {
                   &c->lys, &c->lZ1, &c->lH1, &c->lZ2, &c->lH2, &c->lybar, &c->lcot, &c->lxbar, &c->lcount,
                   &c->rwN, &c->rwt, &c->rdUE, &c->rvec, &c->rcoef, &c->rjv, &c->rjcnt, &c->rjptr, &c->rjidx, &c->rjrow, &c->vgrad, &c->vq, &c->erep,
                   &c->psi_off, &c->psis, &c->lsum, &c->sdir, &c->vmom, &c->obar, &c->torque,
-                  &c->ncscr, &c->cw_misc, &c->cw_keys, &c->cw_epack, &c->fev, &c->gs32};
+                  &c->ncscr, &c->cw_misc, &c->cw_keys, &c->cw_cnt, &c->cw_epack, &c->cw_eoff, &c->cw_rows, &c->fev, &c->gs32};
   for (DBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   if (c->pin) cudaFreeHost(c->pin);
@@ -1443,6 +1466,7 @@ int bop_build_hamiltonian(bop_ctx* c, int n, const double* pos, const double* ce
   CKS(ensure(c, c->cell_start, sizeof(int) * (ncell + 1)));
   CKS(ensure(c, c->cell_fill, sizeof(int) * ncell));
   CKS(ensure(c, c->cell_atoms, sizeof(int) * n));
+  CKS(ensure(c, c->cell_slot, sizeof(int) * n));
   CKS(ensure(c, c->deg, sizeof(int) * (n + 1)));
   CKS(ensure(c, c->row_ptr, sizeof(long long) * (n + 1)));
   CKS(ensure(c, c->frac, sizeof(double) * 6 * 64));
@@ -1455,7 +1479,7 @@ int bop_build_hamiltonian(bop_ctx* c, int n, const double* pos, const double* ce
   bopk::k_bin_atoms<<<gb, TB, 0, s>>>(n, P<double>(c->pos), g, P<int>(c->cell_of), P<int>(c->cell_count));
   CKS(exclusive_scan(c, P<int>(c->cell_count), P<int>(c->cell_start), ncell + 1, s));
   bopk::k_fill_cells<<<gb, TB, 0, s>>>(n, P<int>(c->cell_of), P<int>(c->cell_start), P<int>(c->cell_fill),
-                                       P<int>(c->cell_atoms));
+                                       P<int>(c->cell_atoms), P<int>(c->cell_slot));
   CK(cudaMemsetAsync(c->deg.p, 0, sizeof(int) * (n + 1), s));
   launch_neighbors(0, n, P<double>(c->pos), g, P<int>(c->cell_of), P<int>(c->cell_start), P<int>(c->cell_atoms),
                    P<int>(c->deg), nullptr, nullptr, nullptr, P<unsigned>(c->status), s);
@@ -1513,18 +1537,17 @@ int bop_build_hamiltonian(bop_ctx* c, int n, const double* pos, const double* ce
   }
   }
   CK(cudaGetLastError());
-  // the centres' largest degree (the cluster builder's variant) read back
-  // with the neighbour list's status
-  int md[4] = {0, 0, 0, 0};
-  CKS(ensure(c, c->cw_misc, 4 * sizeof(int)));
-  CK(cudaMemsetAsync(c->cw_misc.p, 0, 4 * sizeof(int), s));
-  launch_max_degree(c->nc, P<long long>(c->row_ptr), P<int>(c->cw_misc), s);
+  // the maxima that the cluster builder is planned with, read back with the
+  // neighbour list's status
+  CKS(ensure(c, c->cw_misc, 8 * sizeof(int)));
+  CK(cudaMemsetAsync(c->cw_misc.p, 0, 8 * sizeof(int), s));
+  launch_grid_maxima(n, P<long long>(c->row_ptr), ncell, P<int>(c->cell_start), nb, P<double>(c->bond_d), g,
+                     P<int>(c->cw_misc), s);
   {
     Readback rb(c, s);
-    CKS(rb.add(md, c->cw_misc.p, 4 * sizeof(int)));
+    CKS(rb.add(c->grid_max, c->cw_misc.p, 5 * sizeof(int)));
     CKS(rb.finish());
   }
-  c->cw_maxdeg = md[0];
   CKS(build_clusters(c, s));
   CKS(size_state(c));
   // per-atom row offsets of a stored Psi sweep

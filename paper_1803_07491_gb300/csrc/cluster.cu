@@ -8,8 +8,9 @@
 // (sx, sy, sz).  Each site's adjacency lists every neighbour inside the
 // cluster as {local index, bond}, ascending local index.
 //
-// One CTA per atom (grid-stride), a hash table of site keys in per-CTA
-// global scratch, the new sites of a level sorted in shared memory.
+// Two builders with the same results: the general one, one CTA per atom
+// (grid-stride), a hash table of site keys in per-CTA global scratch, the new
+// sites of a level sorted in shared memory; and the grid builder below it.
 #include "kernels.h"
 
 namespace {
@@ -303,336 +304,445 @@ k_cluster(int n, int K, const long long* __restrict__ row_ptr, const int* __rest
   }
 }
 
-// ---------------------------------------------------------------- warp builder
+// ---------------------------------------------------------------- grid builder
 // The same clusters (same canonical order, same adjacency and level counts)
-// with one warp per atom: a cluster of a few hundred sites has levels of
-// 1, 14, 50, 110, ... new sites, which a warp covers without block-wide
-// barriers, and every hash probe stays in shared memory.  Pass 0 runs the
-// breadth-first search, counts the adjacency and keeps each atom's site
-// keys in global scratch; pass 1 reloads them, fills the hash table and
-// writes the sites, the sorted adjacency and the level counts.  Clusters of
-// more than CW_MAXS sites, or atoms with more than MAXD neighbours, raise
-// *wfail and the caller falls back to the block builder above.
-constexpr int CW_WARPS = 3;   // warps per CTA (five CTAs of 14 KB per warp fit an SM)
-constexpr int CW_MAXS = 512;  // sites of one cluster
-constexpr int CW_NB = 256;    // new sites of one level
-constexpr int CW_HC = 1024;   // hash slots per warp (a power of two, 2 CW_MAXS)
-// A hash entry is the 48-bit site key with the site's local index + 1 in
-// the top 16 bits (0 while the index is not yet assigned).
-constexpr unsigned long long CW_KEY = (1ull << 48) - 1;
+// through a table in shared memory instead of a hash table.  Every site has
+// an address: its linked cell relative to the cluster's atom, unwrapped over
+// the periodic images, times the slots of a cell, plus its atom's slot in
+// that cell.  The address of a neighbour is the site's address plus an offset
+// that depends on the directed edge alone (k_pack_edges), so that looking a
+// site up is one shared-memory load, with no key, hash or probe.
+//
+// Table size: sites lie within R_K cells of the atom along each axis,
+// neighbours that are looked up within R_{K+1} (grid_plan).  A period of
+// R_K + R_{K+1} + 1 cells keeps the address of every looked-up cell apart
+// from that of every other cell a site can lie in, and only the addresses of
+// sites need storage.
+//
+// Order without sorting the adjacency: a neighbour row is sorted by (atom,
+// image), as the sites of one level are, and the neighbours of a site of
+// level l lie in levels l-1, l, l+1.  An entry's place in its row is its rank
+// among the entries of its own level (a ballot) after the entries of the
+// levels below.  Rows take 16 or 32 lanes, one per edge, so that the loads of
+// a row and its writes are contiguous.
+//
+// G threads per atom.  Pass 0 runs the breadth-first search (new sites are
+// claimed in the table with an atomicOr, sorted per level), counts the
+// adjacency and keeps the site records; pass 1 fills the table from them and
+// writes sites, adjacency and level counts.
+//
+// What bounds it: issue slots (58 to 68 % used), after the table's 14 to 76
+// KB per cluster has limited the CTAs on an SM, hence several warps per
+// cluster.  The hash-table builder it replaces (one warp per atom, 64-bit
+// keys) took 27.9 k and 34.4 k warp instructions per atom in the two passes,
+// this one 16.3 k and 17.1 k: 131,072 bcc atoms at 9 moments 19.8 -> 5.7 ms,
+// 2,000 atoms at 17 moments (one CTA per atom, hash table in global memory
+// before) 10.6 -> 1.1 ms.
+constexpr unsigned short GRID_CLAIM = 0x8000;  // claimed, index not yet assigned; else index + 1
 
-struct CwSmem {
-  unsigned long long hk[CW_HC];
-  unsigned long long sk[CW_MAXS];  // site keys in canonical order
-  unsigned long long nb[CW_NB];    // new keys of one level
-  int lev[BOP_MAX_K + 1];
-  int cnt, fail;
-};
+// site record: atom (24 bits), image bytes + 128 (24 bits), table address (16 bits)
+__device__ __forceinline__ unsigned long long grid_rec(int atom, unsigned img, int addr) {
+  return ((unsigned long long)(unsigned)atom << 40) | ((unsigned long long)img << 16) | (unsigned)addr;
+}
+__device__ __forceinline__ int rec_atom(unsigned long long r) { return (int)(r >> 40); }
+__device__ __forceinline__ int rec_addr(unsigned long long r) { return (int)(r & 0xffff); }
+__device__ __forceinline__ int rec_img(unsigned long long r, int c) { return (int)((r >> (16 + 8 * c)) & 0xff) - 128; }
+// Image bytes of a packed edge or record: component 0 in the high byte, so
+// that records order as (atom, sx, sy, sz).
+__device__ __forceinline__ int epk_img(int y, int c) { return (int)(((unsigned)y >> (16 - 8 * c)) & 0xffu) - 128; }
 
-__device__ __forceinline__ int cw_find(const unsigned long long* hk, unsigned long long key) {
-  unsigned s = hash_slot(key, CW_HC - 1);
-  for (int probe = 0; probe < CW_HC; probe++) {
-    const unsigned long long c = hk[s];
-    if (c == EMPTY) return -1;
-    if ((c & CW_KEY) == key) return (int)s;
-    s = (s + 1) & (CW_HC - 1);
+// Image of a neighbour: the site's plus the edge's, per component, as bytes
+// + 128; false if a component leaves [-127, 127].
+__device__ __forceinline__ bool image_sum(unsigned long long rec, int epk, unsigned* img) {
+  const unsigned ti = (unsigned)(rec >> 16), ei = (unsigned)epk;
+  const unsigned x = ((ti >> 16) & 255u) + ((ei >> 16) & 255u) - 128u, y = ((ti >> 8) & 255u) + ((ei >> 8) & 255u) - 128u,
+                 z = (ti & 255u) + (ei & 255u) - 128u;
+  *img = (x << 16) | (y << 8) | z;
+  return x - 1u < 255u && y - 1u < 255u && z - 1u < 255u;
+}
+
+template <int G>
+__device__ __forceinline__ void group_sync() {
+  if constexpr (G == 32) __syncwarp();
+  else __syncthreads();
+}
+
+// One compare-exchange step with the key of index idx ^ j, in the merge of
+// blocks of k.
+__device__ __forceinline__ unsigned cmp_exchange(unsigned x, unsigned y, int idx, int j, int k) {
+  return ((idx & j) == 0) == ((idx & k) == 0) ? min(x, y) : max(x, y);
+}
+// Strides 32 .. 1 of the merge of blocks of k over 64 keys of one warp: lane
+// holds keys i0 (x0) and i0 + 32 (x1).
+__device__ __forceinline__ void merge64(unsigned& x0, unsigned& x1, int i0, int k) {
+  if (k >= 64) {
+    const unsigned lo = min(x0, x1), hi = max(x0, x1);
+    const bool up = (i0 & k) == 0;
+    x0 = up ? lo : hi;
+    x1 = up ? hi : lo;
   }
-  return -1;
-}
-
-__device__ __forceinline__ int cw_index(const unsigned long long* hk, int slot) {
-  return (int)(hk[slot] >> 48) - 1;
-}
-
-// 1: inserted (index unassigned), 0: present, -1: full.  slot receives the
-// key's slot.
-__device__ __forceinline__ int cw_insert(unsigned long long* hk, unsigned long long key, int* slot) {
-  unsigned s = hash_slot(key, CW_HC - 1);
-  for (int probe = 0; probe < CW_HC; probe++) {
-    const unsigned long long c = hk[s];
-    if (c != EMPTY && (c & CW_KEY) == key) {
-      *slot = (int)s;
-      return 0;
-    }
-    if (c == EMPTY) {
-      const unsigned long long prev = atomicCAS(&hk[s], EMPTY, key);
-      if (prev == EMPTY) {
-        *slot = (int)s;
-        return 1;
-      }
-      if ((prev & CW_KEY) == key) {
-        *slot = (int)s;
-        return 0;
-      }
-    }
-    s = (s + 1) & (CW_HC - 1);
+#pragma unroll
+  for (int j = 16; j > 0; j >>= 1) {
+    if (j >= k) continue;
+    const unsigned y0 = __shfl_xor_sync(0xffffffffu, x0, j), y1 = __shfl_xor_sync(0xffffffffu, x1, j);
+    x0 = cmp_exchange(x0, y0, i0, j, k);
+    x1 = cmp_exchange(x1, y1, i0 + 32, j, k);
   }
-  return -1;
 }
-
-// Ascending bitonic sort of a[0..cnt) by one warp, padded with EMPTY to the
-// next power of two (at most CW_NB).
-__device__ __forceinline__ void cw_sort(unsigned long long* a, int cnt, int lane) {
-  int P = 1;
+// Ascending bitonic sort of a[0..cnt) by the group.  Every warp holds 64
+// keys in registers and exchanges them by shuffles; only strides of 64 and
+// more go through shared memory (three block barriers for 256 keys).  The
+// keys were written before a group barrier.
+template <int G>
+__device__ __forceinline__ void group_sort(unsigned* a, int cnt, int tid) {
+  int P = 64;
   while (P < cnt) P <<= 1;
-  for (int i = cnt + lane; i < P; i += 32) a[i] = EMPTY;
-  __syncwarp();
+  if (P <= 2 * G) {
+    const int i0 = (tid >> 5) * 64 + (tid & 31), i1 = i0 + 32;
+    const bool active = i0 < P;  // whole warps
+    unsigned x0 = ~0u, x1 = ~0u;
+    if (active) {
+      if (i0 < cnt) x0 = a[i0];
+      if (i1 < cnt) x1 = a[i1];
+#pragma unroll
+      for (int k = 2; k <= 64; k <<= 1) merge64(x0, x1, i0, k);
+    }
+    for (int k = 128; k <= P; k <<= 1) {
+      for (int j = k >> 1; j >= 64; j >>= 1) {
+        group_sync<G>();
+        if (active) {
+          a[i0] = x0;
+          a[i1] = x1;
+        }
+        group_sync<G>();
+        if (active) {
+          x0 = cmp_exchange(x0, a[i0 ^ j], i0, j, k);
+          x1 = cmp_exchange(x1, a[i1 ^ j], i1, j, k);
+        }
+      }
+      if (active) merge64(x0, x1, i0, k);
+    }
+    group_sync<G>();
+    if (active) {
+      if (i0 < cnt) a[i0] = x0;
+      if (i1 < cnt) a[i1] = x1;
+    }
+    group_sync<G>();
+    return;
+  }
+  for (int i = cnt + tid; i < P; i += G) a[i] = ~0u;
+  group_sync<G>();
   for (int k = 2; k <= P; k <<= 1)
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = lane; i < P; i += 32) {
-        const int l = i ^ j;
-        if (l > i) {
-          const unsigned long long x = a[i], y = a[l];
-          const bool up = (i & k) == 0;
-          if ((x > y) == up) {
-            a[i] = y;
-            a[l] = x;
-          }
-        }
+      for (int p = tid; p < P / 2; p += G) {
+        const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1)), l = i | j;
+        const unsigned lo = min(a[i], a[l]), hi = max(a[i], a[l]);
+        const bool up = (i & k) == 0;
+        a[i] = up ? lo : hi;
+        a[l] = up ? hi : lo;
       }
-      __syncwarp();
+      group_sync<G>();
     }
 }
 
-// Image of a packed edge record: byte c of y holds image component c + 128.
-__device__ __forceinline__ int epk_img(int y, int c) { return (int)(((unsigned)y >> (8 * c)) & 0xffu) - 128; }
+// What a row step needs of its site, in shared memory (written one thread per
+// site, read by the row's lanes): the first edge, and the address and degree.
+__device__ __forceinline__ int2 site_row(int2 row, int addr) { return make_int2(row.x, addr | (row.y << 16)); }
 
-template <int PASS, bool CUT, int MAXD>
-__global__ void __launch_bounds__(32 * CW_WARPS, MAXD <= 16 ? 5 : 2)
-k_cluster_warp(int n, int K, const long long* __restrict__ row_ptr, const int2* __restrict__ epack,
-               const int* __restrict__ bond_of_edge, PathCut pc,
-               unsigned long long* __restrict__ gkeys, ClusterOut out, int* __restrict__ wfail,
-               unsigned* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char cw_raw[];
-  CwSmem& sm = reinterpret_cast<CwSmem*>(cw_raw)[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  const int nwarps = gridDim.x * CW_WARPS;
-  for (int atom = blockIdx.x * CW_WARPS + (threadIdx.x >> 5); atom < n; atom += nwarps) {
-    for (int q = lane; q < CW_HC; q += 32) sm.hk[q] = EMPTY;
-    if (lane == 0) {
-      sm.fail = 0;
-      sm.cnt = 0;
-    }
-    __syncwarp();
-    unsigned long long* gk = gkeys + (size_t)atom * CW_MAXS;
-    int nsite;
+template <int PASS, bool CUT, int G>
+__global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, ClusterOut out) {
+  extern __shared__ __align__(16) unsigned char grid_raw[];
+  __shared__ int s_lev[BOP_MAX_K + 1];
+  __shared__ int s_cnt, s_fail;
+  __shared__ int s_warp[G / 32 + 1];
+  unsigned short* tab = reinterpret_cast<unsigned short*>(grid_raw);
+  const int tab16 = (A.tsize * 2 + 15) / 16;  // 16-byte words
+  unsigned char* tail = grid_raw + (size_t)tab16 * 16;
+  // pass 0: the new records of a level, their sort keys, site records, site rows
+  unsigned long long* nb = reinterpret_cast<unsigned long long*>(tail);
+  unsigned* keys = reinterpret_cast<unsigned*>(nb + A.newcap);
+  unsigned long long* sk = reinterpret_cast<unsigned long long*>(keys + A.newcap);
+  int2* srow = reinterpret_cast<int2*>(sk + A.maxs);
+  // pass 1: per site {site row, first site of its level | first site of the
+  // next level, row offset}, then entries per class
+  int4* sinf = reinterpret_cast<int4*>(tail);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int K = A.K;
+  const int sub = tid >> A.lpr_shift, j = tid & ((1 << A.lpr_shift) - 1);  // row of the step, edge of the row
+  const int rps = G >> A.lpr_shift;                                        // rows per step
+  const unsigned hm = A.lpr_shift == 5 ? 0xffffffffu : (lane < 16 ? 0xffffu : 0xffff0000u);  // the row's lanes
+  const unsigned below = hm & ((1u << lane) - 1u);
+  constexpr int U = 2;  // row steps in flight
+  unsigned long long prod = 0;
+  for (int atom = blockIdx.x; atom < A.n; atom += gridDim.x) {
+    for (int q = tid; q < tab16; q += G) reinterpret_cast<uint4*>(tab)[q] = make_uint4(0, 0, 0, 0);
+    unsigned long long* gk = A.recs + (size_t)atom * A.maxs;
+    unsigned char* gc = A.counts + (size_t)atom * A.maxs;
+    if (tid == 0) s_fail = s_cnt = 0;
     if (PASS == 0) {
-      // breadth-first search over hop levels
-      if (lane == 0) {
-        const unsigned long long k0 = site_key(atom, 0, 0, 0);
-        int sl = 0;
-        cw_insert(sm.hk, k0, &sl);
-        sm.hk[sl] = k0 | (1ull << 48);
-        sm.sk[0] = k0;
-        sm.lev[0] = 1;
+      group_sync<G>();
+      if (tid == 0) {
+        const int a0 = A.origin + A.slot[atom];
+        tab[a0] = 1;
+        const unsigned long long r = grid_rec(atom, 0x808080u, a0);
+        sk[0] = gk[0] = r;
+        srow[0] = site_row(A.rows[atom], a0);
+        s_lev[0] = 1;
       }
-      __syncwarp();
-      nsite = 1;
+      group_sync<G>();
+      int nsite = 1, f0 = 0;
+      int tot = 0;  // adjacency entries
       for (int k = 1; k <= K; k++) {
-        const int f0 = k >= 2 ? sm.lev[k - 2] : 0, f1 = sm.lev[k - 1];
-        for (int t = f0 + lane; t < f1; t += 32) {
-          const unsigned long long kt = sm.sk[t];
-          const int a = key_atom(kt);
-          const int ix = key_img(kt, 0), iy = key_img(kt, 1), iz = key_img(kt, 2);
-          const long long e0 = row_ptr[a];
-          int deg = (int)(row_ptr[a + 1] - e0);
-          if (deg > MAXD) {
-            atomicOr(wfail, 2);
-            deg = MAXD;
-          }
-          int2 pe[MAXD];  // the atom's edges, all loads in flight together
+        const int f1 = nsite;
+        for (int t0 = f0; t0 < f1; t0 += U * rps) {
+          int2 sr[U];
+          int ad[U];
 #pragma unroll
-          for (int j = 0; j < MAXD; j++)
-            if (j < deg) pe[j] = __ldg(epack + e0 + j);
-#pragma unroll
-          for (int j = 0; j < MAXD; j++) {
-            if (j >= deg) continue;
-            const int sx = ix + epk_img(pe[j].y, 0), sy = iy + epk_img(pe[j].y, 1), sz = iz + epk_img(pe[j].y, 2);
-            if (sx < -127 || sx > 127 || sy < -127 || sy > 127 || sz < -127 || sz > 127) {
-              sm.fail = 1;
-              raise_error(status, BOP_DEV_ERR_IMAGE);
-              continue;
-            }
-            if (CUT) {
-              double d[3];
-              bond_vector(pc.pos + 3 * (size_t)atom, pc.pos + 3 * (size_t)pe[j].x, pc.cell, sx, sy, sz, d);
-              if (!(norm2_rn(d) < pc.r2)) continue;
-            }
-            const unsigned long long key = site_key(pe[j].x, sx, sy, sz);
-            int sl = 0;
-            const int r = cw_insert(sm.hk, key, &sl);
-            if (r == 1) {
-              const int q = atomicAdd(&sm.cnt, 1);
-              if (q < CW_NB) sm.nb[q] = key;
-            } else if (r < 0) {
-              sm.fail = 1;
-            }
-          }
-        }
-        __syncwarp();
-        const int cnt = sm.cnt;
-        if (cnt > CW_NB || cnt > CW_MAXS - nsite) sm.fail = 1;
-        __syncwarp();
-        if (sm.fail) break;
-        // canonical order inside the level: the new keys sorted
-        cw_sort(sm.nb, cnt, lane);
-        for (int q = lane; q < cnt; q += 32) {
-          const unsigned long long key = sm.nb[q];
-          sm.sk[nsite + q] = key;
-          const int sl = cw_find(sm.hk, key);
-          if (sl >= 0) sm.hk[sl] = key | ((unsigned long long)(nsite + q + 1) << 48);
-        }
-        __syncwarp();
-        nsite += cnt;
-        if (lane == 0) {
-          sm.lev[k] = nsite;
-          sm.cnt = 0;
-        }
-        __syncwarp();
-      }
-      if (sm.fail) {
-        if (lane == 0) {
-          atomicOr(wfail, 1);
-          out.atom_nsite[atom] = 0;
-          out.atom_nadj[atom] = 0;
-        }
-        __syncwarp();
-        continue;
-      }
-      for (int t = lane; t < nsite; t += 32) gk[t] = sm.sk[t];
-    } else {
-      // pass 1: the keys of pass 0 (canonical order) and the level ends
-      for (int k = lane; k <= K; k += 32) sm.lev[k] = out.level_end[(size_t)atom * (K + 1) + k];
-      __syncwarp();
-      nsite = sm.lev[K];
-      for (int t = lane; t < nsite; t += 32) {
-        const unsigned long long key = gk[t];
-        sm.sk[t] = key;
-        int sl = 0;
-        cw_insert(sm.hk, key, &sl);
-        sm.hk[sl] = key | ((unsigned long long)(t + 1) << 48);
-      }
-      __syncwarp();
-    }
-    // adjacency of every site: the neighbours inside the cluster, by local index
-    const long long s0 = PASS == 1 ? out.site_off[atom] : 0;
-    const long long a0 = PASS == 1 ? out.adj_base[atom] : 0;
-    int run = 0;
-    unsigned long long prod = 0;
-    for (int tb = 0; tb < nsite; tb += 32) {
-      const int t = tb + lane;
-      unsigned long long ent[MAXD];
-      int deg = 0, c = 0;
-      int lt = 0;
-      if (t < nsite) {
-        const unsigned long long kt = sm.sk[t];
-        const int a = key_atom(kt);
-        const int ix = key_img(kt, 0), iy = key_img(kt, 1), iz = key_img(kt, 2);
-        const long long e0 = row_ptr[a];
-        deg = (int)(row_ptr[a + 1] - e0);
-        if (deg > MAXD) {
-          atomicOr(wfail, 2);
-          deg = MAXD;
-        }
-        // without a path cut every neighbour of a site within K-1 hops is in
-        // the cluster: pass 0 counts those without looking them up
-        const bool inner = !CUT && PASS == 0 && t < sm.lev[K > 0 ? K - 1 : 0] && K > 0;
-        if (inner) {
-          c = deg;
-#pragma unroll
-          for (int j = 0; j < MAXD; j++) ent[j] = ~0ull;
-        } else {
-          int2 pe[MAXD];
-          int bnd[MAXD];
-#pragma unroll
-          for (int j = 0; j < MAXD; j++) {
-            if (j < deg) {
-              pe[j] = __ldg(epack + e0 + j);
-              bnd[j] = PASS == 1 ? __ldg(bond_of_edge + e0 + j) : 0;
-            }
+          for (int u = 0; u < U; u++) {
+            const int t = t0 + u * rps + sub;
+            sr[u] = t < f1 ? srow[t] : make_int2(0, 0);
           }
 #pragma unroll
-          for (int j = 0; j < MAXD; j++) {
-            ent[j] = ~0ull;
-            if (j < deg) {
-              const int sx = ix + epk_img(pe[j].y, 0), sy = iy + epk_img(pe[j].y, 1), sz = iz + epk_img(pe[j].y, 2);
-              if (sx >= -127 && sx <= 127 && sy >= -127 && sy <= 127 && sz >= -127 && sz <= 127) {
-                const int sl = cw_find(sm.hk, site_key(pe[j].x, sx, sy, sz));
-                if (sl >= 0) {
-                  ent[j] = ((unsigned long long)cw_index(sm.hk, sl) << 32) | (unsigned)bnd[j];
-                  c++;
-                }
+          for (int u = 0; u < U; u++)
+            ad[u] = j < (sr[u].y >> 16) ? (sr[u].y & 0xffff) + __ldg(&A.eoff[sr[u].x + j].x) : -1;
+#pragma unroll
+          for (int u = 0; u < U; u++) {
+            // not yet a site of the cluster
+            bool win = ad[u] != -1 && ((unsigned)ad[u] >= (unsigned)A.tsize || tab[ad[u]] == 0);
+            const int t = t0 + u * rps + sub, e = sr[u].x + j;
+            if (CUT && win) {  // path-radius cut: only sites closer than r_path to the atom
+              const int2 pe = __ldg(A.epack + e);
+              unsigned img;
+              if (!image_sum(sk[t], pe.y, &img)) {
+                s_fail = 1;
+                raise_error(A.status, BOP_DEV_ERR_IMAGE);
+                win = false;
+              } else {
+                double d[3];
+                bond_vector(pc.pos + 3 * (size_t)atom, pc.pos + 3 * (size_t)pe.x, pc.cell, (int)(img >> 16) - 128,
+                            (int)((img >> 8) & 255u) - 128, (int)(img & 255u) - 128, d);
+                win = norm2_rn(d) < pc.r2;
+              }
+            }
+            if (win && (unsigned)ad[u] >= (unsigned)A.tsize) {  // outside the planned table: the general builder
+              s_fail = 1;
+              win = false;
+            }
+            if (win) {
+              const int sh = (ad[u] & 1) * 16;
+              const unsigned old = atomicOr(reinterpret_cast<unsigned*>(tab) + (ad[u] >> 1), (unsigned)GRID_CLAIM << sh);
+              if (((old >> sh) & 0xffffu) == 0) {
+                const int q = atomicAdd(&s_cnt, 1);
+                if (q < A.newcap) nb[q] = ((unsigned long long)(unsigned)e << 32) | (unsigned)t;
               }
             }
           }
         }
-        while (lt < K && t >= sm.lev[lt]) lt++;
-      }
-      // offsets of this chunk's rows
-      int incl = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const int off = run + incl - c;
-      run += __shfl_sync(0xffffffffu, incl, 31);
-      if (PASS == 1 && t < nsite) {
-        const unsigned long long kt = sm.sk[t];
-        out.site_atom[s0 + t] = key_atom(kt);
-        out.site_img[3 * (s0 + t)] = (signed char)key_img(kt, 0);
-        out.site_img[3 * (s0 + t) + 1] = (signed char)key_img(kt, 1);
-        out.site_img[3 * (s0 + t) + 2] = (signed char)key_img(kt, 2);
-        out.adj_off[s0 + t] = a0 + off;
-        // level ends in registers (levels above K never match)
-        int lv[BOP_MAX_K];
-#pragma unroll
-        for (int k = 0; k < BOP_MAX_K; k++) lv[k] = k < K ? sm.lev[k] : 0x7fffffff;
-        // the entries' local indices (distinct within a site; unused entries
-        // 0xffffffff): the rank of an entry by its local index is its rank
-        unsigned hi[MAXD];
-#pragma unroll
-        for (int j = 0; j < MAXD; j++) hi[j] = (unsigned)(ent[j] >> 32);
-        // per-level entry counts, one byte per level (at most MAXD each)
-        unsigned long long per_level = 0;
-#pragma unroll
-        for (int j = 0; j < MAXD; j++) {
-          if (ent[j] == ~0ull) continue;
-          int rank = 0;
-#pragma unroll
-          for (int i = 0; i < MAXD; i++) rank += hi[i] < hi[j] ? 1 : 0;
-          const int sidx = (int)hi[j];
-          out.adj[a0 + off + rank] = make_int2(sidx, (int)(unsigned)(ent[j] & 0xffffffffu));
-          int ls = 0;  // level of the entry's site
-#pragma unroll
-          for (int k = 0; k < BOP_MAX_K; k++) ls += sidx >= lv[k] ? 1 : 0;
-          if (ls < K) per_level += 1ull << (8 * ls);
-          const int k0 = lt > ls + 1 ? lt : ls + 1;
-          if (k0 <= K) prod += (unsigned long long)(K - k0 + 1);
+        group_sync<G>();
+        const int cnt = s_cnt;
+        const bool bad = s_fail != 0 || cnt > A.newcap || cnt > A.maxs - nsite;
+        group_sync<G>();
+        if (bad) {
+          if (tid == 0) s_fail = 1;
+          break;
         }
-        // byte k of lvcnt: entries of level <= k, k < K (the byte-wise prefix
-        // sum of per_level: every partial sum is at most MAXD <= 32 < 256)
-        unsigned long long lc = per_level * 0x0101010101010101ull;
-        if (K < 8) lc &= (1ull << (8 * K)) - 1ull;
-        out.lvcnt[s0 + t] = lc;
+        // the claimed (site, edge) pairs become records; canonical order inside the level
+        for (int q = tid; q < cnt; q += G) {
+          const unsigned long long c = nb[q];
+          const unsigned long long rt = sk[(unsigned)c];
+          const int e = (int)(c >> 32);
+          const int2 pe = __ldg(A.epack + e);
+          unsigned img;
+          if (!image_sum(rt, pe.y, &img)) {
+            s_fail = 1;
+            raise_error(A.status, BOP_DEV_ERR_IMAGE);
+          }
+          nb[q] = grid_rec(pe.x, img, rec_addr(rt) + __ldg(&A.eoff[e].x));
+          const unsigned code = (((img >> 16) - 128u + A.mx) * (2u * A.my + 1u) + ((img >> 8) & 255u) - 128u + A.my) *
+                                    (2u * A.mz + 1u) + (img & 255u) - 128u + A.mz;
+          keys[q] = ((unsigned)pe.x * A.ncode + code) << A.qbits | (unsigned)q;
+        }
+        group_sync<G>();
+        group_sort<G>(keys, cnt, tid);
+        for (int q = tid; q < cnt; q += G) {
+          const unsigned long long r = nb[keys[q] & ((1u << A.qbits) - 1u)];
+          const int t = nsite + q;
+          const int2 row = __ldg(A.rows + rec_atom(r));
+          sk[t] = gk[t] = r;
+          srow[t] = site_row(row, rec_addr(r));
+          tab[rec_addr(r)] = (unsigned short)(t + 1);
+          // without a path cut every neighbour of a site within K-1 hops is in the cluster
+          if (!CUT && k < K) {
+            gc[t] = (unsigned char)row.y;
+            tot += row.y;
+          }
+        }
+        f0 = f1;
+        nsite += cnt;
+        if (tid == 0) {
+          s_lev[k] = nsite;
+          s_cnt = 0;
+        }
+        group_sync<G>();
       }
-    }
-    if (PASS == 0) {
-      if (lane == 0) {
-        out.atom_nsite[atom] = nsite;
-        out.atom_nadj[atom] = run;
-        atomicMax(&out.max_level[K + 1], run);
+      group_sync<G>();
+      if (s_fail) {
+        if (tid == 0) {
+          atomicOr(A.fail, 1);
+          out.atom_nsite[atom] = 0;
+          out.atom_nadj[atom] = 0;
+        }
+        group_sync<G>();
+        continue;
       }
-      for (int k = lane; k <= K; k += 32) {
-        out.level_end[(size_t)atom * (K + 1) + k] = sm.lev[k];
-        atomicMax(&out.max_level[k], sm.lev[k]);
+      // adjacency counts of the other sites
+      if (!CUT && tid == 0) {
+        gc[0] = (unsigned char)(srow[0].y >> 16);
+        tot += srow[0].y >> 16;
       }
-    } else {
+      for (int t0 = CUT ? 0 : f0; t0 < nsite; t0 += U * rps) {
+        int2 sr[U];
+        int ad[U];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, o);
-      if (lane == 0 && prod) atomicAdd(out.n_products, prod);
+        for (int u = 0; u < U; u++) {
+          const int t = t0 + u * rps + sub;
+          sr[u] = t < nsite ? srow[t] : make_int2(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          ad[u] = j < (sr[u].y >> 16) ? (sr[u].y & 0xffff) + __ldg(&A.eoff[sr[u].x + j].x) : -1;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const bool hit = (unsigned)ad[u] < (unsigned)A.tsize && tab[ad[u]] != 0;
+          const int c = __popc(__ballot_sync(0xffffffffu, hit) & hm);
+          const int t = t0 + u * rps + sub;
+          if (j == 0 && t < nsite) {
+            gc[t] = (unsigned char)c;
+            tot += c;
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+      if (G > 32) {
+        if (lane == 0) s_warp[tid >> 5] = tot;
+        group_sync<G>();
+        tot = 0;
+        for (int w = 0; w < G / 32; w++) tot += s_warp[w];
+      }
+      if (tid == 0) {
+        out.atom_nsite[atom] = nsite;
+        out.atom_nadj[atom] = tot;
+        if (tot > *(volatile int*)&out.max_level[K + 1]) atomicMax(&out.max_level[K + 1], tot);
+      }
+      for (int k = tid; k <= K; k += G) {
+        out.level_end[(size_t)atom * (K + 1) + k] = s_lev[k];
+        if (s_lev[k] > *(volatile int*)&out.max_level[k]) atomicMax(&out.max_level[k], s_lev[k]);
+      }
+      group_sync<G>();
+    } else {
+      for (int k = tid; k <= K; k += G) s_lev[k] = out.level_end[(size_t)atom * (K + 1) + k];
+      const long long s0 = out.site_off[atom], a0 = out.adj_base[atom];
+      group_sync<G>();
+      const int nsite = s_lev[K];
+      // sites, and the row offsets (exclusive sum of the counts of pass 0)
+      int run = 0;
+      for (int tb = 0; tb < nsite; tb += G) {
+        const int t = tb + tid;
+        int c = 0, lo = 0, hi = 0;
+        int2 sr = make_int2(0, 0);
+        if (t < nsite) {
+          const unsigned long long r = gk[t];
+          c = gc[t];
+          sr = site_row(__ldg(A.rows + rec_atom(r)), rec_addr(r));
+          tab[rec_addr(r)] = (unsigned short)(t + 1);
+          out.site_atom[s0 + t] = rec_atom(r);
+          signed char* si = out.site_img + 3 * (s0 + t);
+          si[0] = (signed char)rec_img(r, 2);
+          si[1] = (signed char)rec_img(r, 1);
+          si[2] = (signed char)rec_img(r, 0);
+          // first site of t's own level, of the one after
+          int lt = 0;
+          while (t >= s_lev[lt]) lt++;
+          lo = lt > 0 ? s_lev[lt - 1] : 0;
+          hi = s_lev[lt];
+        }
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += v;
+        }
+        int base = run;
+        if (G > 32) {
+          if (lane == 31) s_warp[tid >> 5] = incl;
+          group_sync<G>();
+          int tot = 0;
+          for (int w = 0; w < G / 32; w++) {
+            if (w == (tid >> 5)) base = run + tot;
+            tot += s_warp[w];
+          }
+          run += tot;
+          group_sync<G>();
+        } else {
+          run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (t < nsite) {
+          sinf[t] = make_int4(sr.x, sr.y, lo | (hi << 16), base + incl - c);
+          out.adj_off[s0 + t] = a0 + base + incl - c;
+        }
+      }
+      group_sync<G>();
+      int2* adj = out.adj + a0;
+      for (int t0 = 0; t0 < nsite; t0 += U * rps) {
+        int4 si[U];
+        int2 eo[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const int t = t0 + u * rps + sub;
+          si[u] = t < nsite ? sinf[t] : make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) eo[u] = j < (si[u].y >> 16) ? __ldg(A.eoff + si[u].x + j) : make_int2(-65536, 0);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const int ad = (si[u].y & 0xffff) + eo[u].x;
+          const int v = (unsigned)ad < (unsigned)A.tsize ? (int)tab[ad] : 0;  // site + 1, or not in the cluster
+          const int lo = si[u].z & 0xffff, hi = (unsigned)si[u].z >> 16;
+          // the entries of the levels l-1, l, l+1, each in row order
+          const unsigned ball = __ballot_sync(0xffffffffu, v != 0) & hm;
+          const unsigned b1 = __ballot_sync(0xffffffffu, v > lo) & hm;  // levels >= l
+          const unsigned b2 = __ballot_sync(0xffffffffu, v > hi) & hm;  // level l + 1
+          const unsigned b0 = ball & ~b1;
+          const int n0 = __popc(b0), n01 = n0 + __popc(b1 & ~b2);
+          const unsigned mine = v > hi ? b2 : (v > lo ? (b1 & ~b2) : b0);
+          const int first = v > hi ? n01 : (v > lo ? n0 : 0);
+          if (v) adj[si[u].w + first + __popc(mine & below)] = make_int2(v - 1, eo[u].y);
+          // the row's counts replace its offset
+          const int t = t0 + u * rps + sub;
+          if (j == 0 && t < nsite) sinf[t].w = n0 | (n01 << 8) | (__popc(ball) << 16);
+        }
+      }
+      group_sync<G>();
+      for (int t = tid; t < nsite; t += G) {
+        const int w = sinf[t].w, n0 = w & 255, n01 = (w >> 8) & 255, n012 = (w >> 16) & 255;
+        int lt = 0;
+        while (t >= s_lev[lt]) lt++;
+        // byte k: entries of level <= k, k < K
+        unsigned long long lc = 0;
+        for (int k = lt > 0 ? lt - 1 : 0; k < K; k++)
+          lc |= (unsigned long long)(k < lt ? n0 : (k == lt ? n01 : n012)) << (8 * k);
+        out.lvcnt[s0 + t] = lc;
+        // forward levels k = max(lt, ls + 1) .. K use the pair (t, s)
+        prod += (unsigned long long)(n0 * (K - lt + 1) + (n01 - n0) * (K - lt) + (n012 - n01) * (K > lt ? K - lt - 1 : 0));
+      }
+      group_sync<G>();
     }
-    __syncwarp();
+  }
+  if (PASS == 1) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, o);
+    if (lane == 0 && prod) atomicAdd(out.n_products, prod);
   }
 }
 
@@ -652,68 +762,132 @@ int launch_cluster(int pass, int n, int K, const long long* row_ptr, const int* 
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-// Neighbour edges packed as {col, image bytes + 128} for the warp builder.
-__global__ void k_pack_edges(long long E, const int* __restrict__ col, const signed char* __restrict__ img,
-                             int2* __restrict__ out) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (long long)gridDim.x * blockDim.x) {
-    const unsigned b = (unsigned)(img[3 * e] + 128) | ((unsigned)(img[3 * e + 1] + 128) << 8) |
-                       ((unsigned)(img[3 * e + 2] + 128) << 16);
-    out[e] = make_int2(col[e], (int)b);
+// What the grid builder needs of every directed edge i -> (j, image), one
+// warp per atom: {col, image bytes + 128}, {address offset, bond}, and each
+// atom's {first edge, degree}.
+__global__ void k_pack_edges(int n, GridPlan p, Geometry g, const long long* __restrict__ row_ptr,
+                             const int* __restrict__ col, const signed char* __restrict__ img,
+                             const int* __restrict__ bond_of_edge, const int* __restrict__ cell_of,
+                             const int* __restrict__ slot, int2* __restrict__ epack, int2* __restrict__ eoff,
+                             int2* __restrict__ rows) {
+  const int lane = threadIdx.x & 31;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= n) return;
+  const long long e0 = row_ptr[i], e1 = row_ptr[i + 1];
+  if (lane == 0) rows[i] = make_int2((int)e0, (int)(e1 - e0));
+  const int ci = cell_of[i], si = slot[i];
+  const int cx = ci / (g.nc[1] * g.nc[2]), cy = (ci / g.nc[2]) % g.nc[1], cz = ci % g.nc[2];
+  for (long long e = e0 + lane; e < e1; e += 32) {
+    const int jj = col[e], sx = img[3 * e], sy = img[3 * e + 1], sz = img[3 * e + 2];
+    const int cj = cell_of[jj];
+    const int dx = cj / (g.nc[1] * g.nc[2]) + sx * g.nc[0] - cx;
+    const int dy = (cj / g.nc[2]) % g.nc[1] + sy * g.nc[1] - cy;
+    const int dz = cj % g.nc[2] + sz * g.nc[2] - cz;
+    epack[e] = make_int2(jj, (int)(((unsigned)(sx + 128) << 16) | ((unsigned)(sy + 128) << 8) | (unsigned)(sz + 128)));
+    eoff[e] = make_int2(((dx * p.py + dy) * p.pz + dz) * p.slots + slot[jj] - si, bond_of_edge[e]);
   }
 }
 
-void launch_pack_edges(long long E, const int* col, const signed char* img, int2* out, cudaStream_t s) {
-  if (E > 0) k_pack_edges<<<(int)((E + 255) / 256 < 8192 ? (E + 255) / 256 : 8192), 256, 0, s>>>(E, col, img, out);
-}
-
-int launch_cluster_warp(int pass, int n, int K, int max_deg, const long long* row_ptr, const int2* epack,
-                        const int* bond_of_edge, PathCut pc, unsigned long long* gkeys,
-                        ClusterOut out, int* wfail, unsigned* status, cudaStream_t s) {
-  if (n == 0) return 0;
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int need = (n + CW_WARPS - 1) / CW_WARPS;
-  const int grid = need < sms * 5 ? need : sms * 5;
-  const bool cut = pc.r2 > 0.0;
-  const size_t smem = sizeof(CwSmem) * CW_WARPS;
-#define CW_LAUNCH(P, C, D)                                                                                       \
-  do {                                                                                                           \
-    cudaFuncSetAttribute(k_cluster_warp<P, C, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
-    k_cluster_warp<P, C, D><<<grid, 32 * CW_WARPS, smem, s>>>(n, K, row_ptr, epack, bond_of_edge, pc, gkeys, out,  \
-                                                              wfail, status);                                    \
-  } while (0)
-  if (max_deg <= 16) {
-    if (pass == 0) {
-      if (cut) CW_LAUNCH(0, true, 16); else CW_LAUNCH(0, false, 16);
-    } else {
-      if (cut) CW_LAUNCH(1, true, 16); else CW_LAUNCH(1, false, 16);
-    }
-  } else {
-    if (pass == 0) {
-      if (cut) CW_LAUNCH(0, true, 32); else CW_LAUNCH(0, false, 32);
-    } else {
-      if (cut) CW_LAUNCH(1, true, 32); else CW_LAUNCH(1, false, 32);
-    }
-  }
-#undef CW_LAUNCH
+int launch_pack_edges(int n, const GridPlan& p, const Geometry& g, const long long* row_ptr, const int* col,
+                      const signed char* img, const int* bond_of_edge, const int* cell_of, const int* slot,
+                      int2* epack, int2* eoff, int2* rows, cudaStream_t s) {
+  if (n <= 0) return 0;
+  k_pack_edges<<<(n + 7) / 8, 256, 0, s>>>(n, p, g, row_ptr, col, img, bond_of_edge, cell_of, slot, epack, eoff, rows);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int cluster_warp_max_sites() { return CW_MAXS; }
-
-// Largest row_ptr[i+1] - row_ptr[i] into *out (atomic max; *out starts at 0).
-__global__ void k_max_degree(int n, const long long* __restrict__ row_ptr, int* __restrict__ out) {
-  int m = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    m = max(m, (int)(row_ptr[i + 1] - row_ptr[i]));
+// Structure maxima the grid builder is planned with: out[0] the largest
+// degree, out[1] the most atoms of a linked cell, out[2..4] the largest bond
+// component along each axis in units of linked cells, rounded up to
+// 1/GRID_UNIT.  out starts at zero.
+__global__ void k_grid_maxima(int n, const long long* __restrict__ row_ptr, int ncell,
+                              const int* __restrict__ cell_start, long long nb, const double* __restrict__ bond_d,
+                              Geometry g, int* __restrict__ out) {
+  const long long q0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  int m[5] = {0, 0, 0, 0, 0};
+  for (long long i = q0; i < n; i += step) m[0] = max(m[0], (int)(row_ptr[i + 1] - row_ptr[i]));
+  for (long long i = q0; i < ncell; i += step) m[1] = max(m[1], cell_start[i + 1] - cell_start[i]);
+  for (long long b = q0; b < nb; b += step) {
+    const double x = bond_d[3 * b], y = bond_d[3 * b + 1], z = bond_d[3 * b + 2];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    for (int a = 0; a < 3; a++)
+      m[2 + a] = max(m[2 + a], (int)(fabs(x * g.inv[a] + y * g.inv[3 + a] + z * g.inv[6 + a]) * g.nc[a] * GRID_UNIT) + 1);
+  }
+#pragma unroll
+  for (int v = 0; v < 5; v++) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m[v] = max(m[v], __shfl_xor_sync(0xffffffffu, m[v], o));
+    if ((threadIdx.x & 31) == 0 && m[v] > 0) atomicMax(out + v, m[v]);
+  }
 }
 
-void launch_max_degree(int n, const long long* row_ptr, int* out, cudaStream_t s) {
-  if (n > 0) k_max_degree<<<64, 256, 0, s>>>(n, row_ptr, out);
+void launch_grid_maxima(int n, const long long* row_ptr, int ncell, const int* cell_start, long long nb,
+                        const double* bond_d, const Geometry& g, int* out, cudaStream_t s) {
+  const long long work = nb > n ? nb : n;
+  const int grid = (int)((work + 255) / 256 < 304 ? (work + 255) / 256 : 304);
+  if (n > 0) k_grid_maxima<<<grid, 256, 0, s>>>(n, row_ptr, ncell, cell_start, nb, bond_d, g, out);
+}
+
+// Cells within k hops of an atom along one axis: at most the displacement in
+// cells, plus one for the two atoms' places inside their cells (the slack
+// covers atoms up to 1e-9 of the cell outside it, and the rounding of maxima).
+static int hop_reach(int k, int unit_max) { return (int)((double)k * unit_max / GRID_UNIT + 1e-5) + 1; }
+
+bool grid_plan(const Geometry& g, int K, const int* maxima, GridPlan* p) {
+  int r[3], per[3];
+  for (int a = 0; a < 3; a++) {
+    r[a] = hop_reach(K, maxima[2 + a]);
+    per[a] = r[a] + hop_reach(K + 1, maxima[2 + a]) + 1;
+  }
+  const long long half = ((long long)r[0] * per[1] + r[1]) * per[2] + r[2];
+  p->py = per[1];
+  p->pz = per[2];
+  p->slots = maxima[1] > 0 ? maxima[1] : 1;
+  const long long size = (2 * half + 1) * p->slots;
+  if (size > 65535) return false;  // 16-bit addresses
+  p->origin = (int)half * p->slots;
+  // images of sites lie within m of the home cell
+  int* m[3] = {&p->mx, &p->my, &p->mz};
+  for (int a = 0; a < 3; a++) *m[a] = g.pbc[a] ? (r[a] + g.nc[a] - 1) / g.nc[a] : 0;
+  p->tsize = (int)size;
+  return true;
+}
+
+template <int PASS, bool CUT, int G>
+static int run_grid(const GridArgs& a, const PathCut& pc, const ClusterOut& out, int sms, cudaStream_t s) {
+  auto fn = k_cluster_grid<PASS, CUT, G>;
+  const size_t smem = (size_t)(a.tsize * 2 + 15) / 16 * 16 + 
+                      (PASS == 0 ? 16 * (size_t)a.maxs + 12 * (size_t)a.newcap : 16 * (size_t)a.sites);
+  if (smem > 225 * 1024) return -2;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, G, smem) != cudaSuccess) return -1;
+  if (per < 1) return -2;
+  const int grid = a.n < sms * per ? a.n : sms * per;
+  fn<<<grid, G, smem, s>>>(a, pc, out);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+template <int G>
+static int run_grid_pass(int pass, const GridArgs& a, const PathCut& pc, const ClusterOut& out, int sms, cudaStream_t s) {
+  const bool cut = pc.r2 > 0.0;
+  if (pass == 0) return cut ? run_grid<0, true, G>(a, pc, out, sms, s) : run_grid<0, false, G>(a, pc, out, sms, s);
+  return cut ? run_grid<1, true, G>(a, pc, out, sms, s) : run_grid<1, false, G>(a, pc, out, sms, s);
+}
+
+int launch_cluster_grid(int pass, const GridArgs& a, const PathCut& pc, const ClusterOut& out, cudaStream_t s) {
+  if (a.n == 0) return 0;
+  int sms = 0, dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // Threads per cluster: eight rows a step for many clusters (131,072 atoms of
+  // 14 neighbours: 5.7 / 5.9 / 7.5 ms with 128 / 256 / 512 threads; 1,372 atoms
+  // of 18 neighbours, 32 lanes a row: 0.23 / 0.16 / 0.16 ms), 512 where the
+  // clusters do not fill the SMs (250 atoms: 0.051 / 0.037 / 0.033 ms) or are
+  // large (17 moments, 2,000 atoms: 3.6 / 2.0 / 1.1 ms).
+  if (a.maxs <= 512 && a.n > 4 * sms)
+    return a.lpr_shift == 4 ? run_grid_pass<128>(pass, a, pc, out, sms, s) : run_grid_pass<256>(pass, a, pc, out, sms, s);
+  return run_grid_pass<512>(pass, a, pc, out, sms, s);
 }
 
 // Rows of one stored Psi sweep per atom: sum_{k=0..K} |C_k|.

@@ -45,7 +45,8 @@ struct ClusterOut {
 namespace bopk {
 // nbr.cu
 __global__ void k_bin_atoms(int n, const double* pos, Geometry g, int* cell_of, int* cell_count);
-__global__ void k_fill_cells(int n, const int* cell_of, const int* cell_start, int* cell_fill, int* cell_atoms);
+__global__ void k_fill_cells(int n, const int* cell_of, const int* cell_start, int* cell_fill, int* cell_atoms,
+                             int* cell_slot);
 __global__ void k_edge_flags(int n, const long long* row_ptr, const int* col, const signed char* img, int* flag);
 __global__ void k_bonds(int n, const long long* row_ptr, const int* col, const signed char* img, const int* flag,
                         const int* bond_scan, int* bond_of_edge, int* bond_atoms, signed char* bond_img,
@@ -71,18 +72,43 @@ int launch_cluster(int pass, int n, int K, const long long* row_ptr, const int* 
                    unsigned* status, cudaStream_t s);
 
 void launch_level_sums(int n, int K, const int* level_end, long long* out, cudaStream_t s);
-// Warp-per-atom cluster builder (cluster.cu): the same outputs as
-// launch_cluster for clusters of at most cluster_warp_max_sites() sites and
-// atoms of at most 32 neighbours; pass 0 keeps every atom's site keys in
-// gkeys [n][cluster_warp_max_sites()].  *wfail != 0 after a pass: fall back
-// to launch_cluster.
-int launch_cluster_warp(int pass, int n, int K, int max_deg, const long long* row_ptr, const int2* epack,
-                        const int* bond_of_edge, PathCut pc, unsigned long long* gkeys,
-                        ClusterOut out, int* wfail, unsigned* status, cudaStream_t s);
-// epack[e] = {col[e], image bytes + 128} of every directed neighbour edge.
-void launch_pack_edges(long long E, const int* col, const signed char* img, int2* epack, cudaStream_t s);
-int cluster_warp_max_sites();
-void launch_max_degree(int n, const long long* row_ptr, int* out, cudaStream_t s);
+// Grid builder (cluster.cu): the same outputs as launch_cluster through a
+// table of linked cells in shared memory, for rows of at most 32 neighbours.
+constexpr int GRID_UNIT = 1 << 20;
+struct GridPlan {
+  int py, pz;   // periods of the second and third axis, in cells
+  int slots;    // atoms per linked cell
+  int origin;   // address of slot 0 of the cluster's own cell
+  int tsize;    // addresses
+  int mx, my, mz;  // images of sites: [-m, m] along each axis
+};
+// Plan of a structure from its maxima (launch_grid_maxima); false: the table
+// has more than 65,535 addresses.
+bool grid_plan(const Geometry& g, int K, const int* maxima, GridPlan* p);
+void launch_grid_maxima(int n, const long long* row_ptr, int ncell, const int* cell_start, long long nb,
+                        const double* bond_d, const Geometry& g, int* out, cudaStream_t s);
+// {col, image}, {address offset, bond} of every directed edge, {first edge, degree} of every atom
+int launch_pack_edges(int n, const GridPlan& p, const Geometry& g, const long long* row_ptr, const int* col,
+                      const signed char* img, const int* bond_of_edge, const int* cell_of, const int* slot,
+                      int2* epack, int2* eoff, int2* rows, cudaStream_t s);
+struct GridArgs {
+  int n, K;                  // clusters of the first n atoms
+  int origin, tsize;         // GridPlan
+  unsigned mx, my, mz;       // likewise
+  unsigned ncode, qbits;     // images of an atom; log2(newcap): sort keys (atom, image) << qbits | entry
+  int lpr_shift;             // lanes per neighbour row: 4 (16 lanes) or 5 (32)
+  int maxs, newcap;          // sites of one cluster, new sites of one level (a power of two)
+  int sites;                 // pass 1: largest cluster (pass 0 found it)
+  const int2* rows;          // [atoms] {first edge, degree}
+  const int2* epack;         // [E] {col, image bytes + 128}
+  const int2* eoff;          // [E] {address offset, bond}
+  const int* slot;           // [atoms] place of an atom in its linked cell
+  unsigned long long* recs;  // [n][maxs] site records kept from pass 0 to pass 1
+  unsigned char* counts;     // [n][maxs] adjacency counts, likewise
+  int* fail;                 // != 0 after pass 0: a cluster exceeds maxs, newcap or the table
+  unsigned* status;
+};
+int launch_cluster_grid(int pass, const GridArgs& a, const PathCut& pc, const ClusterOut& out, cudaStream_t s);
 
 struct MomentsArgs {
   ClusterView cv;

@@ -30,12 +30,13 @@ __global__ void k_bin_atoms(int n, const double* __restrict__ pos, Geometry g, i
 }
 
 __global__ void k_fill_cells(int n, const int* __restrict__ cell_of, const int* __restrict__ cell_start,
-                             int* __restrict__ cell_fill, int* __restrict__ cell_atoms) {
+                             int* __restrict__ cell_fill, int* __restrict__ cell_atoms, int* __restrict__ cell_slot) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int c = cell_of[i];
   int slot = atomicAdd(&cell_fill[c], 1);
   cell_atoms[cell_start[c] + slot] = i;
+  cell_slot[i] = slot;
 }
 
 // Candidate ranges along one axis: with nc >= 3 the three adjacent cells
