@@ -72,7 +72,9 @@ struct bop_ctx {
   DBuf pos, cell_of, cell_count, cell_start, cell_fill, cell_atoms, cell_slot, deg, row_ptr, col, img, flag, bond_scan,
       bond_of_edge, bond_atoms, bond_img, bond_d, H64, H32, frac;
   DBuf hkeys, hvals, skeys, sslot, scount;
-  DBuf level_end, atom_nsite, atom_nadj, max_level, site_off, adj_base, site_atom, site_img, adj_off, adj, lvcnt;
+  DBuf level_end, atom_nsite, atom_nadj, max_level, site_off, adj_base, site_atom, site_img, adj_off, adj, lvcnt,
+      order, top, ntop, topmask;
+  bool pair_ok = false;  // the clusters carry the pair form of the last level
   DBuf onsite, onsite32, delta, mval, delta_new, m_new, mu, a, b, nlev, a_inf, b_inf, gsig, D, gjack;
   DBuf N, U, dos, fstate, partials, counter, result, e_total, lam, e_atom;
   DBuf w, zscr, adjscr, Hbar, Ebar, ginv;
@@ -107,6 +109,7 @@ struct bop_ctx {
   int cw_tier = 0;
   long long psi_tot = 0;
   bool psi_valid = false;
+  bool psi_pair = false;  // the stored Psi_K holds the selected rows only (MomentsArgs::pair)
   size_t store_budget = (size_t)-1;
   int resp_max_it = 0;     // cap of the SCF-response solve's iterations (0: GM_KRYLOV x GM_CYCLES)
   double resp_rtol = 0.0;  // its relative tolerance (0: the precision's default)
@@ -483,6 +486,8 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     CKS(ensure(c, c->adj_off, sizeof(long long) * (c->nsite + 1)));
     CKS(ensure(c, c->adj, sizeof(int2) * c->nadj));
     CKS(ensure(c, c->lvcnt, sizeof(unsigned long long) * c->nsite));
+    CKS(ensure(c, c->order, sizeof(unsigned) * c->nsite));
+    out.order = P<unsigned>(c->order);
     out.site_off = P<long long>(c->site_off);
     out.adj_base = P<long long>(c->adj_base);
     out.site_atom = P<int>(c->site_atom);
@@ -494,6 +499,17 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     CK(cudaMemsetAsync(c->nprod.p, 0, sizeof(unsigned long long), s));
     out.n_products = P<unsigned long long>(c->nprod);
     a.sites = c->maxlev[K];
+    // every atom a centre and no path cut: H^K between cluster atoms is
+    // symmetric, and the last level needs one side of each pair
+    c->pair_ok = c->nc == c->n && !(c->m.r_path > 0) && !c->m.noncollinear;
+    if (c->pair_ok) {
+      CKS(ensure(c, c->top, sizeof(unsigned) * c->nsite));
+      CKS(ensure(c, c->ntop, sizeof(int) * n));
+      CKS(ensure(c, c->topmask, sizeof(unsigned) * c->nsite));
+      out.top = P<unsigned>(c->top);
+      out.ntop = P<int>(c->ntop);
+      out.topmask = P<unsigned>(c->topmask);
+    }
     {
       Region R1(c, PK_CLUSTER, 1, s);
       if (launch_cluster_grid(1, a, pc, out, s)) return fail(c, BOP_ERR_CUDA, "cluster pass 1 launch failed");
@@ -510,6 +526,7 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
   const int n = c->nc, K = c->K;  // clusters of the centres
   {
     bool done = false;
+    c->pair_ok = false;
     CKS(build_clusters_grid(c, s, &done));
     if (done) return BOP_OK;
   }
@@ -583,6 +600,8 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
     CKS(ensure(c, c->adj_off, sizeof(long long) * (c->nsite + 1)));
     CKS(ensure(c, c->adj, sizeof(int2) * c->nadj));
     CKS(ensure(c, c->lvcnt, sizeof(unsigned long long) * c->nsite));
+    CKS(ensure(c, c->order, sizeof(unsigned) * c->nsite));
+    out.order = P<unsigned>(c->order);
     out.site_off = P<long long>(c->site_off);
     out.adj_base = P<long long>(c->adj_base);
     out.site_atom = P<int>(c->site_atom);
@@ -608,7 +627,9 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
 
 ClusterView cview(bop_ctx* c) {
   return ClusterView{P<long long>(c->site_off), P<int>(c->level_end), P<int>(c->site_atom),
-                     P<long long>(c->adj_off), P<int2>(c->adj), P<unsigned long long>(c->lvcnt), c->K};
+                     P<long long>(c->adj_off), P<int2>(c->adj), P<unsigned long long>(c->lvcnt), c->K,
+                     P<unsigned>(c->order), c->pair_ok ? P<unsigned>(c->top) : nullptr, P<int>(c->ntop),
+                     P<unsigned>(c->topmask)};
 }
 
 int size_state(bop_ctx* c) {
@@ -681,7 +702,10 @@ int nc_args(bop_ctx* c, NcArgs* a) {
   return BOP_OK;
 }
 
-int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s, void* pstore = nullptr) {
+// full: every row of the last level is computed (and stored), for sweeps that
+// keep the work items apart (the rows of the SCF Jacobian).
+int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s, void* pstore = nullptr,
+                bool full = false) {
   if (c->m.noncollinear) {  // the onsite levels are in c->onsite / c->onsite32
     NcArgs a;
     CKS(nc_args(c, &a));
@@ -713,6 +737,7 @@ int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s
   a.pstore = pstore;
   a.psi_off = P<long long>(c->psi_off);
   a.psi_tot = c->psi_tot;
+  a.pair = c->pair_ok && !full;
   Region R(c, PK_MOMENTS, 1, s);
   int r = launch_moments(a, c->fp64, s);
   if (r == -2) return fail(c, BOP_ERR_OVERFLOW, "cluster level too large for shared memory");
@@ -1038,8 +1063,10 @@ int prepare_psi_store(bop_ctx* c, cudaStream_t s) {
   bool fits = false;
   CKS(psi_store_alloc(c, &fits));
   if (!fits) return BOP_OK;
-  CKS(run_moments(c, P<double>(c->onsite), P<double>(c->mu), s, c->psis.p));
+  const bool full = c->m.scf != BOP_SCF_NONE && c->m.scf_response;
+  CKS(run_moments(c, P<double>(c->onsite), P<double>(c->mu), s, c->psis.p, full));
   c->psi_valid = true;
+  c->psi_pair = c->pair_ok && !full;
   return BOP_OK;
 }
 
@@ -1076,8 +1103,11 @@ int adjoint_pass(bop_ctx* c, const double* w, void* Hbar, double* Ebar, cudaStre
     aa.cap_even = ce;
     aa.cap_odd = co;
     aa.max_sites = c->maxlev[c->K] > 0 ? c->maxlev[c->K] : 1;
-    aa.max_adj = c->maxlev[c->K + 1] > 0 ? c->maxlev[c->K + 1] : 1;
     aa.cap_eb = c->maxlev[c->K - 1] > 0 ? c->maxlev[c->K - 1] : 1;
+    aa.max_adj = c->maxlev[c->K + 1] > 0 ? c->maxlev[c->K + 1] : 1;
+    if (aa.max_adj > (long long)aa.cap_eb * c->grid_max[0]) aa.max_adj = aa.cap_eb * c->grid_max[0];
+    aa.pair = c->pair_ok && siteval == nullptr;
+    if (c->psi_pair && !aa.pair) return fail(c, BOP_ERR_STATE, "the stored Psi holds the pair form only");
     aa.siteval = siteval;
     aa.sv_stride = c->nsite;
   } else {
@@ -1421,7 +1451,7 @@ int bop_destroy(bop_ctx* c) {
                   &c->row_ptr, &c->col, &c->img, &c->flag, &c->bond_scan, &c->bond_of_edge, &c->bond_atoms,
                   &c->bond_img, &c->bond_d, &c->H64, &c->H32, &c->frac, &c->hkeys, &c->hvals, &c->skeys,
                   &c->sslot, &c->scount, &c->level_end, &c->atom_nsite, &c->atom_nadj, &c->max_level,
-                  &c->site_off, &c->adj_base, &c->site_atom, &c->site_img, &c->adj_off, &c->adj, &c->lvcnt, &c->onsite,
+                  &c->site_off, &c->adj_base, &c->site_atom, &c->site_img, &c->adj_off, &c->adj, &c->lvcnt, &c->order, &c->top, &c->ntop, &c->topmask, &c->onsite,
                   &c->onsite32, &c->delta, &c->mval, &c->delta_new, &c->m_new, &c->mu, &c->a, &c->b, &c->nlev,
                   &c->a_inf, &c->b_inf, &c->gsig, &c->D, &c->gjack, &c->N, &c->U, &c->dos, &c->fstate,
                   &c->partials, &c->counter, &c->result, &c->e_total, &c->lam, &c->e_atom, &c->w, &c->zscr,
@@ -1735,16 +1765,13 @@ int bop_energy(bop_ctx* c, double* e_atom, double* delta_io, double* m_io, bop_s
   a.grad = nullptr;
   a.J = c->m.j_ii;
   // SCF residual of this iteration (for VARIATIONAL after the gradient sweep)
-  // the variational SCF sweeps back once per iteration, and the response
-  // solve of forces that are expected to follow sweeps back several times:
-  // store Psi in each forward pass when it fits (the last pass is at the
-  // final onsite levels)
+  // the variational SCF sweeps back once per iteration, and without an SCF
+  // the one forward pass serves the single reverse sweep of forces that are
+  // expected to follow: store Psi in the forward pass when it fits.  The
+  // iterations of the other SCFs take the cheaper pass that stores nothing;
+  // their response solve has Psi stored by one more pass (prepare_psi_store)
   bool var_store = false;
-  // (without an SCF the one forward pass stores Psi for the single reverse
-  // sweep of the forces, which then needs no recomputation)
-  const bool resp_store = c->forces_follow && (c->m.scf == BOP_SCF_NONE || ((c->m.scf == BOP_SCF_LCN ||
-                                                                            c->m.scf == BOP_SCF_STONER) &&
-                                                                           c->m.scf_response));
+  const bool resp_store = c->forces_follow && c->m.scf == BOP_SCF_NONE;
   if (variational || resp_store) CKS(psi_store_alloc(c, &var_store));
   c->forces_follow = false;
   auto residual = [&]() -> int {
@@ -1765,6 +1792,7 @@ int bop_energy(bop_ctx* c, double* e_atom, double* delta_io, double* m_io, bop_s
     }
     CKS(run_moments(c, P<double>(c->onsite), P<double>(c->mu), s, var_store ? c->psis.p : nullptr));
     c->psi_valid = var_store;
+    c->psi_pair = c->pair_ok;
     CKS(run_scalar(c, M, P<double>(c->mu), s));
     // warm Fermi start: later SCF iterations, and the first one of a
     // warm-started call after a previous solve

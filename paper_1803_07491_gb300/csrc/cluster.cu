@@ -276,6 +276,7 @@ k_cluster(int n, int K, const long long* __restrict__ row_ptr, const int* __rest
             lc |= (unsigned long long)cnt << (8 * k);
           }
           out.lvcnt[s0 + t] = lc;
+          out.order[s0 + t] = (unsigned)t | ((unsigned)t << 16);
           // forward levels k = max(lt, ls+1) .. K use the pair (t, s)
           int lt = 0;
           while (lt < K && t >= s_lev[lt]) lt++;
@@ -338,7 +339,8 @@ k_cluster(int n, int K, const long long* __restrict__ row_ptr, const int* __rest
 // this one 16.3 k and 17.1 k: 131,072 bcc atoms at 9 moments 19.8 -> 5.7 ms,
 // 2,000 atoms at 17 moments (one CTA per atom, hash table in global memory
 // before) 10.6 -> 1.1 ms.
-constexpr unsigned short GRID_CLAIM = 0x8000;  // claimed, index not yet assigned; else index + 1
+constexpr unsigned short GRID_CLAIM = 0x8000;  // pass 0: claimed, index not yet assigned; else index + 1
+constexpr int ORDER_KEYS = (BOP_MAX_K + 1) * 33;  // (shell, entries) of a row
 
 // site record: atom (24 bits), image bytes + 128 (24 bits), table address (16 bits)
 __device__ __forceinline__ unsigned long long grid_rec(int atom, unsigned img, int addr) {
@@ -445,9 +447,54 @@ __device__ __forceinline__ void group_sort(unsigned* a, int cnt, int tid) {
     }
 }
 
+// Stable order of the sites [0, cnt) by ascending key(t) < nkeys, by one warp:
+// put(rank, t).  off: nkeys counters.  Sites of equal key keep their order, so
+// that the result does not depend on timing.
+template <class Key, class Put>
+__device__ __forceinline__ void warp_order(int cnt, int nkeys, int* off, int lane, Key key, Put put) {
+  for (int q = lane; q < nkeys; q += 32) off[q] = 0;
+  __syncwarp();
+  for (int t = lane; t < cnt; t += 32) atomicAdd(&off[key(t)], 1);
+  __syncwarp();
+  int run = 0;
+  for (int q0 = 0; q0 < nkeys; q0 += 32) {
+    const int q = q0 + lane, c = q < nkeys ? off[q] : 0;
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (q < nkeys) off[q] = run + incl - c;
+    run += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  __syncwarp();
+  for (int t0 = 0; t0 < cnt; t0 += 32) {
+    const int t = t0 + lane;
+    const int k = t < cnt ? key(t) : nkeys;
+    const unsigned same = __match_any_sync(0xffffffffu, k);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    const int base = t < cnt ? off[k] : 0;
+    __syncwarp();
+    if (t < cnt) {
+      if (rank == 0) off[k] = base + __popc(same);
+      put(base + rank, t);
+    }
+    __syncwarp();
+  }
+}
+
 // What a row step needs of its site, in shared memory (written one thread per
 // site, read by the row's lanes): the first edge, and the address and degree.
 __device__ __forceinline__ int2 site_row(int2 row, int addr) { return make_int2(row.x, addr | (row.y << 16)); }
+
+// Bytes of the table; in pass 1 at least those of the orders that follow it
+// in its place.
+__host__ __device__ __forceinline__ size_t grid_front(int pass, const GridArgs& a) {
+  const size_t tab = (size_t)(a.tsize * 2 + 15) / 16 * 16;
+  const size_t ord = (8 * (size_t)((a.sites + 1) & ~1) + 3 * ORDER_KEYS * sizeof(int) + 15) / 16 * 16;
+  return pass == 0 || tab > ord ? tab : ord;
+}
 
 template <int PASS, bool CUT, int G>
 __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, ClusterOut out) {
@@ -457,7 +504,7 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
   __shared__ int s_warp[G / 32 + 1];
   unsigned short* tab = reinterpret_cast<unsigned short*>(grid_raw);
   const int tab16 = (A.tsize * 2 + 15) / 16;  // 16-byte words
-  unsigned char* tail = grid_raw + (size_t)tab16 * 16;
+  unsigned char* tail = grid_raw + grid_front(PASS, A);
   // pass 0: the new records of a level, their sort keys, site records, site rows
   unsigned long long* nb = reinterpret_cast<unsigned long long*>(tail);
   unsigned* keys = reinterpret_cast<unsigned*>(nb + A.newcap);
@@ -466,6 +513,9 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
   // pass 1: per site {site row, first site of its level | first site of the
   // next level, row offset}, then entries per class
   int4* sinf = reinterpret_cast<int4*>(tail);
+  // after the rows, in the table's place: the orders, and the counters of their sorts
+  unsigned short* ord = reinterpret_cast<unsigned short*>(grid_raw);  // [4][sites]
+  int* ocnt = reinterpret_cast<int*>(grid_raw + (size_t)8 * ((A.sites + 1) & ~1));  // [3][ORDER_KEYS]
   const int tid = threadIdx.x, lane = tid & 31;
   const int K = A.K;
   const int sub = tid >> A.lpr_shift, j = tid & ((1 << A.lpr_shift) - 1);  // row of the step, edge of the row
@@ -655,7 +705,8 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
           const unsigned long long r = gk[t];
           c = gc[t];
           sr = site_row(__ldg(A.rows + rec_atom(r)), rec_addr(r));
-          tab[rec_addr(r)] = (unsigned short)(t + 1);
+          const bool sel = pair_selected(atom, rec_atom(r), rec_img(r, 2), rec_img(r, 1), rec_img(r, 0));
+          tab[rec_addr(r)] = (unsigned short)((t + 1) | (sel ? GRID_CLAIM : 0));
           out.site_atom[s0 + t] = rec_atom(r);
           signed char* si = out.site_img + 3 * (s0 + t);
           si[0] = (signed char)rec_img(r, 2);
@@ -707,7 +758,8 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
 #pragma unroll
         for (int u = 0; u < U; u++) {
           const int ad = (si[u].y & 0xffff) + eo[u].x;
-          const int v = (unsigned)ad < (unsigned)A.tsize ? (int)tab[ad] : 0;  // site + 1, or not in the cluster
+          const int w = (unsigned)ad < (unsigned)A.tsize ? (int)tab[ad] : 0;
+          const int v = w & (GRID_CLAIM - 1);  // site + 1, or not in the cluster; the other bit: selected
           const int lo = si[u].z & 0xffff, hi = (unsigned)si[u].z >> 16;
           // the entries of the levels l-1, l, l+1, each in row order
           const unsigned ball = __ballot_sync(0xffffffffu, v != 0) & hm;
@@ -717,10 +769,15 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
           const int n0 = __popc(b0), n01 = n0 + __popc(b1 & ~b2);
           const unsigned mine = v > hi ? b2 : (v > lo ? (b1 & ~b2) : b0);
           const int first = v > hi ? n01 : (v > lo ? n0 : 0);
-          if (v) adj[si[u].w + first + __popc(mine & below)] = make_int2(v - 1, eo[u].y);
-          // the row's counts replace its offset
+          const int pos = first + __popc(mine & below);
+          if (v) adj[si[u].w + pos] = make_int2(v - 1, eo[u].y);
+          const unsigned selm = __reduce_or_sync(hm, v != 0 && w >= GRID_CLAIM ? 1u << pos : 0u);
+          // the row's counts replace its offset, the selected entries its first edge
           const int t = t0 + u * rps + sub;
-          if (j == 0 && t < nsite) sinf[t].w = n0 | (n01 << 8) | (__popc(ball) << 16);
+          if (j == 0 && t < nsite) {
+            sinf[t].x = (int)selm;
+            sinf[t].w = n0 | (n01 << 8) | (__popc(ball) << 16);
+          }
         }
       }
       group_sync<G>();
@@ -728,13 +785,58 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
         const int w = sinf[t].w, n0 = w & 255, n01 = (w >> 8) & 255, n012 = (w >> 16) & 255;
         int lt = 0;
         while (t >= s_lev[lt]) lt++;
+        sinf[t].y = lt;
         // byte k: entries of level <= k, k < K
         unsigned long long lc = 0;
         for (int k = lt > 0 ? lt - 1 : 0; k < K; k++)
           lc |= (unsigned long long)(k < lt ? n0 : (k == lt ? n01 : n012)) << (8 * k);
         out.lvcnt[s0 + t] = lc;
+        if (out.top != nullptr) out.topmask[s0 + t] = (unsigned)sinf[t].x;
         // forward levels k = max(lt, ls + 1) .. K use the pair (t, s)
         prod += (unsigned long long)(n0 * (K - lt + 1) + (n01 - n0) * (K - lt) + (n012 - n01) * (K > lt ? K - lt - 1 : 0));
+      }
+      group_sync<G>();
+      // the orders (one warp each)
+      const int S2 = A.sites;
+      for (int w = tid >> 5; w < 3; w += G / 32) {
+        int* off = ocnt + w * ORDER_KEYS;
+        if (w < 2) {  // by shell, then descending entries of the level below / up to its own
+          const int sh = 8 * w;
+          warp_order(nsite, (K + 1) * 33, off, lane,
+                     [&](int t) { return sinf[t].y * 33 + 32 - ((sinf[t].w >> sh) & 255); },
+                     [&](int q, int t) { ord[w * S2 + q] = (unsigned short)t; });
+        } else if (out.top != nullptr) {  // C_K-1 by descending selected entries
+          warp_order(s_lev[K - 1], 33, off, lane, [&](int t) { return 32 - __popc((unsigned)sinf[t].x); },
+                     [&](int q, int t) { ord[3 * S2 + q] = (unsigned short)t; });
+        }
+      }
+      group_sync<G>();
+      for (int q = tid; q < nsite; q += G) out.order[s0 + q] = (unsigned)ord[q] | ((unsigned)ord[S2 + q] << 16);
+      if (out.top != nullptr) {
+        if (tid < 32) {  // the selected sites in the order of the last level's rows
+          int run = 0;
+          const int l2 = K >= 2 ? s_lev[K - 2] : 0, l1 = s_lev[K - 1];
+          for (int q0 = 0; q0 < nsite; q0 += 32) {
+            const int q = q0 + lane;
+            const int t = q < nsite ? (q < l2 ? q : (q < l1 ? ord[S2 + q] : ord[q])) : 0;
+            bool sel = false;
+            if (q < nsite) {
+              const unsigned long long r = gk[t];
+              sel = pair_selected(atom, rec_atom(r), rec_img(r, 2), rec_img(r, 1), rec_img(r, 0));
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, sel);
+            if (sel) ord[2 * S2 + run + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)t;
+            run += __popc(bal);
+          }
+          if (lane == 0) {
+            s_cnt = run;
+            out.ntop[atom] = run;
+          }
+        }
+        group_sync<G>();
+        const int nt = s_cnt, nr = s_lev[K - 1];
+        for (int q = tid; q < nsite; q += G)
+          out.top[s0 + q] = (q < nt ? (unsigned)ord[2 * S2 + q] : 0u) | ((q < nr ? (unsigned)ord[3 * S2 + q] : 0u) << 16);
       }
       group_sync<G>();
     }
@@ -856,7 +958,7 @@ bool grid_plan(const Geometry& g, int K, const int* maxima, GridPlan* p) {
 template <int PASS, bool CUT, int G>
 static int run_grid(const GridArgs& a, const PathCut& pc, const ClusterOut& out, int sms, cudaStream_t s) {
   auto fn = k_cluster_grid<PASS, CUT, G>;
-  const size_t smem = (size_t)(a.tsize * 2 + 15) / 16 * 16 + 
+  const size_t smem = grid_front(PASS, a) + 
                       (PASS == 0 ? 16 * (size_t)a.maxs + 12 * (size_t)a.newcap : 16 * (size_t)a.sites);
   if (smem > 225 * 1024) return -2;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;

@@ -35,7 +35,30 @@ struct ClusterView {
   const int2* adj;            // {neighbour site (local index), bond}, ascending site
   const unsigned long long* lvcnt;  // [S] byte k = entries with site < level_end[k]
   int K;
+  // Orders of the sites of a cluster by the work of their rows, so that the
+  // rows of a warp are about equally long: within each shell (the sites first
+  // reached at one level) by descending entries, low half: entries of the
+  // level below (the row's work at its own level), high half: entries of the
+  // levels up to its own (its work one level on)
+  const unsigned* order;      // [S]
+  // Pair form of the last level (NULL without it; see pair_selected): low
+  // half: the selected sites by descending row length, ntop of them; high
+  // half: the sites of C_K-1 by descending selected entries
+  const unsigned* top;        // [S]
+  const int* ntop;            // [n]
+  const unsigned* topmask;    // [S] bit e: entry e of the row is a selected site
 };
+
+// Psi_K(t, i) of the pair (centre i, site t = atom j in image s) equals
+// Psi_K(i, t)^T of the pair (centre j, site i in image -s): H^K is symmetric.
+// Each unordered pair is computed from one side only: by the order of the
+// atoms, reversed where their sum is odd (about half of every cluster's pairs
+// whatever the numbering), by the image for two images of one atom.  The
+// centre itself is selected.
+__device__ __forceinline__ bool pair_selected(int i, int j, int sx, int sy, int sz) {
+  if (i != j) return (i < j) != (((i + j) & 1) != 0);
+  return sx > 0 || (sx == 0 && (sy > 0 || (sy == 0 && sz >= 0)));
+}
 
 // ---------------------------------------------------------------- duals
 // Value plus its gradient with respect to the three bond-vector components,

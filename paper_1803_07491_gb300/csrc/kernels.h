@@ -40,6 +40,10 @@ struct ClusterOut {
   int2* adj;             // [A]
   unsigned long long* n_products;  // block products of one moments pass (pass 2)
   unsigned long long* lvcnt;       // [S] per-level entry counts (pass 2)
+  unsigned* order;                 // [S] ClusterView (pass 2)
+  unsigned* top;                   // [S], [n], [S]: the pair form of the last level, may be null (pass 2)
+  int* ntop;
+  unsigned* topmask;
 };
 
 namespace bopk {
@@ -128,6 +132,9 @@ struct MomentsArgs {
   void* pstore;
   const long long* psi_off;  // [n+1] prefix sums of sum_k |C_k| over atoms
   long long psi_tot;
+  // last level in the pair form (needs cv.top; every atom a centre): stores,
+  // then, the selected rows of Psi_K only
+  bool pair;
 };
 int launch_moments(const MomentsArgs& a, int fp64, cudaStream_t s);
 
@@ -151,12 +158,13 @@ struct AdjointArgs {
   long long psi_tot;
   int nc;              // columns per work item used by the forward pass that stored Psi
   int cap_even, cap_odd;  // largest even / odd level |C_k|, k = 1..K
-  int max_sites, max_adj, cap_eb;  // cap_eb: largest |C_K-1|
+  int max_sites, max_adj, cap_eb;  // cap_eb: largest |C_K-1|; max_adj: entries of its rows
   // stored-Psi sweep only: per cluster site t of work item (spin, atom i),
   // sum over the orbitals of dL/dE_t (+=), at siteval[spin * sv_stride +
   // site_off[i] + t] (t < |C_K-1|); may be null
   double* siteval;
   long long sv_stride;
+  bool pair;           // stored-Psi sweep, no siteval: last level in the pair form (MomentsArgs::pair)
 };
 int launch_moments_adjoint(const AdjointArgs& a, int fp64, cudaStream_t s);
 // Elements per bond of the cotangent array Hbar: the unique block elements

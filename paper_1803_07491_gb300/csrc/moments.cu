@@ -181,19 +181,25 @@ __device__ __forceinline__ void ext_adj(const ClusterView& cv, ItemExt& x) {
 }
 
 // One work item's cluster data in shared memory: the adjacency entries of its
-// sites, their adjacency offsets (absolute, as in the cluster arrays), level
-// counts and atoms.
-__device__ __forceinline__ void stage_item(const ClusterView& cv, const ItemExt& x, int2* s_adj, long long* s_aoff,
-                                           unsigned long long* s_lvc, int* s_atom, int tid, int nthr) {
+// first nrow sites, their adjacency offsets (from the item's first entry) and
+// level counts, and the atoms of all its sites.
+__device__ __forceinline__ void stage_item(const ClusterView& cv, const ItemExt& x, int nrow, int nadj, int2* s_adj,
+                                           int* s_off, unsigned long long* s_lvc, int* s_atom, int tid, int nthr) {
   const long long s0 = x.s0, abase = x.abase;
-  const int nsite = x.nsite, nadj = (int)(x.aend - x.abase);
   for (int q = tid; q < nadj; q += nthr) cp_async8(s_adj + q, cv.adj + abase + q);
-  for (int q = tid; q <= nsite; q += nthr) cp_async8(s_aoff + q, cv.adj_off + s0 + q);
-  for (int q = tid; q < nsite; q += nthr) {
-    cp_async8(s_lvc + q, cv.lvcnt + s0 + q);
-    cp_async4(s_atom + q, cv.site_atom + s0 + q);
-  }
+  for (int q = tid; q < nrow; q += nthr) cp_async8(s_lvc + q, cv.lvcnt + s0 + q);
+  for (int q = tid; q < x.nsite; q += nthr) cp_async4(s_atom + q, cv.site_atom + s0 + q);
+  for (int q = tid; q <= nrow; q += nthr) s_off[q] = (int)(cv.adj_off[s0 + q] - abase);
   cp_async_wait_all();
+}
+
+// Its row orders, likewise (before stage_item, whose wait covers these copies).
+__device__ __forceinline__ void stage_order(const ClusterView& cv, const ItemExt& x, bool pair, unsigned* s_ord,
+                                            unsigned* s_top, int tid, int nthr) {
+  for (int q = tid; q < x.nsite; q += nthr) {
+    cp_async4(s_ord + q, cv.order + x.s0 + q);
+    if (pair) cp_async4(s_top + q, cv.top + x.s0 + q);
+  }
 }
 
 template <typename T>
@@ -374,64 +380,156 @@ __device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int cnt
   }
 }
 
-// The reverse sweep's gather with the bond cotangents of the same pairs:
-// for each entry s of row t (t in C_{k-1}, s in C_k), acc += B_ts x[s]
-// (when gather is set) and dL/dB of the forward pair (s, t), x[s] pt^T
-// summed over the columns (x = Psi-bar_k, pt = Psi_k-1(t)), goes to the
-// bond's unique elements; the blocks of the next two entries are in flight.
-template <typename T, int NO, int NC, int PS>
-__device__ __forceinline__ void gather_cot(const int2* __restrict__ ent, int cnt, const T* __restrict__ H, int HS,
-                                           const T* __restrict__ x, T acc[NO][NC], bool gather, const T pt[NO * NC],
-                                           T* __restrict__ Hbar, int HSh) {
+// Adds one bond record of cotangents per lane (v: NO x NO unique elements,
+// padded) to the bonds' cotangent records; bond < 0: none.  All lanes of the
+// warp call it.  FP32: four lanes add one record together, 16 bytes each, so
+// that a reduction instruction touches 8 records instead of 32 (the four
+// quarters are exchanged between the lanes by 12 shuffles; reductions of
+// scattered records cost the L1 unit one cycle per line).
+template <typename T, int NO>
+__device__ __forceinline__ void add_bond_records(T* __restrict__ Hbar, int HSh, int bond, const T G[NO][NO], int lane) {
+  if constexpr (NO == 1 || sizeof(T) == 8) {
+    if (bond >= 0) add_bond_cotangent<T, NO>(Hbar + (size_t)bond * HSh, G);
+  } else {
+    constexpr int HV = hbar_stride<T, NO>();
+    float v[HV];
+#pragma unroll
+    for (int q = 0; q < HV; q++) v[q] = 0.f;
+#pragma unroll
+    for (int b = 0; b < NO; b++)
+#pragma unroll
+      for (int g = b; g < NO; g++) v[UI<NO>(b, g)] = G[b][g] + (b != g ? G[g][b] : 0.f);
+    const int q = lane & 3;
+#pragma unroll
+    for (int d = 0; d < 4; d++) {
+      // quarter q ^ d of this lane's record goes to lane q ^ d, whose quarter q comes here
+      const int o = q ^ d;
+      float4 x;
+      x.x = (o & 2) ? ((o & 1) ? v[12] : v[8]) : ((o & 1) ? v[4] : v[0]);
+      x.y = (o & 2) ? ((o & 1) ? v[13] : v[9]) : ((o & 1) ? v[5] : v[1]);
+      x.z = (o & 2) ? ((o & 1) ? v[14] : v[10]) : ((o & 1) ? v[6] : v[2]);
+      x.w = (o & 2) ? ((o & 1) ? v[15] : v[11]) : ((o & 1) ? v[7] : v[3]);
+      int bd = bond;
+      if (d > 0) {
+        x.x = __shfl_xor_sync(0xffffffffu, x.x, d);
+        x.y = __shfl_xor_sync(0xffffffffu, x.y, d);
+        x.z = __shfl_xor_sync(0xffffffffu, x.z, d);
+        x.w = __shfl_xor_sync(0xffffffffu, x.w, d);
+        bd = __shfl_xor_sync(0xffffffffu, bond, d);
+      }
+      if (bd >= 0) atomicAdd(reinterpret_cast<float4*>(Hbar + (size_t)bd * HSh) + q, x);
+    }
+    if (bond >= 0) {
+      float4* dst = reinterpret_cast<float4*>(Hbar + (size_t)bond * HSh);
+#pragma unroll
+      for (int w = 4; w < HV / 4; w++)
+        atomicAdd(dst + w, make_float4(v[4 * w], v[4 * w + 1], v[4 * w + 2], v[4 * w + 3]));
+    }
+  }
+}
+
+// The reverse sweep's gather of one row by one lane: acc += B_ts x[s] over
+// the entries first, first + step, ... of the row (or those of the bits of
+// mask), with the blocks of two entries in flight.  HBAR: also the bond
+// cotangents dL/dB = x[s] pt^T of the forward pairs (s, t), summed over the
+// columns (x = Psi-bar_k, pt = Psi_k-1(t)); with gather false (level 1) only
+// those.  All lanes of a warp call it (rows of no entries: cnt 0).
+template <typename T, int NO, int NC, int PS, bool HBAR>
+__device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int first, int step, int cnt, unsigned mask,
+                                           bool use_mask, const T* __restrict__ H, int HS, const T* __restrict__ x,
+                                           T acc[NO][NC], bool gather, const T pt[NO * NC], T* __restrict__ Hbar,
+                                           int HSh, int lane) {
   constexpr int HB = hb_count<NO>();
   constexpr int N = NO * NC;
-  if (cnt <= 0) return;
-  int2 e0 = ent[0];
-  int2 e1 = cnt > 1 ? ent[1] : e0;
+  const int mine = use_mask ? __popc(mask) : (cnt > first ? (cnt - first + step - 1) / step : 0);
+  const int rounds = HBAR ? __reduce_max_sync(0xffffffffu, mine) : mine;
+  int e = first;
+  auto next = [&]() -> int2 {  // the row's next entry
+    int i = e;
+    if (use_mask) {
+      i = __ffs(mask) - 1;
+      mask &= mask - 1;
+    }
+    e += step;
+    return ent[i];
+  };
+  int2 e0 = make_int2(0, -1), e1 = make_int2(0, -1);
   T h0[HB], h1[HB];
-  if (gather) {
-    load_bond<T, NO>(H + (size_t)e0.y * HS, h0);
-    if (cnt > 1) load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
+  if (mine > 0) {
+    e0 = next();
+    if (gather) load_bond<T, NO>(H + (size_t)e0.y * HS, h0);
   }
-  for (int e = 0; e < cnt; e++) {
-    const int sidx = e0.x, bond = e0.y;
+  if (mine > 1) {
+    e1 = next();
+    if (gather) load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
+  }
+  for (int it = 0; it < rounds; it++) {
+    const bool on = it < mine;
+    const int sidx = e0.x, bond = on ? e0.y : -1;
     T hc[HB];
 #pragma unroll
     for (int q = 0; q < HB; q++) hc[q] = h0[q];
     e0 = e1;
 #pragma unroll
     for (int q = 0; q < HB; q++) h0[q] = h1[q];
-    if (e + 2 < cnt) {
-      e1 = ent[e + 2];
+    if (it + 2 < mine) {
+      e1 = next();
       if (gather) load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
     }
-    T xs[N];
-    load_row<T, N, PS>(x + (size_t)sidx * PS, xs);
-    if (gather) block_fma<T, NO, NC>(hc, xs, acc);
     T G[NO][NO];
+    if (on) {
+      T xs[N];
+      load_row<T, N, PS>(x + (size_t)sidx * PS, xs);
+      if (gather) block_fma<T, NO, NC>(hc, xs, acc);
+      if constexpr (HBAR) {
 #pragma unroll
-    for (int b = 0; b < NO; b++)
+        for (int b = 0; b < NO; b++)
 #pragma unroll
-      for (int g = 0; g < NO; g++) {
-        T a = T(0);
+          for (int g = 0; g < NO; g++) {
+            T a = T(0);
 #pragma unroll
-        for (int c = 0; c < NC; c++) a += xs[b * NC + c] * pt[g * NC + c];
-        G[b][g] = a;
+            for (int c = 0; c < NC; c++) a += xs[b * NC + c] * pt[g * NC + c];
+            G[b][g] = a;
+          }
       }
-    add_bond_cotangent<T, NO>(Hbar + (size_t)bond * HSh, G);
+    } else if constexpr (HBAR) {
+#pragma unroll
+      for (int b = 0; b < NO; b++)
+#pragma unroll
+        for (int g = 0; g < NO; g++) G[b][g] = T(0);
+    }
+    if constexpr (HBAR) add_bond_records<T, NO>(Hbar, HSh, bond, G, lane);
   }
 }
 
 // Forward kernel.  A persistent CTA takes a run of consecutive work items
 // (spin, atom[, alpha]); neighbouring atoms share most of their clusters'
 // blocks, which then come from L1.  For each item the atom's adjacency,
-// per-site offsets, level counts and site atoms are staged in shared memory
-// (one coalesced copy) when they fit, so that the edge loop only waits for
-// the bond blocks, which are fetched one edge ahead.  Each thread computes
-// all NC columns of one site (NO x NO x NC multiply-adds per edge); Psi
-// rows are padded to 16-byte multiples and kept in two exactly sized
+// per-site offsets, level counts, site atoms and row orders are staged in
+// shared memory (one coalesced copy) when they fit, so that the edge loop only
+// waits for the bond blocks, which are fetched one edge ahead.  Each thread
+// computes all NC columns of one site (NO x NO x NC multiply-adds per edge);
+// Psi rows are padded to 16-byte multiples and kept in two exactly sized
 // buffers (even and odd levels).
-constexpr int FWD_THREADS = 192;
+//
+// Rows run in the order of their length (ClusterView::order): the 1 to 6
+// entries of an outer shell's row and the 14 of an inner one no longer share a
+// warp, whose other lanes would idle for the longest row; odd passes over the
+// threads run backwards, so that the warp with the longest rows of one pass
+// gets the shortest of the next.
+//
+// pair: the last level (68 % of the products of a bcc cluster at 9 moments)
+// computes the selected sites only (pair_selected).  H^K is symmetric, so the
+// block Z = Psi_K(t, i) holds Psi_K(i, t)^T too: its column sums go to this
+// item's last two moments and its row sums to those of the site's atom, all
+// with FP64 atomics onto moments that start at zero.
+template <typename T>
+struct Fwd {
+  // FP64: one DFMA of a warp takes 64 cycles of an SM sub-partition, so that
+  // one warp on each keeps it busy and the CTAs of four warps balance best
+  static constexpr int THREADS = sizeof(T) == 4 ? 192 : 128;
+  static constexpr int MIN_CTAS = 2;
+};
 
 struct FwdSmem {
   int cap_even, cap_odd, max_sites, max_adj;
@@ -439,13 +537,13 @@ struct FwdSmem {
 };
 
 template <typename T, int NO, int NC>
-__global__ void __launch_bounds__(FWD_THREADS, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
 k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
           int n_mom, FwdSmem L, int n_items, int chunk, double* __restrict__ mu, T* __restrict__ pstore,
-          const long long* __restrict__ psi_off, long long psi_tot) {
+          const long long* __restrict__ psi_off, long long psi_tot, bool pair) {
+  constexpr int NT = Fwd<T>::THREADS;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
-  constexpr int HB = hb_count<NO>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf[2];
   buf[0] = reinterpret_cast<T*>(smem_raw);
@@ -453,12 +551,14 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
   unsigned char* tail = align16(reinterpret_cast<unsigned char*>(buf[1] + (size_t)L.cap_odd * PS));
   int2* s_adj = reinterpret_cast<int2*>(tail);
   unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
-  long long* s_aoff = reinterpret_cast<long long*>(s_lvc + (L.stage ? L.max_sites : 0));
-  int* s_atom = reinterpret_cast<int*>(s_aoff + (L.stage ? L.max_sites + 1 : 0));
+  int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.max_sites : 0));
+  int* s_atom = s_off + (L.stage ? L.max_sites + 1 : 0);
+  unsigned* s_ord = reinterpret_cast<unsigned*>(s_atom + (L.stage ? L.max_sites : 0));
+  unsigned* s_top = s_ord + (L.stage ? L.max_sites : 0);
   // per-warp partial sums of the two moments of a level, in two buffers
   // (level parity): the reads of level k's partials need no barrier before
   // level k + 1 starts writing its own
-  __shared__ T red[2][2 * NC][FWD_THREADS / 32];
+  __shared__ T red[2][2 * NC][NT / 32];
   const int K = cv.K;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int w0 = blockIdx.x * chunk, w1 = min(n_items, w0 + chunk);
@@ -476,12 +576,18 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     const int* lev = cv.level_end + (size_t)atom * (K + 1);
     const int2* adj = cv.adj + abase;
     const unsigned long long* lvc = cv.lvcnt + s0;
-    const int* satom = cv.site_atom + s0;
+    const int* satom = L.stage ? s_atom : cv.site_atom + s0;
+    const unsigned* order = L.stage ? s_ord : cv.order + s0;
+    const unsigned* top = L.stage ? s_top : cv.top + s0;
     const T* E = onsite + (size_t)spin * n_on * NO;
-    if (L.stage) stage_item(cv, cur, s_adj, s_aoff, s_lvc, s_atom, tid, FWD_THREADS);
+    if (L.stage) {
+      stage_order(cv, cur, pair, s_ord, s_top, tid, NT);
+      stage_item(cv, cur, cur.nsite, (int)(cur.aend - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
+    }
+    const int ntop = pair ? cv.ntop[atom] : 0;
     const bool more = w + 1 < w1;
     if (more) ext_sites(cv, ((NC == NO) ? w + 1 : ((w + 1) / NO)) % n, nx);
-    for (int q = tid; q < N; q += FWD_THREADS) {
+    for (int q = tid; q < N; q += NT) {
       const int r = q / NC, c = q % NC;
       buf[0][q] = (NC == NO) ? T(r == c ? 1 : 0) : T(r == grp ? 1 : 0);
     }
@@ -489,7 +595,7 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     T* pitem = nullptr;
     if (pstore != nullptr) {
       pitem = pstore + ((size_t)(spin * (NO / NC) + grp) * psi_tot + psi_off[atom]) * PS;
-      for (int q = tid; q < PS; q += FWD_THREADS) {
+      for (int q = tid; q < PS; q += NT) {
         const int r = q / NC, c = q % NC;
         pitem[q] = q < N ? ((NC == NO) ? T(r == c ? 1 : 0) : T(r == grp ? 1 : 0)) : T(0);
       }
@@ -500,64 +606,77 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     if (tid < NC) out[(size_t)tid * n_mom] = 1.0;
     for (int k = 1; k <= K; k++) {
       lo_k += lev[k - 1];
-      const int nrow = lev[k], ncol = lev[k - 1];
+      const bool half = pair && k == K;
+      const int ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
+      const int nrow = half ? ntop : lev[k];
       const T* prev = buf[(k - 1) & 1];
-      T* cur = buf[k & 1];
+      T* next = buf[k & 1];
       T d1[NC], d2[NC];
 #pragma unroll
       for (int c = 0; c < NC; c++) d1[c] = d2[c] = T(0);
-      for (int t = tid; t < nrow; t += FWD_THREADS) {
+      for (int p = 0; p * NT < nrow; p++) {
+        const int r = p * NT + ((p & 1) ? NT - 1 - tid : tid);
+        if (r >= nrow) continue;
+        // rows up to level k-2 are full, shell k-1 has entries up to its own
+        // level, shell k of the one below
+        const int t = half ? (int)(top[r] & 0xffffu)
+                           : (r < inner ? r : (r < ncol ? (int)(order[r] >> 16) : (int)(order[r] & 0xffffu)));
         T acc[NO][NC];
         const bool in_prev = t < ncol;
+        const int atom_t = satom[t];
         if (in_prev) {
           T pt[N];
           load_row<T, N, PS>(prev + (size_t)t * PS, pt);
-          const T* e = E + (size_t)(L.stage ? s_atom[t] : satom[t]) * NO;
+          const T* e = E + (size_t)atom_t * NO;
 #pragma unroll
-          for (int r = 0; r < NO; r++) {
-            const T er = e[r];
+          for (int r_ = 0; r_ < NO; r_++) {
+            const T er = e[r_];
 #pragma unroll
-            for (int c = 0; c < NC; c++) acc[r][c] = er * pt[r * NC + c];
+            for (int c = 0; c < NC; c++) acc[r_][c] = er * pt[r_ * NC + c];
           }
         } else {
 #pragma unroll
-          for (int r = 0; r < NO; r++)
+          for (int r_ = 0; r_ < NO; r_++)
 #pragma unroll
-            for (int c = 0; c < NC; c++) acc[r][c] = T(0);
+            for (int c = 0; c < NC; c++) acc[r_][c] = T(0);
         }
         const unsigned long long lc = L.stage ? s_lvc[t] : lvc[t];
         const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
         if (cnt > 0) {
-          const int q0 = (int)((L.stage ? s_aoff[t] : cv.adj_off[s0 + t]) - abase);
+          const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
           gather_pf2<T, NO, NC, PS>(L.stage ? s_adj + q0 : adj + q0, cnt, H, HS, prev, acc);
         }
-        if (in_prev) {  // row t of Psi_k-1 again (shared memory), rather than kept live over the gather
+        // row t of Psi_k-1 again (shared memory), rather than kept live over the gather
+        const bool other = half && t != 0;
+        double* mt = mu + ((size_t)spin * n + atom_t) * NO * n_mom + 2 * K - 1;  // the last two moments of atom_t
+        if (in_prev) {
           T pt[N];
           load_row<T, N, PS>(prev + (size_t)t * PS, pt);
 #pragma unroll
-          for (int r = 0; r < NO; r++)
+          for (int r_ = 0; r_ < NO; r_++) {
+            T a = T(0);
 #pragma unroll
-            for (int c = 0; c < NC; c++) d1[c] += pt[r * NC + c] * acc[r][c];
+            for (int c = 0; c < NC; c++) {
+              const T v = pt[r_ * NC + c] * acc[r_][c];
+              d1[c] += v;
+              a += v;
+            }
+            if (other) atomicAdd(mt + r_ * n_mom, (double)a);
+          }
         }
 #pragma unroll
-        for (int r = 0; r < NO; r++)
+        for (int r_ = 0; r_ < NO; r_++) {
+          T a = T(0);
 #pragma unroll
-          for (int c = 0; c < NC; c++) d2[c] += acc[r][c] * acc[r][c];
-        if (k < K) {
-          T* dst = cur + (size_t)t * PS;
-#pragma unroll
-          for (int r = 0; r < NO; r++)
-#pragma unroll
-            for (int c = 0; c < NC; c++) dst[r * NC + c] = acc[r][c];
+          for (int c = 0; c < NC; c++) {
+            const T v = acc[r_][c] * acc[r_][c];
+            d2[c] += v;
+            a += v;
+          }
+          if (other) atomicAdd(mt + r_ * n_mom + 1, (double)a);
         }
-        if (pitem != nullptr) {
-          T row[N];
-#pragma unroll
-          for (int r = 0; r < NO; r++)
-#pragma unroll
-            for (int c = 0; c < NC; c++) row[r * NC + c] = acc[r][c];
-          store_row<T, N, PS>(pitem + (size_t)(lo_k + t) * PS, row);
-        }
+        if (k < K) store_row<T, N, PS>(next + (size_t)t * PS, &acc[0][0]);
+        if (pitem != nullptr) store_row<T, N, PS>(pitem + (size_t)(lo_k + t) * PS, &acc[0][0]);
       }
 #pragma unroll
       for (int c = 0; c < NC; c++) {
@@ -572,10 +691,11 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
       __syncthreads();
       if (tid < 2 * NC) {
         T acc = T(0);
-        for (int q = 0; q < FWD_THREADS / 32; q++) acc += red[k & 1][tid][q];
+        for (int q = 0; q < NT / 32; q++) acc += red[k & 1][tid][q];
         const int c = tid % NC;
-        const int m = tid < NC ? 2 * k - 1 : 2 * k;
-        out[(size_t)c * n_mom + m] = (double)acc;
+        double* m = out + (size_t)c * n_mom + (tid < NC ? 2 * k - 1 : 2 * k);
+        if (half) atomicAdd(m, (double)acc);
+        else *m = (double)acc;
       }
     }
     if (more) ext_adj(cv, nx);
@@ -590,14 +710,24 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
 //   Psi-bar_k-1   = H Psi-bar_k (rows < |C_k-1|, columns < |C_k|)
 //                   + 2 w_2k-2 Psi_k-1 + w_2k-1 Psi_k + w_2k-3 Psi_k-2
 // runs like the forward kernel: Psi-bar_k and Psi-bar_k-1 in two shared
-// buffers (even / odd levels), the adjacency staged, one site row per
-// thread.  The onsite cotangents dL/dE_t = sum_k Psi-bar_k[t] . Psi_k-1[t]
-// are accumulated per site in shared memory and added once per item.
-// With HBAR the gather of level k also forms the bond cotangents of its
-// pairs, Psi-bar_k(s) Psi_k-1(t)^T for the forward pair (s in C_k, t in
-// C_{k-1}) (Psi-bar_k(s) is the gather's operand, Psi_k-1(t) one stored row
-// per site), and adds them to the bond's unique elements (gather_cot); at
-// k = 1 only these products run.
+// buffers (even / odd levels), the adjacency of the rows (C_K-1) staged.  The
+// onsite cotangents dL/dE_t = sum_k Psi-bar_k[t] . Psi_k-1[t] are accumulated
+// per site in shared memory and added once per item.  With HBAR the gather of
+// level k also forms the bond cotangents of its pairs, Psi-bar_k(s)
+// Psi_k-1(t)^T for the forward pair (s in C_k, t in C_k-1), and adds them to
+// the bond's unique elements; at k = 1 only these products run.
+//
+// A level of fewer rows than threads gives each row 2 to 16 adjacent lanes
+// that share its entries and add their sums by shuffles (65 rows of 14 entries
+// at level 3 of a bcc cluster, 15 at level 2): the levels' longest chains fall
+// from 14 entries to 7 and 2.
+//
+// pair: the last level in the pair form of the forward kernel.  Z =
+// Psi_K(t, i) enters the moments of the centre i by its columns and those of
+// the site's atom j by its rows, so that its cotangent is 2 (w_i + w_j) Z
+// + (w_i + w_j)' Psi_K-1(t) with column weights w_i and row weights w_j; the
+// gather of level K runs over the selected entries of every row
+// (ClusterView::topmask), rows in the order of their number.
 struct RevSmem {
   int cap_even, cap_odd, max_sites, max_adj, cap_eb;
   bool stage;
@@ -608,17 +738,18 @@ __host__ __device__ constexpr size_t eb_elems(int cap_eb) {
   return ((size_t)cap_eb * NO * sizeof(T) + 15) / 16 * 16 / sizeof(T);
 }
 
+constexpr int REV_SEL_WORDS = 256;  // selected sites as bits (a cluster with a pair form has at most 8,192 sites)
+
 template <typename T, int NO, int NC, bool HBAR>
-__global__ void __launch_bounds__(FWD_THREADS, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
 k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
-          int n_mom,
-          RevSmem L, int n_items, int chunk, const T* __restrict__ pstore,
+          int n_mom, RevSmem L, int n_items, int chunk, const T* __restrict__ pstore,
           const long long* __restrict__ psi_off, long long psi_tot, const double* __restrict__ wts,
           T* __restrict__ Hbar, int HSh, double* __restrict__ Ebar, double* __restrict__ siteval,
-          long long sv_stride) {
+          long long sv_stride, bool pair) {
+  constexpr int NT = Fwd<T>::THREADS;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
-  constexpr int HB = hb_count<NO>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf[2];
   buf[0] = reinterpret_cast<T*>(smem_raw);
@@ -627,13 +758,14 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
   unsigned char* tail = align16(reinterpret_cast<unsigned char*>(eb + eb_elems<T, NO>(L.cap_eb)));
   int2* s_adj = reinterpret_cast<int2*>(tail);
   unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
-  long long* s_aoff = reinterpret_cast<long long*>(s_lvc + (L.stage ? L.max_sites : 0));
-  int* s_atom = reinterpret_cast<int*>(s_aoff + (L.stage ? L.max_sites + 1 : 0));
+  int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.cap_eb : 0));
+  int* s_atom = s_off + (L.stage ? L.cap_eb + 1 : 0);
   __shared__ T ws[NC][BOP_MAX_NMOM];
   __shared__ int s_lev[BOP_MAX_K + 1];
   __shared__ long long s_lo[BOP_MAX_K + 1];
+  __shared__ unsigned s_sel[REV_SEL_WORDS];
   const int K = cv.K;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int w0 = blockIdx.x * chunk, w1 = min(n_items, w0 + chunk);
   ItemExt nx{};
   if (w0 < w1) {
@@ -647,13 +779,17 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     const ItemExt cur = nx;
     const long long s0 = cur.s0, abase = cur.abase;
     const int* lev = cv.level_end + (size_t)atom * (K + 1);
-    const int2* adj = cv.adj + abase;
-    const unsigned long long* lvc = cv.lvcnt + s0;
-    const int* satom = cv.site_atom + s0;
+    const unsigned long long* lvc = L.stage ? s_lvc : cv.lvcnt + s0;
+    const int* satom = L.stage ? s_atom : cv.site_atom + s0;
+    const unsigned* top = cv.top + s0;
     const T* E = onsite + (size_t)spin * n_on * NO;
     const size_t ib = ((size_t)(spin * (NO / NC) + grp) * psi_tot + psi_off[atom]) * PS;
     const T* P = pstore + ib;
-    if (L.stage) stage_item(cv, cur, s_adj, s_aoff, s_lvc, s_atom, tid, FWD_THREADS);
+    if (L.stage) {
+      const int nr = lev[K - 1];
+      stage_item(cv, cur, nr, (int)(cv.adj_off[s0 + nr] - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
+    }
+    const int2* adj = L.stage ? s_adj : cv.adj + abase;
     const bool more = w + 1 < w1;
     if (more) ext_sites(cv, ((NC == NO) ? w + 1 : ((w + 1) / NO)) % n, nx);
     if (tid <= K) s_lev[tid] = lev[tid];
@@ -664,48 +800,86 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
         o += lev[k];
       }
     }
-    for (int q = tid; q < NC * n_mom; q += FWD_THREADS) {
+    for (int q = tid; q < NC * n_mom; q += NT) {
       const int c = q / n_mom, m = q % n_mom;
       ws[c][m] = (T)wts[((size_t)sa * NO + grp + c) * n_mom + m];
     }
+    if (pair)
+      for (int q = tid; q < REV_SEL_WORDS; q += NT) s_sel[q] = 0;
     __syncthreads();
     const int neb = s_lev[K - 1];
-    for (int q = tid; q < neb * NO; q += FWD_THREADS) eb[q] = T(0);
+    for (int q = tid; q < neb * NO; q += NT) eb[q] = T(0);
     // Psi-bar_K
-    {
-      T* xb = buf[K & 1];
-      for (int t = tid; t < s_lev[K]; t += FWD_THREADS) {
-        T pk[N], row[N];
-        load_row<T, N, PS>(P + (size_t)(s_lo[K] + t) * PS, pk);
+    T* xK = buf[K & 1];
+    if (pair) {
+      // rows that are not selected enter with zero
+      const T zero[N] = {};
+      for (int t = tid; t < neb; t += NT) store_row<T, N, PS>(xK + (size_t)t * PS, zero);
+      __syncthreads();
+    }
+    const int nK = pair ? cv.ntop[atom] : s_lev[K];
+    for (int q = tid; q < nK; q += NT) {
+      const int t = pair ? (int)(top[q] & 0xffffu) : q;
+      // weights of the site's atom (rows), in the pair form
+      T wj2[NO], wj1[NO];
 #pragma unroll
-        for (int q = 0; q < N; q++) row[q] = T(2) * ws[q % NC][2 * K] * pk[q];
-        if (t < s_lev[K - 1]) {
-          T pk1[N];
-          load_row<T, N, PS>(P + (size_t)(s_lo[K - 1] + t) * PS, pk1);
+      for (int r = 0; r < NO; r++) wj2[r] = wj1[r] = T(0);
+      if (pair) {
+        if (t < neb) atomicOr(&s_sel[t >> 5], 1u << (t & 31));
+        if (t != 0) {
+          const double* wj = wts + ((size_t)spin * n + satom[t]) * NO * n_mom + 2 * K - 1;
 #pragma unroll
-          for (int q = 0; q < N; q++) row[q] += ws[q % NC][2 * K - 1] * pk1[q];
+          for (int r = 0; r < NO; r++) {
+            wj1[r] = (T)wj[r * n_mom];
+            wj2[r] = (T)wj[r * n_mom + 1];
+          }
         }
-        store_row<T, N, PS>(xb + (size_t)t * PS, row);
       }
+      T pk[N], row[N];
+      load_row<T, N, PS>(P + (size_t)(s_lo[K] + t) * PS, pk);
+#pragma unroll
+      for (int v = 0; v < N; v++) row[v] = T(2) * (ws[v % NC][2 * K] + wj2[v / NC]) * pk[v];
+      if (t < neb) {
+        T pk1[N];
+        load_row<T, N, PS>(P + (size_t)(s_lo[K - 1] + t) * PS, pk1);
+#pragma unroll
+        for (int v = 0; v < N; v++) row[v] += (ws[v % NC][2 * K - 1] + wj1[v / NC]) * pk1[v];
+      }
+      store_row<T, N, PS>(xK + (size_t)t * PS, row);
     }
     __syncthreads();
     for (int k = K; k >= 1; k--) {
+      const bool half = pair && k == K;
       const T* xb = buf[k & 1];
       T* yb = buf[(k - 1) & 1];
       const int nrow = s_lev[k - 1];
-      for (int t = tid; t < nrow; t += FWD_THREADS) {
-        // the stored rows this site needs, towards L2 while the gather runs
+      int psh = 0;  // lanes per row, as a shift
+      if (!half)
+        while (psh < 4 && (nrow << (psh + 1)) <= NT) psh++;
+      const int part = tid & ((1 << psh) - 1);
+      for (int r0 = 0; r0 < nrow; r0 += NT >> psh) {
+        if (r0 + ((tid & ~31) >> psh) >= nrow) continue;  // whole warps
+        const int rr = r0 + (tid >> psh);
+        const bool live = rr < nrow;
+        const int t = !live ? 0 : (half ? (int)(top[rr] >> 16) : rr);
         const T* r1 = P + (size_t)(s_lo[k - 1] + t) * PS;
-        prefetch_row_l2<T, PS>(r1);
-        if (k >= 2) {
-          prefetch_row_l2<T, PS>(P + (size_t)(s_lo[k] + t) * PS);
-          if (t < s_lev[k - 2]) prefetch_row_l2<T, PS>(P + (size_t)(s_lo[k - 2] + t) * PS);
+        if (live && part == 0) {
+          // the stored rows this site needs, towards L2 while the gather runs
+          prefetch_row_l2<T, PS>(r1);
+          if (k >= 2) {
+            prefetch_row_l2<T, PS>(P + (size_t)(s_lo[k] + t) * PS);
+            if (t < s_lev[k - 2]) prefetch_row_l2<T, PS>(P + (size_t)(s_lo[k - 2] + t) * PS);
+          }
         }
         T acc[NO][NC];
-        if (k >= 2) {
+#pragma unroll
+        for (int r = 0; r < NO; r++)
+#pragma unroll
+          for (int c = 0; c < NC; c++) acc[r][c] = T(0);
+        if (k >= 2 && live && part == 0) {
           T xt[N];
           load_row<T, N, PS>(xb + (size_t)t * PS, xt);
-          const T* e = E + (size_t)(L.stage ? s_atom[t] : satom[t]) * NO;
+          const T* e = E + (size_t)satom[t] * NO;
 #pragma unroll
           for (int r = 0; r < NO; r++) {
             const T er = e[r];
@@ -714,26 +888,32 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
           }
         }
         if (k >= 2 || HBAR) {
-          int cnt;
-          if (k < K) {
-            const unsigned long long lc = L.stage ? s_lvc[t] : lvc[t];
-            cnt = (int)((lc >> (8 * k)) & 0xff);
-          } else {
-            cnt = L.stage ? (int)(s_aoff[t + 1] - s_aoff[t]) : (int)(cv.adj_off[s0 + t + 1] - cv.adj_off[s0 + t]);
+          const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+          int cnt = 0;
+          if (live) {
+            if (k < K) cnt = (int)((lvc[t] >> (8 * k)) & 0xff);
+            else cnt = L.stage ? s_off[t + 1] - q0 : (int)(cv.adj_off[s0 + t + 1] - abase) - q0;
           }
-          if (cnt > 0) {
-            const int q0 = (int)((L.stage ? s_aoff[t] : cv.adj_off[s0 + t]) - abase);
-            const int2* ents = L.stage ? s_adj + q0 : adj + q0;
-            if constexpr (HBAR) {
-              // with the bond cotangents of the forward pairs (s, t) of level k
-              T pt[N];
+          const unsigned mask = half && live ? cv.topmask[s0 + t] : 0u;
+          T pt[N];
+          if constexpr (HBAR) {
+            if (live) {
               load_row<T, N, PS>(r1, pt);
-              gather_cot<T, NO, NC, PS>(ents, cnt, H, HS, xb, acc, k >= 2, pt, Hbar, HSh);
             } else {
-              gather_pf2<T, NO, NC, PS>(ents, cnt, H, HS, xb, acc);
+#pragma unroll
+              for (int v = 0; v < N; v++) pt[v] = T(0);
             }
           }
+          gather_rev<T, NO, NC, PS, HBAR>(adj + q0, part, 1 << psh, cnt, mask, half, H, HS, xb, acc, k >= 2, pt, Hbar,
+                                          HSh, lane);
+          for (int o = 1; o < (1 << psh); o <<= 1) {
+#pragma unroll
+            for (int r = 0; r < NO; r++)
+#pragma unroll
+              for (int c = 0; c < NC; c++) acc[r][c] += __shfl_xor_sync(0xffffffffu, acc[r][c], o);
+          }
         }
+        if (!live || part != 0) continue;
         // onsite cotangent of level k: Psi-bar_k[t] . Psi_k-1[t] (rows read after the gather)
         T p1[N];
         {
@@ -749,21 +929,23 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
           }
         }
         if (k >= 2) {
-          T pk[N];
-          load_row<T, N, PS>(P + (size_t)(s_lo[k] + t) * PS, pk);
           T row[N];
 #pragma unroll
-          for (int r = 0; r < NO; r++)
+          for (int v = 0; v < N; v++) row[v] = acc[v / NC][v % NC] + T(2) * ws[v % NC][2 * k - 2] * p1[v];
+          if (!half || (s_sel[t >> 5] >> (t & 31) & 1u)) {
+            T pk[N], wj[NO];
+            load_row<T, N, PS>(P + (size_t)(s_lo[k] + t) * PS, pk);
 #pragma unroll
-            for (int c = 0; c < NC; c++) {
-              const int q = r * NC + c;
-              row[q] = acc[r][c] + T(2) * ws[c][2 * k - 2] * p1[q] + ws[c][2 * k - 1] * pk[q];
-            }
+            for (int r = 0; r < NO; r++)
+              wj[r] = half && t != 0 ? (T)wts[(((size_t)spin * n + satom[t]) * NO + r) * n_mom + 2 * K - 1] : T(0);
+#pragma unroll
+            for (int v = 0; v < N; v++) row[v] += (ws[v % NC][2 * k - 1] + wj[v / NC]) * pk[v];
+          }
           if (t < s_lev[k - 2]) {
             T p2[N];
             load_row<T, N, PS>(P + (size_t)(s_lo[k - 2] + t) * PS, p2);
 #pragma unroll
-            for (int q = 0; q < N; q++) row[q] += ws[q % NC][2 * k - 3] * p2[q];
+            for (int v = 0; v < N; v++) row[v] += ws[v % NC][2 * k - 3] * p2[v];
           }
           store_row<T, N, PS>(yb + (size_t)t * PS, row);
         }
@@ -771,13 +953,13 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
       __syncthreads();
     }
     if (Ebar != nullptr) {
-      for (int q = tid; q < neb * NO; q += FWD_THREADS) {
+      for (int q = tid; q < neb * NO; q += NT) {
         const int t = q / NO, r = q % NO;
-        atomicAdd(Ebar + ((size_t)spin * n_on + (L.stage ? s_atom[t] : satom[t])) * NO + r, (double)eb[q]);
+        atomicAdd(Ebar + ((size_t)spin * n_on + satom[t]) * NO + r, (double)eb[q]);
       }
     }
     if (siteval != nullptr) {  // per-site sums over the orbitals (one row of the SCF Jacobian)
-      for (int t = tid; t < neb; t += FWD_THREADS) {
+      for (int t = tid; t < neb; t += NT) {
         double a = 0.0;
 #pragma unroll
         for (int r = 0; r < NO; r++) a += (double)eb[t * NO + r];
@@ -1387,14 +1569,14 @@ template <typename T, int NO, int NC>
 int run_forward(const MomentsArgs& a, cudaStream_t s) {
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
+  constexpr int NT = Fwd<T>::THREADS;
   FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
   size_t psi = (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T);
-  size_t stage = (size_t)a.max_adj * 8 + (size_t)a.max_sites * 8 + (size_t)(a.max_sites + 1) * 8 +
-                 (size_t)a.max_sites * 4 + 16;
+  size_t stage = (size_t)a.max_adj * 8 + (size_t)a.max_sites * 8 + (size_t)(a.max_sites + 1) * 4 +
+                 (size_t)a.max_sites * 12 + 16;
   size_t smem = psi + stage;
-  // stage the adjacency only while two CTAs (FP32) still fit on an SM
-  const size_t budget = sizeof(T) == 4 ? 110 * 1024 : 200 * 1024;
-  if (smem > budget) {
+  // stage the adjacency only while two CTAs still fit on an SM
+  if (smem > 110 * 1024) {
     L.stage = false;
     smem = psi;
   }
@@ -1403,7 +1585,7 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
   if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int n_items = a.n * a.n_spin * (NO / NC);
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, FWD_THREADS, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem);
   if (per_sm < 1) per_sm = 1;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
@@ -1411,8 +1593,10 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
   const int slots = sms * per_sm;
   const int chunk = (n_items + slots - 1) / slots;
   const int grid = (n_items + chunk - 1) / chunk;
-  fn<<<grid, FWD_THREADS, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L,
-                                      n_items, chunk, a.mu, (T*)a.pstore, a.psi_off, a.psi_tot);
+  if (a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
+    return -1;
+  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
+                            a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1430,20 +1614,21 @@ template <typename T, int NO, int NC, bool HBAR>
 int run_reverse(const AdjointArgs& a, cudaStream_t s) {
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
+  constexpr int NT = Fwd<T>::THREADS;
   RevSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, a.cap_eb, true};
   const size_t psi = (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T) + eb_elems<T, NO>(a.cap_eb) * sizeof(T);
-  const size_t stage = (size_t)a.max_adj * 8 + (size_t)a.max_sites * 8 + (size_t)(a.max_sites + 1) * 8 +
+  const size_t stage = (size_t)a.max_adj * 8 + (size_t)a.cap_eb * 8 + (size_t)(a.cap_eb + 1) * 4 +
                        (size_t)a.max_sites * 4 + 16;
   auto fn = k_adj_rev<T, NO, NC, HBAR>;
   size_t smem = psi + stage;
   int per_sm = 0, per_sm_unstaged = 0;
-  if (smem <= 227 * 1024) {
+  if (smem <= 225 * 1024) {
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, FWD_THREADS, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem);
   }
-  if (psi > 227 * 1024) return -2;
+  if (psi > 225 * 1024) return -2;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psi);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_unstaged, fn, FWD_THREADS, psi);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_unstaged, fn, NT, psi);
   if (per_sm < per_sm_unstaged) {  // staging the adjacency would cost a resident CTA
     L.stage = false;
     smem = psi;
@@ -1459,10 +1644,9 @@ int run_reverse(const AdjointArgs& a, cudaStream_t s) {
   const int slots = sms * per_sm;
   const int chunk = (n_items + slots - 1) / slots;
   const int grid = (n_items + chunk - 1) / chunk;
-  fn<<<grid, FWD_THREADS, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items,
-                                      chunk,
-                                      (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh,
-                                      a.Ebar, a.siteval, a.sv_stride);
+  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
+                            (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
+                            a.sv_stride, a.pair);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
