@@ -16,9 +16,6 @@
 #include "../../include/bopgb.h"
 #include "kernels.h"
 
-int moments_columns(int norb, int cap_sum, int fp64);
-int adjoint_columns(int norb);
-
 constexpr int FERMI_ROUNDS_COLD = 16;  // Newton rounds launched for a cold start
 constexpr int FERMI_ROUNDS_WARM = 5;  // ... and from the previous SCF iteration's E_F
 constexpr int FERMI_ROUNDS_MORE = 64;  // extra rounds if a solve has not converged
@@ -662,15 +659,17 @@ int size_state(bop_ctx* c) {
   return BOP_OK;
 }
 
-// Columns per work item of the forward pass (all 5 starting orbitals when
-// both stored levels fit in shared memory).
-int forward_nc(bop_ctx* c) {
-  int ce = 1, co = 1;
-  for (int k = 0; k < c->K; k++) {
-    int& cap = (k & 1) ? co : ce;
-    if (c->maxlev[k] > cap) cap = c->maxlev[k];
-  }
-  return moments_columns(c->norb, ce + co, c->fp64);
+// Scratch of one slot per CTA (at most four on an SM) for two levels of a work
+// item of cap_sum sites.
+int slot_scratch(bop_ctx* c, int cap_sum, void** p, size_t* bytes) {
+  int sms = 0;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
+  const long long items = (long long)c->S * c->nc;
+  const size_t slots = (size_t)(items < 4ll * sms ? items : 4ll * sms);
+  CKS(ensure(c, c->adjscr, slots * moments_slot_bytes(c->norb, cap_sum, c->fp64)));
+  *p = c->adjscr.p;
+  *bytes = c->adjscr.bytes;
+  return BOP_OK;
 }
 
 // Arguments of the spinor kernel (non-collinear magnetism): per-CTA scratch
@@ -738,6 +737,10 @@ int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s
   a.psi_off = P<long long>(c->psi_off);
   a.psi_tot = c->psi_tot;
   a.pair = c->pair_ok && !full;
+  a.gmem = moments_in_gmem(c->norb, a.cap_even + a.cap_odd, c->fp64);
+  a.scratch = nullptr;
+  a.scratch_bytes = 0;
+  if (a.gmem) CKS(slot_scratch(c, a.cap_even + a.cap_odd, &a.scratch, &a.scratch_bytes));
   Region R(c, PK_MOMENTS, 1, s);
   int r = launch_moments(a, c->fp64, s);
   if (r == -2) return fail(c, BOP_ERR_OVERFLOW, "cluster level too large for shared memory");
@@ -1030,19 +1033,13 @@ int psi_row(int N, int fp64) {
   return fp64 ? (N + 1) / 2 * 2 : (N + 3) / 4 * 4;
 }
 
-// Stores Psi of every work item (one more forward pass at the current
-// onsite levels) when it fits: all starting orbitals share one work item
-// (the stored-Psi sweep keeps two Psi-bar levels of all five columns in
-// shared memory; with one column per item it gathers every block five times
-// and is slower than recomputing), and the store fits in a third of the free
-// device memory and the store budget (psi_store_alloc).  Otherwise the
-// reverse sweeps recompute Psi.
+// Room for the Psi of every work item, when it fits in a third of the free
+// device memory and in the store budget.  Otherwise the reverse sweeps
+// recompute Psi.
 int psi_store_alloc(bop_ctx* c, bool* fits) {
   *fits = false;
-  const int nc = forward_nc(c);
-  if (c->norb > 1 && nc != c->norb) return BOP_OK;
   const size_t esz = c->fp64 ? sizeof(double) : sizeof(float);
-  const size_t bytes = (size_t)c->S * (c->norb / nc) * (size_t)c->psi_tot * psi_row(c->norb * nc, c->fp64) * esz;
+  const size_t bytes = (size_t)c->S * (size_t)c->psi_tot * psi_row(c->norb * c->norb, c->fp64) * esz;
   size_t freeb = 0, totalb = 0;
   CK(cudaMemGetInfo(&freeb, &totalb));
   const size_t held = c->psis.bytes;
@@ -1094,7 +1091,6 @@ int adjoint_pass(bop_ctx* c, const double* w, void* Hbar, double* Ebar, cudaStre
     aa.pstore = c->psis.p;
     aa.psi_off = P<long long>(c->psi_off);
     aa.psi_tot = c->psi_tot;
-    aa.nc = forward_nc(c);
     int ce = 1, co = 1;
     for (int k = 1; k <= c->K; k++) {
       int& cap = (k & 1) ? co : ce;
@@ -1110,14 +1106,15 @@ int adjoint_pass(bop_ctx* c, const double* w, void* Hbar, double* Ebar, cudaStre
     if (c->psi_pair && !aa.pair) return fail(c, BOP_ERR_STATE, "the stored Psi holds the pair form only");
     aa.siteval = siteval;
     aa.sv_stride = c->nsite;
+    aa.gmem = moments_in_gmem(c->norb, ce + co, c->fp64);
+    if (aa.gmem) CKS(slot_scratch(c, ce + co, &aa.scratch, &aa.scratch_bytes));
   } else {
     if (siteval) return fail(c, BOP_ERR_STATE, "per-site cotangents need the stored Psi");
-    int nc = adjoint_columns(c->norb);
-    size_t per_site = (size_t)c->norb * nc;
+    size_t per_site = (size_t)c->norb * c->norb;
     long long levsum = 0;
     for (int k = 0; k <= c->K; k++) levsum += c->maxlev[k];
     size_t slot_elems = (2 * (size_t)levsum) * per_site + 64;
-    int nwork = n * c->S * (c->norb / nc);
+    int nwork = n * c->S;
     int slots = nwork < 1216 ? nwork : 1216;
     size_t esz = c->fp64 ? sizeof(double) : sizeof(float);
     CKS(ensure(c, c->adjscr, esz * slot_elems * slots));

@@ -127,15 +127,22 @@ struct MomentsArgs {
   int max_adj;         // largest adjacency of one cluster
   double* mu;          // [S][n][norb][n_mom]
   // optional store of every Psi_k (NULL = none): rows of the item
-  // (spin, atom[, alpha]) at ((spin (norb/nc) + alpha) psi_tot + psi_off[atom]) rows,
-  // level k at row offset sum_{j<k} |C_j|; row = norb x nc values padded
+  // (spin, atom) at spin psi_tot + psi_off[atom] rows, level k at row offset
+  // sum_{j<k} |C_j|; row = norb x norb values padded
   void* pstore;
   const long long* psi_off;  // [n+1] prefix sums of sum_k |C_k| over atoms
   long long psi_tot;
   // last level in the pair form (needs cv.top; every atom a centre): stores,
   // then, the selected rows of Psi_K only
   bool pair;
+  // Psi of two levels in global memory (moments_in_gmem): in the store, or in
+  // scratch, one slot (moments_slot_bytes) per CTA
+  bool gmem;
+  void* scratch;
+  size_t scratch_bytes;
 };
+size_t moments_slot_bytes(int norb, int cap_sum, int fp64);
+bool moments_in_gmem(int norb, int cap_sum, int fp64);
 int launch_moments(const MomentsArgs& a, int fp64, cudaStream_t s);
 
 struct AdjointArgs {
@@ -156,7 +163,8 @@ struct AdjointArgs {
   const void* pstore;
   const long long* psi_off;
   long long psi_tot;
-  int nc;              // columns per work item used by the forward pass that stored Psi
+  bool gmem;           // stored-Psi sweep: Psi-bar of two levels in scratch (MomentsArgs::gmem)
+  size_t scratch_bytes;
   int cap_even, cap_odd;  // largest even / odd level |C_k|, k = 1..K
   int max_sites, max_adj, cap_eb;  // cap_eb: largest |C_K-1|; max_adj: entries of its rows
   // stored-Psi sweep only: per cluster site t of work item (spin, atom i),

@@ -6,9 +6,9 @@
 // bond and dU/dE for every onsite level from the weights w_n = dU/dmu_n
 // (the Theta-tilde / transfer-path sums of Eqs. theta-tilde, Xi).
 //
-// Forward: one CTA per (spin, atom[, alpha]).  Psi_{k-1} and Psi_k live in
-// shared memory (ping-pong); the last level Psi_K is never stored, only its
-// inner products.  Each thread owns one cluster site per pass and gathers
+// Forward: one CTA per (spin, atom).  Psi_{k-1} and Psi_k live in shared
+// memory (ping-pong) or global scratch; the last level Psi_K is only stored for
+// a reverse sweep.  Each thread owns one cluster site per pass and gathers
 // the 5x5 blocks of its bonds (15 unique elements, 16-element records) from
 // L2 (for sd blocks 21 unique elements in 24-element records).  Products in
 // T (float or double), moments written as double.
@@ -503,14 +503,18 @@ __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int fir
 }
 
 // Forward kernel.  A persistent CTA takes a run of consecutive work items
-// (spin, atom[, alpha]); neighbouring atoms share most of their clusters'
-// blocks, which then come from L1.  For each item the atom's adjacency,
+// (spin, atom); neighbouring atoms share most of their clusters' blocks, which
+// then come from L1.  For each item the atom's adjacency,
 // per-site offsets, level counts, site atoms and row orders are staged in
 // shared memory (one coalesced copy) when they fit, so that the edge loop only
 // waits for the bond blocks, which are fetched one edge ahead.  Each thread
-// computes all NC columns of one site (NO x NO x NC multiply-adds per edge);
-// Psi rows are padded to 16-byte multiples and kept in two exactly sized
-// buffers (even and odd levels).
+// computes all columns of one site (NO^3 multiply-adds per edge); Psi rows are
+// padded to 16-byte multiples and kept in two exactly sized buffers (even and
+// odd levels) in shared memory, or where those do not fit (GMEM: clusters of
+// 11 and more moments) in the Psi store or the CTA's slot of global scratch,
+// from where the L2 serves them: one item with all columns takes 1/5 of the
+// block loads of five items that fit.  FP64 is bound by its DFMA pipe either
+// way (328 bytes per 125 DFMA, 62 cycles of an SM).
 //
 // Rows run in the order of their length (ClusterView::order): the 1 to 6
 // entries of an outer shell's row and the 14 of an inner one no longer share a
@@ -536,19 +540,20 @@ struct FwdSmem {
   bool stage;
 };
 
-template <typename T, int NO, int NC>
+template <typename T, int NO, bool GMEM>
 __global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
 k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
           int n_mom, FwdSmem L, int n_items, int chunk, double* __restrict__ mu, T* __restrict__ pstore,
-          const long long* __restrict__ psi_off, long long psi_tot, bool pair) {
-  constexpr int NT = Fwd<T>::THREADS;
+          const long long* __restrict__ psi_off, long long psi_tot, bool pair, T* __restrict__ scratch,
+          size_t slot_elems) {
+  constexpr int NT = Fwd<T>::THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf[2];
-  buf[0] = reinterpret_cast<T*>(smem_raw);
+  buf[0] = GMEM ? scratch + (size_t)blockIdx.x * slot_elems : reinterpret_cast<T*>(smem_raw);
   buf[1] = buf[0] + (size_t)L.cap_even * PS;
-  unsigned char* tail = align16(reinterpret_cast<unsigned char*>(buf[1] + (size_t)L.cap_odd * PS));
+  unsigned char* tail = align16(GMEM ? smem_raw : reinterpret_cast<unsigned char*>(buf[1] + (size_t)L.cap_odd * PS));
   int2* s_adj = reinterpret_cast<int2*>(tail);
   unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
   int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.max_sites : 0));
@@ -564,13 +569,11 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
   const int w0 = blockIdx.x * chunk, w1 = min(n_items, w0 + chunk);
   ItemExt nx{};
   if (w0 < w1) {
-    ext_sites(cv, ((NC == NO) ? w0 : (w0 / NO)) % n, nx);
+    ext_sites(cv, w0 % n, nx);
     ext_adj(cv, nx);
   }
   for (int w = w0; w < w1; w++) {
-    const int grp = (NC == NO) ? 0 : (w % NO);
-    const int sa = (NC == NO) ? w : (w / NO);
-    const int spin = sa / n, atom = sa % n;
+    const int spin = w / n, atom = w % n;
     const ItemExt cur = nx;
     const long long s0 = cur.s0, abase = cur.abase;
     const int* lev = cv.level_end + (size_t)atom * (K + 1);
@@ -586,30 +589,25 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     }
     const int ntop = pair ? cv.ntop[atom] : 0;
     const bool more = w + 1 < w1;
-    if (more) ext_sites(cv, ((NC == NO) ? w + 1 : ((w + 1) / NO)) % n, nx);
-    for (int q = tid; q < N; q += NT) {
-      const int r = q / NC, c = q % NC;
-      buf[0][q] = (NC == NO) ? T(r == c ? 1 : 0) : T(r == grp ? 1 : 0);
-    }
+    if (more) ext_sites(cv, (w + 1) % n, nx);
     // stored Psi: item rows start at ib, level k at row lo_k = sum_{j<k} |C_j|
     T* pitem = nullptr;
     if (pstore != nullptr) {
-      pitem = pstore + ((size_t)(spin * (NO / NC) + grp) * psi_tot + psi_off[atom]) * PS;
-      for (int q = tid; q < PS; q += NT) {
-        const int r = q / NC, c = q % NC;
-        pitem[q] = q < N ? ((NC == NO) ? T(r == c ? 1 : 0) : T(r == grp ? 1 : 0)) : T(0);
-      }
+      pitem = pstore + ((size_t)spin * psi_tot + psi_off[atom]) * PS;
+      for (int q = tid; q < PS; q += NT) pitem[q] = T(q < N && q / NC == q % NC ? 1 : 0);
     }
+    for (int q = tid; q < PS; q += NT) buf[0][q] = T(q < N && q / NC == q % NC ? 1 : 0);
     long long lo_k = 0;
     __syncthreads();
-    double* out = mu + ((size_t)sa * NO + grp) * n_mom;
+    double* out = mu + (size_t)w * NO * n_mom;
     if (tid < NC) out[(size_t)tid * n_mom] = 1.0;
     for (int k = 1; k <= K; k++) {
+      const bool in_store = GMEM && pstore != nullptr;
+      const T* prev = in_store ? pitem + (size_t)lo_k * PS : buf[(k - 1) & 1];
       lo_k += lev[k - 1];
       const bool half = pair && k == K;
       const int ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
       const int nrow = half ? ntop : lev[k];
-      const T* prev = buf[(k - 1) & 1];
       T* next = buf[k & 1];
       T d1[NC], d2[NC];
 #pragma unroll
@@ -675,7 +673,7 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
           }
           if (other) atomicAdd(mt + r_ * n_mom + 1, (double)a);
         }
-        if (k < K) store_row<T, N, PS>(next + (size_t)t * PS, &acc[0][0]);
+        if (k < K && !in_store) store_row<T, N, PS>(next + (size_t)t * PS, &acc[0][0]);
         if (pitem != nullptr) store_row<T, N, PS>(pitem + (size_t)(lo_k + t) * PS, &acc[0][0]);
       }
 #pragma unroll
@@ -709,8 +707,9 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
 //   Psi-bar_K     = 2 w_2K Psi_K + w_2K-1 Psi_K-1
 //   Psi-bar_k-1   = H Psi-bar_k (rows < |C_k-1|, columns < |C_k|)
 //                   + 2 w_2k-2 Psi_k-1 + w_2k-1 Psi_k + w_2k-3 Psi_k-2
-// runs like the forward kernel: Psi-bar_k and Psi-bar_k-1 in two shared
-// buffers (even / odd levels), the adjacency of the rows (C_K-1) staged.  The
+// runs like the forward kernel: Psi-bar_k and Psi-bar_k-1 in two buffers (even
+// / odd levels) in shared memory or (GMEM) in the CTA's slot of global
+// scratch, the adjacency of the rows (C_K-1) staged.  The
 // onsite cotangents dL/dE_t = sum_k Psi-bar_k[t] . Psi_k-1[t] are accumulated
 // per site in shared memory and added once per item.  With HBAR the gather of
 // level k also forms the bond cotangents of its pairs, Psi-bar_k(s)
@@ -740,21 +739,22 @@ __host__ __device__ constexpr size_t eb_elems(int cap_eb) {
 
 constexpr int REV_SEL_WORDS = 256;  // selected sites as bits (a cluster with a pair form has at most 8,192 sites)
 
-template <typename T, int NO, int NC, bool HBAR>
+template <typename T, int NO, bool HBAR, bool GMEM>
 __global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
 k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
           int n_mom, RevSmem L, int n_items, int chunk, const T* __restrict__ pstore,
           const long long* __restrict__ psi_off, long long psi_tot, const double* __restrict__ wts,
           T* __restrict__ Hbar, int HSh, double* __restrict__ Ebar, double* __restrict__ siteval,
-          long long sv_stride, bool pair) {
-  constexpr int NT = Fwd<T>::THREADS;
+          long long sv_stride, bool pair, T* __restrict__ scratch, size_t slot_elems) {
+  constexpr int NT = Fwd<T>::THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf[2];
-  buf[0] = reinterpret_cast<T*>(smem_raw);
+  buf[0] = GMEM ? scratch + (size_t)blockIdx.x * slot_elems : reinterpret_cast<T*>(smem_raw);
   buf[1] = buf[0] + (size_t)L.cap_even * PS;
-  T* eb = buf[1] + (size_t)L.cap_odd * PS;  // [cap_eb][NO], padded to 16 bytes
+  // [cap_eb][NO], padded to 16 bytes
+  T* eb = GMEM ? reinterpret_cast<T*>(smem_raw) : buf[1] + (size_t)L.cap_odd * PS;
   unsigned char* tail = align16(reinterpret_cast<unsigned char*>(eb + eb_elems<T, NO>(L.cap_eb)));
   int2* s_adj = reinterpret_cast<int2*>(tail);
   unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
@@ -769,13 +769,11 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
   const int w0 = blockIdx.x * chunk, w1 = min(n_items, w0 + chunk);
   ItemExt nx{};
   if (w0 < w1) {
-    ext_sites(cv, ((NC == NO) ? w0 : (w0 / NO)) % n, nx);
+    ext_sites(cv, w0 % n, nx);
     ext_adj(cv, nx);
   }
   for (int w = w0; w < w1; w++) {
-    const int grp = (NC == NO) ? 0 : (w % NO);
-    const int sa = (NC == NO) ? w : (w / NO);
-    const int spin = sa / n, atom = sa % n;
+    const int spin = w / n, atom = w % n;
     const ItemExt cur = nx;
     const long long s0 = cur.s0, abase = cur.abase;
     const int* lev = cv.level_end + (size_t)atom * (K + 1);
@@ -783,7 +781,7 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     const int* satom = L.stage ? s_atom : cv.site_atom + s0;
     const unsigned* top = cv.top + s0;
     const T* E = onsite + (size_t)spin * n_on * NO;
-    const size_t ib = ((size_t)(spin * (NO / NC) + grp) * psi_tot + psi_off[atom]) * PS;
+    const size_t ib = ((size_t)spin * psi_tot + psi_off[atom]) * PS;
     const T* P = pstore + ib;
     if (L.stage) {
       const int nr = lev[K - 1];
@@ -791,7 +789,7 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     }
     const int2* adj = L.stage ? s_adj : cv.adj + abase;
     const bool more = w + 1 < w1;
-    if (more) ext_sites(cv, ((NC == NO) ? w + 1 : ((w + 1) / NO)) % n, nx);
+    if (more) ext_sites(cv, (w + 1) % n, nx);
     if (tid <= K) s_lev[tid] = lev[tid];
     if (tid == 0) {
       long long o = 0;
@@ -802,7 +800,7 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     }
     for (int q = tid; q < NC * n_mom; q += NT) {
       const int c = q / n_mom, m = q % n_mom;
-      ws[c][m] = (T)wts[((size_t)sa * NO + grp + c) * n_mom + m];
+      ws[c][m] = (T)wts[((size_t)w * NO + c) * n_mom + m];
     }
     if (pair)
       for (int q = tid; q < REV_SEL_WORDS; q += NT) s_sel[q] = 0;
@@ -1565,13 +1563,26 @@ int run_nc(const NcArgs& a, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <typename T, int NO, int NC>
+// CTAs of a persistent kernel and the work items of each.
+template <class F>
+void persistent_grid(F fn, int threads, size_t smem, int n_items, int* grid, int* chunk) {
+  int per_sm = 1, sms = 0, dev = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
+  if (per_sm < 1) per_sm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int slots = sms * per_sm;
+  *chunk = (n_items + slots - 1) / slots;
+  *grid = (n_items + *chunk - 1) / *chunk;
+}
+
+template <typename T, int NO, bool GMEM>
 int run_forward(const MomentsArgs& a, cudaStream_t s) {
-  constexpr int N = NO * NC;
+  constexpr int N = NO * NO;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   constexpr int NT = Fwd<T>::THREADS;
   FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
-  size_t psi = (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T);
+  const size_t psi = GMEM ? 0 : (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T);
   size_t stage = (size_t)a.max_adj * 8 + (size_t)a.max_sites * 8 + (size_t)(a.max_sites + 1) * 4 +
                  (size_t)a.max_sites * 12 + 16;
   size_t smem = psi + stage;
@@ -1580,103 +1591,110 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
     L.stage = false;
     smem = psi;
   }
-  if (smem > 227 * 1024) return -2;
-  auto fn = k_moments<T, NO, NC>;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const int n_items = a.n * a.n_spin * (NO / NC);
-  int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem);
-  if (per_sm < 1) per_sm = 1;
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int slots = sms * per_sm;
-  const int chunk = (n_items + slots - 1) / slots;
-  const int grid = (n_items + chunk - 1) / chunk;
+  auto fn = k_moments<T, NO, GMEM>;
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return -1;
+  const int n_items = a.n * a.n_spin;
+  int grid, chunk;
+  persistent_grid(fn, NT, smem, n_items, &grid, &chunk);
+  const size_t slot = (size_t)(a.cap_even + a.cap_odd) * PS;
+  if (GMEM && a.pstore == nullptr && (size_t)grid * slot * sizeof(T) > a.scratch_bytes) {
+    // fewer CTAs than fit on the device: what the scratch holds
+    const size_t most = a.scratch_bytes / (slot * sizeof(T));
+    if (most < 1) return -1;
+    chunk = (int)((n_items + most - 1) / most);
+    grid = (n_items + chunk - 1) / chunk;
+  }
   if (a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
     return -1;
   fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
-                            a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair);
+                            a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <typename T, int NO, int NC>
+template <typename T, int NO>
 int run_adjoint(const AdjointArgs& a, cudaStream_t s) {
-  int nwork = a.n * a.n_spin * (NO / NC);
-  int grid = nwork < a.slots ? nwork : a.slots;
-  k_moments_adj<T, NO, NC><<<grid, MOM_THREADS, 0, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on,
+  const int nwork = a.n * a.n_spin;
+  const int grid = nwork < a.slots ? nwork : a.slots;
+  k_moments_adj<T, NO, NO><<<grid, MOM_THREADS, 0, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on,
                                                        a.n_mom, nwork, a.w, (T*)a.scratch, a.slot_elems,
                                                        (T*)a.Hbar, a.HSh, a.Ebar);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <typename T, int NO, int NC, bool HBAR>
+template <typename T, int NO, bool HBAR, bool GMEM>
 int run_reverse(const AdjointArgs& a, cudaStream_t s) {
-  constexpr int N = NO * NC;
+  constexpr int N = NO * NO;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   constexpr int NT = Fwd<T>::THREADS;
   RevSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, a.cap_eb, true};
-  const size_t psi = (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T) + eb_elems<T, NO>(a.cap_eb) * sizeof(T);
+  const size_t slot = (size_t)(a.cap_even + a.cap_odd) * PS;
+  const size_t psi = (GMEM ? 0 : slot * sizeof(T)) + eb_elems<T, NO>(a.cap_eb) * sizeof(T);
   const size_t stage = (size_t)a.max_adj * 8 + (size_t)a.cap_eb * 8 + (size_t)(a.cap_eb + 1) * 4 +
                        (size_t)a.max_sites * 4 + 16;
-  auto fn = k_adj_rev<T, NO, NC, HBAR>;
+  auto fn = k_adj_rev<T, NO, HBAR, GMEM>;
   size_t smem = psi + stage;
   int per_sm = 0, per_sm_unstaged = 0;
+  if (psi > 225 * 1024) return -2;
   if (smem <= 225 * 1024) {
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem);
   }
-  if (psi > 225 * 1024) return -2;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psi);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_unstaged, fn, NT, psi);
   if (per_sm < per_sm_unstaged) {  // staging the adjacency would cost a resident CTA
     L.stage = false;
     smem = psi;
-    per_sm = per_sm_unstaged;
   } else {
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
-  if (per_sm < 1) per_sm = 1;
-  const int n_items = a.n * a.n_spin * (NO / NC);
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int slots = sms * per_sm;
-  const int chunk = (n_items + slots - 1) / slots;
-  const int grid = (n_items + chunk - 1) / chunk;
+  const int n_items = a.n * a.n_spin;
+  int grid, chunk;
+  persistent_grid(fn, NT, smem, n_items, &grid, &chunk);
+  if (GMEM && (size_t)grid * slot * sizeof(T) > a.scratch_bytes) {
+    const size_t most = a.scratch_bytes / (slot * sizeof(T));
+    if (most < 1) return -1;
+    chunk = (int)((n_items + most - 1) / most);
+    grid = (n_items + chunk - 1) / chunk;
+  }
   fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
                             (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
-                            a.sv_stride, a.pair);
+                            a.sv_stride, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <typename T, int NO, int NC>
+template <typename T, int NO>
 int run_reverse_mode(const AdjointArgs& a, cudaStream_t s) {
-  return a.Hbar ? run_reverse<T, NO, NC, true>(a, s) : run_reverse<T, NO, NC, false>(a, s);
+  if (a.gmem) return a.Hbar ? run_reverse<T, NO, true, true>(a, s) : run_reverse<T, NO, false, true>(a, s);
+  return a.Hbar ? run_reverse<T, NO, true, false>(a, s) : run_reverse<T, NO, false, false>(a, s);
+}
+
+template <typename T, int NO>
+int run_forward_mode(const MomentsArgs& a, cudaStream_t s) {
+  return a.gmem ? run_forward<T, NO, true>(a, s) : run_forward<T, NO, false>(a, s);
 }
 
 }  // namespace
 
-// Column grouping: all starting orbitals of an atom in one CTA when both Psi
-// levels fit in shared memory, one CTA per starting orbital otherwise.
-int moments_columns(int norb, int cap_sum, int fp64) {
-  if (norb == 1) return 1;
-  size_t bytes = (size_t)cap_sum * norb * norb * (fp64 ? 8 : 4);
-  return bytes <= 100 * 1024 ? norb : 1;
+// Psi rows (Psi-bar rows) of two levels of one work item.
+size_t moments_slot_bytes(int norb, int cap_sum, int fp64) {
+  const size_t N = (size_t)norb * norb;
+  const size_t ps = N == 1 ? 1 : (fp64 ? (N + 1) / 2 * 2 : (N + 3) / 4 * 4);
+  return (size_t)cap_sum * ps * (fp64 ? 8 : 4);
+}
+
+// Two levels of an item in shared memory (two CTAs per SM) or in global
+// scratch.
+bool moments_in_gmem(int norb, int cap_sum, int fp64) {
+  return moments_slot_bytes(norb, cap_sum, fp64) > 104 * 1024;
 }
 
 int launch_moments(const MomentsArgs& a, int fp64, cudaStream_t s) {
-  int nc = moments_columns(a.norb, a.cap_even + a.cap_odd, fp64);
-  if (a.norb == 1) return fp64 ? run_forward<double, 1, 1>(a, s) : run_forward<float, 1, 1>(a, s);
-  if (a.norb == 6) {
-    if (nc == 6) return fp64 ? run_forward<double, 6, 6>(a, s) : run_forward<float, 6, 6>(a, s);
-    return fp64 ? run_forward<double, 6, 1>(a, s) : run_forward<float, 6, 1>(a, s);
-  }
-  if (nc == 5) return fp64 ? run_forward<double, 5, 5>(a, s) : run_forward<float, 5, 5>(a, s);
-  return fp64 ? run_forward<double, 5, 1>(a, s) : run_forward<float, 5, 1>(a, s);
+  if (a.norb == 1) return fp64 ? run_forward_mode<double, 1>(a, s) : run_forward_mode<float, 1>(a, s);
+  if (a.norb == 6) return fp64 ? run_forward_mode<double, 6>(a, s) : run_forward_mode<float, 6>(a, s);
+  return fp64 ? run_forward_mode<double, 5>(a, s) : run_forward_mode<float, 5>(a, s);
 }
-
-int adjoint_columns(int norb) { return norb; }
 
 int bond_cotangent_stride(int norb, int fp64) {
   if (norb == 1) return 1;
@@ -1686,17 +1704,13 @@ int bond_cotangent_stride(int norb, int fp64) {
 
 int launch_moments_adjoint(const AdjointArgs& a, int fp64, cudaStream_t s) {
   if (a.pstore != nullptr) {  // reverse sweep over stored Psi
-    if (a.norb == 1) return fp64 ? run_reverse_mode<double, 1, 1>(a, s) : run_reverse_mode<float, 1, 1>(a, s);
-    if (a.norb == 6) {
-      if (a.nc == 6) return fp64 ? run_reverse_mode<double, 6, 6>(a, s) : run_reverse_mode<float, 6, 6>(a, s);
-      return fp64 ? run_reverse_mode<double, 6, 1>(a, s) : run_reverse_mode<float, 6, 1>(a, s);
-    }
-    if (a.nc == 5) return fp64 ? run_reverse_mode<double, 5, 5>(a, s) : run_reverse_mode<float, 5, 5>(a, s);
-    return fp64 ? run_reverse_mode<double, 5, 1>(a, s) : run_reverse_mode<float, 5, 1>(a, s);
+    if (a.norb == 1) return fp64 ? run_reverse_mode<double, 1>(a, s) : run_reverse_mode<float, 1>(a, s);
+    if (a.norb == 6) return fp64 ? run_reverse_mode<double, 6>(a, s) : run_reverse_mode<float, 6>(a, s);
+    return fp64 ? run_reverse_mode<double, 5>(a, s) : run_reverse_mode<float, 5>(a, s);
   }
-  if (a.norb == 1) return fp64 ? run_adjoint<double, 1, 1>(a, s) : run_adjoint<float, 1, 1>(a, s);
-  if (a.norb == 6) return fp64 ? run_adjoint<double, 6, 6>(a, s) : run_adjoint<float, 6, 6>(a, s);
-  return fp64 ? run_adjoint<double, 5, 5>(a, s) : run_adjoint<float, 5, 5>(a, s);
+  if (a.norb == 1) return fp64 ? run_adjoint<double, 1>(a, s) : run_adjoint<float, 1>(a, s);
+  if (a.norb == 6) return fp64 ? run_adjoint<double, 6>(a, s) : run_adjoint<float, 6>(a, s);
+  return fp64 ? run_adjoint<double, 5>(a, s) : run_adjoint<float, 5>(a, s);
 }
 
 int launch_nc(const NcArgs& a, int fp64, cudaStream_t s) {
