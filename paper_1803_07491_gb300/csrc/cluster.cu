@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
       for (int q = tid; q < nsite; q += G) out.order[s0 + q] = (unsigned)ord[q] | ((unsigned)ord[S2 + q] << 16);
       if (out.top != nullptr) {
         if (tid < 32) {  // the selected sites in the order of the last level's rows
-          int run = 0;
+          int run = 0, in = 0;
           const int l2 = K >= 2 ? s_lev[K - 2] : 0, l1 = s_lev[K - 1];
           for (int q0 = 0; q0 < nsite; q0 += 32) {
             const int q = q0 + lane;
@@ -827,10 +827,11 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
             const unsigned bal = __ballot_sync(0xffffffffu, sel);
             if (sel) ord[2 * S2 + run + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)t;
             run += __popc(bal);
+            in += __popc(__ballot_sync(0xffffffffu, sel && q < l1));
           }
           if (lane == 0) {
             s_cnt = run;
-            out.ntop[atom] = run;
+            out.ntop[atom] = run | (in << 16);
           }
         }
         group_sync<G>();

@@ -42,10 +42,10 @@ struct ClusterView {
   // levels up to its own (its work one level on)
   const unsigned* order;      // [S]
   // Pair form of the last level (NULL without it; see pair_selected): low
-  // half: the selected sites by descending row length, ntop of them; high
-  // half: the sites of C_K-1 by descending selected entries
+  // half: the selected sites, those of C_K-1 first, each part by descending
+  // row length; high half: the sites of C_K-1 by descending selected entries
   const unsigned* top;        // [S]
-  const int* ntop;            // [n]
+  const int* ntop;            // [n] selected sites, and << 16 those in C_K-1
   const unsigned* topmask;    // [S] bit e: entry e of the row is a selected site
 };
 

@@ -349,16 +349,17 @@ __device__ __forceinline__ void gather_pf(const int2* __restrict__ adj, long lon
   }
 }
 
-// acc += sum over cnt adjacency entries of B_ts x[s], with the blocks of
-// the next two entries in flight while the current one is applied.
+// acc += sum over cnt adjacency entries (every step-th of ent) of B_ts x[s],
+// with the blocks of the next two entries in flight while the current one is
+// applied.
 template <typename T, int NO, int NC, int PS>
-__device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int cnt, const T* __restrict__ H, int HS,
-                                           const T* __restrict__ x, T acc[NO][NC]) {
+__device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int step, int cnt, const T* __restrict__ H,
+                                           int HS, const T* __restrict__ x, T acc[NO][NC]) {
   constexpr int HB = hb_count<NO>();
   constexpr int N = NO * NC;
   if (cnt <= 0) return;
   int2 e0 = ent[0];
-  int2 e1 = cnt > 1 ? ent[1] : e0;
+  int2 e1 = cnt > 1 ? ent[step] : e0;
   T h0[HB], h1[HB];
   load_bond<T, NO>(H + (size_t)e0.y * HS, h0);
   if (cnt > 1) load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
@@ -371,7 +372,7 @@ __device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int cnt
 #pragma unroll
     for (int q = 0; q < HB; q++) h0[q] = h1[q];
     if (e + 2 < cnt) {
-      e1 = ent[e + 2];
+      e1 = ent[(e + 2) * step];
       load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
     }
     T xs[N];
@@ -520,7 +521,9 @@ __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int fir
 // entries of an outer shell's row and the 14 of an inner one no longer share a
 // warp, whose other lanes would idle for the longest row; odd passes over the
 // threads run backwards, so that the warp with the longest rows of one pass
-// gets the shortest of the next.
+// gets the shortest of the next.  FP64: the long rows of a small level have two
+// lanes each, which halves the longest chain between two barriers (432-atom
+// Stoner cell: 0.83 -> 0.78 ms per pass; in FP32, bound by the L1, 3 %).
 //
 // pair: the last level (68 % of the products of a bcc cluster at 9 moments)
 // computes the selected sites only (pair_selected).  H^K is symmetric, so the
@@ -607,14 +610,20 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
       lo_k += lev[k - 1];
       const bool half = pair && k == K;
       const int ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
-      const int nrow = half ? ntop : lev[k];
+      // rows of C_k-1 (7 to 14 entries in bcc) come first and, at FP64 levels
+      // of at most two passes, get two lanes each; the sites first reached at
+      // this level (1 to 6 entries) one
+      const int nrow = half ? ntop & 0xffff : lev[k];
+      const int nbig = sizeof(T) == 8 && nrow <= 2 * NT ? (half ? ntop >> 16 : ncol) : 0;
       T* next = buf[k & 1];
       T d1[NC], d2[NC];
 #pragma unroll
       for (int c = 0; c < NC; c++) d1[c] = d2[c] = T(0);
-      for (int p = 0; p * NT < nrow; p++) {
-        const int r = p * NT + ((p & 1) ? NT - 1 - tid : tid);
-        if (r >= nrow) continue;
+      for (int p = 0; p * NT < nrow + nbig; p++) {
+        const int v = p * NT + ((p & 1) ? NT - 1 - tid : tid);
+        const bool big = v < 2 * nbig, live = v < nrow + nbig;
+        const int part = big ? v & 1 : 0;
+        const int r = !live ? 0 : (big ? v >> 1 : v - nbig);
         // rows up to level k-2 are full, shell k-1 has entries up to its own
         // level, shell k of the one below
         const int t = half ? (int)(top[r] & 0xffffu)
@@ -622,7 +631,7 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
         T acc[NO][NC];
         const bool in_prev = t < ncol;
         const int atom_t = satom[t];
-        if (in_prev) {
+        if (in_prev && part == 0) {
           T pt[N];
           load_row<T, N, PS>(prev + (size_t)t * PS, pt);
           const T* e = E + (size_t)atom_t * NO;
@@ -638,12 +647,23 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
 #pragma unroll
             for (int c = 0; c < NC; c++) acc[r_][c] = T(0);
         }
-        const unsigned long long lc = L.stage ? s_lvc[t] : lvc[t];
-        const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
-        if (cnt > 0) {
-          const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
-          gather_pf2<T, NO, NC, PS>(L.stage ? s_adj + q0 : adj + q0, cnt, H, HS, prev, acc);
+        if (live) {
+          const unsigned long long lc = L.stage ? s_lvc[t] : lvc[t];
+          const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
+          const int mine = big ? (cnt + 1 - part) >> 1 : cnt;
+          const int q0 = (L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase)) + part;
+          gather_pf2<T, NO, NC, PS>(L.stage ? s_adj + q0 : adj + q0, big ? 2 : 1, mine, H, HS, prev, acc);
         }
+        if (sizeof(T) == 8 && __any_sync(0xffffffffu, big)) {
+#pragma unroll
+          for (int r_ = 0; r_ < NO; r_++)
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+              const T o = __shfl_xor_sync(0xffffffffu, acc[r_][c], 1);
+              if (big) acc[r_][c] += o;
+            }
+        }
+        if (!live || part != 0) continue;
         // row t of Psi_k-1 again (shared memory), rather than kept live over the gather
         const bool other = half && t != 0;
         double* mt = mu + ((size_t)spin * n + atom_t) * NO * n_mom + 2 * K - 1;  // the last two moments of atom_t
@@ -815,7 +835,7 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
       for (int t = tid; t < neb; t += NT) store_row<T, N, PS>(xK + (size_t)t * PS, zero);
       __syncthreads();
     }
-    const int nK = pair ? cv.ntop[atom] : s_lev[K];
+    const int nK = pair ? cv.ntop[atom] & 0xffff : s_lev[K];
     for (int q = tid; q < nK; q += NT) {
       const int t = pair ? (int)(top[q] & 0xffffu) : q;
       // weights of the site's atom (rows), in the pair form
