@@ -483,8 +483,10 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     CKS(ensure(c, c->adj_off, sizeof(long long) * (c->nsite + 1)));
     CKS(ensure(c, c->adj, sizeof(int2) * c->nadj));
     CKS(ensure(c, c->lvcnt, sizeof(unsigned long long) * c->nsite));
-    CKS(ensure(c, c->order, sizeof(unsigned) * c->nsite));
-    out.order = P<unsigned>(c->order);
+    if (c->fp64) {  // row orders of the FP64 kernels
+      CKS(ensure(c, c->order, sizeof(unsigned) * c->nsite));
+      out.order = P<unsigned>(c->order);
+    }
     out.site_off = P<long long>(c->site_off);
     out.adj_base = P<long long>(c->adj_base);
     out.site_atom = P<int>(c->site_atom);
@@ -597,8 +599,10 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
     CKS(ensure(c, c->adj_off, sizeof(long long) * (c->nsite + 1)));
     CKS(ensure(c, c->adj, sizeof(int2) * c->nadj));
     CKS(ensure(c, c->lvcnt, sizeof(unsigned long long) * c->nsite));
-    CKS(ensure(c, c->order, sizeof(unsigned) * c->nsite));
-    out.order = P<unsigned>(c->order);
+    if (c->fp64) {  // row orders of the FP64 kernels
+      CKS(ensure(c, c->order, sizeof(unsigned) * c->nsite));
+      out.order = P<unsigned>(c->order);
+    }
     out.site_off = P<long long>(c->site_off);
     out.adj_base = P<long long>(c->adj_base);
     out.site_atom = P<int>(c->site_atom);
@@ -623,7 +627,7 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
 }
 
 ClusterView cview(bop_ctx* c) {
-  return ClusterView{P<long long>(c->site_off), P<int>(c->level_end), P<int>(c->site_atom),
+  return ClusterView{P<long long>(c->site_off), P<int>(c->level_end), P<int>(c->site_atom), P<signed char>(c->site_img),
                      P<long long>(c->adj_off), P<int2>(c->adj), P<unsigned long long>(c->lvcnt), c->K,
                      P<unsigned>(c->order), c->pair_ok ? P<unsigned>(c->top) : nullptr, P<int>(c->ntop),
                      P<unsigned>(c->topmask)};
@@ -690,6 +694,24 @@ int nc_args(bop_ctx* c, NcArgs* a) {
     int& cap = (k & 1) ? a->cap_odd : a->cap_even;
     if (c->maxlev[k] > cap) cap = c->maxlev[k];
   }
+  a->rev_even = a->rev_odd = 1;
+  for (int k = 1; k <= c->K; k++) {
+    int& cap = (k & 1) ? a->rev_odd : a->rev_even;
+    if (c->maxlev[k] > cap) cap = c->maxlev[k];
+  }
+  a->max_sites = c->maxlev[c->K] > 0 ? c->maxlev[c->K] : 1;
+  a->max_adj = c->maxlev[c->K + 1] > 0 ? c->maxlev[c->K + 1] : 1;
+  a->cap_eb = c->maxlev[c->K - 1] > 0 ? c->maxlev[c->K - 1] : 1;
+  a->rev_adj = a->max_adj;
+  if (a->rev_adj > (long long)a->cap_eb * c->grid_max[0]) a->rev_adj = a->cap_eb * c->grid_max[0];
+  a->psi_off = P<long long>(c->psi_off);
+  a->psi_tot = c->psi_tot;
+  return BOP_OK;
+}
+
+// Per-CTA scratch of k_nc (Psi and Psi-bar of all levels of one work item),
+// which runs where two levels do not fit shared memory or Psi is not stored.
+int nc_scratch(bop_ctx* c, NcArgs* a) {
   long long levsum = 0;
   for (int k = 0; k <= c->K; k++) levsum += c->maxlev[k];
   a->slot_elems = 2 * (size_t)levsum * c->norb * 8 + 64;
@@ -711,6 +733,8 @@ int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s
     CKS(ensure(c, c->vmom, sizeof(double) * (size_t)c->n * c->norb * c->n_mom * 3));
     a.mu = mu;
     a.vmom = P<double>(c->vmom);
+    a.pstore = pstore;
+    if (!nc_in_shared(a, c->fp64)) CKS(nc_scratch(c, &a));
     Region R(c, PK_MOMENTS, 1, s);
     if (launch_nc(a, c->fp64, s)) return fail(c, BOP_ERR_CUDA, "spinor moments launch failed");
     return BOP_OK;
@@ -1039,7 +1063,13 @@ int psi_row(int N, int fp64) {
 int psi_store_alloc(bop_ctx* c, bool* fits) {
   *fits = false;
   const size_t esz = c->fp64 ? sizeof(double) : sizeof(float);
-  const size_t bytes = (size_t)c->S * (size_t)c->psi_tot * psi_row(c->norb * c->norb, c->fp64) * esz;
+  size_t bytes = (size_t)c->S * (size_t)c->psi_tot * psi_row(c->norb * c->norb, c->fp64) * esz;
+  if (c->m.noncollinear) {
+    NcArgs a;
+    CKS(nc_args(c, &a));
+    if (!nc_in_shared(a, c->fp64)) return BOP_OK;
+    bytes = (size_t)c->norb * (size_t)c->psi_tot * c->norb * 8 * esz;
+  }
   size_t freeb = 0, totalb = 0;
   CK(cudaMemGetInfo(&freeb, &totalb));
   const size_t held = c->psis.bytes;
@@ -1052,8 +1082,8 @@ int psi_store_alloc(bop_ctx* c, bool* fits) {
 int prepare_psi_store(bop_ctx* c, cudaStream_t s) {
   // the SCF loop may have stored Psi in its forward passes; the last one is
   // at the final onsite levels
-  c->forces_follow = !c->m.noncollinear;
-  if (c->m.scf == BOP_SCF_VARIATIONAL || c->psi_valid || c->m.noncollinear) return BOP_OK;
+  c->forces_follow = true;
+  if (c->m.scf == BOP_SCF_VARIATIONAL || c->psi_valid) return BOP_OK;
   // a forward pass that stores Psi and the stored-Psi sweeps cost less than
   // the recomputing sweep even for one sweep (131,072 atoms: 12 + 21 ms
   // against 71 ms), so store whenever it fits
@@ -1934,6 +1964,8 @@ int bop_forces(bop_ctx* c, double* forces, double* virial, bop_stats* st, bop_st
       a.Hbar = c->Hbar.p;
       a.HSh = bond_cotangent_stride(c->norb, c->fp64);
       a.obar = P<double>(c->obar);
+      if (c->psi_valid) a.pstore = c->psis.p;
+      else CKS(nc_scratch(c, &a));
       {
         Region R(c, PK_ADJOINT, 1, s);
         if (launch_nc(a, c->fp64, s)) return fail(c, BOP_ERR_CUDA, "spinor reverse sweep launch failed");

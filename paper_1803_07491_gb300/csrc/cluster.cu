@@ -276,7 +276,7 @@ k_cluster(int n, int K, const long long* __restrict__ row_ptr, const int* __rest
             lc |= (unsigned long long)cnt << (8 * k);
           }
           out.lvcnt[s0 + t] = lc;
-          out.order[s0 + t] = (unsigned)t | ((unsigned)t << 16);
+          if (out.order != nullptr) out.order[s0 + t] = (unsigned)t | ((unsigned)t << 16);
           // forward levels k = max(lt, ls+1) .. K use the pair (t, s)
           int lt = 0;
           while (lt < K && t >= s_lev[lt]) lt++;
@@ -800,6 +800,7 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
       const int S2 = A.sites;
       for (int w = tid >> 5; w < 3; w += G / 32) {
         int* off = ocnt + w * ORDER_KEYS;
+        if (w < 2 && out.order == nullptr) continue;
         if (w < 2) {  // by shell, then descending entries of the level below / up to its own
           const int sh = 8 * w;
           warp_order(nsite, (K + 1) * 33, off, lane,
@@ -811,14 +812,15 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
         }
       }
       group_sync<G>();
-      for (int q = tid; q < nsite; q += G) out.order[s0 + q] = (unsigned)ord[q] | ((unsigned)ord[S2 + q] << 16);
+      if (out.order != nullptr)
+        for (int q = tid; q < nsite; q += G) out.order[s0 + q] = (unsigned)ord[q] | ((unsigned)ord[S2 + q] << 16);
       if (out.top != nullptr) {
         if (tid < 32) {  // the selected sites in the order of the last level's rows
           int run = 0, in = 0;
           const int l2 = K >= 2 ? s_lev[K - 2] : 0, l1 = s_lev[K - 1];
           for (int q0 = 0; q0 < nsite; q0 += 32) {
             const int q = q0 + lane;
-            const int t = q < nsite ? (q < l2 ? q : (q < l1 ? ord[S2 + q] : ord[q])) : 0;
+            const int t = q >= nsite ? 0 : (out.order == nullptr || q < l2 ? q : (q < l1 ? ord[S2 + q] : ord[q]));
             bool sel = false;
             if (q < nsite) {
               const unsigned long long r = gk[t];

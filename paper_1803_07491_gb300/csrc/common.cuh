@@ -31,6 +31,7 @@ struct ClusterView {
   const long long* site_off;  // [n+1] first site of each atom
   const int* level_end;       // [n][K+1] sites [0, level_end[k]) form C_k
   const int* site_atom;       // [S] atom of every site
+  const signed char* site_img;  // [S][3] its periodic image
   const long long* adj_off;   // [S+1] adjacency of every site
   const int2* adj;            // {neighbour site (local index), bond}, ascending site
   const unsigned long long* lvcnt;  // [S] byte k = entries with site < level_end[k]
@@ -39,7 +40,7 @@ struct ClusterView {
   // rows of a warp are about equally long: within each shell (the sites first
   // reached at one level) by descending entries, low half: entries of the
   // level below (the row's work at its own level), high half: entries of the
-  // levels up to its own (its work one level on)
+  // levels up to its own (its work one level on); NULL in FP32
   const unsigned* order;      // [S]
   // Pair form of the last level (NULL without it; see pair_selected): low
   // half: the selected sites, those of C_K-1 first, each part by descending

@@ -40,7 +40,7 @@ struct ClusterOut {
   int2* adj;             // [A]
   unsigned long long* n_products;  // block products of one moments pass (pass 2)
   unsigned long long* lvcnt;       // [S] per-level entry counts (pass 2)
-  unsigned* order;                 // [S] ClusterView (pass 2)
+  unsigned* order;                 // [S] ClusterView, may be null (pass 2)
   unsigned* top;                   // [S], [n], [S]: the pair form of the last level, may be null (pass 2)
   int* ntop;
   unsigned* topmask;
@@ -132,8 +132,8 @@ struct MomentsArgs {
   void* pstore;
   const long long* psi_off;  // [n+1] prefix sums of sum_k |C_k| over atoms
   long long psi_tot;
-  // last level in the pair form (needs cv.top; every atom a centre): stores,
-  // then, the selected rows of Psi_K only
+  // pair form (needs cv.top; every atom a centre): FP64 computes, and both
+  // precisions store, the selected rows of Psi_K only
   bool pair;
   // Psi of two levels in global memory (moments_in_gmem): in the store, or in
   // scratch, one slot (moments_slot_bytes) per CTA
@@ -189,6 +189,14 @@ struct NcArgs {
   const double* sdir;  // [n][3] unit moment directions
   int n, norb, n_mom;
   int cap_even, cap_odd;  // largest even / odd level |C_k| (k < K) over atoms (forward in shared memory)
+  int rev_even, rev_odd;  // the same for k = 1..K (Psi-bar), |C_K-1| and the entries of its rows
+  int cap_eb, rev_adj;
+  int max_sites, max_adj; // largest cluster, largest adjacency
+  // store of every Psi_k for the reverse sweep (NULL: none; k_nc recomputes):
+  // rows of norb x 8 reals of item (atom, alpha) at alpha psi_tot + psi_off[atom]
+  void* pstore;
+  const long long* psi_off;
+  long long psi_tot;
   void* scratch;       // per-CTA Psi / Psi-bar storage
   size_t slot_elems;   // elements of T per CTA: 2 sum_k max |C_k| norb 8
   int slots;
@@ -201,6 +209,8 @@ struct NcArgs {
   int HSh;
   double* obar;        // [n][norb][4] (+=): d/d(Ebar, h_x, h_y, h_z)
 };
+// Both sweeps hold two levels (and the onsite cotangents) in shared memory.
+bool nc_in_shared(const NcArgs& a, int fp64);
 int launch_nc(const NcArgs& a, int fp64, cudaStream_t s);
 int launch_torques(int n, int norb, int n_mom, const double* onsite, const double* sdir, const double* w,
                    const double* vmom, const double* obar, double* t, cudaStream_t s);

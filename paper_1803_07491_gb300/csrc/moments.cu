@@ -517,19 +517,25 @@ __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int fir
 // block loads of five items that fit.  FP64 is bound by its DFMA pipe either
 // way (328 bytes per 125 DFMA, 62 cycles of an SM).
 //
-// Rows run in the order of their length (ClusterView::order): the 1 to 6
-// entries of an outer shell's row and the 14 of an inner one no longer share a
-// warp, whose other lanes would idle for the longest row; odd passes over the
-// threads run backwards, so that the warp with the longest rows of one pass
-// gets the shortest of the next.  FP64: the long rows of a small level have two
-// lanes each, which halves the longest chain between two barriers (432-atom
-// Stoner cell: 0.83 -> 0.78 ms per pass; in FP32, bound by the L1, 3 %).
+// FP64: rows run in the order of their length (ClusterView::order): the 1 to
+// 6 entries of an outer shell's row and the 14 of an inner one no longer share
+// a warp, whose other lanes would idle for the longest row; odd passes over
+// the threads run backwards, so that the warp with the longest rows of one
+// pass gets the shortest of the next; and the long rows of a small level have
+// two lanes each, which halves the longest chain between two barriers (432-atom
+// Stoner cell: 1.57 -> 0.78 ms per pass with the pair form).
 //
-// pair: the last level (68 % of the products of a bcc cluster at 9 moments)
-// computes the selected sites only (pair_selected).  H^K is symmetric, so the
-// block Z = Psi_K(t, i) holds Psi_K(i, t)^T too: its column sums go to this
-// item's last two moments and its row sums to those of the site's atom, all
-// with FP64 atomics onto moments that start at zero.
+// FP64, pair: the last level (68 % of the products of a bcc cluster at 9
+// moments) computes the selected sites only (pair_selected).  H^K is
+// symmetric, so the block Z = Psi_K(t, i) holds Psi_K(i, t)^T too: its column
+// sums go to this item's last two moments and its row sums to those of the
+// site's atom, all with FP64 atomics onto moments that start at zero.
+//
+// FP32 keeps one lane per site, in site order, and the sums in that order: the
+// band edges are a maximum over levels, and moments rounded differently send
+// a few orbitals of 100,000 to the other side of a tie, where the forces jump.
+// (Row order and pair form gained 5 % there: the pass is bound by the L1 data
+// path, which idle lanes do not load.)
 template <typename T>
 struct Fwd {
   // FP64: one DFMA of a warp takes 64 cycles of an SM sub-partition, so that
@@ -543,13 +549,22 @@ struct FwdSmem {
   bool stage;
 };
 
+// Whether site t (atom j) of centre i is selected (pair_selected).
+__device__ __forceinline__ bool site_selected(const ClusterView& cv, long long s0, int i, int j, int t) {
+  if (i != j) return pair_selected(i, j, 0, 0, 0);
+  const signed char* im = cv.site_img + 3 * (s0 + t);
+  return pair_selected(i, j, im[0], im[1], im[2]);
+}
+
 template <typename T, int NO, bool GMEM>
 __global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
 k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
           int n_mom, FwdSmem L, int n_items, int chunk, double* __restrict__ mu, T* __restrict__ pstore,
-          const long long* __restrict__ psi_off, long long psi_tot, bool pair, T* __restrict__ scratch,
-          size_t slot_elems) {
+          const long long* __restrict__ psi_off, long long psi_tot, bool pair_form, bool sel_store,
+          T* __restrict__ scratch, size_t slot_elems) {
   constexpr int NT = Fwd<T>::THREADS, NC = NO;
+  constexpr bool ORDERED = sizeof(T) == 8;
+  const bool pair = ORDERED && pair_form;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -562,7 +577,7 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
   int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.max_sites : 0));
   int* s_atom = s_off + (L.stage ? L.max_sites + 1 : 0);
   unsigned* s_ord = reinterpret_cast<unsigned*>(s_atom + (L.stage ? L.max_sites : 0));
-  unsigned* s_top = s_ord + (L.stage ? L.max_sites : 0);
+  unsigned* s_top = s_ord + (L.stage && ORDERED ? L.max_sites : 0);
   // per-warp partial sums of the two moments of a level, in two buffers
   // (level parity): the reads of level k's partials need no barrier before
   // level k + 1 starts writing its own
@@ -587,7 +602,7 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     const unsigned* top = L.stage ? s_top : cv.top + s0;
     const T* E = onsite + (size_t)spin * n_on * NO;
     if (L.stage) {
-      stage_order(cv, cur, pair, s_ord, s_top, tid, NT);
+      if (ORDERED) stage_order(cv, cur, pair, s_ord, s_top, tid, NT);
       stage_item(cv, cur, cur.nsite, (int)(cur.aend - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
     }
     const int ntop = pair ? cv.ntop[atom] : 0;
@@ -614,20 +629,21 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
       // of at most two passes, get two lanes each; the sites first reached at
       // this level (1 to 6 entries) one
       const int nrow = half ? ntop & 0xffff : lev[k];
-      const int nbig = sizeof(T) == 8 && nrow <= 2 * NT ? (half ? ntop >> 16 : ncol) : 0;
+      const int nbig = ORDERED && nrow <= 2 * NT ? (half ? ntop >> 16 : ncol) : 0;
       T* next = buf[k & 1];
       T d1[NC], d2[NC];
 #pragma unroll
       for (int c = 0; c < NC; c++) d1[c] = d2[c] = T(0);
       for (int p = 0; p * NT < nrow + nbig; p++) {
-        const int v = p * NT + ((p & 1) ? NT - 1 - tid : tid);
+        const int v = p * NT + (ORDERED && (p & 1) ? NT - 1 - tid : tid);
         const bool big = v < 2 * nbig, live = v < nrow + nbig;
         const int part = big ? v & 1 : 0;
         const int r = !live ? 0 : (big ? v >> 1 : v - nbig);
         // rows up to level k-2 are full, shell k-1 has entries up to its own
         // level, shell k of the one below
-        const int t = half ? (int)(top[r] & 0xffffu)
-                           : (r < inner ? r : (r < ncol ? (int)(order[r] >> 16) : (int)(order[r] & 0xffffu)));
+        const int t = !ORDERED ? r
+                      : half   ? (int)(top[r] & 0xffffu)
+                               : (r < inner ? r : (r < ncol ? (int)(order[r] >> 16) : (int)(order[r] & 0xffffu)));
         T acc[NO][NC];
         const bool in_prev = t < ncol;
         const int atom_t = satom[t];
@@ -654,7 +670,7 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
           const int q0 = (L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase)) + part;
           gather_pf2<T, NO, NC, PS>(L.stage ? s_adj + q0 : adj + q0, big ? 2 : 1, mine, H, HS, prev, acc);
         }
-        if (sizeof(T) == 8 && __any_sync(0xffffffffu, big)) {
+        if (ORDERED && __any_sync(0xffffffffu, big)) {
 #pragma unroll
           for (int r_ = 0; r_ < NO; r_++)
 #pragma unroll
@@ -675,9 +691,8 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
             T a = T(0);
 #pragma unroll
             for (int c = 0; c < NC; c++) {
-              const T v = pt[r_ * NC + c] * acc[r_][c];
-              d1[c] += v;
-              a += v;
+              d1[c] += pt[r_ * NC + c] * acc[r_][c];
+              a += pt[r_ * NC + c] * acc[r_][c];
             }
             if (other) atomicAdd(mt + r_ * n_mom, (double)a);
           }
@@ -687,14 +702,14 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
           T a = T(0);
 #pragma unroll
           for (int c = 0; c < NC; c++) {
-            const T v = acc[r_][c] * acc[r_][c];
-            d2[c] += v;
-            a += v;
+            d2[c] += acc[r_][c] * acc[r_][c];
+            a += acc[r_][c] * acc[r_][c];
           }
           if (other) atomicAdd(mt + r_ * n_mom + 1, (double)a);
         }
         if (k < K && !in_store) store_row<T, N, PS>(next + (size_t)t * PS, &acc[0][0]);
-        if (pitem != nullptr) store_row<T, N, PS>(pitem + (size_t)(lo_k + t) * PS, &acc[0][0]);
+        if (pitem != nullptr && (half || k < K || !sel_store || site_selected(cv, s0, atom, atom_t, t)))
+          store_row<T, N, PS>(pitem + (size_t)(lo_k + t) * PS, &acc[0][0]);
       }
 #pragma unroll
       for (int c = 0; c < NC; c++) {
@@ -1448,92 +1463,314 @@ k_nc(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsi
   }
 }
 
-// Forward-only form of k_nc: Psi_k-1 and Psi_k in two shared-memory
-// buffers (even and odd levels, each sized for the largest such level
-// below K over all atoms; Psi_K is never stored, only its inner products).
+// The same over stored Psi, as k_moments and k_adj_rev: work items (atom,
+// alpha), the NO items of an atom consecutive in one CTA, which stages the
+// atom's cluster once; Psi (Psi-bar) of two levels in shared memory, blocks of
+// two entries in flight, FP64 rows in the order of their length (FP32 ones in
+// site order over 256 threads, for sums in a fixed order as in k_moments).  One site row
+// holds NO x 8 reals, so that a block feeds 8 NO^2 multiply-adds.
+template <typename T>
+struct NcFwd {
+  static constexpr int THREADS = sizeof(T) == 4 ? 256 : 128;
+};
+
 template <typename T, int NO>
-__global__ void __launch_bounds__(MOM_THREADS)
+__global__ void __launch_bounds__(NcFwd<T>::THREADS, 2)
 k_nc_fwd(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite,
-         const double* __restrict__ sdir, int n, int n_mom, int nwork, int cap_even, double* __restrict__ mu,
-         double* __restrict__ vmom) {
-  constexpr int RW = NO * NCS;
+         const double* __restrict__ sdir, int n, int n_mom, FwdSmem L, int n_items, int chunk,
+         double* __restrict__ mu, double* __restrict__ vmom, T* __restrict__ pstore,
+         const long long* __restrict__ psi_off, long long psi_tot) {
+  constexpr int NT = NcFwd<T>::THREADS;
+  constexpr bool ORDERED = sizeof(T) == 8;
+  constexpr int PS = NO * NCS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* const buf0 = reinterpret_cast<T*>(smem_raw);
-  T* const buf1 = buf0 + (size_t)cap_even * RW;
-  __shared__ int s_lev[BOP_MAX_K + 1];
-  __shared__ T red[8][MOM_THREADS / 32];
+  T* buf[2];
+  buf[0] = reinterpret_cast<T*>(smem_raw);
+  buf[1] = buf[0] + (size_t)L.cap_even * PS;
+  int2* s_adj = reinterpret_cast<int2*>(align16(reinterpret_cast<unsigned char*>(buf[1] + (size_t)L.cap_odd * PS)));
+  unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
+  int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.max_sites : 0));
+  int* s_atom = s_off + (L.stage ? L.max_sites + 1 : 0);
+  unsigned* s_ord = reinterpret_cast<unsigned*>(s_atom + (L.stage ? L.max_sites : 0));
+  __shared__ T red[2][8][NT / 32];
   __shared__ double chi[NCS];
   const int K = cv.K;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
+  const int w0 = blockIdx.x * chunk, w1 = min(n_items, w0 + chunk);
+  int held = -1;  // the atom whose cluster is staged
+  for (int w = w0; w < w1; w++) {
     const int atom = w / NO, al = w % NO;
-    const long long s0 = cv.site_off[atom];
+    ItemExt cur;
+    ext_sites(cv, atom, cur);
+    ext_adj(cv, cur);
+    const long long s0 = cur.s0, abase = cur.abase;
     const int* lev = cv.level_end + (size_t)atom * (K + 1);
-    const int* satom = cv.site_atom + s0;
-    const long long* aoff = cv.adj_off + s0;
-    if (tid <= K) s_lev[tid] = lev[tid];
-    if (tid == 0) start_spinors(sdir + 3 * (size_t)atom, chi);
-    __syncthreads();
-    for (int q = tid; q < RW; q += blockDim.x) buf0[q] = (q / NCS == al) ? (T)chi[q % NCS] : T(0);
+    const unsigned long long* lvc = L.stage ? s_lvc : cv.lvcnt + s0;
+    const int* satom = L.stage ? s_atom : cv.site_atom + s0;
+    const unsigned* order = L.stage ? s_ord : cv.order + s0;
+    const int2* adj = L.stage ? s_adj : cv.adj + abase;
+    if (atom != held) {
+      if (L.stage) {
+        if (ORDERED) stage_order(cv, cur, false, s_ord, nullptr, tid, NT);
+        stage_item(cv, cur, cur.nsite, (int)(cur.aend - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
+      }
+      if (tid == 0) start_spinors(sdir + 3 * (size_t)atom, chi);
+      held = atom;
+      __syncthreads();
+    }
+    T* pitem = pstore != nullptr ? pstore + ((size_t)al * psi_tot + psi_off[atom]) * PS : nullptr;
+    for (int q = tid; q < PS; q += NT) {
+      const T v = (q / NCS == al) ? (T)chi[q % NCS] : T(0);
+      buf[0][q] = v;
+      if (pitem != nullptr) pitem[q] = v;
+    }
     if (tid < 2) {
       mu[(((size_t)tid * n + atom) * NO + al) * n_mom] = 1.0;
       vmom[(((size_t)atom * NO + al) * n_mom) * 3 + tid] = 0.0;
       if (tid == 0) vmom[(((size_t)atom * NO + al) * n_mom) * 3 + 2] = 0.0;
     }
     __syncthreads();
+    long long lo_k = 0;
     for (int k = 1; k <= K; k++) {
-      const T* x = (k & 1) ? buf0 : buf1;  // level k-1
-      T* y = (k & 1) ? buf1 : buf0;        // level k
+      lo_k += lev[k - 1];
+      const int nrow = lev[k], ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
+      const T* prev = buf[(k - 1) & 1];
+      T* next = buf[k & 1];
       T d[8];
 #pragma unroll
       for (int v = 0; v < 8; v++) d[v] = T(0);
-      for (int t = tid; t < s_lev[k]; t += blockDim.x) {
+      for (int p = 0; p * NT < nrow; p++) {
+        const int r = p * NT + (ORDERED && (p & 1) ? NT - 1 - tid : tid);
+        if (r >= nrow) continue;
+        const int t = !ORDERED || r < inner ? r : (r < ncol ? (int)(order[r] >> 16) : (int)(order[r] & 0xffffu));
+        const bool in_prev = t < ncol;
         T acc[NO][NCS];
-        gather_row_nc<T, NO>(cv, H, HS, onsite, sdir, n, satom, aoff, t, s_lev[k - 1], x, acc);
+        if (in_prev) {
+          const int j = satom[t];
+          const T sx = (T)sdir[3 * (size_t)j], sy = (T)sdir[3 * (size_t)j + 1], sz = (T)sdir[3 * (size_t)j + 2];
+          T pt[PS];
+          load_row<T, PS, PS>(prev + (size_t)t * PS, pt);
 #pragma unroll
-        for (int r = 0; r < NO; r++) {
-          const T* a = acc[r];
+          for (int b = 0; b < NO; b++) {
+            const T eu = onsite[(size_t)j * NO + b], ed = onsite[((size_t)n + j) * NO + b];
+            const T f = T(0.5) * (ed - eu);
+            spin_onsite<T>(T(0.5) * (eu + ed), f * sx, f * sy, f * sz, pt + b * NCS, acc[b]);
+          }
+        } else {
+#pragma unroll
+          for (int b = 0; b < NO; b++)
+#pragma unroll
+            for (int c = 0; c < NCS; c++) acc[b][c] = T(0);
+        }
+        const int cnt = (int)((lvc[t] >> (8 * (k - 1))) & 0xff);
+        const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+        gather_pf2<T, NO, NCS, PS>(adj + q0, 1, cnt, H, HS, prev, acc);
+        T pt[PS];
+        if (in_prev) {
+          load_row<T, PS, PS>(prev + (size_t)t * PS, pt);
+        } else {
+#pragma unroll
+          for (int v = 0; v < PS; v++) pt[v] = T(0);
+        }
+        // <Psi^nu|Psi^nu'>: up-up, dn-dn, and Re / Im of up-dn
+#pragma unroll
+        for (int b = 0; b < NO; b++) {
+          const T* a = acc[b];
+          const T* q = pt + b * NCS;
           d[4] += a[0] * a[0] + a[1] * a[1] + a[2] * a[2] + a[3] * a[3];
           d[5] += a[4] * a[4] + a[5] * a[5] + a[6] * a[6] + a[7] * a[7];
           d[6] += a[0] * a[4] + a[1] * a[5] + a[2] * a[6] + a[3] * a[7];
           d[7] += a[0] * a[5] - a[1] * a[4] + a[2] * a[7] - a[3] * a[6];
-          if (t < s_lev[k - 1]) {
-            const T* p = x + ((size_t)t * NO + r) * NCS;
-            d[0] += p[0] * a[0] + p[1] * a[1] + p[2] * a[2] + p[3] * a[3];
-            d[1] += p[4] * a[4] + p[5] * a[5] + p[6] * a[6] + p[7] * a[7];
-            d[2] += p[0] * a[4] + p[1] * a[5] + p[2] * a[6] + p[3] * a[7];
-            d[3] += p[0] * a[5] - p[1] * a[4] + p[2] * a[7] - p[3] * a[6];
-          }
+          d[0] += q[0] * a[0] + q[1] * a[1] + q[2] * a[2] + q[3] * a[3];
+          d[1] += q[4] * a[4] + q[5] * a[5] + q[6] * a[6] + q[7] * a[7];
+          d[2] += q[0] * a[4] + q[1] * a[5] + q[2] * a[6] + q[3] * a[7];
+          d[3] += q[0] * a[5] - q[1] * a[4] + q[2] * a[7] - q[3] * a[6];
         }
-        if (k < K) {
-#pragma unroll
-          for (int r = 0; r < NO; r++)
-#pragma unroll
-            for (int c = 0; c < NCS; c++) y[((size_t)t * NO + r) * NCS + c] = acc[r][c];
-        }
+        if (k < K) store_row<T, PS, PS>(next + (size_t)t * PS, &acc[0][0]);
+        if (pitem != nullptr) store_row<T, PS, PS>(pitem + (size_t)(lo_k + t) * PS, &acc[0][0]);
       }
 #pragma unroll
       for (int v = 0; v < 8; v++) {
         const T r_ = warp_sum(d[v]);
-        if (lane == 0) red[v][wid] = r_;
+        if (lane == 0) red[k & 1][v][wid] = r_;
       }
       __syncthreads();
       if (tid < 2) {  // moment 2k-1 (tid 0) and 2k (tid 1)
-        double L[4];
+        double Lm[4];
         for (int v = 0; v < 4; v++) {
           T a = T(0);
-          for (int q = 0; q < MOM_THREADS / 32; q++) a += red[4 * tid + v][q];
-          L[v] = (double)a;
+          for (int q = 0; q < NT / 32; q++) a += red[k & 1][4 * tid + v][q];
+          Lm[v] = (double)a;
         }
         const int m = 2 * k - 1 + tid;
-        mu[((size_t)atom * NO + al) * n_mom + m] = L[0];
-        mu[(((size_t)n + atom) * NO + al) * n_mom + m] = L[1];
+        mu[((size_t)atom * NO + al) * n_mom + m] = Lm[0];
+        mu[(((size_t)n + atom) * NO + al) * n_mom + m] = Lm[1];
         double v3[3];
-        pauli_from_local(chi, L[0], L[1], L[2], L[3], v3);
+        pauli_from_local(chi, Lm[0], Lm[1], Lm[2], Lm[3], v3);
         for (int xx = 0; xx < 3; xx++) vmom[(((size_t)atom * NO + al) * n_mom + m) * 3 + xx] = v3[xx];
       }
+    }
+    __syncthreads();  // chi and the partials are read before the next item writes them
+  }
+}
+
+// Reverse sweep over the stored spinor Psi (k_nc_fwd), with the bond
+// cotangents and the onsite-matrix cotangents, the latter summed over the
+// levels of an item in shared memory.  2,000 atoms, FP32: 10.2 ms with Psi
+// recomputed in global scratch (k_nc) -> 2.7 ms.  128 threads: a row's Psi-bar, Psi_k-1,
+// sums and blocks take more registers than 168.
+template <typename T, int NO>
+__global__ void __launch_bounds__(128, 2)
+k_nc_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite,
+         const double* __restrict__ sdir, int n, int n_mom, RevSmem L, int n_items, int chunk,
+         const T* __restrict__ pstore, const long long* __restrict__ psi_off, long long psi_tot,
+         const double* __restrict__ wts, T* __restrict__ Hbar, int HSh, double* __restrict__ obar) {
+  constexpr int NT = 128;
+  constexpr int PS = NO * NCS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* buf[2];
+  buf[0] = reinterpret_cast<T*>(smem_raw);
+  buf[1] = buf[0] + (size_t)L.cap_even * PS;
+  T* eb = buf[1] + (size_t)L.cap_odd * PS;  // [cap_eb][NO][4]
+  int2* s_adj = reinterpret_cast<int2*>(align16(reinterpret_cast<unsigned char*>(eb + (size_t)L.cap_eb * NO * 4)));
+  unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
+  int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.cap_eb : 0));
+  int* s_atom = s_off + (L.stage ? L.cap_eb + 1 : 0);
+  __shared__ T ws[2][BOP_MAX_NMOM];
+  const int K = cv.K;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int w0 = blockIdx.x * chunk, w1 = min(n_items, w0 + chunk);
+  int held = -1;
+  for (int w = w0; w < w1; w++) {
+    const int atom = w / NO, al = w % NO;
+    ItemExt cur;
+    ext_sites(cv, atom, cur);
+    cur.abase = cv.adj_off[cur.s0];
+    const long long s0 = cur.s0, abase = cur.abase;
+    const int* lev = cv.level_end + (size_t)atom * (K + 1);
+    const unsigned long long* lvc = L.stage ? s_lvc : cv.lvcnt + s0;
+    const int* satom = L.stage ? s_atom : cv.site_atom + s0;
+    const int2* adj = L.stage ? s_adj : cv.adj + abase;
+    const int neb = lev[K - 1];
+    if (L.stage && atom != held)
+      stage_item(cv, cur, neb, (int)(cv.adj_off[s0 + neb] - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
+    held = atom;
+    for (int q = tid; q < neb * NO * 4; q += NT) eb[q] = T(0);
+    const T* P = pstore + ((size_t)al * psi_tot + psi_off[atom]) * PS;
+    for (int q = tid; q < 2 * n_mom; q += NT) {
+      const int nu = q / n_mom, m = q % n_mom;
+      ws[nu][m] = (T)wts[(((size_t)nu * n + atom) * NO + al) * n_mom + m];
+    }
+    long long lo = 0;  // first stored row of level k
+    for (int k = 0; k < K; k++) lo += lev[k];
+    __syncthreads();
+    // Psi-bar_K
+    for (int t = tid; t < lev[K]; t += NT) {
+      T pk[PS];
+      load_row<T, PS, PS>(P + (size_t)(lo + t) * PS, pk);
+#pragma unroll
+      for (int v = 0; v < PS; v++) pk[v] *= T(2) * ws[(v % NCS) >> 2][2 * K];
+      if (t < neb) {
+        T p1[PS];
+        load_row<T, PS, PS>(P + (size_t)(lo - neb + t) * PS, p1);
+#pragma unroll
+        for (int v = 0; v < PS; v++) pk[v] += ws[(v % NCS) >> 2][2 * K - 1] * p1[v];
+      }
+      store_row<T, PS, PS>(buf[K & 1] + (size_t)t * PS, pk);
+    }
+    __syncthreads();
+    for (int k = K; k >= 1; k--) {
+      const T* xb = buf[k & 1];
+      T* yb = buf[(k - 1) & 1];
+      const int nrow = lev[k - 1], nrow2 = k >= 2 ? lev[k - 2] : 0;
+      const long long lo1 = lo - nrow, lo2 = lo1 - nrow2;  // first rows of levels k-1, k-2
+      int psh = 0;                                         // lanes per row, as a shift
+      while (psh < 4 && (nrow << (psh + 1)) <= NT) psh++;
+      const int part = tid & ((1 << psh) - 1);
+      for (int r0 = 0; r0 < nrow; r0 += NT >> psh) {
+        if (r0 + ((tid & ~31) >> psh) >= nrow) continue;  // whole warps
+        const int rr = r0 + (tid >> psh);
+        const bool live = rr < nrow;
+        const int t = live ? rr : 0;
+        T acc[NO][NCS];
+#pragma unroll
+        for (int b = 0; b < NO; b++)
+#pragma unroll
+          for (int c = 0; c < NCS; c++) acc[b][c] = T(0);
+        const int j = satom[t];
+        const T sx = (T)sdir[3 * (size_t)j], sy = (T)sdir[3 * (size_t)j + 1], sz = (T)sdir[3 * (size_t)j + 2];
+        T pt[PS];
+        if (live) {
+          load_row<T, PS, PS>(P + (size_t)(lo1 + t) * PS, pt);
+        } else {
+#pragma unroll
+          for (int v = 0; v < PS; v++) pt[v] = T(0);
+        }
+        if (live && part == 0) {
+          // d/d(Ebar, h) of the onsite matrix of (atom of t, b), and the onsite term
+          T xt[PS];
+          load_row<T, PS, PS>(xb + (size_t)t * PS, xt);
+#pragma unroll
+          for (int b = 0; b < NO; b++) {
+            T o0 = T(0), ox = T(0), oy = T(0), oz = T(0);
+#pragma unroll
+            for (int nu = 0; nu < 2; nu++) {
+              const T* B = xt + b * NCS + 4 * nu;
+              const T* Q = pt + b * NCS + 4 * nu;
+              o0 += B[0] * Q[0] + B[1] * Q[1] + B[2] * Q[2] + B[3] * Q[3];
+              ox += B[0] * Q[2] + B[1] * Q[3] + B[2] * Q[0] + B[3] * Q[1];
+              oy += B[0] * Q[3] - B[1] * Q[2] - B[2] * Q[1] + B[3] * Q[0];
+              oz += B[0] * Q[0] + B[1] * Q[1] - B[2] * Q[2] - B[3] * Q[3];
+            }
+            T* o = eb + ((size_t)t * NO + b) * 4;
+            o[0] += o0;
+            o[1] += ox;
+            o[2] += oy;
+            o[3] += oz;
+            if (k >= 2) {
+              const T eu = onsite[(size_t)j * NO + b], ed = onsite[((size_t)n + j) * NO + b];
+              const T f = T(0.5) * (ed - eu);
+              spin_onsite<T>(T(0.5) * (eu + ed), f * sx, f * sy, f * sz, xt + b * NCS, acc[b]);
+            }
+          }
+        }
+        const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+        int cnt = 0;
+        if (live) {
+          if (k < K) cnt = (int)((lvc[t] >> (8 * k)) & 0xff);
+          else cnt = L.stage ? s_off[t + 1] - q0 : (int)(cv.adj_off[s0 + t + 1] - abase) - q0;
+        }
+        gather_rev<T, NO, NCS, PS, true>(adj + q0, part, 1 << psh, cnt, 0u, false, H, HS, xb, acc, k >= 2, pt, Hbar,
+                                         HSh, lane);
+        for (int o = 1; o < (1 << psh); o <<= 1) {
+#pragma unroll
+          for (int b = 0; b < NO; b++)
+#pragma unroll
+            for (int c = 0; c < NCS; c++) acc[b][c] += __shfl_xor_sync(0xffffffffu, acc[b][c], o);
+        }
+        if (!live || part != 0 || k < 2) continue;
+        T* row = &acc[0][0];
+#pragma unroll
+        for (int v = 0; v < PS; v++) row[v] += T(2) * ws[(v % NCS) >> 2][2 * k - 2] * pt[v];
+        T p[PS];
+        load_row<T, PS, PS>(P + (size_t)(lo + t) * PS, p);
+#pragma unroll
+        for (int v = 0; v < PS; v++) row[v] += ws[(v % NCS) >> 2][2 * k - 1] * p[v];
+        if (t < nrow2) {
+          load_row<T, PS, PS>(P + (size_t)(lo2 + t) * PS, p);
+#pragma unroll
+          for (int v = 0; v < PS; v++) row[v] += ws[(v % NCS) >> 2][2 * k - 3] * p[v];
+        }
+        store_row<T, PS, PS>(yb + (size_t)t * PS, row);
+      }
+      lo = lo1;
       __syncthreads();
     }
+    for (int q = tid; q < neb * NO * 4; q += NT) {
+      const int t = q / (NO * 4);
+      atomicAdd(obar + (size_t)satom[t] * NO * 4 + q % (NO * 4), (double)eb[q]);
+    }
+    __syncthreads();
   }
 }
 
@@ -1561,28 +1798,6 @@ __global__ void k_torques(int n, int norb, int n_mom, const double* __restrict__
   t[3 * (size_t)i + 2] = g[0] * sy - g[1] * sx;
 }
 
-template <typename T, int NO>
-int run_nc(const NcArgs& a, cudaStream_t s) {
-  const int nwork = a.n * NO;
-  if (nwork == 0) return 0;
-  const int grid = nwork < a.slots ? nwork : a.slots;
-  // forward only: both stored levels in shared memory when they fit
-  const size_t smem = (size_t)(a.cap_even + a.cap_odd) * NO * NCS * sizeof(T);
-  if (a.w == nullptr && a.cap_even >= 1 && a.cap_odd >= 1 && smem <= 200 * 1024) {
-    auto fn = k_nc_fwd<T, NO>;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return -1;
-    fn<<<grid, MOM_THREADS, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, nwork,
-                                       a.cap_even, a.mu, a.vmom);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-  }
-  k_nc<T, NO><<<grid, MOM_THREADS, 0, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom,
-                                           nwork, (T*)a.scratch, a.slot_elems, a.mu, a.vmom, a.w, (T*)a.Hbar, a.HSh,
-                                           a.obar);
-  return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
 // CTAs of a persistent kernel and the work items of each.
 template <class F>
 void persistent_grid(F fn, int threads, size_t smem, int n_items, int* grid, int* chunk) {
@@ -1596,6 +1811,64 @@ void persistent_grid(F fn, int threads, size_t smem, int n_items, int* grid, int
   *grid = (n_items + *chunk - 1) / *chunk;
 }
 
+// Spinor sweeps with two levels in shared memory: -2 where they do not fit.
+template <typename T, int NO>
+int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
+  constexpr int NT = NcFwd<T>::THREADS;
+  FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
+  const size_t psi = (size_t)(a.cap_even + a.cap_odd) * NO * NCS * sizeof(T);
+  size_t smem = psi + (size_t)a.max_adj * 8 + (size_t)a.max_sites * (sizeof(T) == 8 ? 16 : 12) + (size_t)(a.max_sites + 1) * 4 + 16;
+  if (smem > 110 * 1024) {
+    L.stage = false;
+    smem = psi;
+  }
+  if (smem > 225 * 1024) return -2;
+  auto fn = k_nc_fwd<T, NO>;
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return -1;
+  const int n_items = a.n * NO;
+  int grid, chunk;
+  persistent_grid(fn, NT, smem, n_items, &grid, &chunk);
+  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, chunk,
+                            a.mu, a.vmom, (T*)a.pstore, a.psi_off, a.psi_tot);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+template <typename T, int NO>
+int run_nc_rev(const NcArgs& a, cudaStream_t s) {
+  RevSmem L{a.rev_even, a.rev_odd, a.max_sites, a.rev_adj, a.cap_eb, true};
+  const size_t psi = ((size_t)(a.rev_even + a.rev_odd) * NO * NCS + (size_t)a.cap_eb * NO * 4) * sizeof(T) + 16;
+  size_t smem = psi + (size_t)a.rev_adj * 8 + (size_t)a.cap_eb * 8 + (size_t)(a.cap_eb + 1) * 4 +
+                (size_t)a.max_sites * 4;
+  // stage the adjacency where that costs no resident CTA
+  if (smem > (psi > 110 * 1024 ? 225 : 110) * 1024) {
+    L.stage = false;
+    smem = psi;
+  }
+  if (smem > 225 * 1024) return -2;
+  auto fn = k_nc_rev<T, NO>;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  const int n_items = a.n * NO;
+  int grid, chunk;
+  persistent_grid(fn, 128, smem, n_items, &grid, &chunk);
+  fn<<<grid, 128, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, chunk,
+                             (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.obar);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+template <typename T, int NO>
+int run_nc(const NcArgs& a, cudaStream_t s) {
+  const int nwork = a.n * NO;
+  if (nwork == 0) return 0;
+  if (a.scratch == nullptr) return a.w == nullptr ? run_nc_fwd<T, NO>(a, s) : run_nc_rev<T, NO>(a, s);
+  const int grid = nwork < a.slots ? nwork : a.slots;
+  k_nc<T, NO><<<grid, MOM_THREADS, 0, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom,
+                                           nwork, (T*)a.scratch, a.slot_elems, a.mu, a.vmom, a.w, (T*)a.Hbar, a.HSh,
+                                           a.obar);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 template <typename T, int NO, bool GMEM>
 int run_forward(const MomentsArgs& a, cudaStream_t s) {
   constexpr int N = NO * NO;
@@ -1604,7 +1877,7 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
   FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
   const size_t psi = GMEM ? 0 : (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T);
   size_t stage = (size_t)a.max_adj * 8 + (size_t)a.max_sites * 8 + (size_t)(a.max_sites + 1) * 4 +
-                 (size_t)a.max_sites * 12 + 16;
+                 (size_t)a.max_sites * (sizeof(T) == 8 ? 12 : 4) + 16;
   size_t smem = psi + stage;
   // stage the adjacency only while two CTAs still fit on an SM
   if (smem > 110 * 1024) {
@@ -1626,10 +1899,10 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
     chunk = (int)((n_items + most - 1) / most);
     grid = (n_items + chunk - 1) / chunk;
   }
-  if (a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
+  if (sizeof(T) == 8 && a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
     return -1;
   fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
-                            a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
+                            a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1731,6 +2004,13 @@ int launch_moments_adjoint(const AdjointArgs& a, int fp64, cudaStream_t s) {
   if (a.norb == 1) return fp64 ? run_adjoint<double, 1>(a, s) : run_adjoint<float, 1>(a, s);
   if (a.norb == 6) return fp64 ? run_adjoint<double, 6>(a, s) : run_adjoint<float, 6>(a, s);
   return fp64 ? run_adjoint<double, 5>(a, s) : run_adjoint<float, 5>(a, s);
+}
+
+bool nc_in_shared(const NcArgs& a, int fp64) {
+  const size_t esz = fp64 ? 8 : 4;
+  const size_t fwd = (size_t)(a.cap_even + a.cap_odd) * a.norb * NCS * esz;
+  const size_t rev = ((size_t)(a.rev_even + a.rev_odd) * a.norb * NCS + (size_t)a.cap_eb * a.norb * 4) * esz + 16;
+  return fwd <= 225 * 1024 && rev <= 225 * 1024;
 }
 
 int launch_nc(const NcArgs& a, int fp64, cudaStream_t s) {
