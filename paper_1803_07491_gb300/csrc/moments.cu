@@ -1684,8 +1684,10 @@ k_nc_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ 
       T* yb = buf[(k - 1) & 1];
       const int nrow = lev[k - 1], nrow2 = k >= 2 ? lev[k - 2] : 0;
       const long long lo1 = lo - nrow, lo2 = lo1 - nrow2;  // first rows of levels k-1, k-2
-      int psh = 0;                                         // lanes per row, as a shift
-      while (psh < 4 && (nrow << (psh + 1)) <= NT) psh++;
+      // lanes per row, as a shift: level 1 only forms bond cotangents; the sums
+      // of the others stay in entry order (the torques are small differences of
+      // the onsite cotangents: split sums moved them by 1.5e-5)
+      const int psh = k == 1 ? 4 : 0;
       const int part = tid & ((1 << psh) - 1);
       for (int r0 = 0; r0 < nrow; r0 += NT >> psh) {
         if (r0 + ((tid & ~31) >> psh) >= nrow) continue;  // whole warps
@@ -1742,12 +1744,6 @@ k_nc_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ 
         }
         gather_rev<T, NO, NCS, PS, true>(adj + q0, part, 1 << psh, cnt, 0u, false, H, HS, xb, acc, k >= 2, pt, Hbar,
                                          HSh, lane);
-        for (int o = 1; o < (1 << psh); o <<= 1) {
-#pragma unroll
-          for (int b = 0; b < NO; b++)
-#pragma unroll
-            for (int c = 0; c < NCS; c++) acc[b][c] += __shfl_xor_sync(0xffffffffu, acc[b][c], o);
-        }
         if (!live || part != 0 || k < 2) continue;
         T* row = &acc[0][0];
 #pragma unroll
