@@ -29,19 +29,27 @@ namespace {
 constexpr int CT = 32;  // threads per block: one orbital per thread, small blocks so that
                          // a few thousand orbitals still spread over all SMs (FP64-bound)
 
-// Fewer orbitals than one warp per SM sub-partition: the FP64 kernels then
-// give each orbital two lanes (the Fermi sums, the two seeds of the response
-// weights) so that every sub-partition's FP64 unit has work; with more
-// orbitals one lane per orbital avoids duplicating the per-orbital setup.
-int few_orbitals(int M) {
-  static int cap = 0;
-  if (cap == 0) {
-    int dev = 0, sms = 0;
+// A double-precision instruction of a warp takes 64 cycles, whatever its
+// active lanes and however independent the next one is, and an SM completes
+// one per 19 cycles (measured with chains of fused multiply-adds): one warp on
+// every SM sub-partition saturates it, and with fewer warps a kernel's time is
+// its warps' instruction count.  Fewer orbitals than that therefore take 2, 4
+// or 8 lanes each, which share an orbital's sums.
+int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cap = (sms > 0 ? sms : 1) * 4 * 32;
+    if (sms < 1) sms = 1;
   }
-  return M < cap;
+  return sms;
+}
+int few_orbitals(int M) { return M < sm_count() * 4 * 32; }
+// log2 of the lanes per orbital of the sums over the coefficients.
+int lane_shift(int M) {
+  const int full = sm_count() * 4 * 32;  // threads: one warp per sub-partition
+  return !few_orbitals(M) ? 0 : (8ll * M <= full ? 3 : (4ll * M <= full ? 2 : 1));
 }
 
 // moments -> (a, b, a_inf, b_inf) -> g_m sigma_m, m = 0..n_exp, stored
@@ -122,45 +130,81 @@ __device__ __forceinline__ void count_and_dos_f32(const float* __restrict__ gs32
   *dNde = (2.f / pi) * s * c1;
 }
 
-// The same sums by a pair of adjacent lanes (par = lane & 1): with
-// sin(k phi) = s U_{k-1}(x), each sum over U_j splits into its even and odd
-// terms, which obey U_{j+2} = y U_j - U_{j-2} with y = 4x^2 - 2; lane 0 runs
-// the even Clenshaw chains (U_0 = 1, U_2 - y U_0 = 1), lane 1 the odd ones
-// (U_1 = 2x, U_3 - y U_1 = 0), exchanged at the end.  An orbital's FP64
-// work thus runs on two lanes (twice the warps for the same orbitals;
-// measured faster than one lane and than four lanes per orbital when there
-// are fewer orbitals than one warp per SM sub-partition).
-// pm: the pair's lane mask.  Both lanes return N and dNde.
-__device__ __forceinline__ void count_and_dos2(const double* __restrict__ gsig, const double* __restrict__ inv,
-                                               int M, int o, int ne, double x, int par, unsigned pm, double* N,
-                                               double* dNde) {
+// The same sums by L = 2^SH adjacent lanes (r: lane of the orbital).  With
+// sin(k phi) = s U_{k-1}(x), lane r takes the terms U_j of j = r + L i, which
+// obey U_{j+L} = y U_j - U_{j-L} with y = 2 T_L(x); its Clenshaw sum ends in
+// b_0 U_r - b_1 U_{r-L}, U_{r-L} = -U_{L-r-2}.
+template <int SH>
+struct LaneBasis {
+  double y, ur, um;  // 2 T_L, U_r, U_{L-r-2}
+  __device__ __forceinline__ LaneBasis(double x, int r) {
+    constexpr int L = 1 << SH;
+    double t = x;
+#pragma unroll
+    for (int q = 0; q < SH; q++) t = 2.0 * t * t - 1.0;
+    y = 2.0 * t;
+    double u1 = 0.0, u0 = 1.0;  // U_{q-1}, U_q
+    ur = um = 0.0;
+#pragma unroll
+    for (int q = 0; q < L; q++) {
+      if (q == r) ur = u0;
+      if (q == L - r - 2) um = u0;
+      const double u2 = 2.0 * x * u0 - u1;
+      u1 = u0;
+      u0 = u2;
+    }
+  }
+  // sum over the orbital's lanes of b_0 U_r + b_1 U_{L-r-2}
+  __device__ __forceinline__ double finish(double b0, double b1, unsigned pm) const {
+    double v = b0 * ur + b1 * um;
+#pragma unroll
+    for (int o = 1; o < (1 << SH); o <<= 1) v += __shfl_xor_sync(pm, v, o);
+    return v;
+  }
+};
+// The lanes of an orbital, as a shuffle mask.
+template <int SH>
+__device__ __forceinline__ unsigned lane_group() {
+  constexpr int L = 1 << SH;
+  return (L == 32 ? 0xffffffffu : (1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
+}
+
+// All lanes return N and dNde.
+template <int SH>
+__device__ __forceinline__ void count_and_dos_lanes(const double* __restrict__ gsig, const double* __restrict__ inv,
+                                                    int M, int o, int ne, double x, int r, double* N, double* dNde) {
+  constexpr int L = 1 << SH;
+  const unsigned pm = lane_group<SH>();
   auto G = [&](int j) -> double { return (j >= 0 && j <= ne) ? gsig[(size_t)j * M + o] : 0.0; };
-  const double y = 4.0 * x * x - 2.0;
-  // lane par sums the terms U_j with j = 2i + par:
-  //   S_par = sum_i a_{j+1} U_j, a_k = (gs_{k-2} - gs_k)/k;  C_par = sum_i gs_j U_j
+  const LaneBasis<SH> B(x, r);
+  // S = sum_j a_{j+1} U_j, a_k = (gs_{k-2} - gs_k)/k;  C = sum_j gs_j U_j
   double b1 = 0.0, b2 = 0.0, c1 = 0.0, c2 = 0.0;
-  const int top = (ne + 2) / 2;
-  double gp = G(2 * top + par + 1);  // gs_{j+1}
+  const int top = (ne + 1) / L;
+  double gp = G(L * top + r + 1);  // gs_{j+1}; two lanes: the step's gs_{j-1} is the next one's
+#pragma unroll 4  // the loads of four steps in flight
   for (int i = top; i >= 0; i--) {
-    const int j = 2 * i + par;
+    const int j = L * i + r;
     const double gm = G(j - 1), g0 = G(j);
-    const double a = (gm - gp) * inv[j + 1];
-    const double b0 = a + y * b1 - b2;
-    const double c0 = g0 + y * c1 - c2;
+    if (SH != 1) gp = G(j + 1);
+    const double b0 = (j <= ne + 1 ? (gm - gp) * inv[j + 1] : 0.0) + B.y * b1 - b2;
+    const double c0 = g0 + B.y * c1 - c2;
     b2 = b1;
     b1 = b0;
     c2 = c1;
     c1 = c0;
-    gp = gm;
+    if (SH == 1) gp = gm;
   }
-  // even: U_0 = 1, U_2 - y U_0 = 1;  odd: U_1 = 2x, U_3 - y U_1 = 0
-  const double Sp = par == 0 ? b1 + b2 : 2.0 * x * b1;
-  const double Cp = par == 0 ? c1 + c2 : 2.0 * x * c1;
-  const double S = Sp + __shfl_xor_sync(pm, Sp, 1);
-  const double C = Cp + __shfl_xor_sync(pm, Cp, 1);
+  const double S = B.finish(b1, b2, pm), C = B.finish(c1, c2, pm);
   const double phi = acos(x), s = sqrt(fmax(0.0, 1.0 - x * x));
   *N = G(0) * (1.0 - phi / PI) + s * S / PI;
   *dNde = (2.0 / PI) * s * C;
+}
+
+template <int SH>
+__device__ __forceinline__ void count_and_dos_any(const double* __restrict__ gsig, const double* __restrict__ inv,
+                                                  int M, int o, int ne, double x, int r, double* N, double* dNde) {
+  if constexpr (SH == 0) count_and_dos(gsig, inv, M, o, ne, x, N, dNde);
+  else count_and_dos_lanes<SH>(gsig, inv, M, o, ne, x, r, N, dNde);
 }
 
 constexpr int RT2 = 32;  // threads per block of the per-orbital FP64 kernels (see CT)
@@ -351,6 +395,8 @@ __global__ void __launch_bounds__(RT2) k_orbital_N(int M, int ne, const double* 
 //     = (1/pi)[-gs_1 (phi - pi) - (gs_0 + gs_2) sin(phi)
 //              + sum_{k>=2} (gs_{k-3} - gs_{k+1}) sin(k phi)/k],
 // together with N and the DOS.
+// 2^SH lanes per orbital.
+template <int SH>
 __global__ void __launch_bounds__(RT2) k_orbital_NU2(int M, int ne, const double* __restrict__ gsig,
                                                      const double* __restrict__ inv,
                                                      const double* __restrict__ a_inf,
@@ -358,33 +404,52 @@ __global__ void __launch_bounds__(RT2) k_orbital_NU2(int M, int ne, const double
                                                      const double* __restrict__ onsite, const FermiState* st,
                                                      double* __restrict__ N, double* __restrict__ U,
                                                      double* __restrict__ dos) {
-  const int o = blockIdx.x * RT2 + threadIdx.x;
+  constexpr int L = 1 << SH;
+  const int t = blockIdx.x * RT2 + threadIdx.x;
+  const int o = t >> SH, r = t & (L - 1);
   if (o >= M) return;
   const double ai = a_inf[o], bi = b_inf[o];
   const double xr = (st->ef - ai) / (2.0 * bi);
   const double x = clamp1(xr);
   double n, d;
-  count_and_dos(gsig, inv, M, o, ne, x, &n, &d);
+  count_and_dos_any<SH>(gsig, inv, M, o, ne, x, r, &n, &d);
   auto G = [&](int j) -> double { return (j >= 0 && j <= ne) ? gsig[(size_t)j * M + o] : 0.0; };
   const double phi = acos(x), s = sqrt(fmax(0.0, 1.0 - x * x)), x2 = 2.0 * x;
-  double b1 = 0.0, b2 = 0.0;
-  for (int k = ne + 3; k >= 2; k--) {  // sum_{k>=2} e_k sin(k phi) = s sum e_k U_{k-1}
-    const double e = (G(k - 3) - G(k + 1)) * inv[k];
-    const double b0 = e + x2 * b1 - b2;
-    b2 = b1;
-    b1 = b0;
+  // sum_{k>=1} e_k sin(k phi) = s sum e_k U_{k-1}, e_1 = -(gs_0 + gs_2)
+  double sum;
+  if constexpr (SH == 0) {
+    double b1 = 0.0, b2 = 0.0;
+    for (int k = ne + 3; k >= 2; k--) {
+      const double e = (G(k - 3) - G(k + 1)) * inv[k];
+      const double b0 = e + x2 * b1 - b2;
+      b2 = b1;
+      b1 = b0;
+    }
+    // b1 now holds sum_{k>=2} e_k U_{k-1} minus the k = 1 step: finish with e_1
+    sum = -(G(0) + G(2)) + x2 * b1 - b2;
+  } else {
+    const LaneBasis<SH> B(x, r);
+    double b1 = 0.0, b2 = 0.0;
+#pragma unroll 4
+    for (int i = (ne + 2) / L; i >= 0; i--) {
+      const int k = L * i + r + 1;
+      const double e = k == 1 ? -(G(0) + G(2)) : (k <= ne + 3 ? (G(k - 3) - G(k + 1)) * inv[k] : 0.0);
+      const double b0 = e + B.y * b1 - b2;
+      b2 = b1;
+      b1 = b0;
+    }
+    sum = B.finish(b1, b2, lane_group<SH>());
   }
-  // b1 now holds sum_{k>=2} e_k U_{k-1} minus the k = 1 step: finish with e_1
-  const double e1 = -(G(0) + G(2));
-  const double b0 = e1 + x2 * b1 - b2;
-  const double Pv = (-G(1) * (phi - PI) + s * b0) / PI;
+  if (r != 0) return;
+  const double Pv = (-G(1) * (phi - PI) + s * sum) / PI;
   N[o] = n;
   U[o] = bi * Pv - (onsite[o] - ai) * n;
   dos[o] = (xr > -1.0 && xr < 1.0) ? d / (2.0 * bi) : 0.0;
 }
 
 // sum over orbitals of dU/dE_F and dN/dE_F -> lam = sum dU / sum dN (the
-// response of E_F at fixed electron count).
+// response of E_F at fixed electron count).  2^SH lanes per orbital.
+template <int SH>
 __global__ void __launch_bounds__(RT2) k_ef_response2(int M, int ne, const double* __restrict__ gsig,
                                                       const double* __restrict__ inv,
                                                       const double* __restrict__ a_inf,
@@ -393,27 +458,35 @@ __global__ void __launch_bounds__(RT2) k_ef_response2(int M, int ne, const doubl
                                                       double* partials, unsigned* counter, double* lam) {
   __shared__ double sh[RT2 / 32];
   __shared__ bool last;
+  constexpr int L = 1 << SH;
   double aU = 0.0, aN = 0.0;
-  for (int o = blockIdx.x * RT2 + threadIdx.x; o < M; o += gridDim.x * RT2) {
+  for (int t = blockIdx.x * RT2 + threadIdx.x; (t >> SH) < M; t += gridDim.x * RT2) {
+    const int o = t >> SH, r = t & (L - 1);
     const double ai = a_inf[o], bi = b_inf[o];
     const double xr = (st->ef - ai) / (2.0 * bi);
-    if (!(xr > -1.0 && xr < 1.0)) continue;
+    if (!(xr > -1.0 && xr < 1.0)) continue;  // all lanes of the orbital
     // dN/deps = (2/pi) sum gs_m sin((m+1) phi), dP/deps = (2/pi) sum gs_m (sin((m+2) phi) + sin(m phi))
-    const double x2 = 2.0 * xr, s = sqrt(1.0 - xr * xr);
+    const double s = sqrt(1.0 - xr * xr);
+    const LaneBasis<SH> B(xr, r);
     double c1 = 0.0, c2 = 0.0, p1 = 0.0, p2 = 0.0;
     auto G = [&](int j) -> double { return (j >= 0 && j <= ne) ? gsig[(size_t)j * M + o] : 0.0; };
-    for (int k = ne + 2; k >= 1; k--) {  // coefficients of sin(k phi): g_{k-1} (N), g_{k-2} + g_k (P)
-      const double c0 = G(k - 1) + x2 * c1 - c2;
+#pragma unroll 4
+    for (int i = (ne + 1) / L; i >= 0; i--) {  // coefficients of sin(k phi): g_{k-1} (N), g_{k-2} + g_k (P)
+      const int k = L * i + r + 1;
+      const double c0 = G(k - 1) + B.y * c1 - c2;
       c2 = c1;
       c1 = c0;
-      const double q0 = (G(k - 2) + G(k)) + x2 * p1 - p2;
+      const double q0 = (G(k - 2) + (k <= ne ? G(k) : 0.0)) + B.y * p1 - p2;
       p2 = p1;
       p1 = q0;
     }
-    const double dN = (2.0 / PI) * s * c1, dP = (2.0 / PI) * s * p1;
-    const double dU = bi * dP - (onsite[o] - ai) * dN;
-    aU += dU / (2.0 * bi);
-    aN += dN / (2.0 * bi);
+    const unsigned pm = lane_group<SH>();
+    const double dN = (2.0 / PI) * s * B.finish(c1, c2, pm), dP = (2.0 / PI) * s * B.finish(p1, p2, pm);
+    if (r == 0) {
+      const double dU = bi * dP - (onsite[o] - ai) * dN;
+      aU += dU / (2.0 * bi);
+      aN += dN / (2.0 * bi);
+    }
   }
   const double bU = block_sum<RT2>(aU, sh);
   const double bN = block_sum<RT2>(aN, sh);
@@ -467,13 +540,13 @@ __device__ __forceinline__ double coop_block_reduce(double v, double* sh, bool t
 // Rounds evaluate N and the DOS of every orbital at the current iterate and
 // store them; the stored values are those of the last iterate E, within
 // tol of E_F (the SCF residual uses them; the energy is evaluated at E_F).
-template <int FC>
+template <int FC, int SH>
 __global__ void __launch_bounds__(FC) k_fermi_coop(int M, const double* __restrict__ gsig,
                                                    const double* __restrict__ inv, const double* __restrict__ a_inf,
                                                    const double* __restrict__ b_inf, int ne, double sfac,
                                                    double target, FermiState* st, double* part, int warm,
                                                    int max_rounds, double tol, double* __restrict__ Nout,
-                                                   double* __restrict__ dos, int lanes,
+                                                   double* __restrict__ dos,
                                                    const float* __restrict__ gs32) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   __shared__ double sh[FC / 32 + 1];
@@ -536,20 +609,16 @@ __global__ void __launch_bounds__(FC) k_fermi_coop(int M, const double* __restri
   bool done = hi - lo < tol;
   if (done) ef = 0.5 * (lo + hi);
   bool evaluated = false;
-  // lanes (1 or 2) per orbital: thread t takes orbital t / lanes; with two,
-  // the pair shares the sums (count_and_dos2)
-  const int sh_l = lanes == 2 ? 1 : 0;
-  const int par = lanes == 2 ? (threadIdx.x & 1) : 0;
-  const unsigned pm = 3u << ((threadIdx.x & 31) & ~1);
+  // thread t takes orbital t >> SH, whose 2^SH lanes share the sums
+  const int par = threadIdx.x & ((1 << SH) - 1);
   for (int r = 0; !done && r < max_rounds; r++) {
     double aN = 0.0, aD = 0.0;
-    for (int t = b * FC + threadIdx.x; (t >> sh_l) < M; t += stride) {
-      const int o = t >> sh_l;
+    for (int t = b * FC + threadIdx.x; (t >> SH) < M; t += stride) {
+      const int o = t >> SH;
       const double bi = b_inf[o];
       const double xr = (E - a_inf[o]) / (2.0 * bi);
       double Nv, dN;
-      if (sh_l) count_and_dos2(gsig, inv, M, o, ne, clamp1(xr), par, pm, &Nv, &dN);
-      else count_and_dos(gsig, inv, M, o, ne, clamp1(xr), &Nv, &dN);
+      count_and_dos_any<SH>(gsig, inv, M, o, ne, clamp1(xr), par, &Nv, &dN);
       const double d = (xr > -1.0 && xr < 1.0) ? dN / (2.0 * bi) : 0.0;
       if (par == 0) {
         aN += Nv;
@@ -595,13 +664,12 @@ __global__ void __launch_bounds__(FC) k_fermi_coop(int M, const double* __restri
     st->done = done ? 1 : 0;
   }
   if (!evaluated) {  // bracket narrower than tol: N and DOS at its midpoint
-    for (int t = b * FC + threadIdx.x; (t >> sh_l) < M; t += stride) {
-      const int o = t >> sh_l;
+    for (int t = b * FC + threadIdx.x; (t >> SH) < M; t += stride) {
+      const int o = t >> SH;
       const double bi = b_inf[o];
       const double xr = (ef - a_inf[o]) / (2.0 * bi);
       double Nv, dN;
-      if (sh_l) count_and_dos2(gsig, inv, M, o, ne, clamp1(xr), par, pm, &Nv, &dN);
-      else count_and_dos(gsig, inv, M, o, ne, clamp1(xr), &Nv, &dN);
+      count_and_dos_any<SH>(gsig, inv, M, o, ne, clamp1(xr), par, &Nv, &dN);
       if (par == 0) {
         Nout[o] = Nv;
         dos[o] = (xr > -1.0 && xr < 1.0) ? dN / (2.0 * bi) : 0.0;
@@ -853,36 +921,34 @@ int launch_fermi_more(int M, const double* gsig, const double* inv, const double
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <int FC>
-int fermi_coop_grid() {
-  static int g = 0;
-  if (g == 0) {
-    int dev = 0, sms = 0, per = 0, coop = 0;
+template <int FC, int SH>
+int run_fermi_coop(int M, void** args, cudaStream_t s) {
+  static int gmax = 0;
+  if (gmax == 0) {
+    int dev = 0, per = 0, coop = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_fermi_coop<FC>, FC, 0);
-    g = coop && per > 0 ? sms * (per < 4 ? per : 4) : -1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_fermi_coop<FC, SH>, FC, 0);
+    gmax = coop && per > 0 ? sm_count() * (per < 4 ? per : 4) : -1;
   }
-  return g;
+  if (gmax <= 0) return -2;
+  int g = (int)((((long long)M << SH) + FC - 1) / FC);
+  if (g > gmax) g = gmax;
+  if (g < 1) g = 1;
+  return cudaLaunchCooperativeKernel((const void*)k_fermi_coop<FC, SH>, g, FC, args, 0, s) == cudaSuccess ? 0 : -1;
 }
 
 int launch_fermi_coop(int M, const double* gsig, const double* inv, const double* a_inf, const double* b_inf,
                       int n_exp, double spin_factor, double target, FermiState* st, double* partials, int warm,
                       int max_rounds, double tol, double* N, double* dos, cudaStream_t s, const float* gs32) {
-  const bool few = few_orbitals(M);
-  const int fc = few ? FC_SMALL : FC_LARGE;
-  const int gmax = few ? fermi_coop_grid<FC_SMALL>() : fermi_coop_grid<FC_LARGE>();
-  if (gmax <= 0) return -2;
-  int lanes = few ? 2 : 1;
-  int g = (lanes * M + fc - 1) / fc;
-  if (g > gmax) g = gmax;
-  if (g < 1) g = 1;
   void* args[] = {&M, &gsig, &inv, &a_inf, &b_inf, &n_exp, &spin_factor, &target, &st, &partials, &warm,
-                  &max_rounds, &tol, &N, &dos, &lanes, &gs32};
-  const void* fn = few ? (const void*)k_fermi_coop<FC_SMALL> : (const void*)k_fermi_coop<FC_LARGE>;
-  if (cudaLaunchCooperativeKernel(fn, g, fc, args, 0, s) != cudaSuccess) return -1;
-  return 0;
+                  &max_rounds, &tol, &N, &dos, &gs32};
+  switch (lane_shift(M)) {
+    case 0: return run_fermi_coop<FC_LARGE, 0>(M, args, s);
+    case 1: return run_fermi_coop<FC_SMALL, 1>(M, args, s);
+    case 2: return run_fermi_coop<FC_SMALL, 2>(M, args, s);
+    default: return run_fermi_coop<FC_SMALL, 3>(M, args, s);
+  }
 }
 
 __global__ void k_to_f32(long long n, const double* __restrict__ in, float* __restrict__ out) {
@@ -906,13 +972,29 @@ int launch_orbital_N(int M, int n_exp, const double* gsig, const double* inv, co
 int launch_orbital_NU(int M, int n_exp, const double* gsig, const double* inv, const double* a_inf,
                       const double* b_inf, const double* onsite, const FermiState* st, double* N, double* U,
                       double* dos, cudaStream_t s) {
-  k_orbital_NU2<<<(M + RT2 - 1) / RT2, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, N, U, dos);
+  const int sh = lane_shift(M);
+  const int g = (int)((((long long)M << sh) + RT2 - 1) / RT2);
+  switch (sh) {
+    case 0: k_orbital_NU2<0><<<g, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, N, U, dos); break;
+    case 1: k_orbital_NU2<1><<<g, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, N, U, dos); break;
+    case 2: k_orbital_NU2<2><<<g, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, N, U, dos); break;
+    default: k_orbital_NU2<3><<<g, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, N, U, dos); break;
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int launch_ef_response(int M, int n_exp, const double* gsig, const double* inv, const double* a_inf,
                        const double* b_inf, const double* onsite, const FermiState* st, double* red,
                        unsigned* counter, double* lam, cudaStream_t s) {
-  k_ef_response2<<<red_grid2(M), RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, red, counter, lam);
+  const int sh = lane_shift(M), g = red_grid2(M << sh);
+#define EF_RESPONSE(SH) \
+  k_ef_response2<SH><<<g, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, red, counter, lam)
+  switch (sh) {
+    case 0: EF_RESPONSE(0); break;
+    case 1: EF_RESPONSE(1); break;
+    case 2: EF_RESPONSE(2); break;
+    default: EF_RESPONSE(3); break;
+  }
+#undef EF_RESPONSE
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
