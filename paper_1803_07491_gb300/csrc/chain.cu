@@ -817,6 +817,287 @@ __global__ void __launch_bounds__(CT) k_weights_split(WeightArgs A, double cU1, 
 }
 
 
+// ------------------------------------------------------------ few orbitals
+// The recurrences over the coefficients in FP64 for few orbitals (lane_shift),
+// where a warp's instruction count is the time: v_m = in_m - sum_j Q_j v_{m-j}
+// (sigma_m from P, the adjoint lambda from the cotangents of sigma) four
+// coefficients at a time.  Lane s of an orbital's four computes v_{m+s} from
+// v_{m-1}, v_{m-2}, ... by substituting the s recurrences in between:
+//   v_{m+s} = sum_{i<=s} rho_i in_{m+s-i} - sum_j c_j v_{m-j},
+// with rho the impulse response and c the row of the s-fold substituted
+// recurrence, so that the 2 KP multiply-adds of one coefficient yield four.
+template <int NT>  // taps
+struct LookAhead {
+  double c[NT], rho[4];
+  __device__ __forceinline__ LookAhead(const double* q, int s) {  // q[j]: Q_j, j = 0..NT
+    double row[4][NT];
+    rho[0] = 1.0;
+#pragma unroll
+    for (int i = 1; i < 4; i++) {
+      rho[i] = 0.0;
+#pragma unroll
+      for (int j = 1; j <= i; j++)
+        if (j <= NT) rho[i] -= q[j] * rho[i - j];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+      for (int j = 1; j <= NT; j++) {
+        double v = j + r <= NT ? q[j + r] : 0.0;
+#pragma unroll
+        for (int i = 1; i <= r; i++)
+          if (i <= NT) v -= q[i] * row[r - i][j - 1];
+        row[r][j - 1] = v;
+      }
+#pragma unroll
+    for (int j = 0; j < NT; j++) c[j] = s == 0 ? row[0][j] : (s == 1 ? row[1][j] : (s == 2 ? row[2][j] : row[3][j]));
+  }
+  // v_{m+s} from h[j] = v_{m-1-j} and in[i] = in_{m+s-i} (zero for i > s);
+  // then the history advances by the orbital's four values.
+  __device__ __forceinline__ double step(double h[NT], const double in[4]) const {
+    double v = in[0] + rho[1] * in[1] + rho[2] * in[2] + rho[3] * in[3];
+    return advance(h, v);
+  }
+  __device__ __forceinline__ double advance(double h[NT], double v) const {
+#pragma unroll
+    for (int j = 0; j < NT; j++) v -= c[j] * h[j];
+    double n[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) n[i] = __shfl_sync(0xffffffffu, v, i, 4);
+#pragma unroll
+    for (int j = NT - 1; j >= 4; j--) h[j] = h[j - 4];
+#pragma unroll
+    for (int j = 0; j < 4 && j < NT; j++) h[j] = n[3 - j];
+    return v;
+  }
+};
+
+// k_expand with four lanes per orbital (FP64 recurrence).
+template <int KP>
+__global__ void __launch_bounds__(CT) k_expand_few(ScalarArgs A) {
+  const int t = blockIdx.x * CT + threadIdx.x, s = t & 3;
+  const bool live = (t >> 2) < A.M;
+  const int o = live ? t >> 2 : A.M - 1;  // whole warps take part in the exchanges
+  constexpr int NP = 2 * KP + 1;
+  const int M = A.M, ne = A.n_exp, nm = 2 * KP + 1;
+  double mu[BOP_MAX_NMOM];
+  for (int n = 0; n < nm; n++) mu[n] = A.mu[(size_t)o * nm + n];
+  Rec r;
+  recursion(mu, KP, r);
+  const Term tm = bandwidth(r, A.bw);
+  Chain ch;
+  chain_params(r, tm, KP, ch);
+  if (live && s == 0) {
+    for (int k = 0; k < KP; k++) A.a[(size_t)o * KP + k] = r.a[k];
+    for (int k = 0; k <= KP; k++) A.b[(size_t)o * (KP + 1) + k] = r.b[k];
+    A.nlev[o] = r.nlev;
+    A.a_inf[o] = tm.a_inf;
+    A.b_inf[o] = tm.b_inf;
+  }
+  double Q[NP], P[NP];
+  gen_polys<KP>(ch, r.nlev, Q, P);
+  const LookAhead<NP - 1> la(Q, s);
+  double h[NP - 1];
+#pragma unroll
+  for (int j = 0; j < NP - 1; j++) h[j] = 0.0;
+  bool outside = false, finite = true;
+  for (int m0 = 0; m0 <= ne; m0 += 4) {
+    const int m = m0 + s;
+    double v = 0.0;
+    if (m0 < NP) {
+      double in[4];
+#pragma unroll
+      for (int i = 0; i < 4; i++) in[i] = i <= s && m - i < NP ? P[m - i] : 0.0;
+      v = la.step(h, in);
+    } else {
+      v = la.advance(h, 0.0);
+    }
+    if (live && m <= ne) {
+      A.gsig[(size_t)m * M + o] = A.g[m] * v;
+      outside |= A.n_unbounded != nullptr && fabs(v) > (m + 1) * (1.0 + 1e-9);
+      finite &= m < ne || isfinite(v);
+    }
+  }
+  const unsigned out4 = __ballot_sync(0xffffffffu, outside) >> (threadIdx.x & 28) & 15u;
+  if (live && s == 0 && out4) atomicAdd(A.n_unbounded, 1u);
+  if (live && (!isfinite(tm.a_inf) || !isfinite(tm.b_inf) || !finite)) raise_error(A.status, BOP_DEV_ERR_NONFINITE);
+}
+
+// Weights of NS seeds (cU, cN) with eight lanes per orbital, FP64 throughout:
+// the pieces of chain_reverse_ns with the recurrences of sigma and of lambda
+// four coefficients at a time (lanes 0-3 the first seed, 4-7 the second), the
+// sums over the coefficients in eight blocks, and the rest on every lane (128
+// orbitals: 338 -> 144 us).
+// zscratch: sigma [ne+1][M], then the cotangents of each seed.
+template <int KP, int NS>
+__global__ void __launch_bounds__(CT) k_weights_few(WeightArgs A, double cU1, double cN1, double cU2, double cN2,
+                                                    double* __restrict__ w2) {
+  constexpr int NP = 2 * KP + 1;
+  const int t = blockIdx.x * CT + threadIdx.x, lane8 = t & 7, s = t & 3;
+  const bool live = (t >> 3) < A.M;
+  const int o = live ? t >> 3 : A.M - 1;  // dead lanes repeat the last orbital and write nothing
+  const int M = A.M, ne = A.n_exp, nm = 2 * KP + 1;
+  const size_t zl = (size_t)(ne + 1) * M;
+  double* zs = A.zscratch;
+  double cU[NS], cN[NS];
+  cU[0] = NS == 2 ? cU1 : A.cU;
+  cN[0] = NS == 2 ? cN1
+                  : (A.var_q ? cU[0] * (A.var_J * A.var_q[o / A.norb] - A.var_lam[0])
+                             : (A.lam ? -A.cU * A.lam[0] : A.cN0));
+  if (NS == 2) {
+    cU[NS - 1] = cU2;
+    cN[NS - 1] = cN2;
+  }
+  double mu[BOP_MAX_NMOM];
+  for (int n = 0; n < nm; n++) mu[n] = A.mu[(size_t)o * nm + n];
+  Rec r;
+  RecTape<KP> tp;
+  recursion_taped<KP>(mu, r, tp);
+  const Term tm = bandwidth(r, A.bw);
+  Chain ch;
+  chain_params(r, tm, KP, ch);
+  const int Lv = r.nlev;
+  const double ai = tm.a_inf, bi = tm.b_inf, E = A.onsite[o], ef = A.st->ef;
+  ChainPolys<KP> D;
+  chain_polys<KP>(ch, Lv, D);
+  const LookAhead<NP - 1> la(D.k[0], s);
+  // ---- sigma_m
+  {
+    double h[NP - 1];
+#pragma unroll
+    for (int j = 0; j < NP - 1; j++) h[j] = 0.0;
+    for (int m0 = 0; m0 <= ne; m0 += 4) {
+      const int m = m0 + s;
+      double v = 0.0;
+      if (m0 < NP) {
+        double in[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) in[i] = i <= s && m - i < NP ? D.k[1][m - i] : 0.0;
+        v = la.step(h, in);
+      } else {
+        v = la.advance(h, 0.0);
+      }
+      if (live && lane8 < 4 && m <= ne) zs[(size_t)m * M + o] = v;
+    }
+  }
+  __syncwarp();
+  // ---- the sums N, P, dN/deps, dP/deps and the cotangents of sigma_m, in blocks of m
+  const double xr = (ef - ai) / (2.0 * bi);
+  const bool inside = xr > -1.0 && xr < 1.0;
+  const double x = clamp1(xr);
+  const double phi = acos(x);
+  double Nbar[NS], Pbar[NS];
+#pragma unroll
+  for (int q = 0; q < NS; q++) {
+    Nbar[q] = cN[q] - cU[q] * (E - ai);
+    Pbar[q] = cU[q] * bi;
+  }
+  const int blk = (ne + 8) / 8, m_lo = min(ne + 1, lane8 * blk), m_hi = min(ne + 1, m_lo + blk);
+  double sum[4] = {0.0, 0.0, 0.0, 0.0};
+  {
+    constexpr double INV_PI = 1.0 / PI;
+    // s_j = sin(j phi) from s_m on, chi_j from s_{j-1} and s_{j+1}
+    auto chi = [&](int j, double sjm1, double sjp1) -> double {
+      if (j == 0) return 0.0;
+      const double lo = (j == 1) ? (phi - PI) : sjm1 * A.inv[j - 1];
+      return (sjp1 * A.inv[j + 1] - lo) * INV_PI;
+    };
+    const bool edge = x == 1.0 || x == -1.0;  // E_F outside the band: every sine is zero
+    double sm1 = edge ? 0.0 : sin((m_lo - 1) * phi), s0 = edge ? 0.0 : sin(m_lo * phi);
+    double sp1 = 2.0 * x * s0 - sm1, sp2 = 2.0 * x * sp1 - s0, sp3 = 2.0 * x * sp2 - sp1;
+    double c_m = chi(m_lo, sm1, sp1), c_m1 = chi(m_lo + 1, s0, sp2);
+    for (int m = m_lo; m < m_hi; m++) {
+      const double c_m2 = chi(m + 2, sp1, sp3);
+      const double gm = A.g[m], gsm = gm * zs[(size_t)m * M + o], cp = c_m2 + c_m;
+      sum[0] += gsm * c_m1;
+      sum[1] += gsm * cp;
+      sum[2] += gsm * sp1;
+      sum[3] += gsm * (sp2 + s0);
+#pragma unroll
+      for (int q = 0; q < NS; q++)
+        if (live) zs[(1 + q) * zl + (size_t)m * M + o] = gm * (Nbar[q] * c_m1 + Pbar[q] * cp);
+      c_m = c_m1;
+      c_m1 = c_m2;
+      s0 = sp1;
+      sp1 = sp2;
+      sp2 = sp3;
+      sp3 = 2.0 * x * sp2 - sp1;
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < 4; v++)
+#pragma unroll
+    for (int w = 1; w < 8; w <<= 1) sum[v] += __shfl_xor_sync(0xffffffffu, sum[v], w);
+  const double Nv = sum[0], Pv = sum[1], dN = sum[2] * (2.0 / PI), dP = sum[3] * (2.0 / PI);
+  __syncwarp();
+  // ---- lambda_m = cotangent - sum_j [D_0]_j lambda_{m+j}, downwards, in the cotangents' place
+  {
+    double* zb = zs + (1 + (NS == 2 ? lane8 >> 2 : 0)) * zl;
+    double h[NP - 1];
+#pragma unroll
+    for (int j = 0; j < NP - 1; j++) h[j] = 0.0;
+    for (int k0 = 0; k0 <= ne; k0 += 4) {
+      const int k = k0 + s;
+      double in[4];
+#pragma unroll
+      for (int i = 0; i < 4; i++) in[i] = i <= s && k - i <= ne ? zb[(size_t)(ne - (k - i)) * M + o] : 0.0;
+      __syncwarp();
+      const double v = la.step(h, in);
+      if (live && (NS == 2 || lane8 < 4) && k <= ne) zb[(size_t)(ne - k) * M + o] = v;
+    }
+  }
+  __syncwarp();
+  // ---- Pb = dL/d[D_1] (the first lambdas), Qb = dL/d[D_0] = -sum_m lambda_m sigma_{m-j}, in blocks of m
+  for (int q = 0; q < NS; q++) {
+    const double* zb = zs + (1 + q) * zl;
+    double Pb[NP], Qb[NP];
+#pragma unroll
+    for (int j = 0; j < NP; j++) {
+      Pb[j] = j <= ne ? zb[(size_t)j * M + o] : 0.0;
+      Qb[j] = 0.0;
+    }
+    double sw[NP - 1];  // sw[j] = sigma_{m-1-j}
+#pragma unroll
+    for (int j = 0; j < NP - 1; j++) sw[j] = m_lo - 1 - j >= 0 ? zs[(size_t)(m_lo - 1 - j) * M + o] : 0.0;
+    for (int m = m_lo; m < m_hi; m++) {
+      const double lam = zb[(size_t)m * M + o];
+#pragma unroll
+      for (int j = 1; j < NP; j++) Qb[j] -= lam * sw[j - 1];
+#pragma unroll
+      for (int j = NP - 2; j >= 1; j--) sw[j] = sw[j - 1];
+      sw[0] = zs[(size_t)m * M + o];
+    }
+#pragma unroll
+    for (int j = 1; j < NP; j++)
+#pragma unroll
+      for (int w = 1; w < 8; w <<= 1) Qb[j] += __shfl_xor_sync(0xffffffffu, Qb[j], w);
+    double abar[KPMAX + 1], bbar[KPMAX + 2];
+    for (int k = 0; k <= KPMAX; k++) abar[k] = 0.0;
+    for (int k = 0; k <= KPMAX + 1; k++) bbar[k] = 0.0;
+    double abar_inf = cU[q] * Nv, bbar_inf = cU[q] * Pv;
+    if (inside) {
+      const double ebar = Nbar[q] * dN + Pbar[q] * dP;
+      abar_inf += -ebar / (2.0 * bi);
+      bbar_inf += -ebar * xr / bi;
+    }
+    chain_polys_reverse<KP>(ch, Lv, KP, bi, D, Pb, Qb, abar, bbar, abar_inf, bbar_inf);
+    bandwidth_reverse(r, tm, A.bw, abar_inf, bbar_inf, abar, bbar);
+    double mub[BOP_MAX_NMOM];
+    for (int n = 0; n < nm; n++) mub[n] = 0.0;
+    recursion_reverse<KP>(mu, r, tp, abar, bbar, mub);
+    if (live && lane8 == 0) {
+      if (q == 0 && A.dU_dE) A.dU_dE[o] = -cU[0] * Nv;
+      double* w = q == 0 ? A.w : w2;
+      bool bad = false;
+      for (int n = 0; n < nm; n++) {
+        w[(size_t)o * nm + n] = mub[n];
+        bad |= !isfinite(mub[n]);
+      }
+      if (bad) raise_error(A.status, BOP_DEV_ERR_NONFINITE);
+    }
+  }
+}
+
 int red_grid2(int M) {
   int g = (M + RT2 - 1) / RT2;
   return g < 1 ? 1 : (g > 4096 ? 4096 : g);  // the context's partials hold 2 x 4096 values
@@ -829,7 +1110,26 @@ void launch_inverse_table(double* inv, int n, cudaStream_t s) {
 }
 
 int launch_expand(const ScalarArgs& a, cudaStream_t s) {
-  const int g = (a.M + CT - 1) / CT, Kp = (a.n_mom - 1) / 2;
+  const int Kp = (a.n_mom - 1) / 2;
+  // four lanes per orbital while those leave at most one warp per
+  // sub-partition (128 / 4,320 orbitals: 85 / 85 -> 51 / 54 us); the FP32
+  // recurrence takes a fraction of either
+  if (!a.sig32 && lane_shift(a.M) >= 2) {
+    const int g4 = (4 * a.M + CT - 1) / CT;
+    switch (Kp) {
+      case 1: k_expand_few<1><<<g4, CT, 0, s>>>(a); break;
+      case 2: k_expand_few<2><<<g4, CT, 0, s>>>(a); break;
+      case 3: k_expand_few<3><<<g4, CT, 0, s>>>(a); break;
+      case 4: k_expand_few<4><<<g4, CT, 0, s>>>(a); break;
+      case 5: k_expand_few<5><<<g4, CT, 0, s>>>(a); break;
+      case 6: k_expand_few<6><<<g4, CT, 0, s>>>(a); break;
+      case 7: k_expand_few<7><<<g4, CT, 0, s>>>(a); break;
+      case 8: k_expand_few<8><<<g4, CT, 0, s>>>(a); break;
+      default: return -1;
+    }
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  }
+  const int g = (a.M + CT - 1) / CT;
   switch (Kp) {
     case 1: k_expand<1><<<g, CT, 0, s>>>(a); break;
     case 2: k_expand<2><<<g, CT, 0, s>>>(a); break;
@@ -844,7 +1144,29 @@ int launch_expand(const ScalarArgs& a, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+template <int NS>
+int launch_weights_few(const WeightArgs& a, double cU1, double cN1, double cU2, double cN2, double* w2,
+                       cudaStream_t s) {
+  const int g = (8 * a.M + CT - 1) / CT;
+#define WEIGHTS_FEW(KP) \
+  case KP: k_weights_few<KP, NS><<<g, CT, 0, s>>>(a, cU1, cN1, cU2, cN2, w2); break
+  switch ((a.n_mom - 1) / 2) {
+    WEIGHTS_FEW(1);
+    WEIGHTS_FEW(2);
+    WEIGHTS_FEW(3);
+    WEIGHTS_FEW(4);
+    WEIGHTS_FEW(5);
+    WEIGHTS_FEW(6);
+    WEIGHTS_FEW(7);
+    WEIGHTS_FEW(8);
+    default: return -1;
+  }
+#undef WEIGHTS_FEW
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 int launch_weights(const WeightArgs& a, cudaStream_t s) {
+  if (!a.sig32 && lane_shift(a.M) >= 3) return launch_weights_few<1>(a, 0.0, 0.0, 0.0, 0.0, nullptr, s);
   const int g = (a.M + CT - 1) / CT, Kp = (a.n_mom - 1) / 2;
   switch (Kp) {
     case 1: k_weights<1><<<g, CT, 0, s>>>(a); break;
@@ -863,6 +1185,7 @@ int launch_weights(const WeightArgs& a, cudaStream_t s) {
 int launch_weights_pair(const WeightArgs& a, double cU1, double cN1, double cU2, double cN2, double* w2,
                         cudaStream_t s) {
   const int Kp = (a.n_mom - 1) / 2;
+  if (!a.sig32 && lane_shift(a.M) >= 3) return launch_weights_few<2>(a, cU1, cN1, cU2, cN2, w2, s);
   if (!few_orbitals(a.M)) {  // enough warps already: one lane, one forward pass for both seeds
     const int g = (a.M + CT - 1) / CT;
     switch (Kp) {

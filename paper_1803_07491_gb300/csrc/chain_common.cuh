@@ -156,6 +156,77 @@ __device__ inline void recursion_taped(const double* mu, Rec& r, RecTape<KP>& tp
 }
 
 // ------------------------------------------------------------ reverse of the chain
+// The generating polynomials D_0 .. D_{KP+1} of a chain of L levels, all kept.
+template <int KP>
+struct ChainPolys {
+  double k[KP + 2][2 * KP + 1];
+};
+template <int KP>
+__device__ __forceinline__ void chain_polys(const Chain& ch, int L, ChainPolys<KP>& D) {
+  constexpr int NP = 2 * KP + 1;
+  for (int k = 0; k < KP + 2; k++)
+    for (int j = 0; j < NP; j++) D.k[k][j] = 0.0;
+  D.k[L + 1][0] = 1.0;
+  D.k[L][0] = 1.0;
+  for (int k = L - 1; k >= 0; k--) {
+    const double a2 = 2.0 * ch.ah[k], bb = 4.0 * ch.bh[k + 1] * ch.bh[k + 1];
+    for (int j = 0; j < NP; j++) {
+      double v = D.k[k + 1][j];
+      if (j >= 1) v -= a2 * D.k[k + 1][j - 1];
+      if (j >= 2) v += D.k[k + 1][j - 2] - bb * D.k[k + 2][j - 2];
+      D.k[k][j] = v;
+    }
+  }
+}
+// Reverse of the polynomial recursion and of the chain parameters a^_k = (a_k
+// - a_inf)/(2 b_inf), b^_k = b_k/(2 b_inf) (k <= Kb): Pb = dL/d[D_1], Qb =
+// dL/d[D_0] -> cotangents of the raw chain and of its terminator (added).
+template <int KP>
+__device__ __forceinline__ void chain_polys_reverse(const Chain& ch, int L, int Kb, double bi,
+                                                    const ChainPolys<KP>& D, const double* Pb, const double* Qb,
+                                                    double* abar, double* bbar, double& abar_inf, double& bbar_inf) {
+  constexpr int NP = 2 * KP + 1;
+  double ahb[KP + 1], bhb[KP + 2];
+  for (int k = 0; k <= KP; k++) ahb[k] = 0.0;
+  for (int k = 0; k <= KP + 1; k++) bhb[k] = 0.0;
+  double Db[KP + 2][NP];
+  for (int k = 0; k < KP + 2; k++)
+    for (int j = 0; j < NP; j++) Db[k][j] = 0.0;
+  for (int j = 0; j < NP; j++) {
+    Db[0][j] = Qb[j];
+    Db[1][j] = Pb[j];
+  }
+  for (int k = 0; k < L; k++) {
+    const double a2 = 2.0 * ch.ah[k], bb = 4.0 * ch.bh[k + 1] * ch.bh[k + 1];
+    double ga = 0.0, gb = 0.0;
+    for (int j = 0; j < NP; j++) {
+      const double gg = Db[k][j];
+      Db[k + 1][j] += gg;
+      if (j >= 1) {
+        Db[k + 1][j - 1] -= a2 * gg;
+        ga -= 2.0 * gg * D.k[k + 1][j - 1];
+      }
+      if (j >= 2) {
+        Db[k + 1][j - 2] += gg;
+        Db[k + 2][j - 2] -= bb * gg;
+        gb -= 8.0 * ch.bh[k + 1] * gg * D.k[k + 2][j - 2];
+      }
+    }
+    ahb[k] += ga;
+    bhb[k + 1] += gb;
+  }
+  for (int k = 0; k < L; k++) {
+    abar[k] += ahb[k] / (2.0 * bi);
+    abar_inf += -ahb[k] / (2.0 * bi);
+    bbar_inf += -ahb[k] * ch.ah[k] / bi;
+  }
+  for (int k = 1; k <= Kb; k++)
+    if (k <= L) {
+      bbar[k] += bhb[k] / (2.0 * bi);
+      bbar_inf += -bhb[k] * ch.bh[k] / bi;
+    }
+}
+
 // Reverse of chain -> sigma_m -> (N, P) -> L = cU U + cN N for one orbital
 // (fixed E_F and onsite level E), U = b_inf P - (E - a_inf) N, for NS seeds
 // (cU[q], cN[q]) at once: the forward part (generating polynomials, sigma_m,
@@ -172,21 +243,9 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
                                         double (*abar)[KPMAX + 1], double (*bbar)[KPMAX + 2], double* abar_inf,
                                         double* bbar_inf, double* dE, bool f32 = false) {
   constexpr int NP = 2 * KP + 1;
-  // ---- generating polynomials D_0 .. D_{L+1}, all kept
-  double Dk[KP + 2][NP];
-  for (int k = 0; k < KP + 2; k++)
-    for (int j = 0; j < NP; j++) Dk[k][j] = 0.0;
-  Dk[L + 1][0] = 1.0;
-  Dk[L][0] = 1.0;
-  for (int k = L - 1; k >= 0; k--) {
-    const double a2 = 2.0 * ch.ah[k], bb = 4.0 * ch.bh[k + 1] * ch.bh[k + 1];
-    for (int j = 0; j < NP; j++) {
-      double v = Dk[k + 1][j];
-      if (j >= 1) v -= a2 * Dk[k + 1][j - 1];
-      if (j >= 2) v += Dk[k + 1][j - 2] - bb * Dk[k + 2][j - 2];
-      Dk[k][j] = v;
-    }
-  }
+  ChainPolys<KP> D;
+  chain_polys<KP>(ch, L, D);
+  double (&Dk)[KP + 2][NP] = D.k;
   // ---- sigma_m and the sums N, P, dN/deps, dP/deps (with f32 the two
   // recurrences over m, forward and reverse, in FP32 as in sigma_series; the
   // sums and the chi_m stay FP64)
@@ -387,51 +446,8 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
       sw[NP - 2] = mm >= 0 ? zs[(size_t)mm * M + o] : 0.0;
     }
   }
-  // ---- reverse of the polynomial recursion -> a^bar, b^bar; chain parameters
-  for (int q = 0; q < NS; q++) {
-    double ahb[KP + 1], bhb[KP + 2];
-    for (int k = 0; k <= KP; k++) ahb[k] = 0.0;
-    for (int k = 0; k <= KP + 1; k++) bhb[k] = 0.0;
-    {
-      double Db[KP + 2][NP];
-      for (int k = 0; k < KP + 2; k++)
-        for (int j = 0; j < NP; j++) Db[k][j] = 0.0;
-      for (int j = 0; j < NP; j++) {
-        Db[0][j] = Qb[q][j];
-        Db[1][j] = Pb[q][j];
-      }
-      for (int k = 0; k < L; k++) {
-        const double a2 = 2.0 * ch.ah[k], bb = 4.0 * ch.bh[k + 1] * ch.bh[k + 1];
-        double ga = 0.0, gb = 0.0;
-        for (int j = 0; j < NP; j++) {
-          const double gg = Db[k][j];
-          Db[k + 1][j] += gg;
-          if (j >= 1) {
-            Db[k + 1][j - 1] -= a2 * gg;
-            ga -= 2.0 * gg * Dk[k + 1][j - 1];
-          }
-          if (j >= 2) {
-            Db[k + 1][j - 2] += gg;
-            Db[k + 2][j - 2] -= bb * gg;
-            gb -= 8.0 * ch.bh[k + 1] * gg * Dk[k + 2][j - 2];
-          }
-        }
-        ahb[k] += ga;
-        bhb[k + 1] += gb;
-      }
-    }
-    // chain parameters a^_k = (a_k - a_inf)/(2 b_inf), b^_k = b_k/(2 b_inf)
-    for (int k = 0; k < L; k++) {
-      abar[q][k] += ahb[k] / (2.0 * bi);
-      abar_inf[q] += -ahb[k] / (2.0 * bi);
-      bbar_inf[q] += -ahb[k] * ch.ah[k] / bi;
-    }
-    for (int k = 1; k <= Kb; k++)
-      if (k <= L) {
-        bbar[q][k] += bhb[k] / (2.0 * bi);
-        bbar_inf[q] += -bhb[k] * ch.bh[k] / bi;
-      }
-  }
+  for (int q = 0; q < NS; q++)
+    chain_polys_reverse<KP>(ch, L, Kb, bi, D, Pb[q], Qb[q], abar[q], bbar[q], abar_inf[q], bbar_inf[q]);
 }
 
 // One seed (cU, cN); returns dL/dE.
