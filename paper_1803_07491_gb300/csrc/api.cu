@@ -1011,6 +1011,7 @@ int compute_weights(bop_ctx* c, double cU, const double* lam, double cN0, double
   wa.onsite = P<double>(c->onsite);
   wa.st = P<FermiState>(c->fstate);
   wa.g = P<double>(c->gjack);
+    wa.g32 = reinterpret_cast<const float*>(P<double>(c->gjack) + c->n_exp + 1);
   wa.inv = P<double>(c->ginv);
   wa.cU = cU;
   wa.lam = lam;
@@ -1214,6 +1215,7 @@ int scf_response(bop_ctx* c, cudaStream_t s) {
     wa.onsite = P<double>(c->onsite);
     wa.st = P<FermiState>(c->fstate);
     wa.g = P<double>(c->gjack);
+    wa.g32 = reinterpret_cast<const float*>(P<double>(c->gjack) + c->n_exp + 1);
     wa.inv = P<double>(c->ginv);
     wa.cU = 0.0;
     wa.lam = nullptr;
@@ -1448,11 +1450,11 @@ int bop_create(bop_ctx** out, const bop_model* model) {
   c->bm.rep_p = model->rep_p;
   cudaGetDevice(&c->device);
   memset(&c->st, 0, sizeof(c->st));
-  if ((r = ensure(c, c->status, sizeof(unsigned))) || (r = ensure(c, c->gjack, sizeof(double) * (c->n_exp + 1))) ||
+  if ((r = ensure(c, c->status, sizeof(unsigned))) || (r = ensure(c, c->gjack, (sizeof(double) + sizeof(float)) * (c->n_exp + 1))) ||
       (r = ensure(c, c->fstate, sizeof(FermiState))) || (r = ensure(c, c->partials, sizeof(double) * 3 * 4096)) ||
       (r = ensure(c, c->counter, sizeof(unsigned))) || (r = ensure(c, c->result, sizeof(double) * 4)) ||
       (r = ensure(c, c->e_total, sizeof(double))) || (r = ensure(c, c->lam, sizeof(double) * 4)) ||
-      (r = ensure(c, c->ginv, sizeof(double) * (c->n_exp + 8)))) {
+      (r = ensure(c, c->ginv, sizeof(double) * (c->n_exp + 16)))) {
     bop_destroy(c);
     return r;
   }
@@ -1463,7 +1465,7 @@ int bop_create(bop_ctx** out, const bop_model* model) {
     c->pin = nullptr;  // reads go straight to their destinations
   }
   launch_jackson(P<double>(c->gjack), c->n_exp, 0);
-  launch_inverse_table(P<double>(c->ginv), c->n_exp + 8, 0);
+  launch_inverse_table(P<double>(c->ginv), c->n_exp + 16, 0);
   if (cudaDeviceSynchronize() != cudaSuccess) {
     bop_destroy(c);
     return BOP_ERR_CUDA;
@@ -1933,8 +1935,7 @@ int bop_forces(bop_ctx* c, double* forces, double* virial, bop_stats* st, bop_st
     // E_F response (global multiplier), weights, reverse sweep
     {
       Region R(c, PK_EFRESP, 1, s);
-      if (launch_ef_response(M, c->n_exp, P<double>(c->gsig), P<double>(c->ginv), P<double>(c->a_inf),
-                             P<double>(c->b_inf), P<double>(c->onsite), P<FermiState>(c->fstate),
+      if (launch_ef_response(M, P<double>(c->onsite), P<double>(c->dos), P<FermiState>(c->fstate),
                              P<double>(c->partials), P<unsigned>(c->counter), P<double>(c->lam), s))
         return fail(c, BOP_ERR_CUDA, "E_F response launch failed");
     }

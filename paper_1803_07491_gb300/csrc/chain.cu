@@ -97,7 +97,7 @@ __device__ __forceinline__ void count_and_dos(const double* __restrict__ gsig, c
   const double x2 = 2.0 * x;
   double b1 = 0.0, b2 = 0.0, c1 = 0.0, c2 = 0.0;
   for (int k = ne + 2; k >= 1; k--) {  // coefficient of U_{k-1}
-    const double b0 = (G(k - 2) - G(k)) * inv[k] + x2 * b1 - b2;
+    const double b0 = fma(G(k - 2) - G(k), inv[k], fma(x2, b1, -b2));
     b2 = b1;
     b1 = b0;
     const double c0 = G(k - 1) + x2 * c1 - c2;
@@ -118,7 +118,7 @@ __device__ __forceinline__ void count_and_dos_f32(const float* __restrict__ gs32
   const float x2 = 2.f * x;
   float b1 = 0.f, b2 = 0.f, c1 = 0.f, c2 = 0.f;
   for (int k = ne + 2; k >= 1; k--) {
-    const float b0 = (G(k - 2) - G(k)) / (float)k + x2 * b1 - b2;
+    const float b0 = fmaf(G(k - 2) - G(k), __fdividef(1.f, (float)k), fmaf(x2, b1, -b2));
     b2 = b1;
     b1 = b0;
     const float c0 = G(k - 1) + x2 * c1 - c2;
@@ -186,7 +186,7 @@ __device__ __forceinline__ void count_and_dos_lanes(const double* __restrict__ g
     const int j = L * i + r;
     const double gm = G(j - 1), g0 = G(j);
     if (SH != 1) gp = G(j + 1);
-    const double b0 = (j <= ne + 1 ? (gm - gp) * inv[j + 1] : 0.0) + B.y * b1 - b2;
+    const double b0 = fma(gm - gp, inv[j + 1], fma(B.y, b1, -b2));  // j > ne + 1: both zero
     const double c0 = g0 + B.y * c1 - c2;
     b2 = b1;
     b1 = b0;
@@ -420,8 +420,7 @@ __global__ void __launch_bounds__(RT2) k_orbital_NU2(int M, int ne, const double
   if constexpr (SH == 0) {
     double b1 = 0.0, b2 = 0.0;
     for (int k = ne + 3; k >= 2; k--) {
-      const double e = (G(k - 3) - G(k + 1)) * inv[k];
-      const double b0 = e + x2 * b1 - b2;
+      const double b0 = fma(G(k - 3) - G(k + 1), inv[k], fma(x2, b1, -b2));
       b2 = b1;
       b1 = b0;
     }
@@ -448,45 +447,18 @@ __global__ void __launch_bounds__(RT2) k_orbital_NU2(int M, int ne, const double
 }
 
 // sum over orbitals of dU/dE_F and dN/dE_F -> lam = sum dU / sum dN (the
-// response of E_F at fixed electron count).  2^SH lanes per orbital.
-template <int SH>
-__global__ void __launch_bounds__(RT2) k_ef_response2(int M, int ne, const double* __restrict__ gsig,
-                                                      const double* __restrict__ inv,
-                                                      const double* __restrict__ a_inf,
-                                                      const double* __restrict__ b_inf,
-                                                      const double* __restrict__ onsite, const FermiState* st,
+// response of E_F at fixed electron count), from the DOS n at E_F: dN/dE_F = n
+// and, since sin((m+2) phi) + sin(m phi) = 2 cos(phi) sin((m+1) phi) in the
+// energy's series, dU/dE_F = (E_F - E_ialpha) n.
+__global__ void __launch_bounds__(RT2) k_ef_response2(int M, const double* __restrict__ onsite,
+                                                      const double* __restrict__ dos, const FermiState* st,
                                                       double* partials, unsigned* counter, double* lam) {
   __shared__ double sh[RT2 / 32];
   __shared__ bool last;
-  constexpr int L = 1 << SH;
   double aU = 0.0, aN = 0.0;
-  for (int t = blockIdx.x * RT2 + threadIdx.x; (t >> SH) < M; t += gridDim.x * RT2) {
-    const int o = t >> SH, r = t & (L - 1);
-    const double ai = a_inf[o], bi = b_inf[o];
-    const double xr = (st->ef - ai) / (2.0 * bi);
-    if (!(xr > -1.0 && xr < 1.0)) continue;  // all lanes of the orbital
-    // dN/deps = (2/pi) sum gs_m sin((m+1) phi), dP/deps = (2/pi) sum gs_m (sin((m+2) phi) + sin(m phi))
-    const double s = sqrt(1.0 - xr * xr);
-    const LaneBasis<SH> B(xr, r);
-    double c1 = 0.0, c2 = 0.0, p1 = 0.0, p2 = 0.0;
-    auto G = [&](int j) -> double { return (j >= 0 && j <= ne) ? gsig[(size_t)j * M + o] : 0.0; };
-#pragma unroll 4
-    for (int i = (ne + 1) / L; i >= 0; i--) {  // coefficients of sin(k phi): g_{k-1} (N), g_{k-2} + g_k (P)
-      const int k = L * i + r + 1;
-      const double c0 = G(k - 1) + B.y * c1 - c2;
-      c2 = c1;
-      c1 = c0;
-      const double q0 = (G(k - 2) + (k <= ne ? G(k) : 0.0)) + B.y * p1 - p2;
-      p2 = p1;
-      p1 = q0;
-    }
-    const unsigned pm = lane_group<SH>();
-    const double dN = (2.0 / PI) * s * B.finish(c1, c2, pm), dP = (2.0 / PI) * s * B.finish(p1, p2, pm);
-    if (r == 0) {
-      const double dU = bi * dP - (onsite[o] - ai) * dN;
-      aU += dU / (2.0 * bi);
-      aN += dN / (2.0 * bi);
-    }
+  for (int o = blockIdx.x * RT2 + threadIdx.x; o < M; o += gridDim.x * RT2) {
+    aU += (st->ef - onsite[o]) * dos[o];
+    aN += dos[o];
   }
   const double bU = block_sum<RT2>(aU, sh);
   const double bN = block_sum<RT2>(aN, sh);
@@ -599,7 +571,7 @@ __global__ void __launch_bounds__(FC) k_fermi_coop(int M, const double* __restri
       if (!(xn > l32 && xn < h32)) xn = 0.5 * (l32 + h32);
       const double step = fabs(xn - E);
       E = xn;
-      if (step < 1e-5 || h32 - l32 < 1e-5) break;
+      if (step < 1e-7 || h32 - l32 < 1e-7) break;
     }
     if (!(E > lo && E < hi)) E = 0.5 * (lo + hi);
     grid.sync();  // every block has read the last FP32 partials before they are reused
@@ -711,7 +683,7 @@ __global__ void __launch_bounds__(CT) k_weights(WeightArgs A) {
   for (int k = 0; k <= KPMAX; k++) abar[k] = 0.0;
   for (int k = 0; k <= KPMAX + 1; k++) bbar[k] = 0.0;
   double abar_inf = 0.0, bbar_inf = 0.0;
-  const double dE = chain_reverse<KP>(ch, r.nlev, KP, t.a_inf, t.b_inf, A.onsite[o], A.st->ef, A.g, A.inv, A.n_exp,
+  const double dE = chain_reverse<KP>(ch, r.nlev, KP, t.a_inf, t.b_inf, A.onsite[o], A.st->ef, A.g, A.inv, A.g32, A.n_exp,
                                       M, o, cU, cN, A.zscratch, A.zscratch + (size_t)(A.n_exp + 1) * M, abar, bbar,
                                       abar_inf, bbar_inf, A.sig32 != 0);
   if (A.dU_dE) A.dU_dE[o] = dE;
@@ -754,7 +726,7 @@ __global__ void __launch_bounds__(CT) k_weights_pair(WeightArgs A, double cU1, d
   const double cU[2] = {cU1, cU2}, cN[2] = {cN1, cN2};
   const size_t zl = (size_t)(A.n_exp + 1) * M;
   double* zb[2] = {A.zscratch + zl, A.zscratch + 2 * zl};
-  chain_reverse_ns<KP, 2>(ch, r.nlev, KP, t.a_inf, t.b_inf, A.onsite[o], A.st->ef, A.g, A.inv, A.n_exp, M, o, cU,
+  chain_reverse_ns<KP, 2>(ch, r.nlev, KP, t.a_inf, t.b_inf, A.onsite[o], A.st->ef, A.g, A.inv, A.g32, A.n_exp, M, o, cU,
                           cN, A.zscratch, zb, abar, bbar, abar_inf, bbar_inf, dE, A.sig32 != 0);
   if (A.dU_dE) A.dU_dE[o] = dE[0];
   bool bad = false;
@@ -799,7 +771,7 @@ __global__ void __launch_bounds__(CT) k_weights_split(WeightArgs A, double cU1, 
   double abar_inf = 0.0, bbar_inf = 0.0;
   const size_t zl = (size_t)(A.n_exp + 1) * M;
   double* zs = A.zscratch + (size_t)q * 2 * zl;
-  const double dE = chain_reverse<KP>(ch, r.nlev, KP, tm.a_inf, tm.b_inf, A.onsite[o], A.st->ef, A.g, A.inv,
+  const double dE = chain_reverse<KP>(ch, r.nlev, KP, tm.a_inf, tm.b_inf, A.onsite[o], A.st->ef, A.g, A.inv, A.g32,
                                       A.n_exp, M, o, cU, cN, zs, zs + zl, abar, bbar, abar_inf, bbar_inf,
                                       A.sig32 != 0);
   if (q == 0 && A.dU_dE) A.dU_dE[o] = dE;
@@ -981,7 +953,7 @@ __global__ void __launch_bounds__(CT) k_weights_few(WeightArgs A, double cU1, do
     }
   }
   __syncwarp();
-  // ---- the sums N, P, dN/deps, dP/deps and the cotangents of sigma_m, in blocks of m
+  // ---- the sums N, P, dN/deps and the cotangents of sigma_m, in blocks of m
   const double xr = (ef - ai) / (2.0 * bi);
   const bool inside = xr > -1.0 && xr < 1.0;
   const double x = clamp1(xr);
@@ -993,7 +965,7 @@ __global__ void __launch_bounds__(CT) k_weights_few(WeightArgs A, double cU1, do
     Pbar[q] = cU[q] * bi;
   }
   const int blk = (ne + 8) / 8, m_lo = min(ne + 1, lane8 * blk), m_hi = min(ne + 1, m_lo + blk);
-  double sum[4] = {0.0, 0.0, 0.0, 0.0};
+  double sum[3] = {0.0, 0.0, 0.0};
   {
     constexpr double INV_PI = 1.0 / PI;
     // s_j = sin(j phi) from s_m on, chi_j from s_{j-1} and s_{j+1}
@@ -1012,7 +984,6 @@ __global__ void __launch_bounds__(CT) k_weights_few(WeightArgs A, double cU1, do
       sum[0] += gsm * c_m1;
       sum[1] += gsm * cp;
       sum[2] += gsm * sp1;
-      sum[3] += gsm * (sp2 + s0);
 #pragma unroll
       for (int q = 0; q < NS; q++)
         if (live) zs[(1 + q) * zl + (size_t)m * M + o] = gm * (Nbar[q] * c_m1 + Pbar[q] * cp);
@@ -1025,10 +996,10 @@ __global__ void __launch_bounds__(CT) k_weights_few(WeightArgs A, double cU1, do
     }
   }
 #pragma unroll
-  for (int v = 0; v < 4; v++)
+  for (int v = 0; v < 3; v++)
 #pragma unroll
     for (int w = 1; w < 8; w <<= 1) sum[v] += __shfl_xor_sync(0xffffffffu, sum[v], w);
-  const double Nv = sum[0], Pv = sum[1], dN = sum[2] * (2.0 / PI), dP = sum[3] * (2.0 / PI);
+  const double Nv = sum[0], Pv = sum[1], dN = sum[2] * (2.0 / PI), dP = 2.0 * x * dN;
   __syncwarp();
   // ---- lambda_m = cotangent - sum_j [D_0]_j lambda_{m+j}, downwards, in the cotangents' place
   {
@@ -1306,18 +1277,10 @@ int launch_orbital_NU(int M, int n_exp, const double* gsig, const double* inv, c
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int launch_ef_response(int M, int n_exp, const double* gsig, const double* inv, const double* a_inf,
-                       const double* b_inf, const double* onsite, const FermiState* st, double* red,
+int launch_ef_response(int M, const double* onsite, const double* dos, const FermiState* st, double* red,
                        unsigned* counter, double* lam, cudaStream_t s) {
-  const int sh = lane_shift(M), g = red_grid2(M << sh);
-#define EF_RESPONSE(SH) \
-  k_ef_response2<SH><<<g, RT2, 0, s>>>(M, n_exp, gsig, inv, a_inf, b_inf, onsite, st, red, counter, lam)
-  switch (sh) {
-    case 0: EF_RESPONSE(0); break;
-    case 1: EF_RESPONSE(1); break;
-    case 2: EF_RESPONSE(2); break;
-    default: EF_RESPONSE(3); break;
-  }
-#undef EF_RESPONSE
+  int g = red_grid2(M);
+  if (g > 8 * sm_count()) g = 8 * sm_count();
+  k_ef_response2<<<g, RT2, 0, s>>>(M, onsite, dos, st, red, counter, lam);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -125,16 +125,12 @@ __device__ inline void recursion_taped(const double* mu, Rec& r, RecTape<KP>& tp
   tp.C[0][0] = 1.0;
   const double width = fmax(mu[2] - mu[1] * mu[1], 0.0);
   for (int n = 0; n < KP; n++) {
-    double an = 0.0;
-    for (int j = 0; j <= n; j++)
-      for (int l = 0; l <= n; l++) an += c[j] * c[l] * mu[j + l + 1];
+    const double an = hankel_form(c, mu, n + 1, 1);
     r.a[n] = an;
     for (int j = 0; j < KP + 2; j++) d[j] = 0.0;
     for (int j = 0; j <= n + 1; j++) d[j] = (j >= 1 ? c[j - 1] : 0.0) - an * c[j] - r.b[n] * cp[j];
     for (int j = 0; j < KP + 2; j++) tp.Dv[n][j] = d[j];
-    double b2 = 0.0;
-    for (int j = 0; j <= n + 1; j++)
-      for (int l = 0; l <= n + 1; l++) b2 += d[j] * d[l] * mu[j + l];
+    const double b2 = hankel_form(d, mu, n + 2, 0);
     if (b2 <= TRUNC_REL * width) {
       r.b[n + 1] = 0.0;
       r.nlev = n + 1;
@@ -145,11 +141,11 @@ __device__ inline void recursion_taped(const double* mu, Rec& r, RecTape<KP>& tp
       }
       break;
     }
-    const double bn = sqrt(b2);
+    const double bn = sqrt(b2), ib = 1.0 / bn;
     r.b[n + 1] = bn;
     for (int j = 0; j < KP + 2; j++) {
       cp[j] = c[j];
-      c[j] = d[j] / bn;
+      c[j] = d[j] * ib;
       tp.C[n + 1][j] = c[j];
     }
   }
@@ -215,15 +211,17 @@ __device__ __forceinline__ void chain_polys_reverse(const Chain& ch, int L, int 
     ahb[k] += ga;
     bhb[k + 1] += gb;
   }
+  const double ib = 1.0 / bi, i2b = 0.5 * ib;
   for (int k = 0; k < L; k++) {
-    abar[k] += ahb[k] / (2.0 * bi);
-    abar_inf += -ahb[k] / (2.0 * bi);
-    bbar_inf += -ahb[k] * ch.ah[k] / bi;
+    const double g = ahb[k] * i2b;
+    abar[k] += g;
+    abar_inf -= g;
+    bbar_inf -= ahb[k] * ch.ah[k] * ib;
   }
   for (int k = 1; k <= Kb; k++)
     if (k <= L) {
-      bbar[k] += bhb[k] / (2.0 * bi);
-      bbar_inf += -bhb[k] * ch.bh[k] / bi;
+      bbar[k] += bhb[k] * i2b;
+      bbar_inf -= bhb[k] * ch.bh[k] * ib;
     }
 }
 
@@ -238,8 +236,8 @@ __device__ __forceinline__ void chain_polys_reverse(const Chain& ch, int L, int 
 // its cotangent for seed q, [ne+1][M] each.
 template <int KP, int NS>
 __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double ai, double bi, double E, double ef,
-                                        const double* __restrict__ g, const double* __restrict__ inv, int ne, int M,
-                                        int o, const double* cU, const double* cN, double* zs, double* const* zb,
+                                        const double* __restrict__ g, const double* __restrict__ inv,
+                                        const float* __restrict__ g32, int ne, int M, int o, const double* cU, const double* cN, double* zs, double* const* zb,
                                         double (*abar)[KPMAX + 1], double (*bbar)[KPMAX + 2], double* abar_inf,
                                         double* bbar_inf, double* dE, bool f32 = false) {
   constexpr int NP = 2 * KP + 1;
@@ -287,7 +285,8 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
     Nbar[q] = cN[q] - cU[q] * (E - ai);
     Pbar[q] = cU[q] * bi;
   }
-  double Nv = 0.0, Pv = 0.0, dN = 0.0, dP = 0.0;
+  // (dP/deps needs no sum of its own: sin((m+2) phi) + sin(m phi) = 2 x sin((m+1) phi))
+  double Nv = 0.0, Pv = 0.0, dN = 0.0;
   if (f32) {
     // the same sums in FP32 (sigma_m and its cotangent in FP32 scratch): the
     // sines s_j = sin(j phi) = sinpi(j phi/pi) directly (no recurrence, so no
@@ -310,15 +309,14 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
     };
     float s0 = 0.f, sp1 = sinpif(theta), sp2 = sinpif(2.f * theta), sp3 = sinpif(3.f * theta);
     float c_m = 0.f, c_m1 = chi(1, s0, sp2);
-    float Nf = 0.f, Pf = 0.f, dNf = 0.f, dPf = 0.f;
+    float Nf = 0.f, Pf = 0.f, dNf = 0.f;
     for (int m = 0; m <= ne; m++) {
       const float c_m2 = chi(m + 2, sp1, sp3);
-      const float gm = (float)g[m];
+      const float gm = g32[m];
       const float gsm = gm * zsf[(size_t)m * M + o];
       Nf += gsm * c_m1;
       Pf += gsm * (c_m2 + c_m);
       dNf += gsm * sp1;
-      dPf += gsm * (sp2 + s0);
 #pragma unroll
       for (int q = 0; q < NS; q++) zbf[q][(size_t)m * M + o] = gm * (Nbf[q] * c_m1 + Pbf[q] * (c_m2 + c_m));
       c_m = c_m1;
@@ -331,7 +329,6 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
     Nv = Nf;
     Pv = Pf;
     dN = dNf * (2.0 / PI);
-    dP = dPf * (2.0 / PI);
   } else {
     // sines s_j = sin(j phi) by the recurrence; chi_j = (s~_{j+1} - s~_{j-1})/pi,
     // s~_k = sin(k phi)/k, s~_0 = phi - pi
@@ -351,7 +348,6 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
       Nv += gsm * c_m1;
       Pv += gsm * (c_m2 + c_m);
       dN += gsm * sp1;
-      dP += gsm * (sp2 + s0);
 #pragma unroll
       for (int q = 0; q < NS; q++) zb[q][(size_t)m * M + o] = g[m] * (Nbar[q] * c_m1 + Pbar[q] * (c_m2 + c_m));
       c_m = c_m1;
@@ -362,8 +358,8 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
       sp3 = 2.0 * x * sp2 - sp1;
     }
     dN *= 2.0 / PI;
-    dP *= 2.0 / PI;
   }
+  const double dP = 2.0 * x * dN;
 #pragma unroll
   for (int q = 0; q < NS; q++) {
     abar_inf[q] += cU[q] * Nv;
@@ -453,15 +449,15 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
 // One seed (cU, cN); returns dL/dE.
 template <int KP>
 __device__ inline double chain_reverse(const Chain& ch, int L, int Kb, double ai, double bi, double E, double ef,
-                                       const double* __restrict__ g, const double* __restrict__ inv, int ne,
-                                       int M, int o, double cU, double cN, double* zs, double* zb, double* abar,
+                                       const double* __restrict__ g, const double* __restrict__ inv,
+                                       const float* __restrict__ g32, int ne, int M, int o, double cU, double cN, double* zs, double* zb, double* abar,
                                        double* bbar, double& abar_inf, double& bbar_inf, bool f32 = false) {
   double* zbs[1] = {zb};
   double ab[1][KPMAX + 1], bb_[1][KPMAX + 2];
   for (int k = 0; k <= KPMAX; k++) ab[0][k] = abar[k];
   for (int k = 0; k <= KPMAX + 1; k++) bb_[0][k] = bbar[k];
   double ai_[1] = {abar_inf}, bi_[1] = {bbar_inf}, dE[1];
-  chain_reverse_ns<KP, 1>(ch, L, Kb, ai, bi, E, ef, g, inv, ne, M, o, &cU, &cN, zs, zbs, ab, bb_, ai_, bi_, dE, f32);
+  chain_reverse_ns<KP, 1>(ch, L, Kb, ai, bi, E, ef, g, inv, g32, ne, M, o, &cU, &cN, zs, zbs, ab, bb_, ai_, bi_, dE, f32);
   for (int k = 0; k <= KPMAX; k++) abar[k] = ab[0][k];
   for (int k = 0; k <= KPMAX + 1; k++) bbar[k] = bb_[0][k];
   abar_inf = ai_[0];
@@ -537,20 +533,20 @@ __device__ inline void recursion_reverse(const double* mu, const Rec& r, const R
     for (int j = 0; j < KP + 2; j++) db[j] = 0.0;
     const bool made_next = !(r.trunc && n == L - 1);
     if (made_next) {
-      const double bn = r.b[n + 1];
+      const double ib = 1.0 / r.b[n + 1];
       double dotc = 0.0;
       for (int j = 0; j <= n + 1; j++) {
-        db[j] = cb[n + 1][j] / bn;
-        dotc += cb[n + 1][j] * tp.Dv[n][j];
+        db[j] = cb[n + 1][j] * ib;
+        dotc += db[j] * tp.Dv[n][j];
       }
-      const double bnb = bbar[n + 1] - dotc / (bn * bn);
-      const double b2b = bnb / (2.0 * bn);
+      const double b2b = (bbar[n + 1] - dotc * ib) * (0.5 * ib);
       for (int j = 0; j <= n + 1; j++) {
         double acc = 0.0;
-        for (int l = 0; l <= n + 1; l++) {
-          acc += mu[j + l] * tp.Dv[n][l];
-          mub[j + l] += b2b * tp.Dv[n][j] * tp.Dv[n][l];
-        }
+        for (int l = 0; l <= n + 1; l++) acc += mu[j + l] * tp.Dv[n][l];
+        // d/dmu of the form: each unordered pair of coefficients once
+        const double g = b2b * tp.Dv[n][j], g2 = 2.0 * g;
+        mub[2 * j] += g * tp.Dv[n][j];
+        for (int l = j + 1; l <= n + 1; l++) mub[j + l] += g2 * tp.Dv[n][l];
         db[j] += 2.0 * b2b * acc;
       }
     }
@@ -566,10 +562,10 @@ __device__ inline void recursion_reverse(const double* mu, const Rec& r, const R
     }
     for (int j = 0; j <= n; j++) {
       double acc = 0.0;
-      for (int l = 0; l <= n; l++) {
-        acc += mu[j + l + 1] * tp.C[n][l];
-        mub[j + l + 1] += an_b * tp.C[n][j] * tp.C[n][l];
-      }
+      for (int l = 0; l <= n; l++) acc += mu[j + l + 1] * tp.C[n][l];
+      const double g = an_b * tp.C[n][j], g2 = 2.0 * g;
+      mub[2 * j + 1] += g * tp.C[n][j];
+      for (int l = j + 1; l <= n; l++) mub[j + l + 1] += g2 * tp.C[n][l];
       cb[n][j] += 2.0 * an_b * acc;
     }
   }

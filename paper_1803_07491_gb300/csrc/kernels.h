@@ -321,7 +321,8 @@ struct WeightArgs {
   const double* onsite;  // [M]
   const FermiState* st;
   const double* g;
-  const double* inv;     // [n_exp+8] 1/k
+  const float* g32;      // the same in FP32 (a conversion costs a double-precision instruction)
+  const double* inv;     // [n_exp+16] 1/k
   double cU;             // L = cU*U + cN*N
   const double* lam;     // device scalar: cN = -cU * (*lam)  (E_F response); NULL: cN = cN0
   double cN0;
@@ -342,8 +343,7 @@ int launch_weights(const WeightArgs& a, cudaStream_t s);
 // fixed E_F (a.lam unused), one lane per seed; a.zscratch: [4][n_exp+1][M].
 int launch_weights_pair(const WeightArgs& a, double cU1, double cN1, double cU2, double cN2, double* w2,
                         cudaStream_t s);
-int launch_ef_response(int M, int n_exp, const double* gsig, const double* inv, const double* a_inf,
-                       const double* b_inf, const double* onsite, const FermiState* st, double* red,
+int launch_ef_response(int M, const double* onsite, const double* dos, const FermiState* st, double* red,
                        unsigned* counter, double* lam, cudaStream_t s);
 
 // learned.cu: the learned terminator (n_mom = 9, continued to 8 levels)

@@ -29,24 +29,54 @@ constexpr int NB = 10;         // base record: a_0..a_3, b_1..b_4, a_inf, b_inf
 __device__ __forceinline__ double ldv(const float* p, size_t i) { return p[i]; }
 __device__ __forceinline__ double ldv(const double* p, size_t i) { return p[i]; }
 
+// The normalisation vector in FP64 in shared memory, with the reciprocals of
+// the input deviations in their place: once per block, where a conversion of
+// every orbital would cost as much as a multiplication and a division nine.
+struct NormTable {
+  double v[BOP_MLP_NNORM];
+};
+__device__ __forceinline__ void load_norm(const float* __restrict__ norm, NormTable& n) {
+  for (int j = threadIdx.x; j < BOP_MLP_NNORM; j += CT) {
+    const double x = (double)norm[j];
+    n.v[j] = j >= NORM_XS && j < NORM_XS + NI ? 1.0 / x : x;
+  }
+  __syncthreads();
+}
+
+// Moments about a: m_n = sum_l C(n,l) (-a)^l mu_{n-l} (n <= 8) by repeated
+// differences, m_k -= a m_{k-1}.
+__device__ __forceinline__ void shift_moments(double m[9], double a) {
+#pragma unroll
+  for (int p = 1; p <= 8; p++)
+#pragma unroll
+    for (int k = 8; k >= p; k--) m[k] -= a * m[k - 1];
+}
+// Its transpose.
+__device__ __forceinline__ void shift_moments_transposed(double y[9], double a) {
+#pragma unroll
+  for (int p = 8; p >= 1; p--)
+#pragma unroll
+    for (int k = p; k <= 8; k++) y[k - 1] -= a * y[k];
+}
+
 // Inputs of the network for one orbital (9-moment chain r, terminator t).
 __device__ inline void features9(const double* mu, const Rec& r, const Term& t, double x[NI]) {
-  const double ai = t.a_inf, bi = t.b_inf;
-  for (int k = 0; k < KB; k++) x[k] = (r.a[k] - ai) / bi;
-  for (int k = 1; k <= KB; k++) x[KB + k - 1] = r.b[k] / bi;
+  const double ai = t.a_inf, bi = t.b_inf, ib = 1.0 / bi;
+  for (int k = 0; k < KB; k++) x[k] = (r.a[k] - ai) * ib;
+  for (int k = 1; k <= KB; k++) x[KB + k - 1] = r.b[k] * ib;
   x[8] = ai;
   x[9] = bi;
   // mu-hat_n = (2 b_inf)^-n sum_l C(n,l) (-a_inf)^l mu_{n-l}
+  double m[9];
+#pragma unroll
+  for (int n = 0; n < 9; n++) m[n] = mu[n];
+  shift_moments(m, ai);
+  const double i2b = 0.5 * ib;
   double s = 1.0;
+#pragma unroll
   for (int n = 1; n <= 8; n++) {
-    s /= (2.0 * bi);
-    double acc = 0.0, c = 1.0, p = 1.0;  // C(n,l), (-a_inf)^l
-    for (int l = 0; l <= n; l++) {
-      acc += c * p * mu[n - l];
-      c = c * (double)(n - l) / (double)(l + 1);
-      p *= -ai;
-    }
-    x[9 + n] = acc * s;
+    s *= i2b;
+    x[9 + n] = m[n] * s;
   }
 }
 
@@ -95,15 +125,16 @@ __device__ inline void base_chain(const double* base, int nlev, Rec& r, Term& t)
 }
 
 template <class T>
-__device__ inline void destandardise(const LearnedArgs& A, int o, double yh[NO]) {
+__device__ inline void destandardise(const LearnedArgs& A, const NormTable& nt, int o, double yh[NO]) {
   const T* ys = static_cast<const T*>(A.ys);
-  for (int j = 0; j < NO; j++)
-    yh[j] = (double)A.norm[NORM_YM + j] + (double)A.norm[NORM_YS + j] * ldv(ys, (size_t)o * NO + j);
+  for (int j = 0; j < NO; j++) yh[j] = nt.v[NORM_YM + j] + nt.v[NORM_YS + j] * ldv(ys, (size_t)o * NO + j);
 }
 
 // mu[9] -> base record, nlev, standardised inputs, in-range flag.
 template <class T>
 __global__ void __launch_bounds__(CT) k_features(LearnedArgs A) {
+  __shared__ NormTable nt;
+  load_norm(A.norm, nt);
   const int o = blockIdx.x * CT + threadIdx.x;
   if (o >= A.M) return;
   double mu[9];
@@ -122,8 +153,8 @@ __global__ void __launch_bounds__(CT) k_features(LearnedArgs A) {
   bool inside = r.nlev == KB;
   T* xs = static_cast<T*>(A.xs);
   for (int j = 0; j < NI; j++) {
-    inside &= x[j] >= (double)A.norm[NORM_LO + j] && x[j] <= (double)A.norm[NORM_HI + j];
-    xs[(size_t)o * NI + j] = (T)((x[j] - (double)A.norm[NORM_XM + j]) / (double)A.norm[NORM_XS + j]);
+    inside &= x[j] >= nt.v[NORM_LO + j] && x[j] <= nt.v[NORM_HI + j];
+    xs[(size_t)o * NI + j] = (T)((x[j] - nt.v[NORM_XM + j]) * nt.v[NORM_XS + j]);
   }
   A.flag[o] = inside ? 1 : 0;
 }
@@ -131,11 +162,13 @@ __global__ void __launch_bounds__(CT) k_features(LearnedArgs A) {
 // Continued chain -> a*_inf, b*_inf, g_m sigma_m (n_exp + 1 terms).
 template <class T>
 __global__ void __launch_bounds__(CT) k_expand_learned(LearnedArgs A) {
+  __shared__ NormTable nt;
+  load_norm(A.norm, nt);
   const int o = blockIdx.x * CT + threadIdx.x;
   bool ok = false;
   if (o < A.M) {
     double yh[NO];
-    destandardise<T>(A, o, yh);
+    destandardise<T>(A, nt, o, yh);
     const double* base = A.base + (size_t)o * NB;
     Rec r;
     Term t;
@@ -160,6 +193,8 @@ __global__ void __launch_bounds__(CT) k_expand_learned(LearnedArgs A) {
 // standardised) and of the base record (cot).
 template <class T>
 __global__ void __launch_bounds__(CT) k_weights_learned_a(LearnedArgs A) {
+  __shared__ NormTable nt;
+  load_norm(A.norm, nt);
   const int o = blockIdx.x * CT + threadIdx.x;
   if (o >= A.M) return;
   const WeightArgs& W = A.W;
@@ -168,7 +203,7 @@ __global__ void __launch_bounds__(CT) k_weights_learned_a(LearnedArgs A) {
   const double cN = W.var_q ? cU * (W.var_J * W.var_q[o / W.norb] - W.var_lam[0])
                             : (W.lam ? -W.cU * W.lam[0] : W.cN0);
   double yh[NO];
-  destandardise<T>(A, o, yh);
+  destandardise<T>(A, nt, o, yh);
   const double* base = A.base + (size_t)o * NB;
   const bool learned = (A.flag[o] & 2) != 0;
   Rec r;
@@ -182,7 +217,7 @@ __global__ void __launch_bounds__(CT) k_weights_learned_a(LearnedArgs A) {
   for (int k = 0; k <= KPMAX + 1; k++) bbar[k] = 0.0;
   double abar_inf = 0.0, bbar_inf = 0.0;
   const double dE = chain_reverse<KX>(ch, r.nlev, learned ? KX : KB, t.a_inf, t.b_inf, W.onsite[o], W.st->ef, W.g,
-                                      W.inv, W.n_exp, M, o, cU, cN, W.zscratch,
+                                      W.inv, W.g32, W.n_exp, M, o, cU, cN, W.zscratch,
                                       W.zscratch + (size_t)(W.n_exp + 1) * M, abar, bbar, abar_inf, bbar_inf,
                                       A.sig32 != 0);
   if (W.dU_dE) W.dU_dE[o] = dE;
@@ -211,7 +246,7 @@ __global__ void __launch_bounds__(CT) k_weights_learned_a(LearnedArgs A) {
     bib = bbar_inf;
   }
   T* ybar = static_cast<T*>(A.ybar);
-  for (int j = 0; j < NO; j++) ybar[(size_t)o * NO + j] = (T)(yb[j] * (double)A.norm[NORM_YS + j]);
+  for (int j = 0; j < NO; j++) ybar[(size_t)o * NO + j] = (T)(yb[j] * nt.v[NORM_YS + j]);
   double* cot = A.cot + (size_t)o * NB;
   for (int k = 0; k < KB; k++) cot[k] = abar[k];
   for (int k = 1; k <= KB; k++) cot[KB + k - 1] = bbar[k];
@@ -222,6 +257,8 @@ __global__ void __launch_bounds__(CT) k_weights_learned_a(LearnedArgs A) {
 // Reverse of the features, Gershgorin and the moment recursion -> w.
 template <class T>
 __global__ void __launch_bounds__(CT) k_weights_learned_b(LearnedArgs A) {
+  __shared__ NormTable nt;
+  load_norm(A.norm, nt);
   const int o = blockIdx.x * CT + threadIdx.x;
   if (o >= A.M) return;
   double mu[9];
@@ -242,37 +279,41 @@ __global__ void __launch_bounds__(CT) k_weights_learned_b(LearnedArgs A) {
   if (A.flag[o] & 2) {
     const T* xbar = static_cast<const T*>(A.xbar);
     double xb[NI];
-    for (int j = 0; j < NI; j++) xb[j] = ldv(xbar, (size_t)o * NI + j) / (double)A.norm[NORM_XS + j];
-    const double ai = t.a_inf, bi = t.b_inf;
+    for (int j = 0; j < NI; j++) xb[j] = ldv(xbar, (size_t)o * NI + j) * nt.v[NORM_XS + j];
+    const double ai = t.a_inf, bi = t.b_inf, ib = 1.0 / bi;
     for (int k = 0; k < KB; k++) {  // x_k = (a_k - a_inf)/b_inf
-      const double xk = (r.a[k] - ai) / bi;
-      abar[k] += xb[k] / bi;
-      abar_inf -= xb[k] / bi;
-      bbar_inf -= xb[k] * xk / bi;
+      const double g = xb[k] * ib;
+      abar[k] += g;
+      abar_inf -= g;
+      bbar_inf -= g * ((r.a[k] - ai) * ib);
     }
     for (int k = 1; k <= KB; k++) {  // x = b_k/b_inf
-      const double xk = r.b[k] / bi;
-      bbar[k] += xb[KB + k - 1] / bi;
-      bbar_inf -= xb[KB + k - 1] * xk / bi;
+      const double g = xb[KB + k - 1] * ib;
+      bbar[k] += g;
+      bbar_inf -= g * (r.b[k] * ib);
     }
     abar_inf += xb[8];
     bbar_inf += xb[9];
+    // mu-hat_n = s_n m_n, s_n = (2 b_inf)^-n, m_n the moments about a_inf with
+    // dm_n/da_inf = -n m_{n-1}
+    double m[9], y[9];
+#pragma unroll
+    for (int n = 0; n < 9; n++) m[n] = mu[n];
+    shift_moments(m, ai);
+    const double i2b = 0.5 * ib;
     double s = 1.0;
-    for (int n = 1; n <= 8; n++) {  // mu-hat_n
-      s /= (2.0 * bi);
-      const double g = xb[9 + n];
-      double acc = 0.0, dacc = 0.0, c = 1.0, p = 1.0, pm = 0.0;  // pm = (-a_inf)^(l-1)
-      for (int l = 0; l <= n; l++) {
-        acc += c * p * mu[n - l];
-        mub[n - l] += g * s * c * p;
-        if (l >= 1) dacc += c * (double)l * pm * mu[n - l];  // d/d(-a_inf) of (-a_inf)^l
-        c = c * (double)(n - l) / (double)(l + 1);
-        pm = p;
-        p *= -ai;
-      }
-      abar_inf += -g * s * dacc;
-      bbar_inf += -g * (double)n / bi * acc * s;
+    y[0] = 0.0;
+#pragma unroll
+    for (int n = 1; n <= 8; n++) {
+      s *= i2b;
+      y[n] = xb[9 + n] * s;
+      const double ny = (double)n * y[n];
+      abar_inf -= ny * m[n - 1];
+      bbar_inf -= ny * ib * m[n];
     }
+    shift_moments_transposed(y, ai);
+#pragma unroll
+    for (int n = 0; n < 9; n++) mub[n] += y[n];
   }
   gershgorin_reverse(t, abar_inf, bbar_inf, abar, bbar);
   recursion_reverse<KB>(mu, r, tp, abar, bbar, mub);

@@ -15,12 +15,14 @@
 namespace {
 using namespace scal;
 
+// g: [n_exp + 1] doubles, then the same in FP32
 __global__ void k_jackson(double* g, int n_exp) {
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m > n_exp) return;
   const double N = n_exp, x = PI / (N + 1.0);
   auto gJ = [&](double mm) { return ((N - mm + 1.0) * cos(mm * x) + sin(mm * x) / tan(x)) / (N + 1.0); };
   g[m] = gJ(m + 1.0) / gJ(1.0);
+  reinterpret_cast<float*>(g + n_exp + 1)[m] = (float)g[m];
 }
 
 // N(phi) per orbital from the sine series by Clenshaw's recurrence.

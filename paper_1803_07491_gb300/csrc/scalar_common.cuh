@@ -20,6 +20,19 @@ struct Rec {
   bool trunc;
 };
 
+// sum_j sum_l v_j v_l mu_{j+l+off} over j, l < cnt (the inner sums first: half
+// the multiplications of the double sum term by term; a double-precision
+// division costs nine of them, hence the reciprocals below).
+__device__ __forceinline__ double hankel_form(const double* v, const double* mu, int cnt, int off) {
+  double t = 0.0;
+  for (int j = 0; j < cnt; j++) {
+    double u = 0.0;
+    for (int l = 0; l < cnt; l++) u += v[l] * mu[j + l + off];
+    t += v[j] * u;
+  }
+  return t;
+}
+
 // a_n = sum c_j c_l mu_{j+l+1};  b_{n+1} c^{n+1} = c^n shifted - a_n c^n - b_n c^{n-1}
 __device__ inline void recursion(const double* mu, int Kp, Rec& r) {
   double c[KPMAX + 2], cp[KPMAX + 2], d[KPMAX + 2];
@@ -30,14 +43,10 @@ __device__ inline void recursion(const double* mu, int Kp, Rec& r) {
   r.trunc = false;
   double width = fmax(mu[2] - mu[1] * mu[1], 0.0);
   for (int n = 0; n < Kp; n++) {
-    double an = 0.0;
-    for (int j = 0; j <= n; j++)
-      for (int l = 0; l <= n; l++) an += c[j] * c[l] * mu[j + l + 1];
+    const double an = hankel_form(c, mu, n + 1, 1);
     r.a[n] = an;
     for (int j = 0; j <= n + 1; j++) d[j] = (j >= 1 ? c[j - 1] : 0.0) - an * c[j] - r.b[n] * cp[j];
-    double b2 = 0.0;
-    for (int j = 0; j <= n + 1; j++)
-      for (int l = 0; l <= n + 1; l++) b2 += d[j] * d[l] * mu[j + l];
+    const double b2 = hankel_form(d, mu, n + 2, 0);
     if (b2 <= TRUNC_REL * width) {
       r.b[n + 1] = 0.0;
       r.nlev = n + 1;
@@ -48,11 +57,11 @@ __device__ inline void recursion(const double* mu, int Kp, Rec& r) {
       }
       return;
     }
-    double bn = sqrt(b2);
+    const double bn = sqrt(b2), ib = 1.0 / bn;
     r.b[n + 1] = bn;
     for (int j = 0; j <= n + 1; j++) {
       cp[j] = c[j];
-      c[j] = d[j] / bn;
+      c[j] = d[j] * ib;
     }
   }
 }
@@ -167,9 +176,10 @@ __device__ inline void chain_params(const Rec& r, const Term& t, int Kp, Chain& 
   for (int k = 0; k <= KPMAX; k++) ch.ah[k] = 0.0;
   for (int k = 0; k <= KPMAX + 1; k++) ch.bh[k] = 0.5;
   ch.bh[0] = 0.0;
-  for (int k = 0; k < r.nlev; k++) ch.ah[k] = (r.a[k] - t.a_inf) / (2.0 * t.b_inf);
+  const double i2b = 1.0 / (2.0 * t.b_inf);
+  for (int k = 0; k < r.nlev; k++) ch.ah[k] = (r.a[k] - t.a_inf) * i2b;
   for (int k = 1; k <= Kp; k++)
-    if (k <= r.nlev) ch.bh[k] = r.b[k] / (2.0 * t.b_inf);
+    if (k <= r.nlev) ch.bh[k] = r.b[k] * i2b;
 }
 __device__ __forceinline__ double AH(const Chain& ch, int k) { return k <= KPMAX ? ch.ah[k] : 0.0; }
 __device__ __forceinline__ double BH(const Chain& ch, int k) { return k <= KPMAX + 1 ? ch.bh[k] : 0.5; }
