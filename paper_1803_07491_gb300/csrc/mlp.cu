@@ -1,15 +1,15 @@
 // The learned-terminator network 18 -> 128 -> 128 -> 10 (GELU): training
-// (FP32 forward, reverse mode, Adam) and inference (bfloat16 weights,
-// FP32 or FP64 activations) as tiled GEMMs with fused bias / GELU /
-// GELU-derivative epilogues (the FP32 inference on the tensor pipe, the rest
-// as SIMT tiles), plus the bop_mlp object of the C ABI.
+// (FP32 forward and reverse of a batch in one kernel, then the sum of its
+// partial gradients, then Adam) and inference (bfloat16 weights, FP32 or FP64
+// activations) as tiled GEMMs with fused bias / GELU / GELU-derivative
+// epilogues (FP32 on the tensor pipe, FP64 as SIMT tiles), plus the bop_mlp
+// object of the C ABI.
 //
 // The layers are small dense contractions (K = 18, 128, 10) applied to
-// every orbital of a structure (hundreds of thousands of rows); the MLP is
-// a few per cent of an energy + force evaluation, so the kernels are plain
-// 64 x 64 register-blocked tiles.  Every reduction (weight gradients over a
-// batch, the loss, the bias gradients, the normalisation statistics) runs
-// in a fixed order, so training is deterministic.
+// every orbital of a structure (hundreds of thousands of rows).  Every
+// reduction (weight gradients over a batch, the loss, the bias gradients, the
+// normalisation statistics) runs in a fixed order, so training is
+// deterministic.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -32,12 +32,7 @@ constexpr int NORM_XM = 0, NORM_XS = NI, NORM_LO = 2 * NI, NORM_HI = 3 * NI, NOR
 static_assert(NORM_YS + NO == BOP_MLP_NNORM, "normalisation layout");
 
 constexpr int GBM = 64, GBN = 64, GBK = 16, GT = 256;
-constexpr int KCHUNK = 512;  // batch rows per split of a weight-gradient GEMM
 constexpr int RT = 256;
-
-__device__ __forceinline__ float ld(const float* p, size_t i) { return p[i]; }
-__device__ __forceinline__ double ld(const double* p, size_t i) { return p[i]; }
-__device__ __forceinline__ float ld(const __nv_bfloat16* p, size_t i) { return __bfloat162float(p[i]); }
 
 __device__ __forceinline__ float ncdf(float x) { return normcdff(x); }
 __device__ __forceinline__ double ncdf(double x) { return normcdf(x); }
@@ -57,7 +52,7 @@ __device__ __forceinline__ T gelu_d(T z) {
 enum { EPI_NONE = 0, EPI_BIAS = 1, EPI_BIAS_GELU = 2, EPI_DGELU = 3 };
 
 struct GemmArgs {
-  int M, N, K, lda, ldb, ldc, kchunk;
+  int M, N, K, lda, ldb, ldc;
   const void* A;
   const void* B;
   void* C;
@@ -65,42 +60,36 @@ struct GemmArgs {
   void* Z;            // EPI_BIAS_GELU: pre-activation out [M][ldc]; EPI_DGELU: pre-activation in
 };
 
-// C[m][n] = sum_k opA(m,k) opB(k,n) with
-//   opA(m,k) = TA ? A[k lda + m] : A[m lda + k],
-//   opB(k,n) = TB ? B[n ldb + k] : B[k ldb + n],
-// over k in [z kchunk, min(K, (z+1) kchunk)) for split z = blockIdx.z (the
-// output of split z starts at C + z M ldc).  Tiles of 64 x 64, 16-deep
-// slabs in shared memory, 4 x 4 outputs per thread; ragged edges guarded.
-template <class T, class TAe, class TBe, bool TA, bool TB, int EPI>
+// C[m][n] = sum_k A[m lda + k] opB(k,n), opB(k,n) = TB ? B[n ldb + k] : B[k ldb + n].
+// Tiles of 64 x 64, 16-deep slabs in shared memory, 4 x 4 outputs per thread;
+// ragged edges guarded.
+template <class T, bool TB, int EPI>
 __global__ void __launch_bounds__(GT) k_gemm(GemmArgs g) {
   __shared__ T As[GBK][GBM + 4];
   __shared__ T Bs[GBK][GBN + 4];
-  const TAe* A = static_cast<const TAe*>(g.A);
-  const TBe* B = static_cast<const TBe*>(g.B);
+  const T* A = static_cast<const T*>(g.A);
+  const __nv_bfloat16* B = static_cast<const __nv_bfloat16*>(g.B);
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   const int m0 = blockIdx.x * GBM, n0 = blockIdx.y * GBN;
-  const int kb = blockIdx.z * g.kchunk;
-  const int ke = min(g.K, kb + g.kchunk);
   T acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
     for (int j = 0; j < 4; j++) acc[i][j] = T(0);
-  for (int k0 = kb; k0 < ke; k0 += GBK) {
+  for (int k0 = 0; k0 < g.K; k0 += GBK) {
 #pragma unroll
     for (int q = 0; q < 4; q++) {
       const int e = tid + q * GT;
-      int ml, kl;
-      if (TA) { ml = e % GBM; kl = e / GBM; } else { ml = e / GBK; kl = e % GBK; }
+      const int ml = e / GBK, kl = e % GBK;
       const int m = m0 + ml, k = k0 + kl;
       T v = T(0);
-      if (m < g.M && k < ke) v = (T)ld(A, TA ? (size_t)k * g.lda + m : (size_t)m * g.lda + k);
+      if (m < g.M && k < g.K) v = A[(size_t)m * g.lda + k];
       As[kl][ml] = v;
       int nl, kl2;
       if (TB) { kl2 = e % GBK; nl = e / GBK; } else { nl = e % GBN; kl2 = e / GBN; }
       const int n = n0 + nl, k2 = k0 + kl2;
       T w = T(0);
-      if (n < g.N && k2 < ke) w = (T)ld(B, TB ? (size_t)n * g.ldb + k2 : (size_t)k2 * g.ldb + n);
+      if (n < g.N && k2 < g.K) w = (T)__bfloat162float(B[TB ? (size_t)n * g.ldb + k2 : (size_t)k2 * g.ldb + n]);
       Bs[kl2][nl] = w;
     }
     __syncthreads();
@@ -118,7 +107,7 @@ __global__ void __launch_bounds__(GT) k_gemm(GemmArgs g) {
     }
     __syncthreads();
   }
-  T* C = static_cast<T*>(g.C) + (size_t)blockIdx.z * g.M * g.ldc;
+  T* C = static_cast<T*>(g.C);
   T* Z = static_cast<T*>(g.Z);
 #pragma unroll
   for (int i = 0; i < 4; i++) {
@@ -144,14 +133,13 @@ __global__ void __launch_bounds__(GT) k_gemm(GemmArgs g) {
   }
 }
 
-template <class T, class TAe, class TBe, bool TA, bool TB, int EPI>
+template <class T, bool TB, int EPI>
 int gemm(int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc, const float* bias,
-         void* Z, int kchunk, cudaStream_t s) {
+         void* Z, cudaStream_t s) {
   if (M <= 0 || N <= 0) return 0;
-  GemmArgs g{M, N, K, lda, ldb, ldc, kchunk > 0 ? kchunk : K, A, B, C, bias, Z};
-  const int splits = kchunk > 0 ? (K + kchunk - 1) / kchunk : 1;
-  dim3 grid((M + GBM - 1) / GBM, (N + GBN - 1) / GBN, splits < 1 ? 1 : splits);
-  k_gemm<T, TAe, TBe, TA, TB, EPI><<<grid, GT, 0, s>>>(g);
+  GemmArgs g{M, N, K, lda, ldb, ldc, A, B, C, bias, Z};
+  dim3 grid((M + GBM - 1) / GBM, (N + GBN - 1) / GBN);
+  k_gemm<T, TB, EPI><<<grid, GT, 0, s>>>(g);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -285,7 +273,7 @@ int gemm_tc(int M, int N, int K, const float* A, int lda, const __nv_bfloat16* B
             const float* bias, float* Z, cudaStream_t s) {
   if (M <= 0 || N <= 0) return 0;
   if (K > KP || N > NP) return -1;
-  GemmArgs g{M, N, K, lda, ldb, ldc, K, A, B, C, bias, Z};
+  GemmArgs g{M, N, K, lda, ldb, ldc, A, B, C, bias, Z};
   constexpr size_t smem = (size_t)NP * (KP + 8) * sizeof(__nv_bfloat16) + (size_t)TC_ROWS * (KP + 8) * sizeof(float);
   auto fn = k_gemm_tc<KP, NP, TB, EPI>;
   static int per_sm = 0, sms = 0;
@@ -304,110 +292,389 @@ int gemm_tc(int M, int N, int K, const float* A, int lda, const __nv_bfloat16* B
 }
 
 // ---------------------------------------------------------------- training kernels
-// Batch rows idx[b] of the raw data, standardised; den = 10 sum mask by the
-// last block (fixed order).  A row index outside [0, M) is read as a masked
-// row of zeros and flagged in bad[0].
-__global__ void __launch_bounds__(RT) k_gather(int B, long long M, unsigned* bad, const int* __restrict__ idx,
-                                               const float* __restrict__ x,
-                                               const float* __restrict__ t, const float* __restrict__ mask,
-                                               const float* __restrict__ norm, float* xs, float* ts, float* mb,
-                                               double* part, unsigned* counter, float* den) {
-  __shared__ double sh[RT / 32 + 1];
-  __shared__ bool last;
-  const int b = blockIdx.x * RT + threadIdx.x;
-  double mv = 0.0;
-  if (b < B) {
+// One batch, forward and reverse, in a single persistent kernel: a block
+// holds the FP32 weights in shared memory, takes tiles of 32 rows of the
+// batch through the three layers and back, and keeps the sums of its weight
+// gradients in registers over its tiles; k_gradient adds the blocks' sums.
+//
+// Bound: the shared-memory reads and the FP32 pipe: 60k multiply-adds per
+// row are 15k issue cycles per tile and SM quarter, of 25k instructions in
+// all.  Layer by layer through global memory (64 x 64 tiles, the batch in
+// splits of 512 rows) the same work was 14 launches of 3 to 40 us on 16 to
+// 128 blocks.  A tile of 32 rows puts a batch of 4,096 on 128 blocks; the
+// products read 16-byte weights and broadcast activations, 64 multiply-adds
+// per 10 loads.  Measured with Adam: 215 -> 41 us at a batch of 4,096 (27 us
+// of it here; about 21 us per tile beyond the first), 211 -> 39 us at 512.
+// The 1 / den of the loss (den = 10 sum of the batch's masks, known only at
+// the end) is applied by k_gradient: the reverse is linear in it.
+constexpr int TR = 32;        // batch rows per tile
+constexpr int TT = 256;       // threads
+constexpr int HS = NH + 4;    // row stride of the 128-wide arrays (16-byte rows, no bank conflicts)
+constexpr int XS = 24;        // inputs 0..8 at 0, 9..17 at 12, zeros between: 16-byte halves
+constexpr int WS1 = XS + 4;   // row stride of W1 in the same order
+constexpr int YS = 16;        // outputs 0..4 at 0, 5..9 at 8
+constexpr int PSTRIDE = (NPAR + 3) & ~3;  // floats of one block's sums
+static_assert(NI == 18 && NH == 128 && NO == 10 && TT == 256 && TR == 32, "thread mappings of k_train");
+static_assert(OFF_W2 % 4 == 0 && OFF_W3 % 4 == 0 && NPAR % 2 == 0, "16-byte rows of the parameters");
+
+__device__ __forceinline__ int xslot(int j) { return j < 9 ? j : j + 3; }
+__device__ __forceinline__ int yslot(int o) { return o < 5 ? o : o + 3; }
+
+struct TrainSmem {
+  float W2[NH * HS], W1[NH * WS1], W3[NO * HS];
+  float H1[TR * HS], G1[TR * HS];  // GELU and its derivative; G1 becomes dL/dZ1
+  float H2[TR * HS], G2[TR * HS];  // G2 becomes dL/dZ2
+  float xs[TR * XS], dy[TR * YS];
+  float b1[NH], b2[NH], b3[NO];
+  double red[2 * TT / 32];
+};
+
+template <int N>  // N bytes, both addresses multiples of N
+__device__ __forceinline__ void copy_async(float* dst, const float* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if (N == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// acc[i][j] = sum_k A[i][k] W[32 j][k]: 8 rows of A (stride SA; the same for
+// a warp), 2 rows of W (stride SW; lane by lane), k ascending.
+template <int K, int SA, int SW>
+__device__ __forceinline__ void rows_product(const float* A, const float* W, float acc[8][2]) {
+#pragma unroll
+  for (int i = 0; i < 8; i++) acc[i][0] = acc[i][1] = 0.f;
+#pragma unroll 2
+  for (int k = 0; k < K; k += 4) {
+    const float4 w0 = *reinterpret_cast<const float4*>(W + k);
+    const float4 w1 = *reinterpret_cast<const float4*>(W + 32 * SW + k);
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      const float4 a = *reinterpret_cast<const float4*>(A + i * SA + k);
+      acc[i][0] = fmaf(a.w, w0.w, fmaf(a.z, w0.z, fmaf(a.y, w0.y, fmaf(a.x, w0.x, acc[i][0]))));
+      acc[i][1] = fmaf(a.w, w1.w, fmaf(a.z, w1.z, fmaf(a.y, w1.y, fmaf(a.x, w1.x, acc[i][1]))));
+    }
+  }
+}
+
+__device__ __forceinline__ void gelu_both(float z, float& h, float& g) {
+  const float c = ncdf(z);
+  h = z * c;
+  g = c + z * nexp(-0.5f * z * z) * 0.39894228040143267794f;
+}
+
+// parts[block][NPAR]: the block's sums of den dL/dparam;
+// red[2 block], red[2 block + 1]: its sums of m (Y - T)^2 and of m.  A row
+// index outside [0, M) is a masked row of zeros and flagged in bad[0].
+__global__ void __launch_bounds__(TT, 1) k_train(int B, long long M, unsigned* bad, const int* __restrict__ idx,
+                                                 const float* __restrict__ x, const float* __restrict__ t,
+                                                 const float* __restrict__ mask, const float* __restrict__ norm,
+                                                 const float* __restrict__ P, float* parts, double* red) {
+  extern __shared__ __align__(16) unsigned char train_raw[];
+  TrainSmem& S = *reinterpret_cast<TrainSmem*>(train_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int gr = tid >> 3, gl = tid & 7;                       // gather and layer 3: row, lane of the row
+  const int r0 = 8 * (warp & 3), ch = 64 * (warp >> 2);        // layers: 8 rows, 64 columns per warp
+  const int kt = 4 * (tid & 15), nt = 4 * (tid >> 4);          // dW2: rows nt + {0,64} + 0..3, columns kt likewise
+  const int c1 = tid & 127, half = tid >> 7;                   // dW1, dW3, biases: column, half of the others
+
+  // weights in flight first, then the rows of the first tile
+  for (int q = tid; q < NH * NH / 4; q += TT)
+    copy_async<16>(S.W2 + (q / (NH / 4)) * HS + 4 * (q % (NH / 4)), P + OFF_W2 + 4 * q);
+  for (int q = tid; q < NO * NH / 4; q += TT)
+    copy_async<16>(S.W3 + (q / (NH / 4)) * HS + 4 * (q % (NH / 4)), P + OFF_W3 + 4 * q);
+  for (int q = tid; q < NH * NI; q += TT) copy_async<4>(S.W1 + (q / NI) * WS1 + xslot(q % NI), P + OFF_W1 + q);
+  if (tid < NH) {
+    copy_async<4>(S.b1 + tid, P + OFF_B1 + tid);
+    copy_async<4>(S.b2 + tid, P + OFF_B2 + tid);
+  }
+  if (tid < NO) copy_async<4>(S.b3 + tid, P + OFF_B3 + tid);
+  const int tiles = (B - 1) / TR + 1;
+  float xm[3], xd[3], tm[2], td[2];
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const int j = gl + 8 * q < NI ? gl + 8 * q : 0;
+    xm[q] = norm[NORM_XM + j];
+    xd[q] = norm[NORM_XS + j];
+  }
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const int o = gl + 8 * q < NO ? gl + 8 * q : 0;
+    tm[q] = norm[NORM_YM + o];
+    td[q] = norm[NORM_YS + o];
+  }
+  // the row of a tile: inputs gl, gl + 8, gl + 16 (< 18), targets gl, gl + 8 (< 10)
+  float xv[3], tv[2], mv;
+  auto fetch = [&](int tile) {
+    const unsigned b = (unsigned)tile * TR + gr;
+    xv[0] = xv[1] = xv[2] = tv[0] = tv[1] = mv = 0.f;
+    if (b >= (unsigned)B) return;
     const long long r = idx[b];
-    if (r >= 0 && r < M) {
-      for (int j = 0; j < NI; j++)
-        xs[(size_t)b * NI + j] = (x[r * NI + j] - norm[NORM_XM + j]) / norm[NORM_XS + j];
-      for (int j = 0; j < NO; j++)
-        ts[(size_t)b * NO + j] = (t[r * NO + j] - norm[NORM_YM + j]) / norm[NORM_YS + j];
-      mb[b] = mask[r];
-      mv = mask[r];
-    } else {
-      for (int j = 0; j < NI; j++) xs[(size_t)b * NI + j] = 0.f;
-      for (int j = 0; j < NO; j++) ts[(size_t)b * NO + j] = 0.f;
-      mb[b] = 0.f;
-      atomicOr(bad, 1u);
+    if (r < 0 || r >= M) {
+      if (gl == 0) atomicOr(bad, 1u);
+#pragma unroll
+      for (int q = 0; q < 3; q++) xv[q] = xm[q];  // standardised to zero
+#pragma unroll
+      for (int q = 0; q < 2; q++) tv[q] = tm[q];
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; q++)
+      if (gl + 8 * q < NI) xv[q] = x[r * NI + gl + 8 * q];
+#pragma unroll
+    for (int q = 0; q < 2; q++)
+      if (gl + 8 * q < NO) tv[q] = t[r * NO + gl + 8 * q];
+    mv = mask[r];
+  };
+  fetch(blockIdx.x);
+  for (int q = tid; q < (NH + TR) * 6; q += TT) {  // the gaps of W1 and xs
+    const int r = q / 6, g = q % 6, k = g < 3 ? 9 + g : 18 + g;
+    (r < NH ? S.W1 + r * WS1 : S.xs + (r - NH) * XS)[k] = 0.f;
+  }
+
+  float dW2[8][8], dW1[9], dW3[5], db12 = 0.f, db3 = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; i++)
+#pragma unroll
+    for (int j = 0; j < 8; j++) dW2[i][j] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 9; j++) dW1[j] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 5; j++) dW3[j] = 0.f;
+  double loss = 0.0, msum = 0.0;
+
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const bool in = (unsigned)tile * TR + gr < (unsigned)B;
+    const float tg[2] = {(tv[0] - tm[0]) / td[0], (tv[1] - tm[1]) / td[1]}, m = mv;
+#pragma unroll
+    for (int q = 0; q < 3; q++)
+      if (gl + 8 * q < NI) S.xs[gr * XS + xslot(gl + 8 * q)] = in ? (xv[q] - xm[q]) / xd[q] : 0.f;
+    copy_wait();
+    __syncthreads();
+    if (tile + (int)gridDim.x < tiles) fetch(tile + gridDim.x);  // in flight through this tile
+    float acc[8][2];
+    // layer 1
+    rows_product<XS, XS, WS1>(S.xs + r0 * XS, S.W1 + (ch + lane) * WS1, acc);
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      const int n = ch + lane + 32 * j;
+#pragma unroll
+      for (int i = 0; i < 8; i++) gelu_both(acc[i][j] + S.b1[n], S.H1[(r0 + i) * HS + n], S.G1[(r0 + i) * HS + n]);
+    }
+    __syncthreads();
+    // layer 2
+    rows_product<NH, HS, HS>(S.H1 + r0 * HS, S.W2 + (ch + lane) * HS, acc);
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      const int n = ch + lane + 32 * j;
+#pragma unroll
+      for (int i = 0; i < 8; i++) gelu_both(acc[i][j] + S.b2[n], S.H2[(r0 + i) * HS + n], S.G2[(r0 + i) * HS + n]);
+    }
+    __syncthreads();
+    // layer 3: eight lanes per row, 16 of its 128 products each
+    {
+      float y[NO];
+#pragma unroll
+      for (int o = 0; o < NO; o++) y[o] = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int k = 4 * gl + 32 * q;
+        const float4 h = *reinterpret_cast<const float4*>(S.H2 + gr * HS + k);
+#pragma unroll
+        for (int o = 0; o < NO; o++) {
+          const float4 w = *reinterpret_cast<const float4*>(S.W3 + o * HS + k);
+          y[o] = fmaf(h.w, w.w, fmaf(h.z, w.z, fmaf(h.y, w.y, fmaf(h.x, w.x, y[o]))));
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < NO; o++)
+#pragma unroll
+        for (int d = 4; d > 0; d >>= 1) y[o] += __shfl_xor_sync(0xffffffffu, y[o], d);
+#pragma unroll
+      for (int o = 0; o < NO; o++)
+        if ((o & 7) == gl) {
+          const float r = in ? (y[o] + S.b3[o] - tg[o >> 3]) * m : 0.f;
+          S.dy[gr * YS + yslot(o)] = 2.0f * r;
+          loss += (double)r * r;
+        }
+      if (gl == 0) msum += m;
+    }
+    __syncthreads();
+    // dW3 = dy^T H2, db3; dZ2 = (dy W3) gelu'(Z2)
+#pragma unroll 4
+    for (int r = 0; r < TR; r++) {
+      const float h = S.H2[r * HS + c1];
+      const float4 d = *reinterpret_cast<const float4*>(S.dy + r * YS + 8 * half);
+      dW3[0] = fmaf(d.x, h, dW3[0]);
+      dW3[1] = fmaf(d.y, h, dW3[1]);
+      dW3[2] = fmaf(d.z, h, dW3[2]);
+      dW3[3] = fmaf(d.w, h, dW3[3]);
+      dW3[4] = fmaf(S.dy[r * YS + 8 * half + 4], h, dW3[4]);
+    }
+    if (tid < NO)
+      for (int r = 0; r < TR; r++) db3 += S.dy[r * YS + yslot(tid)];
+    {
+      float w[NO][2];
+#pragma unroll
+      for (int o = 0; o < NO; o++)
+#pragma unroll
+        for (int j = 0; j < 2; j++) w[o][j] = S.W3[o * HS + ch + lane + 32 * j];
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const float* d = S.dy + (r0 + i) * YS;
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+          float v = 0.f;
+#pragma unroll
+          for (int o = 0; o < NO; o++) v = fmaf(d[o < 5 ? o : o + 3], w[o][j], v);
+          S.G2[(r0 + i) * HS + ch + lane + 32 * j] *= v;
+        }
+      }
+    }
+    __syncthreads();
+    // dZ1 = (dZ2 W2) gelu'(Z1)
+#pragma unroll
+    for (int i = 0; i < 8; i++) acc[i][0] = acc[i][1] = 0.f;
+#pragma unroll 2
+    for (int n = 0; n < NH; n += 4) {
+      float2 w[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) w[q] = *reinterpret_cast<const float2*>(S.W2 + (n + q) * HS + ch + 2 * lane);
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const float4 d = *reinterpret_cast<const float4*>(S.G2 + (r0 + i) * HS + n);
+        acc[i][0] = fmaf(d.w, w[3].x, fmaf(d.z, w[2].x, fmaf(d.y, w[1].x, fmaf(d.x, w[0].x, acc[i][0]))));
+        acc[i][1] = fmaf(d.w, w[3].y, fmaf(d.z, w[2].y, fmaf(d.y, w[1].y, fmaf(d.x, w[0].y, acc[i][1]))));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      float2* g = reinterpret_cast<float2*>(S.G1 + (r0 + i) * HS + ch + 2 * lane);
+      const float2 v = *g;
+      *g = make_float2(v.x * acc[i][0], v.y * acc[i][1]);
+    }
+    // dW2 = dZ2^T H1
+#pragma unroll 2
+    for (int r = 0; r < TR; r++) {
+      float d[8], h[8];
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        *reinterpret_cast<float4*>(d + 4 * q) = *reinterpret_cast<const float4*>(S.G2 + r * HS + nt + 64 * q);
+        *reinterpret_cast<float4*>(h + 4 * q) = *reinterpret_cast<const float4*>(S.H1 + r * HS + kt + 64 * q);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i++)
+#pragma unroll
+        for (int j = 0; j < 8; j++) dW2[i][j] = fmaf(d[i], h[j], dW2[i][j]);
+    }
+    if (half == 1)
+      for (int r = 0; r < TR; r++) db12 += S.G2[r * HS + c1];
+    __syncthreads();
+    // dW1 = dZ1^T xs, db1
+#pragma unroll 4
+    for (int r = 0; r < TR; r++) {
+      const float d = S.G1[r * HS + c1];
+      const float* xr = S.xs + r * XS + 12 * half;
+      const float4 x0 = *reinterpret_cast<const float4*>(xr);
+      const float4 x1 = *reinterpret_cast<const float4*>(xr + 4);
+      dW1[0] = fmaf(d, x0.x, dW1[0]);
+      dW1[1] = fmaf(d, x0.y, dW1[1]);
+      dW1[2] = fmaf(d, x0.z, dW1[2]);
+      dW1[3] = fmaf(d, x0.w, dW1[3]);
+      dW1[4] = fmaf(d, x1.x, dW1[4]);
+      dW1[5] = fmaf(d, x1.y, dW1[5]);
+      dW1[6] = fmaf(d, x1.z, dW1[6]);
+      dW1[7] = fmaf(d, x1.w, dW1[7]);
+      dW1[8] = fmaf(d, xr[8], dW1[8]);
+      if (half == 0) db12 += d;
+    }
+    __syncthreads();  // xs and the activations are free for the next tile
+  }
+
+  float* out = parts + (size_t)blockIdx.x * PSTRIDE;
+#pragma unroll
+  for (int i = 0; i < 8; i++)
+#pragma unroll
+    for (int q = 0; q < 2; q++)
+      *reinterpret_cast<float4*>(out + OFF_W2 + (nt + (i & 3) + 64 * (i >> 2)) * NH + kt + 64 * q) =
+          make_float4(dW2[i][4 * q], dW2[i][4 * q + 1], dW2[i][4 * q + 2], dW2[i][4 * q + 3]);
+#pragma unroll
+  for (int j = 0; j < 9; j++) out[OFF_W1 + c1 * NI + 9 * half + j] = dW1[j];
+#pragma unroll
+  for (int j = 0; j < 5; j++) out[OFF_W3 + (5 * half + j) * NH + c1] = dW3[j];
+  out[(half ? OFF_B2 : OFF_B1) + c1] = db12;
+  if (tid < NO) out[OFF_B3 + tid] = db3;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    msum += __shfl_xor_sync(0xffffffffu, msum, o);
+  }
+  if (lane == 0) {
+    S.red[2 * warp] = loss;
+    S.red[2 * warp + 1] = msum;
+  }
+  __syncthreads();
+  if (tid < 2) {
+    double q = 0.0;
+    for (int w = 0; w < TT / 32; w++) q += S.red[2 * w + tid];
+    red[2 * blockIdx.x + tid] = q;
+  }
+}
+
+// grad = sum over the blocks of k_train / den, loss = sum m (Y - T)^2 / den,
+// den = 10 max(1, sum of the masks); grad_out, loss_out may be NULL.  64
+// parameters per block, its eight warps take the blocks' sums in turn
+// (80 KB per block of k_train, read once from L2), fixed order.
+__global__ void __launch_bounds__(TT) k_gradient(int nb, const float* __restrict__ parts,
+                                                 const double* __restrict__ red, float* grad, float* grad_out,
+                                                 float* loss_out) {
+  __shared__ float2 sh[TT / 32][32];
+  __shared__ double sd[2][TT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i = blockIdx.x * 64 + 2 * lane;
+  float2 v = make_float2(0.f, 0.f);
+  if (i < NPAR) {
+#pragma unroll 8
+    for (int b = warp; b < nb; b += TT / 32) {
+      const float2 p = *reinterpret_cast<const float2*>(parts + (size_t)b * PSTRIDE + i);
+      v.x += p.x;
+      v.y += p.y;
     }
   }
-  for (int o = 16; o > 0; o >>= 1) mv += __shfl_xor_sync(0xffffffffu, mv, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mv;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double q = 0.0;
-    for (int w = 0; w < RT / 32; w++) q += sh[w];
-    part[blockIdx.x] = q;
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  double l = 0.0, m = 0.0;
+  for (int b = tid; b < nb; b += TT) {
+    l += red[2 * b];
+    m += red[2 * b + 1];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    l += __shfl_xor_sync(0xffffffffu, l, o);
+    m += __shfl_xor_sync(0xffffffffu, m, o);
+  }
+  sh[warp][lane] = v;
+  if (lane == 0) {
+    sd[0][warp] = l;
+    sd[1][warp] = m;
   }
   __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  double q = 0.0;
-  for (int k = 0; k < (int)gridDim.x; k++) q += __ldcg(part + k);
-  den[0] = (float)(NO * (q > 1.0 ? q : 1.0));
-  *counter = 0;
-}
-
-// dY = 2 (Y - T) m / den; loss = sum m (Y - T)^2 / den (last block).
-__global__ void __launch_bounds__(RT) k_mse(int B, const float* __restrict__ y, const float* __restrict__ ts,
-                                            const float* __restrict__ mb, const float* __restrict__ den, float* dy,
-                                            double* part, unsigned* counter, float* loss) {
-  __shared__ double sh[RT / 32 + 1];
-  __shared__ bool last;
-  const int b = blockIdx.x * RT + threadIdx.x;
-  const float d = den[0];
-  double acc = 0.0;
-  if (b < B) {
-    const float m = mb[b];
-    for (int j = 0; j < NO; j++) {
-      const float r = (y[(size_t)b * NO + j] - ts[(size_t)b * NO + j]) * m;
-      dy[(size_t)b * NO + j] = 2.0f * r / d;
-      acc += (double)r * r;
-    }
+  if (warp != 0) return;
+  l = m = 0.0;
+  for (int w = 0; w < TT / 32; w++) {
+    l += sd[0][w];
+    m += sd[1][w];
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double q = 0.0;
-    for (int w = 0; w < RT / 32; w++) q += sh[w];
-    part[blockIdx.x] = q;
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  const float den = (float)(NO * (m > 1.0 ? m : 1.0));
+  if (blockIdx.x == 0 && lane == 0 && loss_out) loss_out[0] = (float)(l / den);
+  if (i >= NPAR) return;
+  for (int w = 1; w < TT / 32; w++) {
+    v.x += sh[w][lane].x;
+    v.y += sh[w][lane].y;
   }
-  __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  double q = 0.0;
-  for (int k = 0; k < (int)gridDim.x; k++) q += __ldcg(part + k);
-  if (loss) loss[0] = (float)(q / d);
-  *counter = 0;
-}
-
-// out[i] = sum_s parts[s][i], s ascending.
-__global__ void k_sum_splits(int n, int S, const float* __restrict__ parts, float* out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float v = 0.f;
-  for (int s = 0; s < S; s++) v += parts[(size_t)s * n + i];
-  out[i] = v;
-}
-
-// out[n] = sum_b X[b][n]: one block per column, strided partial sums and a
-// fixed shuffle tree.
-__global__ void __launch_bounds__(RT) k_colsum(int B, int N, const float* __restrict__ X, float* out) {
-  __shared__ float sh[RT / 32];
-  const int n = blockIdx.x;
-  float v = 0.f;
-  for (int b = threadIdx.x; b < B; b += RT) v += X[(size_t)b * N + n];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float q = 0.f;
-    for (int w = 0; w < RT / 32; w++) q += sh[w];
-    out[n] = q;
+  v.x /= den;
+  v.y /= den;
+  grad[i] = v.x;
+  grad[i + 1] = v.y;
+  if (grad_out) {
+    grad_out[i] = v.x;
+    grad_out[i + 1] = v.y;
   }
 }
 
@@ -536,12 +803,12 @@ int mlp_infer_forward(int fp64, int M, const void* xs, const float* params, cons
   const __nv_bfloat16* w = static_cast<const __nv_bfloat16*>(wbf);
   int r = 0;
   if (fp64) {
-    r |= gemm<double, double, __nv_bfloat16, false, true, EPI_BIAS_GELU>(M, NH, NI, xs, NI, w + OFF_W1, NI, H1, NH,
-                                                                         params + OFF_B1, Z1, 0, s);
-    r |= gemm<double, double, __nv_bfloat16, false, true, EPI_BIAS_GELU>(M, NH, NH, H1, NH, w + OFF_W2, NH, H2, NH,
-                                                                         params + OFF_B2, Z2, 0, s);
-    r |= gemm<double, double, __nv_bfloat16, false, true, EPI_BIAS>(M, NO, NH, H2, NH, w + OFF_W3, NH, ys, NO,
-                                                                    params + OFF_B3, nullptr, 0, s);
+    r |= gemm<double, true, EPI_BIAS_GELU>(M, NH, NI, xs, NI, w + OFF_W1, NI, H1, NH,
+                                                                         params + OFF_B1, Z1, s);
+    r |= gemm<double, true, EPI_BIAS_GELU>(M, NH, NH, H1, NH, w + OFF_W2, NH, H2, NH,
+                                                                         params + OFF_B2, Z2, s);
+    r |= gemm<double, true, EPI_BIAS>(M, NO, NH, H2, NH, w + OFF_W3, NH, ys, NO,
+                                                                    params + OFF_B3, nullptr, s);
   } else {  // tensor pipe (three bfloat16 parts per FP32 activation)
     r |= gemm_tc<32, 128, true, EPI_BIAS_GELU>(M, NH, NI, (const float*)xs, NI, w + OFF_W1, NI, (float*)H1, NH,
                                                params + OFF_B1, (float*)Z1, s);
@@ -559,12 +826,12 @@ int mlp_infer_backward(int fp64, int M, const void* ybar, const void* wbf, void*
   const __nv_bfloat16* w = static_cast<const __nv_bfloat16*>(wbf);
   int r = 0;
   if (fp64) {
-    r |= gemm<double, double, __nv_bfloat16, false, false, EPI_DGELU>(M, NH, NO, ybar, NO, w + OFF_W3, NH, dZ2, NH,
-                                                                      nullptr, Z2, 0, s);
-    r |= gemm<double, double, __nv_bfloat16, false, false, EPI_DGELU>(M, NH, NH, dZ2, NH, w + OFF_W2, NH, dZ1, NH,
-                                                                      nullptr, Z1, 0, s);
-    r |= gemm<double, double, __nv_bfloat16, false, false, EPI_NONE>(M, NI, NH, dZ1, NH, w + OFF_W1, NI, xbar, NI,
-                                                                     nullptr, nullptr, 0, s);
+    r |= gemm<double, false, EPI_DGELU>(M, NH, NO, ybar, NO, w + OFF_W3, NH, dZ2, NH,
+                                                                      nullptr, Z2, s);
+    r |= gemm<double, false, EPI_DGELU>(M, NH, NH, dZ2, NH, w + OFF_W2, NH, dZ1, NH,
+                                                                      nullptr, Z1, s);
+    r |= gemm<double, false, EPI_NONE>(M, NI, NH, dZ1, NH, w + OFF_W1, NI, xbar, NI,
+                                                                     nullptr, nullptr, s);
   } else {  // tensor pipe (three bfloat16 parts per FP32 cotangent)
     r |= gemm_tc<16, 128, false, EPI_DGELU>(M, NH, NO, (const float*)ybar, NO, w + OFF_W3, NH, (float*)dZ2, NH,
                                             nullptr, (float*)Z2, s);
@@ -584,7 +851,7 @@ struct MBuf {
 
 struct bop_mlp {
   MBuf params, grad, am, av, wbf, norm;
-  MBuf xs, ts, mb, Z1, H1, Z2, H2, y, dy, parts, red, counter, den, loss, bad;
+  MBuf xs, Z1, H1, Z2, H2, y, parts, red, bad;
   int adam_t = 0;
   int batch_cap = 0;
   char err[256];
@@ -627,18 +894,14 @@ T* MP(MBuf& b) {
     if (e_ != cudaSuccess) return mfail(net, BOP_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_));     \
   } while (0)
 
+// Buffers of a prediction over B rows.
 int size_batch(bop_mlp* net, int B) {
   if (B <= net->batch_cap) return BOP_OK;
   int r;
   const size_t b = (size_t)B;
-  const int S = (B + KCHUNK - 1) / KCHUNK;
-  if ((r = mensure(net, net->xs, sizeof(float) * b * NI)) || (r = mensure(net, net->ts, sizeof(float) * b * NO)) ||
-      (r = mensure(net, net->mb, sizeof(float) * b)) || (r = mensure(net, net->Z1, sizeof(float) * b * NH)) ||
+  if ((r = mensure(net, net->xs, sizeof(float) * b * NI)) || (r = mensure(net, net->Z1, sizeof(float) * b * NH)) ||
       (r = mensure(net, net->H1, sizeof(float) * b * NH)) || (r = mensure(net, net->Z2, sizeof(float) * b * NH)) ||
-      (r = mensure(net, net->H2, sizeof(float) * b * NH)) || (r = mensure(net, net->y, sizeof(float) * b * NO)) ||
-      (r = mensure(net, net->dy, sizeof(float) * b * NO)) ||
-      (r = mensure(net, net->parts, sizeof(float) * (size_t)S * NH * NH)) ||
-      (r = mensure(net, net->red, sizeof(double) * (b / RT + 2))))
+      (r = mensure(net, net->H2, sizeof(float) * b * NH)) || (r = mensure(net, net->y, sizeof(float) * b * NO)))
     return r;
   net->batch_cap = B;
   return BOP_OK;
@@ -662,8 +925,7 @@ int bop_mlp_create(bop_mlp** out, const float* params_host) {
   if ((r = mensure(net, net->params, sizeof(float) * NPAR)) || (r = mensure(net, net->grad, sizeof(float) * NPAR)) ||
       (r = mensure(net, net->am, sizeof(float) * NPAR)) || (r = mensure(net, net->av, sizeof(float) * NPAR)) ||
       (r = mensure(net, net->wbf, sizeof(__nv_bfloat16) * NPAR)) ||
-      (r = mensure(net, net->norm, sizeof(float) * BOP_MLP_NNORM)) || (r = mensure(net, net->counter, 16)) ||
-      (r = mensure(net, net->den, 16)) || (r = mensure(net, net->loss, 16)) || (r = mensure(net, net->bad, 16))) {
+      (r = mensure(net, net->norm, sizeof(float) * BOP_MLP_NNORM)) || (r = mensure(net, net->bad, 16))) {
     bop_mlp_destroy(net);
     return r;
   }
@@ -679,7 +941,7 @@ int bop_mlp_create(bop_mlp** out, const float* params_host) {
       cudaMemcpy(net->norm.p, norm0, sizeof(norm0), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(net->am.p, 0, sizeof(float) * NPAR) != cudaSuccess ||
       cudaMemset(net->av.p, 0, sizeof(float) * NPAR) != cudaSuccess ||
-      cudaMemset(net->counter.p, 0, 16) != cudaSuccess || cudaMemset(net->bad.p, 0, 16) != cudaSuccess) {
+      cudaMemset(net->bad.p, 0, 16) != cudaSuccess) {
     bop_mlp_destroy(net);
     return BOP_ERR_CUDA;
   }
@@ -694,9 +956,8 @@ int bop_mlp_create(bop_mlp** out, const float* params_host) {
 
 int bop_mlp_destroy(bop_mlp* net) {
   if (!net) return BOP_OK;
-  for (MBuf* b : {&net->params, &net->grad, &net->am, &net->av, &net->wbf, &net->norm, &net->xs, &net->ts, &net->mb,
-                  &net->Z1, &net->H1, &net->Z2, &net->H2, &net->y, &net->dy, &net->parts, &net->red, &net->counter,
-                  &net->den, &net->loss, &net->bad})
+  for (MBuf* b : {&net->params, &net->grad, &net->am, &net->av, &net->wbf, &net->norm, &net->xs, &net->Z1,
+                  &net->H1, &net->Z2, &net->H2, &net->y, &net->parts, &net->red, &net->bad})
     if (b->p) cudaFree(b->p);
   delete net;
   return BOP_OK;
@@ -735,54 +996,21 @@ int bop_mlp_gradient(bop_mlp* net, long long M, const float* x, const float* t, 
   if (!net || M < 1 || !x || !t || !mask || !idx || batch < 1)
     return mfail(net, BOP_ERR_ARG, "need M >= 1, x, t, mask, idx and batch >= 1");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int r = size_batch(net, batch);
-  if (r) return r;
-  const int B = batch;
-  const int nb = grid1(B, RT);
-  float* P = MP<float>(net->params);
-  float* G = MP<float>(net->grad);
-  float* xs = MP<float>(net->xs);
-  float* Z1 = MP<float>(net->Z1);
-  float* H1 = MP<float>(net->H1);
-  float* Z2 = MP<float>(net->Z2);
-  float* H2 = MP<float>(net->H2);
-  float* y = MP<float>(net->y);
-  float* dy = MP<float>(net->dy);
+  int dev = 0, sms = 0;
+  MCK(cudaGetDevice(&dev));
+  MCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  MCK(cudaFuncSetAttribute(k_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)));
+  const int tiles = (batch - 1) / TR + 1;
+  const int nb = tiles < sms ? tiles : sms;
+  int r;
+  if ((r = mensure(net, net->parts, sizeof(float) * (size_t)nb * PSTRIDE)) ||
+      (r = mensure(net, net->red, sizeof(double) * 2 * nb)))
+    return r;
   float* parts = MP<float>(net->parts);
-  k_gather<<<nb, RT, 0, s>>>(B, M, MP<unsigned>(net->bad), idx, x, t, mask, MP<float>(net->norm), xs, MP<float>(net->ts), MP<float>(net->mb),
-                             MP<double>(net->red), MP<unsigned>(net->counter), MP<float>(net->den));
-  int e = 0;
-  // forward (FP32 master weights)
-  e |= gemm<float, float, float, false, true, EPI_BIAS_GELU>(B, NH, NI, xs, NI, P + OFF_W1, NI, H1, NH, P + OFF_B1,
-                                                             Z1, 0, s);
-  e |= gemm<float, float, float, false, true, EPI_BIAS_GELU>(B, NH, NH, H1, NH, P + OFF_W2, NH, H2, NH, P + OFF_B2,
-                                                             Z2, 0, s);
-  e |= gemm<float, float, float, false, true, EPI_BIAS>(B, NO, NH, H2, NH, P + OFF_W3, NH, y, NO, P + OFF_B3, nullptr,
-                                                        0, s);
-  k_mse<<<nb, RT, 0, s>>>(B, y, MP<float>(net->ts), MP<float>(net->mb), MP<float>(net->den), dy,
-                          MP<double>(net->red), MP<unsigned>(net->counter), loss_out ? loss_out : MP<float>(net->loss));
-  const int S = (B + KCHUNK - 1) / KCHUNK;
-  // layer 3: dW3 = dy^T H2, db3 = sum dy
-  e |= gemm<float, float, float, true, false, EPI_NONE>(NO, NH, B, dy, NO, H2, NH, parts, NH, nullptr, nullptr,
-                                                        KCHUNK, s);
-  k_sum_splits<<<grid1(NO * NH, 256), 256, 0, s>>>(NO * NH, S, parts, G + OFF_W3);
-  k_colsum<<<NO, RT, 0, s>>>(B, NO, dy, G + OFF_B3);
-  // dZ2 = (dy W3) * gelu'(Z2), in place of Z2
-  e |= gemm<float, float, float, false, false, EPI_DGELU>(B, NH, NO, dy, NO, P + OFF_W3, NH, Z2, NH, nullptr, Z2, 0,
-                                                          s);
-  e |= gemm<float, float, float, true, false, EPI_NONE>(NH, NH, B, Z2, NH, H1, NH, parts, NH, nullptr, nullptr,
-                                                        KCHUNK, s);
-  k_sum_splits<<<grid1(NH * NH, 256), 256, 0, s>>>(NH * NH, S, parts, G + OFF_W2);
-  k_colsum<<<NH, RT, 0, s>>>(B, NH, Z2, G + OFF_B2);
-  // dZ1 = (dZ2 W2) * gelu'(Z1), in place of Z1
-  e |= gemm<float, float, float, false, false, EPI_DGELU>(B, NH, NH, Z2, NH, P + OFF_W2, NH, Z1, NH, nullptr, Z1, 0,
-                                                          s);
-  e |= gemm<float, float, float, true, false, EPI_NONE>(NH, NI, B, Z1, NH, xs, NI, parts, NI, nullptr, nullptr,
-                                                        KCHUNK, s);
-  k_sum_splits<<<grid1(NH * NI, 256), 256, 0, s>>>(NH * NI, S, parts, G + OFF_W1);
-  k_colsum<<<NH, RT, 0, s>>>(B, NH, Z1, G + OFF_B1);
-  if (e) return mfail(net, BOP_ERR_CUDA, "gemm launch failed");
-  if (grad_out) MCK(cudaMemcpyAsync(grad_out, G, sizeof(float) * NPAR, cudaMemcpyDeviceToDevice, s));
+  double* red = MP<double>(net->red);
+  k_train<<<nb, TT, sizeof(TrainSmem), s>>>(batch, M, MP<unsigned>(net->bad), idx, x, t, mask, MP<float>(net->norm),
+                                            MP<float>(net->params), parts, red);
+  k_gradient<<<grid1(NPAR, 64), TT, 0, s>>>(nb, parts, red, MP<float>(net->grad), grad_out, loss_out);
   MCK(cudaGetLastError());
   return BOP_OK;
 }

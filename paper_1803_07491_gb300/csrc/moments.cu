@@ -323,32 +323,6 @@ __device__ __forceinline__ void block_fma(const T* u, const T* x, T acc[NO][NC])
   }
 }
 
-// acc += sum over the first cnt adjacency entries of t of B_ts x[s]; the
-// next entry and its block are fetched while the current one is applied.
-template <typename T, int NO, int NC, int PS>
-__device__ __forceinline__ void gather_pf(const int2* __restrict__ adj, long long q0, int cnt,
-                                          const T* __restrict__ H, int HS, const T* __restrict__ x,
-                                          T acc[NO][NC]) {
-  if (cnt <= 0) return;
-  constexpr int HB = hb_count<NO>();
-  int2 en = __ldg(adj + q0);
-  T hb[HB];
-  load_bond<T, NO>(H + (size_t)en.y * HS, hb);
-  for (int e = 0; e < cnt; e++) {
-    const int s = en.x;
-    T hc[HB];
-#pragma unroll
-    for (int q = 0; q < HB; q++) hc[q] = hb[q];
-    if (e + 1 < cnt) {
-      en = __ldg(adj + q0 + e + 1);
-      load_bond<T, NO>(H + (size_t)en.y * HS, hb);
-    }
-    T xs[NO * NC];
-    load_row<T, NO * NC, PS>(x + (size_t)s * PS, xs);
-    block_fma<T, NO, NC>(hc, xs, acc);
-  }
-}
-
 // acc += sum over cnt adjacency entries (every step-th of ent) of B_ts x[s],
 // with the blocks of the next two entries in flight while the current one is
 // applied.

@@ -200,3 +200,41 @@ def test_trained_network_beats_constant_terminator(bop):
     assert atom_learned < atom_plain
     assert err_learned < 0.5 * err_plain
     net.close()
+
+
+@pytest.mark.parametrize("batch", [1, 31, 32, 33, 4865, 10007])
+def test_gradient_at_tile_edges(bop, om, batch):
+    """Batches around one 32-row tile, one tile beyond 152 blocks' first and a
+    ragged third round, with masked, repeated and out-of-range rows.  FP32
+    sums of at most 128 products through three layers and back against FP64:
+    6 x 128 x 2^-24 = 5e-5 of the largest gradient; 1e-4 as above."""
+    rng = np.random.default_rng(50 + batch)
+    p0, q0, M = I.mlp_init_params(51), I.mlp_fixed_norm(), 2000
+    x = rng.normal(size=(M, 18)).astype(np.float32)
+    t = rng.normal(size=(M, 10)).astype(np.float32)
+    mk = (rng.uniform(size=M) > 0.3).astype(np.float32)
+    idx = rng.integers(0, M, batch).astype(np.int32)
+    mk[idx[0]] = 1.0
+    outside = batch > 32
+    if outside:
+        idx[5], idx[batch - 1] = -1, M
+    xd, td, md, ii = (torch.tensor(a, device="cuda") for a in (x, t, mk, idx))
+    net = bop.Network(p0)
+    net.set_norm(q0)
+    g = [torch.empty(om.N_PARAM, dtype=torch.float32, device="cuda") for _ in range(2)]
+    loss = torch.empty(1, dtype=torch.float32, device="cuda")
+    for k in range(2):
+        bop.bop_mlp_gradient(net.h, xd, td, md, ii, g[k], loss)
+    assert torch.equal(g[0], g[1])
+    assert bop.lib().bop_mlp_check(net.h, None) == (bop.BOP_ERR_ARG if outside else 0)
+    ok = (idx >= 0) & (idx < M)
+    xm, xsd, _, _, ym, ysd = om.unpack_norm(q0)
+    lr_, gr = om.loss_and_grad(p0, (x[idx[ok]].astype(np.float64) - xm) / xsd,
+                               (t[idx[ok]].astype(np.float64) - ym) / ysd, mk[idx[ok]])
+    assert abs(loss.item() - lr_) < 1e-5 * lr_
+    assert np.max(np.abs(g[0].cpu().numpy() - gr)) < 1e-4 * np.abs(gr).max()
+    # nothing but masked rows: zero loss and gradient
+    md.zero_()
+    bop.bop_mlp_gradient(net.h, xd, td, md, ii, g[0], loss)
+    assert loss.item() == 0.0 and not g[0].any()
+    net.close()
