@@ -1160,8 +1160,6 @@ int adjoint_pass(bop_ctx* c, const double* w, void* Hbar, double* Ebar, cudaStre
   return BOP_OK;
 }
 
-constexpr int GM_KRYLOV = 40;   // GMRES basis size per cycle
-constexpr int GM_CYCLES = 3;    // cycles (restarts + 1)
 
 // Reads nv doubles from the device (synchronises s).
 int read_back(bop_ctx* c, const double* d, double* h, int nv, cudaStream_t s) {
@@ -1189,7 +1187,7 @@ int scf_response(bop_ctx* c, cudaStream_t s) {
   CKS(ensure(c, c->rvec, sizeof(double) * (size_t)nu * (GM_KRYLOV + 6)));
   // coef: [0, K+2) host-set coefficients; then the Gram-Schmidt passes and
   // the norm of one Arnoldi step, read back together
-  CKS(ensure(c, c->rcoef, sizeof(double) * (3 * GM_KRYLOV + 8)));
+  CKS(ensure(c, c->rcoef, sizeof(double) * (3 * GM_KRYLOV + 8 + GMRES_PART)));
   double* V = P<double>(c->rvec);                 // Krylov basis [GM_KRYLOV + 1][nu]
   double* rhs = V + (size_t)(GM_KRYLOV + 1) * nu;  // dE/du
   double* Pd = rhs + nu;                           // diagonal preconditioner
@@ -1283,15 +1281,31 @@ int scf_response(bop_ctx* c, cudaStream_t s) {
     if (launch_dots(nu, 1, a, b, coef, s)) return fail(c, BOP_ERR_CUDA, "response kernels failed");
     return read_back(c, coef, h, 1, s);
   };
-  CK(cudaMemsetAsync(y, 0, sizeof(double) * nu, s));
-  double bnorm = 0.0;
-  CKS(dot(rhs, rhs, &bnorm));
-  bnorm = std::sqrt(bnorm);
   int iters = 0;
-  double rel = 0.0;
-  bool conv = bnorm == 0.0;
+  double rel = 0.0, bnorm = 0.0;
+  bool conv = false, solved = false;
+  if (use_rows) {
+    GmresArgs ga{n,   nu,  max_it, c->nsite, P<long long>(c->rjptr), P<long long>(c->rjidx), P<int>(c->rjrow),
+                 P<double>(c->rjv), rhs, Pd, c->sfac, I, rtol, V, tmp, yc, y, coef + 3 * GM_KRYLOV + 8, coef};
+    Region R(c, PK_SCF, 1, s);
+    const int r = launch_gmres(ga, s);
+    if (r != 0 && r != -2) return fail(c, BOP_ERR_CUDA, "response kernels failed");
+    solved = r == 0;
+  }
+  if (solved) {
+    double o[3];
+    CKS(read_back(c, coef, o, 3, s));
+    iters = (int)o[0];
+    rel = o[1];
+    conv = o[2] != 0.0;
+  } else {
+    CK(cudaMemsetAsync(y, 0, sizeof(double) * nu, s));
+    CKS(dot(rhs, rhs, &bnorm));
+    bnorm = std::sqrt(bnorm);
+    conv = bnorm == 0.0;
+  }
   const double one = 1.0, minus_one = -1.0;
-  for (int cyc = 0; cyc < GM_CYCLES && !conv && iters < max_it; cyc++) {
+  for (int cyc = 0; !solved && cyc < GM_CYCLES && !conv && iters < max_it; cyc++) {
     // residual r = g - J^T y into V_0
     CK(cudaMemcpyAsync(V, rhs, sizeof(double) * nu, cudaMemcpyDeviceToDevice, s));
     if (cyc > 0) {

@@ -391,6 +391,26 @@ int launch_var_lambda(int n, int norb, double s, double J, double n0, const doub
                       const double* onsite, const FermiState* st, double* q, double* lam, double* red,
                       unsigned* counter, cudaStream_t stream);
 int launch_scale_by_inv_norm(int nu, double* u, const double* nsq, cudaStream_t stream);
+// The GMRES solve J^T y = rhs over the rows of J as per-site values
+// (launch_jt_build, AdjointArgs.siteval): right preconditioner diag(P),
+// cycles of GM_KRYLOV steps, relative residual rtol or max_it steps.
+// V [GM_KRYLOV + 1][nu], x, xy [nu] scratch; part GMRES_PART doubles;
+// out: iterations, relative residual, converged.  -2: cooperative launch not
+// possible.
+constexpr int GM_KRYLOV = 40;      // basis size per cycle
+constexpr int GM_CYCLES = 3;       // cycles (restarts + 1)
+constexpr int GMRES_BLOCKS = 512;  // most blocks of the launch
+constexpr int GMRES_PART = GMRES_BLOCKS * (2 * (GM_KRYLOV + 1) + 1);
+struct GmresArgs {
+  int n, nu, max_it;           // nu = n, or 2n with the Stoner moments
+  long long stride;            // val: spin s at val + s stride
+  const long long *ptr, *idx;
+  const int* row;
+  const double *val, *rhs, *P;
+  double s, I, rtol;
+  double *V, *x, *xy, *y, *part, *out;
+};
+int launch_gmres(const GmresArgs& g, cudaStream_t stream);
 // J^T v of the SCF response from the per-site values of one sweep with the
 // dN/dmu weights (AdjointArgs.siteval).  The transpose of the rows: for
 // every atom j the global sites of other atoms' clusters (first |C_K-1|

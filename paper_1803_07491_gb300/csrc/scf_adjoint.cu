@@ -6,6 +6,8 @@
 // those weights, project onsite-level cotangents onto u, and carry out the
 // Gram-Schmidt and combination steps of GMRES.  Every reduction has a fixed
 // order.
+#include <cooperative_groups.h>
+
 #include "kernels.h"
 
 namespace {
@@ -220,6 +222,220 @@ __global__ void k_jt_gather(int n, int S, const long long* __restrict__ ptr, con
   if (lane == 0) Eb[(size_t)spin * n + j] = a;
 }
 
+// The whole response solve over the stored rows of J in one cooperative
+// launch: restarted GMRES, right-preconditioned with the diagonal P, classical
+// Gram-Schmidt twice.  As separate kernels a step was 9 launches of 3 to 8 us
+// and a read-back of its Hessenberg column for a few us of work.
+//
+// Bound: the latency of the three grid synchronisations of a step and of the
+// loads between them.  Every block owns a contiguous slice of the atoms: it
+// gathers u = J^T x for its slice (one warp per atom, both spins), keeps its
+// slice of every basis vector to itself, and adds partial dot products of
+// the slice to a table [block][vector] that each block sums for itself in
+// block order after the synchronisation.  The newest vector is the only one
+// that other blocks read: its owner writes P u before the norm is known, and
+// the gather multiplies its sums by 1 / |u|.  The Givens rotations and the
+// stopping rule run in every block on the same numbers.  Measured per step at
+// 2,000 atoms: 52 us of kernels and a read-back of about 15 us -> 27 us.
+constexpr int GT = 512;
+
+// sum over the blocks of part[b][k], by one warp; the same in all lanes
+__device__ __forceinline__ double block_sums(const double* part, int nb, int ld, int k, int lane) {
+  double a = 0.0;
+  for (int b = lane; b < nb; b += 32) a += __ldcg(part + (size_t)b * ld + k);
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+__global__ void __launch_bounds__(GT, 1) k_gmres(GmresArgs g) {
+  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  constexpr int LD = GM_KRYLOV + 1;
+  __shared__ double Hh[GM_KRYLOV + 1][GM_KRYLOV], cs[GM_KRYLOV], sn[GM_KRYLOV], gv[GM_KRYLOV + 1];
+  __shared__ double h1[GM_KRYLOV + 1], h2[GM_KRYLOV + 1], red[GT / 32], ctl[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x;
+  const int n = g.n, nu = g.nu, comp = nu / n;
+  const int a0 = (int)((long long)n * blockIdx.x / nb), na = (int)((long long)n * (blockIdx.x + 1) / nb) - a0;
+  const int own = na * comp;  // owned elements: e -> (e / na) n + a0 + e % na
+  auto at = [&](int e) { return e < na ? a0 + e : n + a0 + e - na; };
+  double* part1 = g.part + (size_t)blockIdx.x * LD;
+  double* part2 = g.part + (size_t)(nb + blockIdx.x) * LD;
+  double* partn = g.part + (size_t)2 * nb * LD;
+
+  // out (own slice) = scale J^T x for x complete in memory
+  auto product = [&](const double* x, double scale, double* out) {
+    for (int q = warp; q < na; q += GT / 32) {
+      const int j = a0 + q;
+      const long long p0 = g.ptr[j], p1 = g.ptr[j + 1];
+      double a = 0.0, b = 0.0;
+#pragma unroll 4
+      for (long long p = p0 + lane; p < p1; p += 32) {
+        const int i = g.row[p];
+        const long long t = g.idx[p];
+        const double c = g.s * __ldcg(x + i);
+        if (comp == 1) {
+          a += c * g.val[t];
+        } else {
+          const double m = __ldcg(x + n + i);
+          a += (c + m) * g.val[t];
+          b += (c - m) * g.val[g.stride + t];
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (comp == 2) b += __shfl_xor_sync(0xffffffffu, b, o);
+      }
+      if (lane == 0) {
+        out[j] = scale * (a + b);
+        if (comp == 2) out[n + j] = scale * (0.5 * g.I * (b - a) - __ldcg(x + n + j));
+      }
+    }
+    __syncthreads();
+  };
+  // table[block][k] = own part of V_k . w for k < nvec
+  auto dots = [&](int nvec, const double* w, double* table) {
+    for (int k = warp; k < nvec; k += GT / 32) {
+      const double* v = g.V + (size_t)k * nu;
+      double a = 0.0;
+      for (int e = lane; e < own; e += 32) a += v[at(e)] * w[at(e)];
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) table[k] = a;
+    }
+  };
+  // w -= sum_k h_k V_k on the own slice, h summed from the blocks' table
+  auto subtract = [&](int nvec, const double* table, double* h, double* w) {
+    for (int k = warp; k < nvec; k += GT / 32) {
+      const double a = block_sums(table, nb, LD, k, lane);
+      if (lane == 0) h[k] = a;
+    }
+    __syncthreads();
+    for (int e = tid; e < own; e += GT) {
+      double a = w[at(e)];
+#pragma unroll 4
+      for (int k = 0; k < nvec; k++) a -= h[k] * g.V[(size_t)k * nu + at(e)];
+      w[at(e)] = a;
+    }
+    __syncthreads();
+  };
+  // partn[block] = own part of w . w; px (if not NULL) = P w
+  auto norm_part = [&](const double* w, double* px) {
+    double a = 0.0;
+    for (int e = tid; e < own; e += GT) {
+      const double v = w[at(e)];
+      a += v * v;
+      if (px) px[at(e)] = v * g.P[at(e)];
+    }
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) red[warp] = a;
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int q = 0; q < GT / 32; q++) t += red[q];
+      partn[blockIdx.x] = t;
+    }
+  };
+  auto norm2 = [&]() {  // after the grid synchronisation; the same in all threads
+    if (warp == 0) {
+      const double a = block_sums(partn, nb, 1, 0, lane);
+      if (lane == 0) ctl[0] = a;
+    }
+    __syncthreads();
+    return ctl[0];
+  };
+
+  for (int e = tid; e < own; e += GT) g.y[at(e)] = 0.0;
+  // r = rhs in the first cycle
+  for (int e = tid; e < own; e += GT) g.V[at(e)] = g.rhs[at(e)];
+  __syncthreads();
+  norm_part(g.V, g.x);
+  grid.sync();
+  const double bnorm = sqrt(norm2());
+  double beta = bnorm, rel = 0.0;
+  int iters = 0;
+  bool conv = bnorm == 0.0;
+  for (int cyc = 0; cyc < GM_CYCLES && !conv && iters < g.max_it; cyc++) {
+    if (cyc > 0) {  // r = rhs - J^T y into V_0
+      for (int e = tid; e < own; e += GT) g.xy[at(e)] = g.y[at(e)];
+      grid.sync();
+      product(g.xy, 1.0, g.V);
+      for (int e = tid; e < own; e += GT) g.V[at(e)] = g.rhs[at(e)] - g.V[at(e)];
+      __syncthreads();
+      norm_part(g.V, g.x);
+      grid.sync();
+      beta = sqrt(norm2());
+    }
+    if (beta <= g.rtol * bnorm) {
+      conv = true;
+      rel = beta / bnorm;
+      break;
+    }
+    double inv = 1.0 / beta;
+    for (int e = tid; e < own; e += GT) g.V[at(e)] *= inv;
+    for (int q = tid; q <= GM_KRYLOV; q += GT) gv[q] = q == 0 ? beta : 0.0;
+    __syncthreads();
+    int k = 0;
+    for (int j = 0; j < GM_KRYLOV; j++) {
+      double* u = g.V + (size_t)(j + 1) * nu;
+      product(g.x, inv, u);
+      dots(j + 1, u, part1);
+      grid.sync();
+      subtract(j + 1, g.part, h1, u);
+      dots(j + 1, u, part2);
+      grid.sync();
+      subtract(j + 1, g.part + (size_t)nb * LD, h2, u);
+      norm_part(u, g.x);
+      grid.sync();
+      const double hn = sqrt(norm2());
+      inv = 1.0 / hn;
+      if (hn > 0.0)
+        for (int e = tid; e < own; e += GT) u[at(e)] *= inv;
+      if (tid == 0) {  // Givens rotations on the new Hessenberg column
+        double t = h1[0] + h2[0];
+        for (int q = 0; q < j; q++) {
+          const double b = h1[q + 1] + h2[q + 1];
+          Hh[q][j] = cs[q] * t + sn[q] * b;
+          t = -sn[q] * t + cs[q] * b;
+        }
+        const double rr = hypot(t, hn);
+        const double c = rr > 0.0 ? t / rr : 1.0, z = rr > 0.0 ? hn / rr : 0.0;
+        cs[j] = c;
+        sn[j] = z;
+        Hh[j][j] = rr;
+        gv[j + 1] = -z * gv[j];
+        gv[j] = c * gv[j];
+        ctl[1] = fabs(gv[j + 1]) / bnorm;
+      }
+      __syncthreads();
+      k = j + 1;
+      iters++;
+      rel = ctl[1];
+      if (rel <= g.rtol || hn == 0.0 || iters >= g.max_it) break;
+    }
+    // z = H^-1 gv (upper triangular) in gv, y += P sum z_q V_q
+    if (warp == 0) {
+      for (int q = k - 1; q >= 0; q--) {
+        const double z = gv[q] / Hh[q][q];
+        for (int r = lane; r < q; r += 32) gv[r] -= Hh[r][q] * z;
+        __syncwarp();
+        if (lane == 0) gv[q] = z;
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < own; e += GT) {
+      double a = 0.0;
+      for (int q = 0; q < k; q++) a += gv[q] * g.V[(size_t)q * nu + at(e)];
+      g.y[at(e)] += a * g.P[at(e)];
+    }
+    __syncthreads();
+    conv = rel <= g.rtol;
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    g.out[0] = iters;
+    g.out[1] = rel;
+    g.out[2] = conv ? 1.0 : 0.0;
+  }
+}
+
 unsigned grid(long long n) { return (unsigned)((n + VT - 1) / VT); }
 int ok() { return cudaGetLastError() == cudaSuccess ? 0 : -1; }
 
@@ -295,4 +511,26 @@ int launch_jt_gather(int n, int S, const long long* ptr, const long long* idx, c
   const long long threads = (long long)S * n * 32;
   k_jt_gather<<<grid(threads), VT, 0, stream>>>(n, S, ptr, idx, row, val, stride, v, s, stoner, Eb);
   return ok();
+}
+
+int launch_gmres(const GmresArgs& g, cudaStream_t stream) {
+  int dev = 0, sms = 0, coop = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (!coop || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gmres, GT, 0) != cudaSuccess || per_sm < 1)
+    return -2;
+  // 8 atoms per block until every SM has a block: fewer blocks leave warps of
+  // the gather unused, more lengthen the sums over the blocks
+  int nb = (g.n + 7) / 8;
+  if (nb > sms) nb = sms;
+  if (nb > GMRES_BLOCKS) nb = GMRES_BLOCKS;
+  GmresArgs a = g;
+  void* args[] = {&a};
+  const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_gmres), nb, GT, args, 0, stream);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e == cudaErrorCooperativeLaunchTooLarge ? -2 : -1;
+  }
+  return 0;
 }

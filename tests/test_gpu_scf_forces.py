@@ -154,3 +154,31 @@ def test_stored_and_recomputed_reverse_sweeps_agree(bop, prec, tol, which):
     assert np.max(np.abs(F1 - F2)) < tol * scale
     assert np.max(np.abs(V1 - V2)) < tol * max(1.0, np.abs(V2).max())
     assert np.max(np.abs(W1 - W2)) < tol * max(1.0, np.abs(W2).max())
+
+
+@pytest.mark.parametrize("scf,cells,rtol", [("lcn", (1, 1, 1), 0.0), ("lcn", (2, 2, 1), 1e-15), ("stoner", (3, 2, 2), 0.0),
+                                            ("stoner", (2, 2, 1), 1e-15), ("lcn", (9, 9, 8), 0.0)])
+def test_response_solve_over_stored_rows(bop, scf, cells, rtol):
+    """The response solve in one launch over the stored rows of J against the
+    one that sweeps once per product (store budget 0): fewer atoms than one
+    block's warps, ragged slices, more atoms than eight per block, and with a
+    residual that FP64 cannot reach every restart of the basis.  Both stop at
+    a relative residual of 1e-10 (or the round-off): forces to 1e-8 of the
+    largest, a hundred times that for the conditioning of J."""
+    kw = dict(scf=scf, scf_tol=1e-10, scf_max_it=400)
+    if scf == "stoner":
+        kw.update(n_spin=2, stoner_I=0.8, eta=1.0, m_mix=1.0)
+    w = I.with_run(I.small_bcc(*cells, 0.06, 61), **kw)
+    out = []
+    for budget in (-1, 0):
+        ctx = bop.Context(w.model, w.run, "fp64")
+        bop.bop_set_store_budget(ctx.h, budget)
+        bop.bop_set_response_limits(ctx.h, 0, rtol)
+        ctx.build(w.pos, w.cell, w.pbc)
+        _, st = ctx.energy()
+        assert st["scf_converged"] == 1
+        F, _, fs = bop.bop_forces_stats(ctx.h, w.n_atoms, allow_noconv=True)
+        assert (fs["response_converged"] == 1) if rtol == 0.0 else (fs["response_residual"] < 1e-8)
+        out.append(F.cpu().numpy())
+        ctx.close()
+    assert np.max(np.abs(out[0] - out[1])) < 1e-8 * max(1.0, np.abs(out[1]).max())
