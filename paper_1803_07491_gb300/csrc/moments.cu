@@ -323,17 +323,17 @@ __device__ __forceinline__ void block_fma(const T* u, const T* x, T acc[NO][NC])
   }
 }
 
-// acc += sum over cnt adjacency entries (every step-th of ent) of B_ts x[s],
+// acc += sum over cnt adjacency entries of B_ts x[s],
 // with the blocks of the next two entries in flight while the current one is
 // applied.
 template <typename T, int NO, int NC, int PS>
-__device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int step, int cnt, const T* __restrict__ H,
+__device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int cnt, const T* __restrict__ H,
                                            int HS, const T* __restrict__ x, T acc[NO][NC]) {
   constexpr int HB = hb_count<NO>();
   constexpr int N = NO * NC;
   if (cnt <= 0) return;
   int2 e0 = ent[0];
-  int2 e1 = cnt > 1 ? ent[step] : e0;
+  int2 e1 = cnt > 1 ? ent[1] : e0;
   T h0[HB], h1[HB];
   load_bond<T, NO>(H + (size_t)e0.y * HS, h0);
   if (cnt > 1) load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
@@ -346,7 +346,7 @@ __device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int ste
 #pragma unroll
     for (int q = 0; q < HB; q++) h0[q] = h1[q];
     if (e + 2 < cnt) {
-      e1 = ent[(e + 2) * step];
+      e1 = ent[e + 2];
       load_bond<T, NO>(H + (size_t)e1.y * HS, h1);
     }
     T xs[N];
@@ -477,10 +477,10 @@ __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int fir
   }
 }
 
-// Forward kernel.  A persistent CTA takes a run of consecutive work items
-// (spin, atom); neighbouring atoms share most of their clusters' blocks, which
-// then come from L1.  For each item the atom's adjacency,
-// per-site offsets, level counts, site atoms and row orders are staged in
+// Forward kernel, FP32 (FP64: k_moments64).  A persistent CTA takes a run of
+// consecutive work items (spin, atom); neighbouring atoms share most of their
+// clusters' blocks, which then come from L1.  For each item the atom's
+// adjacency, per-site offsets, level counts and site atoms are staged in
 // shared memory (one coalesced copy) when they fit, so that the edge loop only
 // waits for the bond blocks, which are fetched one edge ahead.  Each thread
 // computes all columns of one site (NO^3 multiply-adds per edge); Psi rows are
@@ -488,35 +488,14 @@ __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int fir
 // odd levels) in shared memory, or where those do not fit (GMEM: clusters of
 // 11 and more moments) in the Psi store or the CTA's slot of global scratch,
 // from where the L2 serves them: one item with all columns takes 1/5 of the
-// block loads of five items that fit.  FP64 is bound by its DFMA pipe either
-// way (328 bytes per 125 DFMA, 62 cycles of an SM).
+// block loads of five items that fit.
 //
-// FP64: rows run in the order of their length (ClusterView::order): the 1 to
-// 6 entries of an outer shell's row and the 14 of an inner one no longer share
-// a warp, whose other lanes would idle for the longest row; odd passes over
-// the threads run backwards, so that the warp with the longest rows of one
-// pass gets the shortest of the next; and the long rows of a small level have
-// two lanes each, which halves the longest chain between two barriers (432-atom
-// Stoner cell: 1.57 -> 0.78 ms per pass with the pair form).
-//
-// FP64, pair: the last level (68 % of the products of a bcc cluster at 9
-// moments) computes the selected sites only (pair_selected).  H^K is
-// symmetric, so the block Z = Psi_K(t, i) holds Psi_K(i, t)^T too: its column
-// sums go to this item's last two moments and its row sums to those of the
-// site's atom, all with FP64 atomics onto moments that start at zero.
-//
-// FP32 keeps one lane per site, in site order, and the sums in that order: the
-// band edges are a maximum over levels, and moments rounded differently send
-// a few orbitals of 100,000 to the other side of a tie, where the forces jump.
-// (Row order and pair form gained 5 % there: the pass is bound by the L1 data
-// path, which idle lanes do not load.)
-template <typename T>
-struct Fwd {
-  // FP64: one DFMA of a warp takes 64 cycles of an SM sub-partition, so that
-  // one warp on each keeps it busy and the CTAs of four warps balance best
-  static constexpr int THREADS = sizeof(T) == 4 ? 192 : 128;
-  static constexpr int MIN_CTAS = 2;
-};
+// One lane per site, in site order, and the sums in that order: the band edges
+// are a maximum over levels, and moments rounded differently send a few
+// orbitals of 100,000 to the other side of a tie, where the forces jump.
+// (Rows ordered by length and the pair form of k_moments64 gained 5 % here: the
+// pass is bound by the L1 data path, which idle lanes do not load.)
+constexpr int F32_THREADS = 192;
 
 struct FwdSmem {
   int cap_even, cap_odd, max_sites, max_adj;
@@ -530,15 +509,14 @@ __device__ __forceinline__ bool site_selected(const ClusterView& cv, long long s
   return pair_selected(i, j, im[0], im[1], im[2]);
 }
 
-template <typename T, int NO, bool GMEM>
-__global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
-k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
-          int n_mom, FwdSmem L, int n_items, int chunk, double* __restrict__ mu, T* __restrict__ pstore,
-          const long long* __restrict__ psi_off, long long psi_tot, bool pair_form, bool sel_store,
-          T* __restrict__ scratch, size_t slot_elems) {
-  constexpr int NT = Fwd<T>::THREADS, NC = NO;
-  constexpr bool ORDERED = sizeof(T) == 8;
-  const bool pair = ORDERED && pair_form;
+template <int NO, bool GMEM>
+__global__ void __launch_bounds__(F32_THREADS, 2)
+k_moments(ClusterView cv, const float* __restrict__ H, int HS, const float* __restrict__ onsite, int n, int n_on,
+          int n_mom, FwdSmem L, int n_items, int chunk, double* __restrict__ mu, float* __restrict__ pstore,
+          const long long* __restrict__ psi_off, long long psi_tot, bool sel_store,
+          float* __restrict__ scratch, size_t slot_elems) {
+  using T = float;
+  constexpr int NT = F32_THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -550,8 +528,6 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
   unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
   int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.max_sites : 0));
   int* s_atom = s_off + (L.stage ? L.max_sites + 1 : 0);
-  unsigned* s_ord = reinterpret_cast<unsigned*>(s_atom + (L.stage ? L.max_sites : 0));
-  unsigned* s_top = s_ord + (L.stage && ORDERED ? L.max_sites : 0);
   // per-warp partial sums of the two moments of a level, in two buffers
   // (level parity): the reads of level k's partials need no barrier before
   // level k + 1 starts writing its own
@@ -572,14 +548,9 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
     const int2* adj = cv.adj + abase;
     const unsigned long long* lvc = cv.lvcnt + s0;
     const int* satom = L.stage ? s_atom : cv.site_atom + s0;
-    const unsigned* order = L.stage ? s_ord : cv.order + s0;
-    const unsigned* top = L.stage ? s_top : cv.top + s0;
     const T* E = onsite + (size_t)spin * n_on * NO;
-    if (L.stage) {
-      if (ORDERED) stage_order(cv, cur, pair, s_ord, s_top, tid, NT);
+    if (L.stage)
       stage_item(cv, cur, cur.nsite, (int)(cur.aend - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
-    }
-    const int ntop = pair ? cv.ntop[atom] : 0;
     const bool more = w + 1 < w1;
     if (more) ext_sites(cv, (w + 1) % n, nx);
     // stored Psi: item rows start at ib, level k at row lo_k = sum_{j<k} |C_j|
@@ -597,31 +568,16 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
       const bool in_store = GMEM && pstore != nullptr;
       const T* prev = in_store ? pitem + (size_t)lo_k * PS : buf[(k - 1) & 1];
       lo_k += lev[k - 1];
-      const bool half = pair && k == K;
-      const int ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
-      // rows of C_k-1 (7 to 14 entries in bcc) come first and, at FP64 levels
-      // of at most two passes, get two lanes each; the sites first reached at
-      // this level (1 to 6 entries) one
-      const int nrow = half ? ntop & 0xffff : lev[k];
-      const int nbig = ORDERED && nrow <= 2 * NT ? (half ? ntop >> 16 : ncol) : 0;
+      const int ncol = lev[k - 1], nrow = lev[k];
       T* next = buf[k & 1];
       T d1[NC], d2[NC];
 #pragma unroll
       for (int c = 0; c < NC; c++) d1[c] = d2[c] = T(0);
-      for (int p = 0; p * NT < nrow + nbig; p++) {
-        const int v = p * NT + (ORDERED && (p & 1) ? NT - 1 - tid : tid);
-        const bool big = v < 2 * nbig, live = v < nrow + nbig;
-        const int part = big ? v & 1 : 0;
-        const int r = !live ? 0 : (big ? v >> 1 : v - nbig);
-        // rows up to level k-2 are full, shell k-1 has entries up to its own
-        // level, shell k of the one below
-        const int t = !ORDERED ? r
-                      : half   ? (int)(top[r] & 0xffffu)
-                               : (r < inner ? r : (r < ncol ? (int)(order[r] >> 16) : (int)(order[r] & 0xffffu)));
+      for (int t = tid; t < nrow; t += NT) {
         T acc[NO][NC];
         const bool in_prev = t < ncol;
         const int atom_t = satom[t];
-        if (in_prev && part == 0) {
+        if (in_prev) {
           T pt[N];
           load_row<T, N, PS>(prev + (size_t)t * PS, pt);
           const T* e = E + (size_t)atom_t * NO;
@@ -637,52 +593,25 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
 #pragma unroll
             for (int c = 0; c < NC; c++) acc[r_][c] = T(0);
         }
-        if (live) {
-          const unsigned long long lc = L.stage ? s_lvc[t] : lvc[t];
-          const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
-          const int mine = big ? (cnt + 1 - part) >> 1 : cnt;
-          const int q0 = (L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase)) + part;
-          gather_pf2<T, NO, NC, PS>(L.stage ? s_adj + q0 : adj + q0, big ? 2 : 1, mine, H, HS, prev, acc);
-        }
-        if (ORDERED && __any_sync(0xffffffffu, big)) {
-#pragma unroll
-          for (int r_ = 0; r_ < NO; r_++)
-#pragma unroll
-            for (int c = 0; c < NC; c++) {
-              const T o = __shfl_xor_sync(0xffffffffu, acc[r_][c], 1);
-              if (big) acc[r_][c] += o;
-            }
-        }
-        if (!live || part != 0) continue;
+        const unsigned long long lc = L.stage ? s_lvc[t] : lvc[t];
+        const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
+        const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+        gather_pf2<T, NO, NC, PS>(L.stage ? s_adj + q0 : adj + q0, cnt, H, HS, prev, acc);
         // row t of Psi_k-1 again (shared memory), rather than kept live over the gather
-        const bool other = half && t != 0;
-        double* mt = mu + ((size_t)spin * n + atom_t) * NO * n_mom + 2 * K - 1;  // the last two moments of atom_t
         if (in_prev) {
           T pt[N];
           load_row<T, N, PS>(prev + (size_t)t * PS, pt);
 #pragma unroll
-          for (int r_ = 0; r_ < NO; r_++) {
-            T a = T(0);
+          for (int r_ = 0; r_ < NO; r_++)
 #pragma unroll
-            for (int c = 0; c < NC; c++) {
-              d1[c] += pt[r_ * NC + c] * acc[r_][c];
-              a += pt[r_ * NC + c] * acc[r_][c];
-            }
-            if (other) atomicAdd(mt + r_ * n_mom, (double)a);
-          }
+            for (int c = 0; c < NC; c++) d1[c] += pt[r_ * NC + c] * acc[r_][c];
         }
 #pragma unroll
-        for (int r_ = 0; r_ < NO; r_++) {
-          T a = T(0);
+        for (int r_ = 0; r_ < NO; r_++)
 #pragma unroll
-          for (int c = 0; c < NC; c++) {
-            d2[c] += acc[r_][c] * acc[r_][c];
-            a += acc[r_][c] * acc[r_][c];
-          }
-          if (other) atomicAdd(mt + r_ * n_mom + 1, (double)a);
-        }
+          for (int c = 0; c < NC; c++) d2[c] += acc[r_][c] * acc[r_][c];
         if (k < K && !in_store) store_row<T, N, PS>(next + (size_t)t * PS, &acc[0][0]);
-        if (pitem != nullptr && (half || k < K || !sel_store || site_selected(cv, s0, atom, atom_t, t)))
+        if (pitem != nullptr && (k < K || !sel_store || site_selected(cv, s0, atom, atom_t, t)))
           store_row<T, N, PS>(pitem + (size_t)(lo_k + t) * PS, &acc[0][0]);
       }
 #pragma unroll
@@ -700,15 +629,251 @@ k_moments(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
         T acc = T(0);
         for (int q = 0; q < NT / 32; q++) acc += red[k & 1][tid][q];
         const int c = tid % NC;
-        double* m = out + (size_t)c * n_mom + (tid < NC ? 2 * k - 1 : 2 * k);
-        if (half) atomicAdd(m, (double)acc);
-        else *m = (double)acc;
+        out[(size_t)c * n_mom + (tid < NC ? 2 * k - 1 : 2 * k)] = (double)acc;
       }
     }
     if (more) ext_adj(cv, nx);
   }
 }
 
+// ------------------------------------------------------------------ FP64: a lane per row of a site's block
+// FP64 is bound by the DFMA pipe (a warp's instruction takes 64 cycles of an SM
+// sub-partition, whatever its active lanes), so the work goes into warps that
+// are full and equally long: NO lanes per site, lane r holding row r of its
+// NO x NO block (32 / NO sites per warp, 25 multiply-adds per entry and lane at
+// NO = 5), and the warps of a CTA taking the next sites of a level from a
+// counter, longest rows first.  The lanes of a site read the same Psi row
+// (one shared-memory broadcast) and the NO elements of their row of the bond
+// block.  With one lane per site (and two for long rows of small levels) the
+// lanes were 82 % and the pipe 81 % busy, the SMs 88 %, at 9 moments.  The
+// work items go round the CTAs, so that cheap ones (surfaces) spread over
+// them.
+constexpr int F64_THREADS = 256;      // forward
+constexpr int F64_REV_THREADS = 128;  // reverse (twice the registers per lane)
+// (row entries of one lane in flight: two)
+
+// Sums of NV values over the warp with 10 instead of 5 NV additions at NV =
+// 10: every exchange halves the values a lane keeps.  Returns the sum of
+// value *which (-1: none); lanes may hold the same one.
+template <int NV>
+__device__ __forceinline__ double warp_sums(double (&v)[NV], int lane, int* which) {
+  int n = NV, base = 0, held = NV;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+    if (n > 1) {
+      const int h = (n + 1) / 2;
+#pragma unroll
+      for (int i = 0; i < NV; i++) {
+        if (i < h) {
+          const double a = v[i], b = i + h < n ? v[i + h < NV ? i + h : 0] : 0.0;
+          v[i] = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, o);
+        }
+      }
+      if (up) base += h;
+      held = up ? held - h : min(held, h);
+      n = h;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  *which = held > 0 ? base : -1;
+  return v[0];
+}
+
+// Row r of NO x NO blocks: acc[c] += sum over the entries of sum_g B[r][g]
+// x[s][g][c], with the block rows of two entries in flight.  u: positions of
+// B[r][g] in the bond record.
+template <int NO, int PS>
+__device__ __forceinline__ void gather64(const int2* __restrict__ ent, int cnt, const double* __restrict__ H, int HS,
+                                         const double* __restrict__ x, const int u[NO], double acc[NO]) {
+  if (cnt <= 0) return;
+  int2 e0 = ent[0], e1 = e0;
+  double b0[NO], b1[NO];
+#pragma unroll
+  for (int g = 0; g < NO; g++) b0[g] = __ldg(H + (size_t)e0.y * HS + u[g]);
+  if (cnt > 1) {
+    e1 = ent[1];
+#pragma unroll
+    for (int g = 0; g < NO; g++) b1[g] = __ldg(H + (size_t)e1.y * HS + u[g]);
+  }
+  for (int e = 0; e < cnt; e++) {
+    const int s = e0.x;
+    double b[NO];
+#pragma unroll
+    for (int g = 0; g < NO; g++) {
+      b[g] = b0[g];
+      b0[g] = b1[g];
+    }
+    e0 = e1;
+    if (e + 2 < cnt) {
+      e1 = ent[e + 2];
+#pragma unroll
+      for (int g = 0; g < NO; g++) b1[g] = __ldg(H + (size_t)e1.y * HS + u[g]);
+    }
+    double xs[NO * NO];
+    load_row<double, NO * NO, PS>(x + (size_t)s * PS, xs);
+#pragma unroll
+    for (int g = 0; g < NO; g++)
+#pragma unroll
+      for (int c = 0; c < NO; c++) acc[c] += b[g] * xs[g * NO + c];
+  }
+}
+
+// Forward.  pair: the last level computes the selected sites only
+// (pair_selected).  H^K is symmetric, so the block Z = Psi_K(t, i) holds
+// Psi_K(i, t)^T too: its column sums go to this item's last two moments and
+// its row sums to those of the site's atom, all with FP64 atomics onto moments
+// that start at zero (68 % of a bcc cluster's products at 9 moments are in
+// that level).  GMEM as k_moments.
+template <int NO, bool GMEM>
+__global__ void __launch_bounds__(F64_THREADS, 2)
+k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* __restrict__ onsite, int n, int n_on,
+            int n_mom, FwdSmem L, int n_items, double* __restrict__ mu, double* __restrict__ pstore,
+            const long long* __restrict__ psi_off, long long psi_tot, bool pair, double* __restrict__ scratch,
+            size_t slot_elems) {
+  constexpr int NT = F64_THREADS, NC = NO, RPW = 32 / NO;
+  constexpr int N = NO * NC;
+  constexpr int PS = (N == 1) ? 1 : Row<double, N>::PS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* buf[2];
+  buf[0] = GMEM ? scratch + (size_t)blockIdx.x * slot_elems : reinterpret_cast<double*>(smem_raw);
+  buf[1] = buf[0] + (size_t)L.cap_even * PS;
+  unsigned char* tail = align16(GMEM ? smem_raw : reinterpret_cast<unsigned char*>(buf[1] + (size_t)L.cap_odd * PS));
+  int2* s_adj = reinterpret_cast<int2*>(tail);
+  unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
+  int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.max_sites : 0));
+  int* s_atom = s_off + (L.stage ? L.max_sites + 1 : 0);
+  unsigned* s_ord = reinterpret_cast<unsigned*>(s_atom + (L.stage ? L.max_sites : 0));
+  unsigned* s_top = s_ord + (L.stage ? L.max_sites : 0);
+  // per-warp partial sums of the two moments of a level, in two buffers
+  // (level parity), as k_moments
+  __shared__ double red[2][2 * NC][NT / 32];
+  __shared__ int s_next[BOP_MAX_K + 1];  // next sites of a level
+  const int K = cv.K;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int sub = lane / NO, r = lane % NO;  // this lane's site of the warp's and its block row
+  int u[NO];
+#pragma unroll
+  for (int g = 0; g < NO; g++) u[g] = UI<NO>(r, g);
+  ItemExt nx{};
+  if ((int)blockIdx.x < n_items) {
+    ext_sites(cv, blockIdx.x % n, nx);
+    ext_adj(cv, nx);
+  }
+  for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
+    const int spin = w / n, atom = w % n;
+    const ItemExt cur = nx;
+    const long long s0 = cur.s0, abase = cur.abase;
+    const int* lev = cv.level_end + (size_t)atom * (K + 1);
+    const int2* adj = cv.adj + abase;
+    const int* satom = L.stage ? s_atom : cv.site_atom + s0;
+    const unsigned* order = L.stage ? s_ord : cv.order + s0;
+    const unsigned* top = L.stage ? s_top : cv.top + s0;
+    const double* E = onsite + (size_t)spin * n_on * NO;
+    if (L.stage) {
+      stage_order(cv, cur, pair, s_ord, s_top, tid, NT);
+      stage_item(cv, cur, cur.nsite, (int)(cur.aend - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
+    }
+    const int ntop = pair ? cv.ntop[atom] & 0xffff : 0;
+    const bool more = n_items - w > (int)gridDim.x;
+    if (more) ext_sites(cv, (w + gridDim.x) % n, nx);
+    // stored Psi: item rows start at psi_off, level k at row lo_k = sum_{j<k} |C_j|
+    double* pitem = nullptr;
+    if (pstore != nullptr) {
+      pitem = pstore + ((size_t)spin * psi_tot + psi_off[atom]) * PS;
+      for (int q = tid; q < PS; q += NT) pitem[q] = q < N && q / NC == q % NC ? 1.0 : 0.0;
+    }
+    for (int q = tid; q < PS; q += NT) buf[0][q] = q < N && q / NC == q % NC ? 1.0 : 0.0;
+    if (tid <= K) s_next[tid] = 0;
+    long long lo_k = 0;
+    __syncthreads();
+    double* out = mu + (size_t)w * NO * n_mom;
+    if (tid < NC) out[(size_t)tid * n_mom] = 1.0;
+    for (int k = 1; k <= K; k++) {
+      const bool in_store = GMEM && pstore != nullptr;
+      const double* prev = in_store ? pitem + (size_t)lo_k * PS : buf[(k - 1) & 1];
+      lo_k += lev[k - 1];
+      const bool half = pair && k == K;
+      const int ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
+      const int nrow = half ? ntop : lev[k];
+      double* next = buf[k & 1];
+      double d[2 * NC];
+#pragma unroll
+      for (int c = 0; c < 2 * NC; c++) d[c] = 0.0;
+      while (true) {
+        int first = 0;
+        if (lane == 0) first = atomicAdd(&s_next[k], RPW);
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (first >= nrow) break;
+        const int q = first + sub;
+        if (sub >= RPW || q >= nrow) continue;  // (the shuffle above reconverges the warp)
+        // rows up to level k-2 are full, shell k-1 has entries up to its own
+        // level, shell k of the one below
+        const int t = half ? (int)(top[q] & 0xffffu)
+                           : (q < inner ? q : (q < ncol ? (int)(order[q] >> 16) : (int)(order[q] & 0xffffu)));
+        const bool in_prev = t < ncol;
+        const int atom_t = satom[t];
+        const double* pt = prev + (size_t)t * PS + r * NC;
+        double acc[NC];
+        if (in_prev) {
+          const double er = E[(size_t)atom_t * NO + r];
+#pragma unroll
+          for (int c = 0; c < NC; c++) acc[c] = er * pt[c];
+        } else {
+#pragma unroll
+          for (int c = 0; c < NC; c++) acc[c] = 0.0;
+        }
+        const unsigned long long lc = L.stage ? s_lvc[t] : cv.lvcnt[s0 + t];
+        const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
+        const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+        gather64<NO, PS>(L.stage ? s_adj + q0 : adj + q0, cnt, H, HS, prev, u, acc);
+        const bool other = half && t != 0;
+        double* mt = mu + (((size_t)spin * n + atom_t) * NO + r) * n_mom + 2 * K - 1;  // the last two moments of (atom_t, r)
+        if (in_prev) {
+          double a = 0.0;
+#pragma unroll
+          for (int c = 0; c < NC; c++) {
+            const double p = pt[c];
+            d[c] += p * acc[c];
+            if (half) a += p * acc[c];
+          }
+          if (other) atomicAdd(mt, a);
+        }
+        double a = 0.0;
+#pragma unroll
+        for (int c = 0; c < NC; c++) {
+          d[NC + c] += acc[c] * acc[c];
+          if (half) a += acc[c] * acc[c];
+        }
+        if (other) atomicAdd(mt + 1, a);
+        if (k < K && !in_store) {
+#pragma unroll
+          for (int c = 0; c < NC; c++) next[(size_t)t * PS + r * NC + c] = acc[c];
+        }
+        if (pitem != nullptr) {
+#pragma unroll
+          for (int c = 0; c < NC; c++) pitem[(size_t)(lo_k + t) * PS + r * NC + c] = acc[c];
+        }
+      }
+      int which;
+      const double sum = warp_sums<2 * NC>(d, lane, &which);
+      if (which >= 0) red[k & 1][which][wid] = sum;
+      // level k's rows and partials are complete; level k + 1 writes the
+      // other Psi buffer (read last at level k - 1) and the other partials
+      __syncthreads();
+      if (tid < 2 * NC) {
+        double a = 0.0;
+        for (int q = 0; q < NT / 32; q++) a += red[k & 1][tid][q];
+        const int c = tid % NC;
+        double* m = out + (size_t)c * n_mom + (tid < NC ? 2 * k - 1 : 2 * k);
+        if (half) atomicAdd(m, a);
+        else *m = a;
+      }
+    }
+    if (more) ext_adj(cv, nx);
+  }
+}
 
 // ------------------------------------------------------------------ reverse sweep over stored Psi
 // With every Psi_k of every work item stored in global memory (rows of the
@@ -748,14 +913,15 @@ __host__ __device__ constexpr size_t eb_elems(int cap_eb) {
 
 constexpr int REV_SEL_WORDS = 256;  // selected sites as bits (a cluster with a pair form has at most 8,192 sites)
 
-template <typename T, int NO, bool HBAR, bool GMEM>
-__global__ void __launch_bounds__(Fwd<T>::THREADS, Fwd<T>::MIN_CTAS)
-k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on,
-          int n_mom, RevSmem L, int n_items, int chunk, const T* __restrict__ pstore,
+template <int NO, bool HBAR, bool GMEM>
+__global__ void __launch_bounds__(F32_THREADS, 2)
+k_adj_rev(ClusterView cv, const float* __restrict__ H, int HS, const float* __restrict__ onsite, int n, int n_on,
+          int n_mom, RevSmem L, int n_items, int chunk, const float* __restrict__ pstore,
           const long long* __restrict__ psi_off, long long psi_tot, const double* __restrict__ wts,
-          T* __restrict__ Hbar, int HSh, double* __restrict__ Ebar, double* __restrict__ siteval,
-          long long sv_stride, bool pair, T* __restrict__ scratch, size_t slot_elems) {
-  constexpr int NT = Fwd<T>::THREADS, NC = NO;
+          float* __restrict__ Hbar, int HSh, double* __restrict__ Ebar, double* __restrict__ siteval,
+          long long sv_stride, bool pair, float* __restrict__ scratch, size_t slot_elems) {
+  using T = float;
+  constexpr int NT = F32_THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -970,6 +1136,316 @@ k_adj_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__
         double a = 0.0;
 #pragma unroll
         for (int r = 0; r < NO; r++) a += (double)eb[t * NO + r];
+        atomicAdd(siteval + (size_t)spin * sv_stride + s0 + t, a);
+      }
+    }
+    if (more) ext_adj(cv, nx);
+    __syncthreads();
+  }
+}
+
+// FP64 (see k_moments64): lane r of a site holds row r of its block.  HBAR: for
+// the bond cotangents dL/dB = x[s] pt^T (x = Psi-bar_k, pt = Psi_k-1(t)) lane r
+// forms column r from its row of pt and the whole x[s], rows taken in the order
+// r, r + 1, .. (mod NO): what its unique elements (r, r), (r, r + 1), (r, r + 2)
+// still lack then sits in the same place of another lane of the site, and two
+// shuffles replace a sum over lanes.
+//
+// The entries first, first + step, ... of the row, or those of the bits of
+// mask.  All lanes of a warp call it (rows of no entries: cnt 0); rounds run
+// together with HBAR.  u[j], o[j]: positions of B[r][(r + j) % NO] in the bond
+// record and of row (r + j) % NO in a Psi row.
+template <int NO, int PS, bool HBAR>
+__device__ __forceinline__ void gather_rev64(const int2* __restrict__ ent, int first, int step, int cnt, unsigned mask,
+                                             bool use_mask, const double* __restrict__ H, int HS,
+                                             const double* __restrict__ x, const int u[NO], const int o[NO],
+                                             double acc[NO], bool gather, const double pt[NO],
+                                             double* __restrict__ Hbar, int HSh, int lane, int r) {
+  const int mine = use_mask ? __popc(mask) : (cnt > first ? (cnt - first + step - 1) / step : 0);
+  const int rounds = HBAR ? __reduce_max_sync(0xffffffffu, mine) : mine;
+  int e = first;
+  auto next = [&]() -> int2 {  // the row's next entry
+    int i = e;
+    if (use_mask) {
+      i = __ffs(mask) - 1;
+      mask &= mask - 1;
+    }
+    e += step;
+    return ent[i];
+  };
+  int2 e0 = make_int2(0, -1), e1 = make_int2(0, -1);
+  double b0[NO], b1[NO];
+#pragma unroll
+  for (int j = 0; j < NO; j++) b0[j] = b1[j] = 0.0;
+  auto load = [&](int bond, double b[NO]) {
+#pragma unroll
+    for (int j = 0; j < NO; j++) b[j] = __ldg(H + (size_t)bond * HS + u[j]);
+  };
+  if (mine > 0) {
+    e0 = next();
+    if (gather) load(e0.y, b0);
+  }
+  if (mine > 1) {
+    e1 = next();
+    if (gather) load(e1.y, b1);
+  }
+  for (int it = 0; it < rounds; it++) {
+    const bool on = it < mine;
+    const int s = e0.x, bond = on ? e0.y : -1;
+    double b[NO];
+#pragma unroll
+    for (int j = 0; j < NO; j++) {
+      b[j] = b0[j];
+      b0[j] = b1[j];
+    }
+    e0 = e1;
+    if (it + 2 < mine) {
+      e1 = next();
+      if (gather) load(e1.y, b1);
+    }
+    if constexpr (!HBAR) {
+      double xs[NO * NO];
+      load_row<double, NO * NO, PS>(x + (size_t)s * PS, xs);
+      // (u is not rotated without HBAR)
+#pragma unroll
+      for (int g = 0; g < NO; g++)
+#pragma unroll
+        for (int c = 0; c < NO; c++) acc[c] += b[g] * xs[g * NO + c];
+    } else {
+      double G[NO];  // G[j] = dL/dB[(r + j) % NO][r]
+#pragma unroll
+      for (int j = 0; j < NO; j++) G[j] = 0.0;
+      if (on) {
+        const double* xr = x + (size_t)s * PS;
+#pragma unroll
+        for (int j = 0; j < NO; j++)
+#pragma unroll
+          for (int c = 0; c < NO; c++) {
+            const double v = xr[o[j] + c];
+            acc[c] += b[j] * v;
+            G[j] += v * pt[c];
+          }
+      }
+      double* hb = Hbar + (size_t)(bond < 0 ? 0 : bond) * HSh;
+      if (bond >= 0) atomicAdd(hb + u[0], G[0]);
+#pragma unroll
+      for (int j = 1; j <= NO / 2; j++) {
+        // lane (r + j) % NO of the site holds dL/dB[r][(r + j) % NO] as its G[NO - j]
+        const double other = __shfl_sync(0xffffffffu, G[NO - j], lane + (r + j < NO ? j : j - NO));
+        if (bond >= 0 && (2 * j < NO || r < j)) atomicAdd(hb + u[j], G[j] + other);
+      }
+    }
+  }
+}
+
+template <int NO, bool HBAR, bool GMEM>
+__global__ void __launch_bounds__(F64_REV_THREADS, 3)
+k_adj_rev64(ClusterView cv, const double* __restrict__ H, int HS, const double* __restrict__ onsite, int n, int n_on,
+            int n_mom, RevSmem L, int n_items, const double* __restrict__ pstore,
+            const long long* __restrict__ psi_off, long long psi_tot, const double* __restrict__ wts,
+            double* __restrict__ Hbar, int HSh, double* __restrict__ Ebar, double* __restrict__ siteval,
+            long long sv_stride, bool pair, double* __restrict__ scratch, size_t slot_elems) {
+  constexpr int NT = F64_REV_THREADS, NC = NO, RPW = 32 / NO;
+  constexpr int N = NO * NC;
+  constexpr int PS = (N == 1) ? 1 : Row<double, N>::PS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* buf[2];
+  buf[0] = GMEM ? scratch + (size_t)blockIdx.x * slot_elems : reinterpret_cast<double*>(smem_raw);
+  buf[1] = buf[0] + (size_t)L.cap_even * PS;
+  // [cap_eb][NO], padded to 16 bytes
+  double* eb = GMEM ? reinterpret_cast<double*>(smem_raw) : buf[1] + (size_t)L.cap_odd * PS;
+  unsigned char* tail = align16(reinterpret_cast<unsigned char*>(eb + eb_elems<double, NO>(L.cap_eb)));
+  int2* s_adj = reinterpret_cast<int2*>(tail);
+  unsigned long long* s_lvc = reinterpret_cast<unsigned long long*>(s_adj + (L.stage ? L.max_adj : 0));
+  int* s_off = reinterpret_cast<int*>(s_lvc + (L.stage ? L.cap_eb : 0));
+  int* s_atom = s_off + (L.stage ? L.cap_eb + 1 : 0);
+  __shared__ double ws[NC][BOP_MAX_NMOM];
+  __shared__ int s_lev[BOP_MAX_K + 1], s_next[BOP_MAX_K + 1];
+  __shared__ long long s_lo[BOP_MAX_K + 1];
+  __shared__ unsigned s_sel[REV_SEL_WORDS];
+  const int K = cv.K;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int grp = lane / NO, r = lane % NO;
+  int u[NO], o[NO];
+#pragma unroll
+  for (int j = 0; j < NO; j++) {
+    const int g = HBAR ? (r + j) % NO : j;
+    u[j] = UI<NO>(r, g);
+    o[j] = g * NC;
+  }
+  ItemExt nx{};
+  if ((int)blockIdx.x < n_items) {
+    ext_sites(cv, blockIdx.x % n, nx);
+    ext_adj(cv, nx);
+  }
+  for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
+    const int spin = w / n, atom = w % n;
+    const ItemExt cur = nx;
+    const long long s0 = cur.s0, abase = cur.abase;
+    const int* lev = cv.level_end + (size_t)atom * (K + 1);
+    const unsigned long long* lvc = L.stage ? s_lvc : cv.lvcnt + s0;
+    const int* satom = L.stage ? s_atom : cv.site_atom + s0;
+    const unsigned* top = cv.top + s0;
+    const double* E = onsite + (size_t)spin * n_on * NO;
+    const double* P = pstore + ((size_t)spin * psi_tot + psi_off[atom]) * PS;
+    if (L.stage) {
+      const int nr = lev[K - 1];
+      stage_item(cv, cur, nr, (int)(cv.adj_off[s0 + nr] - abase), s_adj, s_off, s_lvc, s_atom, tid, NT);
+    }
+    const int2* adj = L.stage ? s_adj : cv.adj + abase;
+    const bool more = n_items - w > (int)gridDim.x;
+    if (more) ext_sites(cv, (w + gridDim.x) % n, nx);
+    if (tid <= K) {
+      s_lev[tid] = lev[tid];
+      s_next[tid] = 0;
+    }
+    if (tid == 0) {
+      long long lo = 0;
+      for (int k = 0; k <= K; k++) {
+        s_lo[k] = lo;
+        lo += lev[k];
+      }
+    }
+    for (int q = tid; q < NC * n_mom; q += NT) {
+      const int c = q / n_mom, m = q % n_mom;
+      ws[c][m] = wts[((size_t)w * NO + c) * n_mom + m];
+    }
+    if (pair)
+      for (int q = tid; q < REV_SEL_WORDS; q += NT) s_sel[q] = 0;
+    __syncthreads();
+    const int neb = s_lev[K - 1];
+    for (int q = tid; q < neb * NO; q += NT) eb[q] = 0.0;
+    // Psi-bar_K
+    double* xK = buf[K & 1];
+    if (pair) {  // rows that are not selected enter with zero
+      for (int q = tid; q < neb * PS; q += NT) xK[q] = 0.0;
+      __syncthreads();
+    }
+    const int nK = pair ? cv.ntop[atom] & 0xffff : s_lev[K];
+    for (int q = tid; q < nK * NO; q += NT) {
+      const int i = q / NO, b = q % NO;
+      const int t = pair ? (int)(top[i] & 0xffffu) : i;
+      // weights of the site's atom (rows), in the pair form
+      double wj2 = 0.0, wj1 = 0.0;
+      if (pair) {
+        if (b == 0 && t < neb) atomicOr(&s_sel[t >> 5], 1u << (t & 31));
+        if (t != 0) {
+          const double* wj = wts + (((size_t)spin * n + satom[t]) * NO + b) * n_mom + 2 * K - 1;
+          wj1 = wj[0];
+          wj2 = wj[1];
+        }
+      }
+      const double* pk = P + (size_t)(s_lo[K] + t) * PS + b * NC;
+      double* row = xK + (size_t)t * PS + b * NC;
+      const double* p1 = P + (size_t)(s_lo[K - 1] + t) * PS + b * NC;
+#pragma unroll
+      for (int c = 0; c < NC; c++) {
+        double v = 2.0 * (ws[c][2 * K] + wj2) * pk[c];
+        if (t < neb) v += (ws[c][2 * K - 1] + wj1) * p1[c];
+        row[c] = v;
+      }
+    }
+    __syncthreads();
+    for (int k = K; k >= 1; k--) {
+      const bool half = pair && k == K;
+      const double* xb = buf[k & 1];
+      double* yb = buf[(k - 1) & 1];
+      const int nrow = s_lev[k - 1];
+      // lanes of few rows: P parts of a row's entries (2 to 14 in bcc) each on
+      // its own lanes, where that shortens the rounds of the CTA's warps
+      int parts = 1, rows = RPW;  // rows of a warp
+      if (!half) {
+        int best = 1 << 30;
+#pragma unroll
+        for (int p = 1; p <= (RPW < 8 ? RPW : 8); p++) {
+          const int rp = RPW / p, len = (nrow + rp * (NT / 32) - 1) / (rp * (NT / 32)) * (16 / p + 1);
+          if (len < best) {
+            best = len;
+            parts = p;
+            rows = rp;
+          }
+        }
+      }
+      const int part = grp % parts, sub = grp / parts;
+      while (true) {
+        int first = 0;
+        if (lane == 0) first = atomicAdd(&s_next[k], rows);
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (first >= nrow) break;
+        const int rr = first + sub;
+        const bool live = sub < rows && rr < nrow;
+        const int t = !live ? 0 : (half ? (int)(top[rr] >> 16) : rr);
+        const double* r1 = P + (size_t)(s_lo[k - 1] + t) * PS + r * NC;
+        double pt[NC], acc[NC];
+#pragma unroll
+        for (int c = 0; c < NC; c++) {
+          pt[c] = live ? r1[c] : 0.0;
+          acc[c] = 0.0;
+        }
+        const bool own = live && part == 0;
+        const double* xt = xb + (size_t)t * PS + r * NC;
+        if (own) {
+          if (r == 0 && k >= 2) {  // the stored rows this site needs, towards L2 while the gather runs
+            prefetch_row_l2<double, PS>(P + (size_t)(s_lo[k] + t) * PS);
+            if (t < s_lev[k - 2]) prefetch_row_l2<double, PS>(P + (size_t)(s_lo[k - 2] + t) * PS);
+          }
+          if (k >= 2) {
+            const double er = E[(size_t)satom[t] * NO + r];
+#pragma unroll
+            for (int c = 0; c < NC; c++) acc[c] = er * xt[c];
+          }
+        }
+        if (k >= 2 || HBAR) {
+          const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+          int cnt = 0;
+          if (live) {
+            if (k < K) cnt = (int)((lvc[t] >> (8 * k)) & 0xff);
+            else cnt = L.stage ? s_off[t + 1] - q0 : (int)(cv.adj_off[s0 + t + 1] - abase) - q0;
+          }
+          const unsigned mask = half && live ? cv.topmask[s0 + t] : 0u;
+          gather_rev64<NO, PS, HBAR>(adj + q0, part, parts, cnt, mask, half, H, HS, xb, u, o, acc, k >= 2, pt, Hbar,
+                                     HSh, lane, r);
+          __syncwarp();
+          for (int p = 1; p < parts; p++)
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+              const double v = __shfl_sync(0xffffffffu, acc[c], lane + p * NO);
+              if (part == 0) acc[c] += v;
+            }
+        }
+        if (!own) continue;
+        // onsite cotangent of level k: Psi-bar_k[t] . Psi_k-1[t]
+        double a = 0.0;
+#pragma unroll
+        for (int c = 0; c < NC; c++) a += xt[c] * pt[c];
+        eb[t * NO + r] += a;
+        if (k >= 2) {
+          const bool has_k = !half || (s_sel[t >> 5] >> (t & 31) & 1u), has_2 = t < s_lev[k - 2];
+          const double wj = half && t != 0 ? wts[(((size_t)spin * n + satom[t]) * NO + r) * n_mom + 2 * K - 1] : 0.0;
+          const double* pk = P + (size_t)(s_lo[k] + t) * PS + r * NC;
+          const double* p2 = P + (size_t)(s_lo[k - 2] + t) * PS + r * NC;
+#pragma unroll
+          for (int c = 0; c < NC; c++) {
+            double v = acc[c] + 2.0 * ws[c][2 * k - 2] * pt[c];
+            if (has_k) v += (ws[c][2 * k - 1] + wj) * pk[c];
+            if (has_2) v += ws[c][2 * k - 3] * p2[c];
+            yb[(size_t)t * PS + r * NC + c] = v;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    if (Ebar != nullptr) {
+      for (int q = tid; q < neb * NO; q += NT) {
+        const int t = q / NO, b = q % NO;
+        atomicAdd(Ebar + ((size_t)spin * n_on + satom[t]) * NO + b, eb[q]);
+      }
+    }
+    if (siteval != nullptr) {  // per-site sums over the orbitals (one row of the SCF Jacobian)
+      for (int t = tid; t < neb; t += NT) {
+        double a = 0.0;
+#pragma unroll
+        for (int b = 0; b < NO; b++) a += eb[t * NO + b];
         atomicAdd(siteval + (size_t)spin * sv_stride + s0 + t, a);
       }
     }
@@ -1538,7 +2014,7 @@ k_nc_fwd(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ 
         }
         const int cnt = (int)((lvc[t] >> (8 * (k - 1))) & 0xff);
         const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
-        gather_pf2<T, NO, NCS, PS>(adj + q0, 1, cnt, H, HS, prev, acc);
+        gather_pf2<T, NO, NCS, PS>(adj + q0, cnt, H, HS, prev, acc);
         T pt[PS];
         if (in_prev) {
           load_row<T, PS, PS>(prev + (size_t)t * PS, pt);
@@ -1768,17 +2244,19 @@ __global__ void k_torques(int n, int norb, int n_mom, const double* __restrict__
   t[3 * (size_t)i + 2] = g[0] * sy - g[1] * sx;
 }
 
-// CTAs of a persistent kernel and the work items of each.
+// CTAs of a persistent kernel (at most `most`) and the work items of each: a
+// run of consecutive ones, or with `round` those a grid apart.
 template <class F>
-void persistent_grid(F fn, int threads, size_t smem, int n_items, int* grid, int* chunk) {
+void persistent_grid(F fn, int threads, size_t smem, int n_items, size_t most, bool round, int* grid, int* chunk) {
   int per_sm = 1, sms = 0, dev = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
   if (per_sm < 1) per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int slots = sms * per_sm;
+  int slots = sms * per_sm;
+  if ((size_t)slots > most) slots = (int)most;
   *chunk = (n_items + slots - 1) / slots;
-  *grid = (n_items + *chunk - 1) / *chunk;
+  *grid = round ? (n_items < slots ? n_items : slots) : (n_items + *chunk - 1) / *chunk;
 }
 
 // Spinor sweeps with two levels in shared memory: -2 where they do not fit.
@@ -1799,7 +2277,7 @@ int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
     return -1;
   const int n_items = a.n * NO;
   int grid, chunk;
-  persistent_grid(fn, NT, smem, n_items, &grid, &chunk);
+  persistent_grid(fn, NT, smem, n_items, n_items, false, &grid, &chunk);
   fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, chunk,
                             a.mu, a.vmom, (T*)a.pstore, a.psi_off, a.psi_tot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -1821,7 +2299,7 @@ int run_nc_rev(const NcArgs& a, cudaStream_t s) {
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
   const int n_items = a.n * NO;
   int grid, chunk;
-  persistent_grid(fn, 128, smem, n_items, &grid, &chunk);
+  persistent_grid(fn, 128, smem, n_items, n_items, false, &grid, &chunk);
   fn<<<grid, 128, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, chunk,
                              (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.obar);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -1843,7 +2321,8 @@ template <typename T, int NO, bool GMEM>
 int run_forward(const MomentsArgs& a, cudaStream_t s) {
   constexpr int N = NO * NO;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
-  constexpr int NT = Fwd<T>::THREADS;
+  constexpr bool F64 = sizeof(T) == 8;
+  constexpr int NT = F64 ? F64_THREADS : F32_THREADS;
   FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
   const size_t psi = GMEM ? 0 : (size_t)(a.cap_even + a.cap_odd) * PS * sizeof(T);
   size_t stage = (size_t)a.max_adj * 8 + (size_t)a.max_sites * 8 + (size_t)(a.max_sites + 1) * 4 +
@@ -1854,25 +2333,28 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
     L.stage = false;
     smem = psi;
   }
-  auto fn = k_moments<T, NO, GMEM>;
+  auto fn = [] {
+    if constexpr (F64) return k_moments64<NO, GMEM>;
+    else return k_moments<NO, GMEM>;
+  }();
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return -1;
   const int n_items = a.n * a.n_spin;
   int grid, chunk;
-  persistent_grid(fn, NT, smem, n_items, &grid, &chunk);
   const size_t slot = (size_t)(a.cap_even + a.cap_odd) * PS;
-  if (GMEM && a.pstore == nullptr && (size_t)grid * slot * sizeof(T) > a.scratch_bytes) {
-    // fewer CTAs than fit on the device: what the scratch holds
-    const size_t most = a.scratch_bytes / (slot * sizeof(T));
-    if (most < 1) return -1;
-    chunk = (int)((n_items + most - 1) / most);
-    grid = (n_items + chunk - 1) / chunk;
-  }
-  if (sizeof(T) == 8 && a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
+  // with Psi in global scratch no more CTAs than its slots
+  const size_t most = GMEM && a.pstore == nullptr ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
+  if (most < 1) return n_items == 0 ? 0 : -1;
+  persistent_grid(fn, NT, smem, n_items, most, F64, &grid, &chunk);
+  if (F64 && a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
     return -1;
-  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
-                            a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, a.pair, (T*)a.scratch, slot);
+  if constexpr (F64)
+    fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, a.mu,
+                              (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
+  else
+    fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
+                              a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1890,13 +2372,17 @@ template <typename T, int NO, bool HBAR, bool GMEM>
 int run_reverse(const AdjointArgs& a, cudaStream_t s) {
   constexpr int N = NO * NO;
   constexpr int PS = (N == 1) ? 1 : Row<T, N>::PS;
-  constexpr int NT = Fwd<T>::THREADS;
+  constexpr bool F64 = sizeof(T) == 8;
+  constexpr int NT = F64 ? F64_REV_THREADS : F32_THREADS;
   RevSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, a.cap_eb, true};
   const size_t slot = (size_t)(a.cap_even + a.cap_odd) * PS;
   const size_t psi = (GMEM ? 0 : slot * sizeof(T)) + eb_elems<T, NO>(a.cap_eb) * sizeof(T);
   const size_t stage = (size_t)a.max_adj * 8 + (size_t)a.cap_eb * 8 + (size_t)(a.cap_eb + 1) * 4 +
                        (size_t)a.max_sites * 4 + 16;
-  auto fn = k_adj_rev<T, NO, HBAR, GMEM>;
+  auto fn = [] {
+    if constexpr (F64) return k_adj_rev64<NO, HBAR, GMEM>;
+    else return k_adj_rev<NO, HBAR, GMEM>;
+  }();
   size_t smem = psi + stage;
   int per_sm = 0, per_sm_unstaged = 0;
   if (psi > 225 * 1024) return -2;
@@ -1914,16 +2400,17 @@ int run_reverse(const AdjointArgs& a, cudaStream_t s) {
   }
   const int n_items = a.n * a.n_spin;
   int grid, chunk;
-  persistent_grid(fn, NT, smem, n_items, &grid, &chunk);
-  if (GMEM && (size_t)grid * slot * sizeof(T) > a.scratch_bytes) {
-    const size_t most = a.scratch_bytes / (slot * sizeof(T));
-    if (most < 1) return -1;
-    chunk = (int)((n_items + most - 1) / most);
-    grid = (n_items + chunk - 1) / chunk;
-  }
-  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
-                            (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
-                            a.sv_stride, a.pair, (T*)a.scratch, slot);
+  const size_t most = GMEM ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
+  if (most < 1) return n_items == 0 ? 0 : -1;
+  persistent_grid(fn, NT, smem, n_items, most, F64, &grid, &chunk);
+  if constexpr (F64)
+    fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items,
+                              (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
+                              a.sv_stride, a.pair, (T*)a.scratch, slot);
+  else
+    fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, chunk,
+                              (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
+                              a.sv_stride, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
