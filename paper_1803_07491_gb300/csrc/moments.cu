@@ -650,36 +650,6 @@ k_moments(ClusterView cv, const float* __restrict__ H, int HS, const float* __re
 // them.
 constexpr int F64_THREADS = 256;      // forward
 constexpr int F64_REV_THREADS = 128;  // reverse (twice the registers per lane)
-// (row entries of one lane in flight: two)
-
-// Sums of NV values over the warp with 10 instead of 5 NV additions at NV =
-// 10: every exchange halves the values a lane keeps.  Returns the sum of
-// value *which (-1: none); lanes may hold the same one.
-template <int NV>
-__device__ __forceinline__ double warp_sums(double (&v)[NV], int lane, int* which) {
-  int n = NV, base = 0, held = NV;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const bool up = (lane & o) != 0;
-    if (n > 1) {
-      const int h = (n + 1) / 2;
-#pragma unroll
-      for (int i = 0; i < NV; i++) {
-        if (i < h) {
-          const double a = v[i], b = i + h < n ? v[i + h < NV ? i + h : 0] : 0.0;
-          v[i] = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, o);
-        }
-      }
-      if (up) base += h;
-      held = up ? held - h : min(held, h);
-      n = h;
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-    }
-  }
-  *which = held > 0 ? base : -1;
-  return v[0];
-}
 
 // Row r of NO x NO blocks: acc[c] += sum over the entries of sum_g B[r][g]
 // x[s][g][c], with the block rows of two entries in flight.  u: positions of
@@ -732,7 +702,7 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
             int n_mom, FwdSmem L, int n_items, double* __restrict__ mu, double* __restrict__ pstore,
             const long long* __restrict__ psi_off, long long psi_tot, bool pair, double* __restrict__ scratch,
             size_t slot_elems) {
-  constexpr int NT = F64_THREADS, NC = NO, RPW = 32 / NO;
+  constexpr int NT = F64_THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<double, N>::PS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -752,10 +722,6 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
   __shared__ int s_next[BOP_MAX_K + 1];  // next sites of a level
   const int K = cv.K;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int sub = lane / NO, r = lane % NO;  // this lane's site of the warp's and its block row
-  int u[NO];
-#pragma unroll
-  for (int g = 0; g < NO; g++) u[g] = UI<NO>(r, g);
   ItemExt nx{};
   if ((int)blockIdx.x < n_items) {
     ext_sites(cv, blockIdx.x % n, nx);
@@ -803,11 +769,15 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
       for (int c = 0; c < 2 * NC; c++) d[c] = 0.0;
       while (true) {
         int first = 0;
-        if (lane == 0) first = atomicAdd(&s_next[k], RPW);
+        if (lane == 0) first = atomicAdd(&s_next[k], 32);
         first = __shfl_sync(0xffffffffu, first, 0);
-        if (first >= nrow) break;
-        const int q = first + sub;
-        if (sub >= RPW || q >= nrow) continue;  // (the shuffle above reconverges the warp)
+        if (first >= nrow * NO) break;
+        // (the lanes of a site need not be in one warp: 32 / NO is no whole number)
+        const int q = (first + lane) / NO, r = (first + lane) % NO;
+        if (q >= nrow) continue;  // (the shuffle above reconverges the warp)
+        int u[NO];
+#pragma unroll
+        for (int g = 0; g < NO; g++) u[g] = UI<NO>(r, g);
         // rows up to level k-2 are full, shell k-1 has entries up to its own
         // level, shell k of the one below
         const int t = half ? (int)(top[q] & 0xffffu)

@@ -182,3 +182,38 @@ def test_response_solve_over_stored_rows(bop, scf, cells, rtol):
         out.append(F.cpu().numpy())
         ctx.close()
     assert np.max(np.abs(out[0] - out[1])) < 1e-8 * max(1.0, np.abs(out[1]).max())
+
+
+@pytest.mark.parametrize("model,n_mom,scf", [("s", 3, "none"), ("s", 17, "none"), ("d", 3, "none"), ("d", 7, "lcn"), ("d", 11, "none"),
+                                             ("d", 17, "none"), ("sd", 5, "lcn"), ("sd", 13, "none")])
+def test_fp64_sweeps_on_a_slab(bop, ob, model, n_mom, scf):
+    """FP64 moments against the oracle, and the forces of the sweeps over the
+    stored Psi against the recomputing ones, on 31 atoms with two free
+    surfaces and a vacancy: rows of 4 to 14 entries, levels of one site and of
+    several hundred, orbitals that do not divide a warp.  Both sides sum at
+    most 14 products per row and level, so the moments agree to 1e-12 of
+    their size and the forces to 1e-10."""
+    M = {"s": I.MODEL_S, "d": I.MODEL_D, "sd": I.MODEL_SD}[model]
+    pos, cell, _ = I.slab_with_vacancies(2, 2, 4, 1, 0.08, 71)
+    run = I.RunParams(n_e={1: 0.7, 5: 6.8, 6: 8.0}[M.norb], n_mom=n_mom)
+    w = I.Workload("slab", pos, cell, (1, 1, 0), M, run)
+    if scf == "lcn":
+        w = I.with_run(w, scf="lcn", scf_tol=1e-10)
+    out = []
+    for budget in (-1, 0):
+        ctx = bop.Context(w.model, w.run, "fp64")
+        bop.bop_set_store_budget(ctx.h, budget)
+        res = ctx.evaluate(w.pos, w.cell, w.pbc)
+        orb = bop.bop_get_orbital_state(ctx.h, w.n_atoms * M.norb, n_mom)
+        out.append((res.forces.cpu().numpy(), res.virial.cpu().numpy()))
+        ctx.close()
+    for a, b in zip(*out):
+        assert np.max(np.abs(a - b)) < 1e-10 * max(1.0, np.abs(b).max())
+    om = oracle_model(M)
+    nbr = ob.neighbors(w.pos, w.cell, w.pbc, om.rc)
+    H = ob.blocks(om, w.pos, w.cell, nbr)
+    onsite = orb["onsite"].cpu().numpy().reshape(w.n_atoms, M.norb)
+    ref = ob.moments(nbr, H, onsite, n_mom)
+    mu = orb["mu"].cpu().numpy().reshape(ref.shape)
+    size = np.sqrt(np.abs(ref[:, :, 2:3])) ** np.arange(n_mom)
+    assert np.max(np.abs(mu - ref) / np.maximum(np.abs(ref), size)) < 1e-12
