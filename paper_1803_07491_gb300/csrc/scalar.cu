@@ -227,14 +227,23 @@ __global__ void __launch_bounds__(RT) k_scf_residual(ScfArgs A) {
   // tree per quantity, then one thread per quantity over the warps in order)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int q = 0; q < nv; q++) {
+  for (int q = 0; q < 2; q++) {
     double v = acc[q];
-    for (int o = 16; o > 0; o >>= 1) {
-      const double w = __shfl_xor_sync(0xffffffffu, v, o);
-      v = q < 2 ? fmax(v, w) : v + w;
-    }
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     if (lane == 0) sh[q][wid] = v;
   }
+  auto sums = [&](auto first, auto count) {  // of acc[first .. first + count)
+    constexpr int F = decltype(first)::value, C = decltype(count)::value;
+    double v[C];
+#pragma unroll
+    for (int q = 0; q < C; q++) v[q] = acc[F + q];
+    int which;
+    const double a = warp_sums<C>(v, lane, &which);
+    if (which >= 0) sh[F + which][wid] = a;
+  };
+  constexpr int C1 = nv - 2 < 32 ? nv - 2 : 32, C2 = nv - 2 - C1;
+  sums(std::integral_constant<int, 2>{}, std::integral_constant<int, C1>{});
+  if constexpr (C2 > 0) sums(std::integral_constant<int, 2 + C1>{}, std::integral_constant<int, C2>{});
   __syncthreads();
   if (threadIdx.x < nv) {
     const int q = threadIdx.x;
@@ -258,81 +267,74 @@ __global__ void __launch_bounds__(RT) k_scf_residual(ScfArgs A) {
     tot_s[q] = v;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
+  if (threadIdx.x >= 32) return;
   const bool conv = tot_s[0] < A.tol && (A.mode != 2 || tot_s[1] < 10.0 * A.tol);
-  A.result[0] = tot_s[0];
-  A.result[1] = tot_s[1];
-  A.result[2] = conv ? 1.0 : 0.0;
-  if (A.mixer == 0 || h == 0) {
-    A.result[3] = tot_s[2] / A.n;  // mean of delta_new (linear) or of x + F (no history yet)
-  } else {
-    // normal equations of the least-squares problem, Gaussian elimination
-    // with partial pivoting (row exchanges as predicated swaps of fixed rows)
-    double G[h > 0 ? h : 1][h + 1];
-    double dmax = 0.0;
-#pragma unroll
-    for (int j = 0; j < h; j++)
-#pragma unroll
-      for (int l = j; l < h; l++) {
-        const double g = tot_s[3 + j * h - j * (j - 1) / 2 + (l - j)];
-        G[j][l] = g;
-        G[l][j] = g;
-        if (j == l) dmax = fmax(dmax, g);
-      }
+  double mean = tot_s[2];  // of delta_new (linear) or of x + F (no history yet)
+  if (A.mixer != 0 && h > 0) {
+    // normal equations of the least-squares problem, Gaussian elimination with
+    // partial pivoting, lane r holding row r (by one thread it was 560
+    // double-precision instructions of 64 cycles; rows side by side take 190)
+    const int r = lane < h ? lane : 0;
+    double R[h + 1], dmax = 0.0;
 #pragma unroll
     for (int j = 0; j < h; j++) {
-      G[j][h] = tot_s[3 + nA + j];
-      G[j][j] += 1e-12 * dmax + 1e-300;
+      const int a = r < j ? r : j, b = r < j ? j : r;
+      R[j] = tot_s[3 + a * h - a * (a - 1) / 2 + (b - a)];
+      dmax = fmax(dmax, tot_s[3 + j * h - j * (j - 1) / 2]);
     }
+    R[h] = tot_s[3 + nA + r];
+#pragma unroll
+    for (int j = 0; j < h; j++)
+      if (r == j) R[j] += 1e-12 * dmax + 1e-300;
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < h; c++) {
       int pr = c;
-      double best = fabs(G[c][c]);
+      double best = fabs(__shfl_sync(0xffffffffu, R[c], c));
 #pragma unroll
-      for (int r = c + 1; r < h; r++)
-        if (fabs(G[r][c]) > best) {
-          best = fabs(G[r][c]);
-          pr = r;
+      for (int q = c + 1; q < h; q++) {
+        const double v = fabs(__shfl_sync(0xffffffffu, R[c], q));
+        if (v > best) {
+          best = v;
+          pr = q;
         }
+      }
       if (!(best > 0.0)) ok = false;
+      const int src = lane == c ? pr : (lane == pr ? c : lane);
 #pragma unroll
-      for (int r = c + 1; r < h; r++)
-        if (r == pr)
-#pragma unroll
-          for (int k = 0; k <= h; k++) {
-            const double t = G[c][k];
-            G[c][k] = G[r][k];
-            G[r][k] = t;
-          }
+      for (int k = 0; k <= h; k++) R[k] = __shfl_sync(0xffffffffu, R[k], src);
       if (ok) {
+        const double f = R[c] / __shfl_sync(0xffffffffu, R[c], c);
 #pragma unroll
-        for (int r = c + 1; r < h; r++) {
-          const double f = G[r][c] / G[c][c];
-#pragma unroll
-          for (int k = c; k <= h; k++) G[r][k] -= f * G[c][k];
+        for (int k = c; k <= h; k++) {
+          const double p = __shfl_sync(0xffffffffu, R[k], c);
+          if (lane > c) R[k] -= f * p;
         }
       }
     }
     double gam[h > 0 ? h : 1];
 #pragma unroll
     for (int j = h - 1; j >= 0; j--) {
-      double v = ok ? G[j][h] : 0.0;
+      double v = ok ? R[h] : 0.0;
       if (ok) {
 #pragma unroll
-        for (int k = j + 1; k < h; k++) v -= G[j][k] * gam[k];
-        v /= G[j][j];
+        for (int k = j + 1; k < h; k++) v -= R[k] * gam[k];
+        v /= R[j];
       }
+      v = __shfl_sync(0xffffffffu, v, j);
       gam[j] = isfinite(v) ? v : 0.0;
     }
-    double mean = tot_s[2];
 #pragma unroll
     for (int j = 0; j < h; j++) {
-      A.gamma[j] = gam[j];
+      if (lane == 0) A.gamma[j] = gam[j];
       mean -= gam[j] * tot_s[3 + nA + h + j];
     }
-    A.result[3] = mean / A.n;  // mean of the updated delta before the gauge shift
   }
+  if (lane != 0) return;
+  A.result[0] = tot_s[0];
+  A.result[1] = tot_s[1];
+  A.result[2] = conv ? 1.0 : 0.0;
+  A.result[3] = mean / A.n;  // mean of the updated delta before the gauge shift
   *A.counter = 0;
 }
 
