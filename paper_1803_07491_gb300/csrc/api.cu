@@ -219,41 +219,60 @@ double fermi_tol(const bop_ctx* c) {
   return std::fmax(t, FERMI_TOL);
 }
 
+constexpr int GRID_FAIL = 6;  // word of cw_misc (the maxima are words 0 to 4): the grid builder's failure flag
 constexpr size_t PIN_BYTES = 16384;
 
 // The small device-to-host reads of one synchronisation point: each lands in
-// the context's pinned staging area (an asynchronous copy, where a copy into
-// pageable memory synchronises the stream by itself), and all of them are
+// the context's pinned staging area (a copy into pageable memory would
+// synchronise the stream by itself), and all of them are
 // copied to their destinations once the stream has synchronised.  A read
 // that does not fit goes straight to its destination.
+// All staged reads go in one launch, a single one as a copy.
 struct Readback {
   bop_ctx* c;
   cudaStream_t s;
   int n = 0;
+  bool sent = true;  // the staged reads are on their way
   size_t used = 0;
-  void* dst[16];
-  size_t off[16], len[16];
+  void* dst[COLLECT_MAX];
+  const void* src[COLLECT_MAX];
+  size_t off[COLLECT_MAX], len[COLLECT_MAX];
   Readback(bop_ctx* c_, cudaStream_t s_) : c(c_), s(s_) {}
-  // an error return between add and sync: the staged copies land before the
+  // an error return between send and sync: the staged copies land before the
   // staging area is used again
   ~Readback() {
-    if (n > 0) cudaStreamSynchronize(s);
+    if (n > 0 && sent) cudaStreamSynchronize(s);
   }
   int add(void* h, const void* d, size_t bytes) {
     const size_t at = (used + 15) & ~(size_t)15;
-    if (c->pin == nullptr || n == 16 || at + bytes > PIN_BYTES) {
+    if (c->pin == nullptr || n == COLLECT_MAX || at + bytes > PIN_BYTES || bytes % 4 != 0) {
       CK(cudaMemcpyAsync(h, d, bytes, cudaMemcpyDeviceToHost, s));
       return BOP_OK;
     }
-    CK(cudaMemcpyAsync(static_cast<char*>(c->pin) + at, d, bytes, cudaMemcpyDeviceToHost, s));
+    sent = false;
+    src[n] = d;
     dst[n] = h;
     off[n] = at;
     len[n++] = bytes;
     used = at + bytes;
     return BOP_OK;
   }
-  // synchronises s and copies the staged reads out
+  // sends the staged reads, synchronises s and copies them out
   int sync() {
+    if (n == 1) {
+      CK(cudaMemcpyAsync(static_cast<char*>(c->pin) + off[0], src[0], len[0], cudaMemcpyDeviceToHost, s));
+    } else if (n > 1) {
+      CollectArgs a;
+      a.n = n;
+      a.dst = static_cast<unsigned*>(c->pin);
+      for (int q = 0; q < n; q++) {
+        a.src[q] = static_cast<const unsigned*>(src[q]);
+        a.at[q] = (int)(off[q] / 4);
+        a.words[q] = (int)(len[q] / 4);
+      }
+      if (launch_collect(a, s)) return fail(c, BOP_ERR_CUDA, "readback launch: %s", cudaGetErrorString(cudaPeekAtLastError()));
+    }
+    sent = true;
     CK(cudaStreamSynchronize(s));
     for (int q = 0; q < n; q++) memcpy(dst[q], static_cast<char*>(c->pin) + off[q], len[q]);
     n = 0;
@@ -291,6 +310,10 @@ int check_status(bop_ctx* c, cudaStream_t s) {
 // summed into 64-bit offsets must not wrap at 2^31).
 template <class Tin, class Tout>
 int exclusive_scan(bop_ctx* c, const Tin* in, Tout* out, long long n, cudaStream_t s) {
+  if (n <= SCAN_SMALL) {  // one launch instead of two
+    if (launch_scan_small<Tin, Tout>(in, out, nullptr, nullptr, (int)n, s)) return fail(c, BOP_ERR_CUDA, "scan launch failed");
+    return BOP_OK;
+  }
   size_t tmp = 0;
   CK(cub::DeviceScan::ExclusiveScan(nullptr, tmp, in, out, cuda::std::plus<Tout>{}, Tout(0), (int)n, s));
   CKS(ensure(c, c->cub_tmp, tmp));
@@ -390,6 +413,19 @@ int geometry(bop_ctx* c, const double* cell, const int* pbc, Geometry* g) {
   return BOP_OK;
 }
 
+// The offsets of the sites and of the adjacency entries from every atom's counts.
+int scan_cluster_sizes(bop_ctx* c, int n, cudaStream_t s) {
+  if (n + 1 <= SCAN_SMALL) {
+    if (launch_scan_small<int, long long>(P<int>(c->atom_nsite), P<long long>(c->site_off), P<int>(c->atom_nadj),
+                                          P<long long>(c->adj_base), n + 1, s))
+      return fail(c, BOP_ERR_CUDA, "scan launch failed");
+    return BOP_OK;
+  }
+  CKS(exclusive_scan(c, P<int>(c->atom_nsite), P<long long>(c->site_off), n + 1, s));
+  CKS(exclusive_scan(c, P<int>(c->atom_nadj), P<long long>(c->adj_base), n + 1, s));
+  return BOP_OK;
+}
+
 // Grid builder (rows of at most 32 neighbours, a table that fits shared
 // memory); *done = false when it does not apply, and the block builder below
 // runs instead.  Capacities by tier: a cluster that outgrows one tier sends
@@ -401,9 +437,6 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
   GridPlan plan;
   if (n == 0 || c->n >= (1 << 24) || c->grid_max[0] > 32 || !grid_plan(c->g, K, c->grid_max, &plan)) return BOP_OK;
   CKS(ensure(c, c->level_end, sizeof(int) * (size_t)n * (K + 1)));
-  CKS(ensure(c, c->atom_nsite, sizeof(int) * (n + 1)));
-  CKS(ensure(c, c->atom_nadj, sizeof(int) * (n + 1)));
-  CKS(ensure(c, c->max_level, sizeof(int) * (K + 2)));
   CKS(ensure(c, c->site_off, sizeof(long long) * (n + 1)));
   CKS(ensure(c, c->adj_base, sizeof(long long) * (n + 1)));
   CKS(ensure(c, c->cw_epack, sizeof(int2) * (size_t)(c->E > 0 ? c->E : 1)));
@@ -418,11 +451,15 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
   for (int q = 0; q < 9; q++) pc.cell[q] = c->g.cell[q];
   pc.r2 = c->m.r_path > 0 ? c->m.r_path * c->m.r_path : 0.0;
   const int first = c->m.r_path > 0 || K <= 4 ? 0 : (K <= 6 ? 1 : 2);
+  bool clean = true;  // zeroed by the structure build
   for (int tier = c->cw_tier > first ? c->cw_tier : first; tier < 4; tier++) {
-    CK(cudaMemsetAsync(c->atom_nsite.p, 0, sizeof(int) * (n + 1), s));
-    CK(cudaMemsetAsync(c->atom_nadj.p, 0, sizeof(int) * (n + 1), s));
-    CK(cudaMemsetAsync(c->max_level.p, 0, sizeof(int) * (K + 2), s));
-    CK(cudaMemsetAsync(c->cw_misc.p, 0, sizeof(int), s));
+    if (!clean) {  // a tier that failed left its counts
+      CK(cudaMemsetAsync(c->atom_nsite.p, 0, sizeof(int) * (n + 1), s));
+      CK(cudaMemsetAsync(c->atom_nadj.p, 0, sizeof(int) * (n + 1), s));
+      CK(cudaMemsetAsync(c->max_level.p, 0, sizeof(int) * (K + 2), s));
+      CK(cudaMemsetAsync(P<int>(c->cw_misc) + GRID_FAIL, 0, sizeof(int), s));
+    }
+    clean = false;
     GridArgs a;
     a.n = n;
     a.K = K;
@@ -447,7 +484,7 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     a.slot = P<int>(c->cell_slot);
     a.recs = P<unsigned long long>(c->cw_keys);
     a.counts = P<unsigned char>(c->cw_cnt);
-    a.fail = P<int>(c->cw_misc);
+    a.fail = P<int>(c->cw_misc) + GRID_FAIL;
     a.status = P<unsigned>(c->status);
     ClusterOut out{};
     out.level_end = P<int>(c->level_end);
@@ -462,8 +499,7 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     }
     // the sizes and the flag of pass 0 in one synchronisation (the scans run
     // before it is known whether pass 0 succeeded; they are discarded if not)
-    CKS(exclusive_scan(c, P<int>(c->atom_nsite), P<long long>(c->site_off), n + 1, s));
-    CKS(exclusive_scan(c, P<int>(c->atom_nadj), P<long long>(c->adj_base), n + 1, s));
+    CKS(scan_cluster_sizes(c, n, s));
     long long tot[2];
     int failed = 0;
     {
@@ -471,7 +507,7 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
       CKS(rb.add(&tot[0], P<long long>(c->site_off) + n, sizeof(long long)));
       CKS(rb.add(&tot[1], P<long long>(c->adj_base) + n, sizeof(long long)));
       CKS(rb.add(c->maxlev, c->max_level.p, sizeof(int) * (K + 2)));
-      CKS(rb.add(&failed, c->cw_misc.p, sizeof(int)));
+      CKS(rb.add(&failed, P<int>(c->cw_misc) + GRID_FAIL, sizeof(int)));
       CKS(rb.finish());  // synchronises
     }
     if (failed) continue;
@@ -494,8 +530,6 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     out.adj_off = P<long long>(c->adj_off);
     out.adj = P<int2>(c->adj);
     out.lvcnt = P<unsigned long long>(c->lvcnt);
-    CKS(ensure(c, c->nprod, sizeof(unsigned long long)));
-    CK(cudaMemsetAsync(c->nprod.p, 0, sizeof(unsigned long long), s));
     out.n_products = P<unsigned long long>(c->nprod);
     a.sites = c->maxlev[K];
     // every atom a centre and no path cut: H^K between cluster atoms is
@@ -582,8 +616,7 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
     CKS(check_status(c, s));
     c->cl_maxs = maxs;
     // offsets
-    CKS(exclusive_scan(c, P<int>(c->atom_nsite), P<long long>(c->site_off), n + 1, s));
-    CKS(exclusive_scan(c, P<int>(c->atom_nadj), P<long long>(c->adj_base), n + 1, s));
+    CKS(scan_cluster_sizes(c, n, s));
     long long tot[2];
     {
       Readback rb(c, s);
@@ -1543,17 +1576,36 @@ int bop_build_hamiltonian(bop_ctx* c, int n, const double* pos, const double* ce
   CKS(ensure(c, c->deg, sizeof(int) * (n + 1)));
   CKS(ensure(c, c->row_ptr, sizeof(long long) * (n + 1)));
   CKS(ensure(c, c->frac, sizeof(double) * 6 * 64));
+  CKS(ensure(c, c->cw_misc, 8 * sizeof(int)));
+  CKS(ensure(c, c->atom_nsite, sizeof(int) * (c->nc + 1)));
+  CKS(ensure(c, c->atom_nadj, sizeof(int) * (c->nc + 1)));
+  CKS(ensure(c, c->max_level, sizeof(int) * (c->K + 2)));
+  CKS(ensure(c, c->nprod, sizeof(unsigned long long)));
+  CKS(ensure(c, c->lsum, sizeof(long long) * (c->nc + 1)));
   const int TB = 256, gb = (n + TB - 1) / TB;
   {
   Region Rn(c, PK_NBR, 5, s);
+  // every counter of the build in one launch (ten memsets of 2 us otherwise)
+  ZeroArgs z{};
+  auto zero = [&](DBuf& b, size_t bytes) {
+    z.p[z.n] = P<unsigned>(b);
+    z.words[z.n++] = (long long)(bytes / 4);
+  };
+  zero(c->cell_count, sizeof(int) * (ncell + 1));
+  zero(c->cell_fill, sizeof(int) * ncell);
+  zero(c->deg, sizeof(int) * (n + 1));
+  zero(c->cw_misc, sizeof(int) * 8);
+  zero(c->atom_nsite, sizeof(int) * (c->nc + 1));
+  zero(c->atom_nadj, sizeof(int) * (c->nc + 1));
+  zero(c->max_level, sizeof(int) * (c->K + 2));
+  zero(c->nprod, sizeof(unsigned long long));
+  zero(c->lsum, sizeof(long long) * (c->nc + 1));
+  if (launch_zero(z, s)) return fail(c, BOP_ERR_CUDA, "zeroing launch failed");
   bopk::k_frac_range<<<64, 256, 0, s>>>(n, P<double>(c->pos), g, P<double>(c->frac));
-  CK(cudaMemsetAsync(c->cell_count.p, 0, sizeof(int) * (ncell + 1), s));
-  CK(cudaMemsetAsync(c->cell_fill.p, 0, sizeof(int) * ncell, s));
   bopk::k_bin_atoms<<<gb, TB, 0, s>>>(n, P<double>(c->pos), g, P<int>(c->cell_of), P<int>(c->cell_count));
   CKS(exclusive_scan(c, P<int>(c->cell_count), P<int>(c->cell_start), ncell + 1, s));
   bopk::k_fill_cells<<<gb, TB, 0, s>>>(n, P<int>(c->cell_of), P<int>(c->cell_start), P<int>(c->cell_fill),
                                        P<int>(c->cell_atoms), P<int>(c->cell_slot));
-  CK(cudaMemsetAsync(c->deg.p, 0, sizeof(int) * (n + 1), s));
   launch_neighbors(0, n, P<double>(c->pos), g, P<int>(c->cell_of), P<int>(c->cell_start), P<int>(c->cell_atoms),
                    P<int>(c->deg), nullptr, nullptr, nullptr, P<unsigned>(c->status), s);
   CK(cudaGetLastError());
@@ -1612,8 +1664,6 @@ int bop_build_hamiltonian(bop_ctx* c, int n, const double* pos, const double* ce
   CK(cudaGetLastError());
   // the maxima that the cluster builder is planned with, read back with the
   // neighbour list's status
-  CKS(ensure(c, c->cw_misc, 8 * sizeof(int)));
-  CK(cudaMemsetAsync(c->cw_misc.p, 0, 8 * sizeof(int), s));
   launch_grid_maxima(n, P<long long>(c->row_ptr), ncell, P<int>(c->cell_start), nb, P<double>(c->bond_d), g,
                      P<int>(c->cw_misc), s);
   {
@@ -1625,9 +1675,7 @@ int bop_build_hamiltonian(bop_ctx* c, int n, const double* pos, const double* ce
   CKS(size_state(c));
   // per-atom row offsets of a stored Psi sweep
   const int nc = c->nc;
-  CKS(ensure(c, c->lsum, sizeof(long long) * (nc + 1)));
   CKS(ensure(c, c->psi_off, sizeof(long long) * (nc + 1)));
-  CK(cudaMemsetAsync(c->lsum.p, 0, sizeof(long long) * (nc + 1), s));
   launch_level_sums(nc, c->K, P<int>(c->level_end), P<long long>(c->lsum), s);
   CKS(exclusive_scan(c, P<long long>(c->lsum), P<long long>(c->psi_off), nc + 1, s));
   unsigned long long np = 0;

@@ -447,3 +447,30 @@ int launch_rep_energy(int n, BondModel m, const long long* row_ptr, const int* b
                       double* erep, cudaStream_t s);
 int launch_forces(int nb, BondModel m, const double* bond_d, const int* bond_atoms, const void* Hbar, int HSh, int fp64,
                   double* forces, double* virial, cudaStream_t s);
+
+// batch.cu
+// Up to ZERO_MAX arrays of 4-byte words set to zero in one launch (blocks is
+// filled in by the launcher).
+constexpr int ZERO_MAX = 10, ZERO_WORDS = 4096;
+struct ZeroArgs {
+  int n;
+  unsigned* p[ZERO_MAX];
+  long long words[ZERO_MAX];
+  int blocks[ZERO_MAX];
+};
+int launch_zero(ZeroArgs z, cudaStream_t s);
+// Up to COLLECT_MAX pieces of 4-byte words copied to dst + at[q] (pinned host
+// memory).
+constexpr int COLLECT_MAX = 16;
+struct CollectArgs {
+  int n;
+  const unsigned* src[COLLECT_MAX];
+  int at[COLLECT_MAX], words[COLLECT_MAX];
+  unsigned* dst;
+};
+int launch_collect(const CollectArgs& a, cudaStream_t s);
+// Exclusive prefix sums of n <= SCAN_SMALL elements, of a second array too
+// where in1 is not NULL.
+constexpr int SCAN_SMALL = 8192;
+template <class Tin, class Tout>
+int launch_scan_small(const Tin* in0, Tout* out0, const Tin* in1, Tout* out1, int n, cudaStream_t s);

@@ -184,7 +184,7 @@ def test_response_solve_over_stored_rows(bop, scf, cells, rtol):
     assert np.max(np.abs(out[0] - out[1])) < 1e-8 * max(1.0, np.abs(out[1]).max())
 
 
-@pytest.mark.parametrize("model,n_mom,scf", [("s", 3, "none"), ("s", 17, "none"), ("d", 3, "none"), ("d", 7, "lcn"), ("d", 11, "none"),
+@pytest.mark.parametrize("model,n_mom,scf", [("s", 3, "none"), ("s", 17, "none"), ("d", 3, "none"), ("d", 5, "none"), ("d", 9, "lcn"), ("d", 11, "none"),
                                              ("d", 17, "none"), ("sd", 5, "lcn"), ("sd", 13, "none")])
 def test_fp64_sweeps_on_a_slab(bop, ob, model, n_mom, scf):
     """FP64 moments against the oracle, and the forces of the sweeps over the
