@@ -285,8 +285,11 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
     Nbar[q] = cN[q] - cU[q] * (E - ai);
     Pbar[q] = cU[q] * bi;
   }
-  // (dP/deps needs no sum of its own: sin((m+2) phi) + sin(m phi) = 2 x sin((m+1) phi))
-  double Nv = 0.0, Pv = 0.0, dN = 0.0;
+  // (in FP64 dP/deps needs no sum of its own: sin((m+2) phi) + sin(m phi) = 2 x
+  // sin((m+1) phi).  In FP32 it keeps one: recursions near a truncation amplify
+  // its rounding by 1e3 and more, and there the two forms differ as much as
+  // either does from the 64-bit value.)
+  double Nv = 0.0, Pv = 0.0, dN = 0.0, dP = 0.0;
   if (f32) {
     // the same sums in FP32 (sigma_m and its cotangent in FP32 scratch): the
     // sines s_j = sin(j phi) = sinpi(j phi/pi) directly (no recurrence, so no
@@ -309,7 +312,7 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
     };
     float s0 = 0.f, sp1 = sinpif(theta), sp2 = sinpif(2.f * theta), sp3 = sinpif(3.f * theta);
     float c_m = 0.f, c_m1 = chi(1, s0, sp2);
-    float Nf = 0.f, Pf = 0.f, dNf = 0.f;
+    float Nf = 0.f, Pf = 0.f, dNf = 0.f, dPf = 0.f;
     for (int m = 0; m <= ne; m++) {
       const float c_m2 = chi(m + 2, sp1, sp3);
       const float gm = g32[m];
@@ -317,6 +320,7 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
       Nf += gsm * c_m1;
       Pf += gsm * (c_m2 + c_m);
       dNf += gsm * sp1;
+      dPf += gsm * (sp2 + s0);
 #pragma unroll
       for (int q = 0; q < NS; q++) zbf[q][(size_t)m * M + o] = gm * (Nbf[q] * c_m1 + Pbf[q] * (c_m2 + c_m));
       c_m = c_m1;
@@ -329,6 +333,7 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
     Nv = Nf;
     Pv = Pf;
     dN = dNf * (2.0 / PI);
+    dP = dPf * (2.0 / PI);
   } else {
     // sines s_j = sin(j phi) by the recurrence; chi_j = (s~_{j+1} - s~_{j-1})/pi,
     // s~_k = sin(k phi)/k, s~_0 = phi - pi
@@ -358,8 +363,8 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
       sp3 = 2.0 * x * sp2 - sp1;
     }
     dN *= 2.0 / PI;
+    dP = 2.0 * x * dN;
   }
-  const double dP = 2.0 * x * dN;
 #pragma unroll
   for (int q = 0; q < NS; q++) {
     abar_inf[q] += cU[q] * Nv;
