@@ -8,15 +8,15 @@
 //
 // Forward: one CTA per (spin, atom).  Psi_{k-1} and Psi_k live in shared
 // memory (ping-pong) or global scratch; the last level Psi_K is only stored for
-// a reverse sweep.  Each thread owns one cluster site per pass and gathers
+// a reverse sweep.  FP32: a thread per cluster site and pass, which gathers
 // the 5x5 blocks of its bonds (15 unique elements, 16-element records) from
-// L2 (for sd blocks 21 unique elements in 24-element records).  Products in
-// T (float or double), moments written as double.
+// L2 (for sd blocks 21 unique elements in 24-element records).  FP64: a thread
+// per row of a site's block.  Moments written as double.
 //
-// Adjoint: one CTA per work item as well, Psi_0..Psi_K and the cotangents
-// Psi-bar_1..Psi-bar_K kept in the CTA's slot of global scratch; the bond
-// cotangents are summed over levels per cluster edge and added to the
-// bond's unique elements with FP64 atomics.
+// Reverse: over the stored Psi, one CTA per work item with Psi-bar of two
+// levels at a time; where the store does not fit, Psi_0..Psi_K and the
+// cotangents Psi-bar_1..Psi-bar_K are recomputed in the CTA's slot of global
+// scratch and the bond cotangents summed over levels per cluster edge.
 #include "kernels.h"
 
 namespace {
