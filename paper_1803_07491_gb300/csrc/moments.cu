@@ -2229,12 +2229,21 @@ __global__ void k_torques(int n, int norb, int n_mom, const double* __restrict__
   t[3 * (size_t)i + 2] = g[0] * sy - g[1] * sx;
 }
 
-// CTAs of a persistent kernel, at most `most`.
+// Allows fn every size of dynamic shared memory that the launches below ask
+// for.  The 48 KB that need no permission cover the static arrays too, so a
+// size a little below them is refused like a larger one; and the limit does
+// not depend on the size, which another thread's launch may not share.
+constexpr size_t SMEM_MAX = 225 * 1024;
+template <class F>
+bool allow_smem(F fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX) == cudaSuccess;
+}
+
+// CTAs of a persistent kernel, at most `most`; 0: not one fits an SM.
 template <class F>
 int persistent_grid(F fn, int threads, size_t smem, int n_items, size_t most) {
-  int per_sm = 1, sms = 0, dev = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-  if (per_sm < 1) per_sm = 1;
+  int per_sm = 0, sms = 0, dev = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) return 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int slots = sms * per_sm;
@@ -2255,11 +2264,10 @@ int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
   }
   if (smem > 225 * 1024) return -2;
   auto fn = k_nc_fwd<T, NO>;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return -1;
+  if (!allow_smem(fn)) return -1;
   const int n_items = a.n * NO;
   const int grid = persistent_grid(fn, NT, smem, n_items, n_items);
+  if (grid < 1) return -1;
   fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, a.mu, a.vmom, (T*)a.pstore, a.psi_off, a.psi_tot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -2280,6 +2288,7 @@ int run_nc_rev(const NcArgs& a, cudaStream_t s) {
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
   const int n_items = a.n * NO;
   const int grid = persistent_grid(fn, 128, smem, n_items, n_items);
+  if (grid < 1) return -1;
   fn<<<grid, 128, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.obar);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -2316,15 +2325,14 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
     if constexpr (F64) return k_moments64<NO, GMEM>;
     else return k_moments<NO, GMEM>;
   }();
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return -1;
+  if (!allow_smem(fn)) return -1;
   const int n_items = a.n * a.n_spin;
   const size_t slot = (size_t)(a.cap_even + a.cap_odd) * PS;
   // with Psi in global scratch no more CTAs than its slots
   const size_t most = GMEM && a.pstore == nullptr ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
   if (most < 1) return n_items == 0 ? 0 : -1;
   const int grid = persistent_grid(fn, NT, smem, n_items, most);
+  if (grid < 1) return -1;
   if (F64 && a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
     return -1;
   if constexpr (F64)
@@ -2379,6 +2387,7 @@ int run_reverse(const AdjointArgs& a, cudaStream_t s) {
   const size_t most = GMEM ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
   if (most < 1) return n_items == 0 ? 0 : -1;
   const int grid = persistent_grid(fn, NT, smem, n_items, most);
+  if (grid < 1) return -1;
   if constexpr (F64)
     fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items,
                               (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
