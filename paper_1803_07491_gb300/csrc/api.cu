@@ -2195,6 +2195,7 @@ int bop_set_store_budget(bop_ctx* c, long long bytes) {
         b->p = nullptr;
         b->bytes = 0;
       }
+    c->psi_valid = false;  // between energy and forces: the reverse sweep recomputes Psi
   }
   return BOP_OK;
 }

@@ -2274,6 +2274,7 @@ int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
 
 template <typename T, int NO>
 int run_nc_rev(const NcArgs& a, cudaStream_t s) {
+  if (a.pstore == nullptr) return -1;
   RevSmem L{a.rev_even, a.rev_odd, a.max_sites, a.rev_adj, a.cap_eb, true};
   const size_t psi = ((size_t)(a.rev_even + a.rev_odd) * NO * NCS + (size_t)a.cap_eb * NO * 4) * sizeof(T) + 16;
   size_t smem = psi + (size_t)a.rev_adj * 8 + (size_t)a.cap_eb * 8 + (size_t)(a.cap_eb + 1) * 4 +

@@ -1,0 +1,75 @@
+"""The Psi store's routes: forces, virial and torques of a reverse sweep
+without a store (the budget forbids it, or it is released between the energy
+and the forces) against those of the stored sweep.  Both evaluate the same
+sums in another order: FP64 to 1e-9 of the largest value, FP32 products to
+twice the 1e-3 that the FP32 mode keeps to the oracle."""
+import numpy as np
+import pytest
+
+from paper_1803_07491_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MODELS = {"s": I.MODEL_S, "d": I.MODEL_D, "sd": I.MODEL_SD}
+
+
+@pytest.fixture(scope="module")
+def bop():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1803_07491_gb300 import build, bop as b
+    build.build()
+    return b
+
+
+def _forces(bop, w, kw, prec, budget=None, release=False):
+    ctx = bop.Context(w.model, w.run, prec)
+    if budget is not None:
+        bop.bop_set_store_budget(ctx.h, budget)
+    out = []
+    for _ in range(2):  # the second energy stores Psi in its own pass, forces being expected to follow
+        ctx.build(w.pos, w.cell, w.pbc)
+        if "spin_dir" in kw:
+            ctx.set_spin_directions(kw["spin_dir"])
+        m = kw.get("m")
+        ctx.energy(m=None if m is None else torch.as_tensor(m, dtype=torch.float64, device="cuda").clone())
+        if release:
+            bop.bop_set_store_budget(ctx.h, 0)
+        F, W = ctx.forces()
+        out.append([F.cpu().numpy(), W.cpu().numpy()])
+        if "spin_dir" in kw:
+            out[-1].append(ctx.torques().cpu().numpy())
+        if release:
+            bop.bop_set_store_budget(ctx.h, -1)
+    ctx.close()
+    return out
+
+
+def _close(a, b, tol):
+    for x, y in zip(a, b):
+        assert np.max(np.abs(x - y)) <= tol * max(1.0, np.abs(y).max())
+
+
+@pytest.mark.parametrize("model", ["s", "d", "sd"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("how", ["budget", "release"])
+def test_noncollinear_without_a_store(bop, model, prec, how):
+    """Forward pass without a store, reverse sweep with Psi recomputed."""
+    w = I.small_bcc(3, 2, 2, 0.06, 61, model=MODELS[model])
+    w = I.with_run(w, n_spin=2, scf="none", stoner_I=1.5 if model == "s" else 0.8, noncollinear=True)
+    kw = dict(spin_dir=I.random_directions(w.n_atoms, 62),
+              m=np.random.default_rng(63).uniform(0.2, 0.6 if model == "s" else 2.5, w.n_atoms))
+    ref = _forces(bop, w, kw, prec)
+    got = _forces(bop, w, kw, prec, budget=0 if how == "budget" else None, release=how == "release")
+    for r, g in zip(ref, got):
+        _close(g, r, 1e-9 if prec == "fp64" else 2e-3)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_store_released_between_energy_and_forces(bop, prec):
+    w = I.small_bcc(3, 3, 2, 0.06, 64, model=I.MODEL_D)
+    ref = _forces(bop, w, {}, prec)
+    got = _forces(bop, w, {}, prec, release=True)
+    for r, g in zip(ref, got):
+        _close(g, r, 1e-9 if prec == "fp64" else 2e-3)
