@@ -862,7 +862,7 @@ int launch_cluster(int pass, int n, int K, const long long* row_ptr, const int* 
   const bool cut = pc.r2 > 0.0;
   auto fn = pass == 0 ? (cut ? k_cluster<0, true> : k_cluster<0, false>)
                       : (cut ? k_cluster<1, true> : k_cluster<1, false>);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!allow_smem(fn)) return -1;
   fn<<<grid, CL_THREADS, smem, s>>>(n, K, row_ptr, col, img, bond_of_edge, pc, sc, out, status);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -963,8 +963,8 @@ static int run_grid(const GridArgs& a, const PathCut& pc, const ClusterOut& out,
   auto fn = k_cluster_grid<PASS, CUT, G>;
   const size_t smem = grid_front(PASS, a) + 
                       (PASS == 0 ? 16 * (size_t)a.maxs + 12 * (size_t)a.newcap : 16 * (size_t)a.sites);
-  if (smem > 225 * 1024) return -2;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (smem > SMEM_MAX) return -2;
+  if (!allow_smem(fn)) return -1;
   int per = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, G, smem) != cudaSuccess) return -1;
   if (per < 1) return -2;

@@ -6,6 +6,17 @@
 #include "../../include/bopgb.h"
 #include "common.cuh"
 
+// Allows fn every size of dynamic shared memory that a launch here asks for.
+// The 48 KB that need no permission cover the static arrays too, so a size a
+// little below them is refused like a larger one; and the permission does not
+// follow the size of one call, which would take it from another thread's
+// launch of the same kernel.
+constexpr size_t SMEM_MAX = 225 * 1024;
+template <class F>
+bool allow_smem(F fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX) == cudaSuccess;
+}
+
 // Cell, its inverse and the linked-cell grid of one structure.
 struct Geometry {
   double cell[9];  // rows = lattice vectors

@@ -2229,16 +2229,6 @@ __global__ void k_torques(int n, int norb, int n_mom, const double* __restrict__
   t[3 * (size_t)i + 2] = g[0] * sy - g[1] * sx;
 }
 
-// Allows fn every size of dynamic shared memory that the launches below ask
-// for.  The 48 KB that need no permission cover the static arrays too, so a
-// size a little below them is refused like a larger one; and the limit does
-// not depend on the size, which another thread's launch may not share.
-constexpr size_t SMEM_MAX = 225 * 1024;
-template <class F>
-bool allow_smem(F fn) {
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX) == cudaSuccess;
-}
-
 // CTAs of a persistent kernel, at most `most`; 0: not one fits an SM.
 template <class F>
 int persistent_grid(F fn, int threads, size_t smem, int n_items, size_t most) {
@@ -2262,7 +2252,7 @@ int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
     L.stage = false;
     smem = psi;
   }
-  if (smem > 225 * 1024) return -2;
+  if (smem > SMEM_MAX) return -2;
   auto fn = k_nc_fwd<T, NO>;
   if (!allow_smem(fn)) return -1;
   const int n_items = a.n * NO;
@@ -2284,9 +2274,9 @@ int run_nc_rev(const NcArgs& a, cudaStream_t s) {
     L.stage = false;
     smem = psi;
   }
-  if (smem > 225 * 1024) return -2;
+  if (smem > SMEM_MAX) return -2;
   auto fn = k_nc_rev<T, NO>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (!allow_smem(fn)) return -1;
   const int n_items = a.n * NO;
   const int grid = persistent_grid(fn, 128, smem, n_items, n_items);
   if (grid < 1) return -1;
@@ -2371,18 +2361,13 @@ int run_reverse(const AdjointArgs& a, cudaStream_t s) {
   }();
   size_t smem = psi + stage;
   int per_sm = 0, per_sm_unstaged = 0;
-  if (psi > 225 * 1024) return -2;
-  if (smem <= 225 * 1024) {
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem);
-  }
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psi);
+  if (psi > SMEM_MAX) return -2;
+  if (!allow_smem(fn)) return -1;
+  if (smem <= SMEM_MAX) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_unstaged, fn, NT, psi);
   if (per_sm < per_sm_unstaged) {  // staging the adjacency would cost a resident CTA
     L.stage = false;
     smem = psi;
-  } else {
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
   const int n_items = a.n * a.n_spin;
   const size_t most = GMEM ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
@@ -2452,7 +2437,7 @@ bool nc_in_shared(const NcArgs& a, int fp64) {
   const size_t esz = fp64 ? 8 : 4;
   const size_t fwd = (size_t)(a.cap_even + a.cap_odd) * a.norb * NCS * esz;
   const size_t rev = ((size_t)(a.rev_even + a.rev_odd) * a.norb * NCS + (size_t)a.cap_eb * a.norb * 4) * esz + 16;
-  return fwd <= 225 * 1024 && rev <= 225 * 1024;
+  return fwd <= SMEM_MAX && rev <= SMEM_MAX;
 }
 
 int launch_nc(const NcArgs& a, int fp64, cudaStream_t s) {
