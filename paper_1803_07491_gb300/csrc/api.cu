@@ -767,7 +767,7 @@ int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s
     a.mu = mu;
     a.vmom = P<double>(c->vmom);
     a.pstore = pstore;
-    if (!nc_in_shared(a, c->fp64)) CKS(nc_scratch(c, &a));
+    if (!nc_fwd_in_shared(a, c->fp64)) CKS(nc_scratch(c, &a));
     Region R(c, PK_MOMENTS, 1, s);
     if (launch_nc(a, c->fp64, s)) return fail(c, BOP_ERR_CUDA, "spinor moments launch failed");
     return BOP_OK;
@@ -1101,7 +1101,7 @@ int psi_store_alloc(bop_ctx* c, bool* fits) {
   if (c->m.noncollinear) {
     NcArgs a;
     CKS(nc_args(c, &a));
-    if (!nc_in_shared(a, c->fp64)) return BOP_OK;
+    if (!nc_fwd_in_shared(a, c->fp64) || !nc_rev_in_shared(a, c->fp64)) return BOP_OK;
     bytes = (size_t)c->norb * (size_t)c->psi_tot * c->norb * 8 * esz;
   }
   if (bytes > c->store_budget) return BOP_OK;

@@ -220,8 +220,11 @@ struct NcArgs {
   int HSh;
   double* obar;        // [n][norb][4] (+=): d/d(Ebar, h_x, h_y, h_z)
 };
-// Both sweeps hold two levels (and the onsite cotangents) in shared memory.
-bool nc_in_shared(const NcArgs& a, int fp64);
+// Two levels of the forward sweep, and of the reverse sweep with its onsite
+// cotangents, fit shared memory.  The reverse one needs up to three times as
+// much: it has a route of its own.
+bool nc_fwd_in_shared(const NcArgs& a, int fp64);
+bool nc_rev_in_shared(const NcArgs& a, int fp64);
 int launch_nc(const NcArgs& a, int fp64, cudaStream_t s);
 int launch_torques(int n, int norb, int n_mom, const double* onsite, const double* sdir, const double* w,
                    const double* vmom, const double* obar, double* t, cudaStream_t s);

@@ -2433,11 +2433,13 @@ int launch_moments_adjoint(const AdjointArgs& a, int fp64, cudaStream_t s) {
   return fp64 ? run_adjoint<double, 5>(a, s) : run_adjoint<float, 5>(a, s);
 }
 
-bool nc_in_shared(const NcArgs& a, int fp64) {
-  const size_t esz = fp64 ? 8 : 4;
-  const size_t fwd = (size_t)(a.cap_even + a.cap_odd) * a.norb * NCS * esz;
-  const size_t rev = ((size_t)(a.rev_even + a.rev_odd) * a.norb * NCS + (size_t)a.cap_eb * a.norb * 4) * esz + 16;
-  return fwd <= SMEM_MAX && rev <= SMEM_MAX;
+bool nc_fwd_in_shared(const NcArgs& a, int fp64) {
+  return (size_t)(a.cap_even + a.cap_odd) * a.norb * NCS * (fp64 ? 8 : 4) <= SMEM_MAX;
+}
+
+bool nc_rev_in_shared(const NcArgs& a, int fp64) {
+  const size_t rows = (size_t)(a.rev_even + a.rev_odd) * a.norb * NCS + (size_t)a.cap_eb * a.norb * 4;
+  return rows * (fp64 ? 8 : 4) + 16 <= SMEM_MAX;
 }
 
 int launch_nc(const NcArgs& a, int fp64, cudaStream_t s) {
