@@ -366,6 +366,20 @@ __device__ __forceinline__ void gather_pf2(const int2* __restrict__ ent, int cnt
   }
 }
 
+// The same, one entry at a time: fewer registers by two blocks.
+template <typename T, int NO, int NC, int PS>
+__device__ __forceinline__ void gather_plain(const int2* __restrict__ ent, int cnt, const T* __restrict__ H, int HS,
+                                             const T* __restrict__ x, T acc[NO][NC]) {
+  constexpr int N = NO * NC;
+  for (int e = 0; e < cnt; e++) {
+    const int2 en = ent[e];
+    T hb[hb_count<NO>()], xs[N];
+    load_bond<T, NO>(H + (size_t)en.y * HS, hb);
+    load_row<T, N, PS>(x + (size_t)en.x * PS, xs);
+    block_fma<T, NO, NC>(hb, xs, acc);
+  }
+}
+
 // Adds one bond record of cotangents per lane (v: NO x NO unique elements,
 // padded) to the bonds' cotangent records; bond < 0: none.  All lanes of the
 // warp call it.  FP32: four lanes add one record together, 16 bytes each, so
@@ -1898,22 +1912,30 @@ k_nc(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsi
 
 // The same over stored Psi, as k_moments and k_adj_rev: work items (atom,
 // alpha), the NO items of an atom consecutive in one CTA, which stages the
-// atom's cluster once; Psi (Psi-bar) of two levels in shared memory, blocks of
-// two entries in flight, FP64 rows in the order of their length (FP32 ones in
-// site order over 256 threads, for sums in a fixed order as in k_moments).  One site row
-// holds NO x 8 reals, so that a block feeds 8 NO^2 multiply-adds.
-template <typename T>
+// atom's cluster once; Psi (Psi-bar) of two levels in shared memory, FP64 rows
+// in the order of their length (FP32 ones in site order over 256 threads, for
+// sums in a fixed order as in k_moments).  One site row holds NO x 8 reals, so
+// that a block feeds 8 NO^2 multiply-adds.
+//
+// Forward in FP32 the resident warps hide the loads: blocks of two entries in
+// flight cost registers (sd blocks spilled at the 128 of two CTAs, s blocks
+// kept two CTAs where four fit).  Moments of 2,000 atoms at 9 moments, two
+// entries in flight -> one at a time, s with four CTAs: s 0.155 -> 0.116, d
+// 1.59 -> 1.47, sd 2.79 -> 2.34 ms.  In FP64, with half the threads, two in
+// flight stay ahead for d and sd (432 atoms: 4.63 against 4.82 ms).
+template <typename T, int NO>
 struct NcFwd {
   static constexpr int THREADS = sizeof(T) == 4 ? 256 : 128;
+  static constexpr int CTAS = NO == 1 ? 4 : 2;
 };
 
 template <typename T, int NO>
-__global__ void __launch_bounds__(NcFwd<T>::THREADS, 2)
+__global__ void __launch_bounds__(NcFwd<T, NO>::THREADS, NcFwd<T, NO>::CTAS)
 k_nc_fwd(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite,
          const double* __restrict__ sdir, int n, int n_mom, FwdSmem L, int n_items,
          double* __restrict__ mu, double* __restrict__ vmom, T* __restrict__ pstore,
          const long long* __restrict__ psi_off, long long psi_tot) {
-  constexpr int NT = NcFwd<T>::THREADS;
+  constexpr int NT = NcFwd<T, NO>::THREADS;
   constexpr bool ORDERED = sizeof(T) == 8;
   constexpr int PS = NO * NCS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1998,7 +2020,8 @@ k_nc_fwd(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ 
         }
         const int cnt = (int)((lvc[t] >> (8 * (k - 1))) & 0xff);
         const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
-        gather_pf2<T, NO, NCS, PS>(adj + q0, cnt, H, HS, prev, acc);
+        if constexpr (sizeof(T) == 4) gather_plain<T, NO, NCS, PS>(adj + q0, cnt, H, HS, prev, acc);
+        else gather_pf2<T, NO, NCS, PS>(adj + q0, cnt, H, HS, prev, acc);
         T pt[PS];
         if (in_prev) {
           load_row<T, PS, PS>(prev + (size_t)t * PS, pt);
@@ -2244,7 +2267,7 @@ int persistent_grid(F fn, int threads, size_t smem, int n_items, size_t most) {
 // Spinor sweeps with two levels in shared memory: -2 where they do not fit.
 template <typename T, int NO>
 int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
-  constexpr int NT = NcFwd<T>::THREADS;
+  constexpr int NT = NcFwd<T, NO>::THREADS;
   FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
   const size_t psi = (size_t)(a.cap_even + a.cap_odd) * NO * NCS * sizeof(T);
   size_t smem = psi + (size_t)a.max_adj * 8 + (size_t)a.max_sites * (sizeof(T) == 8 ? 16 : 12) + (size_t)(a.max_sites + 1) * 4 + 16;
