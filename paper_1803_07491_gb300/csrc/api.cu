@@ -1977,8 +1977,9 @@ int bop_forces(bop_ctx* c, double* forces, double* virial, bop_stats* st, bop_st
   CKS(ensure(c, c->w, sizeof(double) * (size_t)M * c->n_mom));
   CKS(ensure(c, c->zscr, sizeof(double) * (size_t)M * (c->n_exp + 1) * 2));
   // bond cotangents in the product type (FP32: float4 reductions)
-  const size_t hbar_bytes = (c->fp64 ? sizeof(double) : sizeof(float)) * (size_t)(c->nb > 0 ? c->nb : 1) *
-                            bond_cotangent_stride(c->norb, c->fp64);
+  const size_t hbar_elems = (size_t)(c->nb > 0 ? c->nb : 1) * bond_cotangent_stride(c->norb, c->fp64);
+  const size_t second = c->m.noncollinear && !c->fp64 ? hbar_elems : 0;  // NcArgs::second
+  const size_t hbar_bytes = (c->fp64 ? sizeof(double) : sizeof(float)) * (hbar_elems + second);
   CKS(ensure(c, c->Hbar, hbar_bytes));
   CKS(ensure(c, c->Ebar, sizeof(double) * (size_t)c->S * n * c->norb));  // onsite cotangents of every atom
   CK(cudaMemsetAsync(c->Hbar.p, 0, hbar_bytes, s));
@@ -2028,6 +2029,7 @@ int bop_forces(bop_ctx* c, double* forces, double* virial, bop_stats* st, bop_st
       a.w = P<double>(c->w);
       a.Hbar = c->Hbar.p;
       a.HSh = bond_cotangent_stride(c->norb, c->fp64);
+      a.second = second;
       a.obar = P<double>(c->obar);
       if (c->psi_valid) a.pstore = c->psis.p;
       else CKS(nc_scratch(c, &a));
@@ -2062,7 +2064,7 @@ int bop_forces(bop_ctx* c, double* forces, double* virial, bop_stats* st, bop_st
   {
     Region Rf(c, PK_FORCES, c->nb > 0 ? 1 : 0, s);
     if (c->nb > 0 && launch_forces((int)c->nb, c->bm, P<double>(c->bond_d), P<int>(c->bond_atoms),
-                                   c->Hbar.p, bond_cotangent_stride(c->norb, c->fp64), c->fp64, F, W, s))
+                                   c->Hbar.p, bond_cotangent_stride(c->norb, c->fp64), second, c->fp64, F, W, s))
       return fail(c, BOP_ERR_CUDA, "forces launch failed");
   }
   int r = check_status(c, s);

@@ -15,7 +15,8 @@ constexpr int FT = 256;
 template <typename HT>
 __global__ void __launch_bounds__(FT) k_forces(int nb, BondModel m, const double* __restrict__ bond_d,
                                                const int* __restrict__ bond_atoms, const HT* __restrict__ Hbar,
-                                               int HSh, double* __restrict__ F, double* __restrict__ W) {
+                                               int HSh, size_t second, double* __restrict__ F,
+                                               double* __restrict__ W) {
   __shared__ double sw[9][FT / 32];
   double w9[9];
   for (int q = 0; q < 9; q++) w9[q] = 0.0;
@@ -34,7 +35,8 @@ __global__ void __launch_bounds__(FT) k_forces(int nb, BondModel m, const double
     const int nu = block_unique(m.norb);
     ST a0 = ST(0), a1 = ST(0), a2 = ST(0);
     for (int q = 0; q < nu; q++) {
-      const ST hb = (ST)Hbar[(size_t)b * HSh + q];
+      ST hb = (ST)Hbar[(size_t)b * HSh + q];
+      if (second > 0) hb += (ST)Hbar[second + (size_t)b * HSh + q];
       a0 += hb * u[q].g0;
       a1 += hb * u[q].g1;
       a2 += hb * u[q].g2;
@@ -95,13 +97,13 @@ int launch_rep_energy(int n, BondModel m, const long long* row_ptr, const int* b
 }
 
 int launch_forces(int nb, BondModel m, const double* bond_d, const int* bond_atoms, const void* Hbar, int HSh,
-                  int fp64, double* forces, double* virial, cudaStream_t s) {
+                  size_t second, int fp64, double* forces, double* virial, cudaStream_t s) {
   int g = (nb + FT - 1) / FT;
   if (g > 4096) g = 4096;
   if (g < 1) g = 1;
   if (fp64)
-    k_forces<double><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const double*)Hbar, HSh, forces, virial);
+    k_forces<double><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const double*)Hbar, HSh, second, forces, virial);
   else
-    k_forces<float><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const float*)Hbar, HSh, forces, virial);
+    k_forces<float><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const float*)Hbar, HSh, second, forces, virial);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -73,3 +73,23 @@ def test_store_released_between_energy_and_forces(bop, prec):
     got = _forces(bop, w, {}, prec, release=True)
     for r, g in zip(ref, got):
         _close(g, r, 1e-9 if prec == "fp64" else 2e-3)
+
+
+@pytest.mark.parametrize("model,bound", [("d", 2.75e-6), ("sd", 3.65e-6)])
+def test_noncollinear_fp32_force_rounding(bop, model, bound):
+    """Rounding of the FP32 forces of the sweep over stored Psi (rms against
+    the FP64 mode, four seeds of a 432-atom cell): no more than that of the
+    sweep that recomputes Psi and adds to a bond once per item, 2.69e-6 (d) and
+    3.56e-6 (sd) eV/A with 2 % for the order of the atomic additions."""
+    err = []
+    for seed in range(4):
+        w = I.with_run(I.small_bcc(6, 6, 6, 0.05, 100 + seed, model=MODELS[model]), n_spin=2, scf="none",
+                       stoner_I=0.8, noncollinear=True)
+        sdir = I.random_directions(w.n_atoms, seed)
+        F = []
+        for prec in ("fp64", "fp32"):
+            ctx = bop.Context(w.model, w.run, prec)
+            F.append(ctx.evaluate(w.pos, w.cell, w.pbc, spin_dir=sdir, m=np.full(w.n_atoms, 2.0)).forces.cpu().numpy())
+            ctx.close()
+        err.append(np.sqrt(np.mean((F[1] - F[0]) ** 2)))
+    assert np.mean(err) < bound
