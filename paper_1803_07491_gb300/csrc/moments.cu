@@ -2255,13 +2255,13 @@ __global__ void k_torques(int n, int norb, int n_mom, const double* __restrict__
 
 // CTAs of a persistent kernel, at most `most`; 0: not one fits an SM.
 template <class F>
-int persistent_grid(F fn, int threads, size_t smem, int n_items, size_t most) {
+int persistent_grid(F fn, int threads, size_t smem, int n_items, int most) {
   int per_sm = 0, sms = 0, dev = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) return 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int slots = sms * per_sm;
-  if ((size_t)slots > most) slots = (int)most;
+  if (slots > most) slots = most;
   return n_items < slots ? n_items : slots;
 }
 
@@ -2321,6 +2321,19 @@ int run_nc(const NcArgs& a, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+}  // namespace
+
+// Most CTAs of a sweep: with Psi of two levels in global memory each CTA has a
+// slot of the scratch, also where Psi_1 .. Psi_K are in the store (Psi_0 is
+// written to the slot).
+extern "C" int launch_max_ctas(int gmem, size_t scratch_bytes, size_t slot_bytes, int n_items) {
+  if (!gmem) return n_items;
+  const size_t slots = scratch_bytes / slot_bytes;
+  return slots < (size_t)n_items ? (int)slots : n_items;
+}
+
+namespace {
+
 template <typename T, int NO, bool GMEM>
 int run_forward(const MomentsArgs& a, cudaStream_t s) {
   constexpr int N = NO * NO;
@@ -2344,8 +2357,7 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
   if (!allow_smem(fn)) return -1;
   const int n_items = a.n * a.n_spin;
   const size_t slot = (size_t)(a.cap_even + a.cap_odd) * PS;
-  // with Psi in global scratch no more CTAs than its slots
-  const size_t most = GMEM && a.pstore == nullptr ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
+  const int most = launch_max_ctas(GMEM, a.scratch_bytes, slot * sizeof(T), n_items);
   if (most < 1) return n_items == 0 ? 0 : -1;
   const int grid = persistent_grid(fn, NT, smem, n_items, most);
   if (grid < 1) return -1;
@@ -2395,7 +2407,7 @@ int run_reverse(const AdjointArgs& a, cudaStream_t s) {
     smem = psi;
   }
   const int n_items = a.n * a.n_spin;
-  const size_t most = GMEM ? a.scratch_bytes / (slot * sizeof(T)) : (size_t)n_items;
+  const int most = launch_max_ctas(GMEM, a.scratch_bytes, slot * sizeof(T), n_items);
   if (most < 1) return n_items == 0 ? 0 : -1;
   const int grid = persistent_grid(fn, NT, smem, n_items, most);
   if (grid < 1) return -1;
