@@ -606,6 +606,7 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
           if (!image_sum(rt, pe.y, &img)) {
             s_fail = 1;
             raise_error(A.status, BOP_DEV_ERR_IMAGE);
+            img = 0x808080u;  // an image beyond a byte would reach the record's atom
           }
           nb[q] = grid_rec(pe.x, img, rec_addr(rt) + __ldg(&A.eoff[e].x));
           const unsigned code = (((img >> 16) - 128u + A.mx) * (2u * A.my + 1u) + ((img >> 8) & 255u) - 128u + A.my) *
