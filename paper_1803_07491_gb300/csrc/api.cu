@@ -472,12 +472,19 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     a.mx = plan.mx;
     a.my = plan.my;
     a.mz = plan.mz;
-    a.ncode = (2 * a.mx + 1) * (2 * a.my + 1) * (2 * a.mz + 1);
+    const int codes = cluster_key_codes(c->n, (2 * a.mx + 1) * (2 * a.my + 1) * (2 * a.mz + 1), a.newcap);
+    if (codes < 0) return BOP_OK;
+    a.ncode = codes;
     a.qbits = 0;
     while ((1 << a.qbits) < a.newcap) a.qbits++;
-    if ((unsigned long long)c->n * a.ncode >= 1ull << (32 - a.qbits)) return BOP_OK;  // 32-bit sort keys
-    CKS(ensure(c, c->cw_keys, sizeof(unsigned long long) * (size_t)n * a.maxs));
-    CKS(ensure(c, c->cw_cnt, (size_t)n * a.maxs));
+    const size_t recs = (size_t)n * a.maxs;
+    if (sizeof(unsigned long long) * recs > c->cw_keys.bytes) {  // a third of the free memory at most
+      size_t freeb = 0, totalb = 0;
+      CK(cudaMemGetInfo(&freeb, &totalb));
+      if ((sizeof(unsigned long long) + 1) * recs > (freeb + c->cw_keys.bytes + c->cw_cnt.bytes) / 3) return BOP_OK;
+    }
+    CKS(ensure(c, c->cw_keys, sizeof(unsigned long long) * recs));
+    CKS(ensure(c, c->cw_cnt, recs));
     a.rows = P<int2>(c->cw_rows);
     a.epack = P<int2>(c->cw_epack);
     a.eoff = P<int2>(c->cw_eoff);

@@ -484,6 +484,25 @@ __device__ __forceinline__ void warp_order(int cnt, int nkeys, int* off, int lan
   }
 }
 
+// Keys of the atom alone: how far entry q of the sorted keys lies from its
+// place among the images of its atom, which stand side by side.
+__device__ __forceinline__ int image_rank(const unsigned* keys, const unsigned long long* nb, int q, int cnt,
+                                          unsigned mask) {
+  const unsigned long long r = nb[keys[q] & mask];
+  int d = 0;
+  for (int p = q - 1; p >= 0; p--) {
+    const unsigned long long o = nb[keys[p] & mask];
+    if (rec_atom(o) != rec_atom(r)) break;
+    d -= o > r ? 1 : 0;
+  }
+  for (int p = q + 1; p < cnt; p++) {
+    const unsigned long long o = nb[keys[p] & mask];
+    if (rec_atom(o) != rec_atom(r)) break;
+    d += o < r ? 1 : 0;
+  }
+  return d;
+}
+
 // What a row step needs of its site, in shared memory (written one thread per
 // site, read by the row's lanes): the first edge, and the address and degree.
 __device__ __forceinline__ int2 site_row(int2 row, int addr) { return make_int2(row.x, addr | (row.y << 16)); }
@@ -611,13 +630,13 @@ __global__ void __launch_bounds__(G) k_cluster_grid(GridArgs A, PathCut pc, Clus
           nb[q] = grid_rec(pe.x, img, rec_addr(rt) + __ldg(&A.eoff[e].x));
           const unsigned code = (((img >> 16) - 128u + A.mx) * (2u * A.my + 1u) + ((img >> 8) & 255u) - 128u + A.my) *
                                     (2u * A.mz + 1u) + (img & 255u) - 128u + A.mz;
-          keys[q] = ((unsigned)pe.x * A.ncode + code) << A.qbits | (unsigned)q;
+          keys[q] = (A.ncode > 0 ? (unsigned)pe.x * A.ncode + code : (unsigned)pe.x) << A.qbits | (unsigned)q;
         }
         group_sync<G>();
         group_sort<G>(keys, cnt, tid);
         for (int q = tid; q < cnt; q += G) {
           const unsigned long long r = nb[keys[q] & ((1u << A.qbits) - 1u)];
-          const int t = nsite + q;
+          const int t = nsite + q + (A.ncode > 0 ? 0 : image_rank(keys, nb, q, cnt, (1u << A.qbits) - 1u));
           const int2 row = __ldg(A.rows + rec_atom(r));
           sk[t] = gk[t] = r;
           srow[t] = site_row(row, rec_addr(r));
@@ -957,6 +976,18 @@ bool grid_plan(const Geometry& g, int K, const int* maxima, GridPlan* p) {
   for (int a = 0; a < 3; a++) *m[a] = g.pbc[a] ? (r[a] + g.nc[a] - 1) / g.nc[a] : 0;
   p->tsize = (int)size;
   return true;
+}
+
+// Codes per atom in the 32-bit sort keys of a level (newcap entries) of a
+// structure of n atoms with ncode images each: ncode where they fit, 0 (keys of
+// the atom alone, its images put in order after the sort) up to 2^24 atoms at
+// 256 entries, -1 beyond.  With 27 images the codes end at 621,378 atoms.
+extern "C" int cluster_key_codes(int n, int ncode, int newcap) {
+  int qbits = 0;
+  while ((1 << qbits) < newcap) qbits++;
+  const unsigned long long limit = 1ull << (32 - qbits);
+  if ((unsigned long long)n * (unsigned)ncode < limit) return ncode;
+  return (unsigned long long)n <= limit ? 0 : -1;
 }
 
 template <int PASS, bool CUT, int G>

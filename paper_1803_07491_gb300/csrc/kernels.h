@@ -110,7 +110,7 @@ struct GridArgs {
   int n, K;                  // clusters of the first n atoms
   int origin, tsize;         // GridPlan
   unsigned mx, my, mz;       // likewise
-  unsigned ncode, qbits;     // images of an atom; log2(newcap): sort keys (atom, image) << qbits | entry
+  unsigned ncode, qbits;     // cluster_key_codes, log2(newcap): sort keys (atom, image) << qbits | entry
   int lpr_shift;             // lanes per neighbour row: 4 (16 lanes) or 5 (32)
   int maxs, newcap;          // sites of one cluster, new sites of one level (a power of two)
   int sites;                 // pass 1: largest cluster (pass 0 found it)
@@ -123,6 +123,7 @@ struct GridArgs {
   int* fail;                 // != 0 after pass 0: a cluster exceeds maxs, newcap or the table
   unsigned* status;
 };
+extern "C" int cluster_key_codes(int n, int ncode, int newcap);
 int launch_cluster_grid(int pass, const GridArgs& a, const PathCut& pc, const ClusterOut& out, cudaStream_t s);
 
 struct MomentsArgs {
