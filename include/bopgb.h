@@ -300,7 +300,9 @@ int bop_recursion(bop_ctx* ctx, int M, const double* mu, double* a, double* b, i
  *   m_io      device [n] Stoner moments, same convention (NULL = m0)
  *   stats_host optional host struct
  * Synchronises stream once per SCF iteration (convergence flag) and at
- * the end. */
+ * the end.  Moments, energies, E_F and onsite levels of two calls on the same
+ * input are the same bits (scf VARIATIONAL excepted: it sweeps back in every
+ * iteration); forces, virial and torques are summed by atomics and are not. */
 int bop_energy(bop_ctx* ctx, double* e_atom, double* delta_io, double* m_io, bop_stats* stats_host,
                bop_stream stream);
 

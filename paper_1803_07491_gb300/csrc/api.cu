@@ -70,8 +70,9 @@ struct bop_ctx {
       bond_of_edge, bond_atoms, bond_img, bond_d, H64, H32, frac;
   DBuf hkeys, hvals, skeys, sslot, scount;
   DBuf level_end, atom_nsite, atom_nadj, max_level, site_off, adj_base, site_atom, site_img, adj_off, adj, lvcnt,
-      order, top, ntop, topmask;
+      order, top, ntop, topmask, mirror, rowsum;
   bool pair_ok = false;  // the clusters carry the pair form of the last level
+  bool mirror_ok = false;  // mirror is that of the built structure
   DBuf onsite, onsite32, delta, mval, delta_new, m_new, mu, a, b, nlev, a_inf, b_inf, gsig, D, gjack;
   DBuf N, U, dos, fstate, partials, counter, result, e_total, lam, e_atom;
   DBuf w, zscr, adjscr, Hbar, Ebar, ginv;
@@ -566,7 +567,7 @@ int build_clusters(bop_ctx* c, cudaStream_t s) {
   const int n = c->nc, K = c->K;  // clusters of the centres
   {
     bool done = false;
-    c->pair_ok = false;
+    c->pair_ok = c->mirror_ok = false;
     CKS(build_clusters_grid(c, s, &done));
     if (done) return BOP_OK;
   }
@@ -763,6 +764,34 @@ int nc_scratch(bop_ctx* c, NcArgs* a) {
   return BOP_OK;
 }
 
+// What the FP64 pair form needs beside the clusters, made by the first pass of a
+// structure.  Row sums that take more than a third of the free memory: the full
+// form instead.
+int pair_scratch(bop_ctx* c, MomentsArgs* a, cudaStream_t s) {
+  const size_t bytes = sizeof(double2) * (size_t)c->S * c->nsite * c->norb;
+  if (bytes > c->rowsum.bytes) {
+    size_t freeb = 0, totalb = 0;
+    CK(cudaMemGetInfo(&freeb, &totalb));
+    if (bytes > (freeb + c->rowsum.bytes) / 3 || c->nsite >= 1ll << 32) {
+      a->pair = false;
+      return BOP_OK;
+    }
+    CKS(ensure(c, c->rowsum, bytes));
+  }
+  if (!c->mirror_ok) {
+    CKS(ensure(c, c->mirror, sizeof(unsigned) * (size_t)c->nsite));
+    Region R(c, PK_CLUSTER, 1, s);
+    if (launch_pair_mirror(c->nc, c->K, P<long long>(c->site_off), P<int>(c->level_end), P<int>(c->site_atom),
+                           P<signed char>(c->site_img), P<unsigned>(c->mirror), P<unsigned>(c->status), s))
+      return fail(c, BOP_ERR_CUDA, "pair mirror launch failed");
+    c->mirror_ok = true;
+  }
+  a->mirror = P<unsigned>(c->mirror);
+  a->rowsum = P<double2>(c->rowsum);
+  a->nsite = c->nsite;
+  return BOP_OK;
+}
+
 // full: every row of the last level is computed (and stored), for sweeps that
 // keep the work items apart (the rows of the SCF Jacobian).
 int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s, void* pstore = nullptr,
@@ -801,11 +830,12 @@ int run_moments(bop_ctx* c, const double* onsite_dev, double* mu, cudaStream_t s
   a.psi_off = P<long long>(c->psi_off);
   a.psi_tot = c->psi_tot;
   a.pair = c->pair_ok && !full;
+  if (a.pair && c->fp64) CKS(pair_scratch(c, &a, s));
   a.gmem = moments_in_gmem(c->norb, a.cap_even + a.cap_odd, c->fp64);
   a.scratch = nullptr;
   a.scratch_bytes = 0;
   if (a.gmem) CKS(slot_scratch(c, a.cap_even + a.cap_odd, &a.scratch, &a.scratch_bytes));
-  Region R(c, PK_MOMENTS, 1, s);
+  Region R(c, PK_MOMENTS, a.pair && c->fp64 ? 2 : 1, s);
   int r = launch_moments(a, c->fp64, s);
   if (r == -2) return fail(c, BOP_ERR_OVERFLOW, "cluster level too large for shared memory");
   if (r) return fail(c, BOP_ERR_CUDA, "moments launch: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1536,7 +1566,8 @@ int bop_destroy(bop_ctx* c) {
                   &c->row_ptr, &c->col, &c->img, &c->flag, &c->bond_scan, &c->bond_of_edge, &c->bond_atoms,
                   &c->bond_img, &c->bond_d, &c->H64, &c->H32, &c->frac, &c->hkeys, &c->hvals, &c->skeys,
                   &c->sslot, &c->scount, &c->level_end, &c->atom_nsite, &c->atom_nadj, &c->max_level,
-                  &c->site_off, &c->adj_base, &c->site_atom, &c->site_img, &c->adj_off, &c->adj, &c->lvcnt, &c->order, &c->top, &c->ntop, &c->topmask, &c->onsite,
+                  &c->site_off, &c->adj_base, &c->site_atom, &c->site_img, &c->adj_off, &c->adj, &c->lvcnt, &c->order, &c->top, &c->ntop, &c->topmask,
+                   &c->mirror, &c->rowsum, &c->onsite,
                   &c->onsite32, &c->delta, &c->mval, &c->delta_new, &c->m_new, &c->mu, &c->a, &c->b, &c->nlev,
                   &c->a_inf, &c->b_inf, &c->gsig, &c->D, &c->gjack, &c->N, &c->U, &c->dos, &c->fstate,
                   &c->partials, &c->counter, &c->result, &c->e_total, &c->lam, &c->e_atom, &c->w, &c->zscr,

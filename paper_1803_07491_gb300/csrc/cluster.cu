@@ -1027,6 +1027,81 @@ int launch_cluster_grid(int pass, const GridArgs& a, const PathCut& pc, const Cl
   return run_grid_pass<512>(pass, a, pc, out, sms, s);
 }
 
+// The pair form's way back, one block per atom j: a site (i, s) of its cluster
+// that is not selected is the selected site (j, -s) of i's cluster, in the same
+// shell.  mirror + site_off[j]: the places of those among the sites of all
+// clusters (a binary search of the shell's canonical order), in the order of
+// j's sites.
+constexpr int MIR_THREADS = 512;
+
+__global__ void __launch_bounds__(MIR_THREADS) k_pair_mirror(int K, const long long* __restrict__ site_off,
+                                                             const int* __restrict__ level_end,
+                                                             const int* __restrict__ site_atom,
+                                                             const signed char* __restrict__ site_img,
+                                                             unsigned* __restrict__ mirror,
+                                                             unsigned* __restrict__ status) {
+  __shared__ int s_lev[BOP_MAX_K + 1], s_cnt[MIR_THREADS / 32];
+  const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const long long s0 = site_off[j];
+  if (tid <= K) s_lev[tid] = level_end[(size_t)j * (K + 1) + tid];
+  __syncthreads();
+  const int nsite = s_lev[K];
+  int done = 0;  // entries of the rounds before
+  for (int u0 = 0; u0 < nsite; u0 += MIR_THREADS) {
+    const int u = u0 + tid;
+    int i = j, sx = 0, sy = 0, sz = 0;  // (the centre is selected)
+    if (u < nsite) {
+      const signed char* im = site_img + 3 * (s0 + u);
+      i = site_atom[s0 + u];
+      sx = im[0];
+      sy = im[1];
+      sz = im[2];
+    }
+    const bool mine = !pair_selected(j, i, sx, sy, sz);
+    const unsigned bal = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) s_cnt[wid] = __popc(bal);
+    __syncthreads();
+    int at = done + __popc(bal & ((1u << lane) - 1u));
+    for (int w = 0; w < MIR_THREADS / 32; w++) {
+      if (w < wid) at += s_cnt[w];
+      done += s_cnt[w];
+    }
+    __syncthreads();
+    if (!mine) continue;  // (barriers above only)
+    int l = 1;
+    while (u >= s_lev[l]) l++;
+    const int* li = level_end + (size_t)i * (K + 1);
+    const long long b = site_off[i];
+    int lo = li[l - 1], hi = li[l];
+    const int end = hi;
+    auto order = [&](int m) {  // site m of i's cluster against (j, -s)
+      const int a = site_atom[b + m];
+      if (a != j) return a < j ? -1 : 1;
+      const signed char* q = site_img + 3 * (b + m);
+      if (q[0] != -sx) return q[0] < -sx ? -1 : 1;
+      if (q[1] != -sy) return q[1] < -sy ? -1 : 1;
+      return q[2] != -sz ? (q[2] < -sz ? -1 : 1) : 0;
+    };
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (order(mid) < 0) lo = mid + 1;
+      else hi = mid;
+    }
+    if (lo >= end || order(lo) != 0) {  // cannot happen: hops are symmetric
+      raise_error(status, BOP_DEV_ERR_CLUSTER);
+      lo = 0;
+    }
+    mirror[s0 + at] = (unsigned)(b + lo);
+  }
+}
+
+int launch_pair_mirror(int n, int K, const long long* site_off, const int* level_end, const int* site_atom,
+                       const signed char* site_img, unsigned* mirror, unsigned* status, cudaStream_t s) {
+  if (n <= 0) return 0;
+  k_pair_mirror<<<n, MIR_THREADS, 0, s>>>(K, site_off, level_end, site_atom, site_img, mirror, status);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 // Rows of one stored Psi sweep per atom: sum_{k=0..K} |C_k|.
 __global__ void k_level_sums(int n, int K, const int* __restrict__ level_end, long long* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -123,6 +123,8 @@ struct GridArgs {
   int* fail;                 // != 0 after pass 0: a cluster exceeds maxs, newcap or the table
   unsigned* status;
 };
+int launch_pair_mirror(int n, int K, const long long* site_off, const int* level_end, const int* site_atom,
+                       const signed char* site_img, unsigned* mirror, unsigned* status, cudaStream_t s);
 extern "C" int cluster_key_codes(int n, int ncode, int newcap);
 int launch_cluster_grid(int pass, const GridArgs& a, const PathCut& pc, const ClusterOut& out, cudaStream_t s);
 
@@ -147,6 +149,11 @@ struct MomentsArgs {
   // pair form (needs cv.top; every atom a centre): FP64 computes, and both
   // precisions store, the selected rows of Psi_K only
   bool pair;
+  // FP64 pair form: launch_pair_mirror's, and scratch of {row sum with Psi_K-1,
+  // row sum of squares} per spin, site of every cluster and orbital
+  const unsigned* mirror;
+  double2* rowsum;
+  long long nsite;     // sites of all clusters
   // Psi of two levels in global memory (moments_in_gmem): in the store, or in
   // scratch, one slot (moments_slot_bytes) per CTA
   bool gmem;

@@ -667,8 +667,7 @@ k_moments(ClusterView cv, const float* __restrict__ H, int HS, const float* __re
 // sub-partition, whatever its active lanes), so the work goes into warps that
 // are full and equally long: NO lanes per site, lane r holding row r of its
 // NO x NO block (32 / NO sites per warp, 25 multiply-adds per entry and lane at
-// NO = 5), and the warps of a CTA taking the next sites of a level from a
-// counter, longest rows first.  The lanes of a site read the same Psi row
+// NO = 5), longest rows first.  The lanes of a site read the same Psi row
 // (one shared-memory broadcast) and the NO elements of their row of the bond
 // block.  With one lane per site (and two for long rows of small levels) the
 // lanes were 82 % and the pipe 81 % busy, the SMs 88 %, at 9 moments.  The
@@ -718,16 +717,18 @@ __device__ __forceinline__ void gather64(const int2* __restrict__ ent, int cnt, 
 
 // Forward.  pair: the last level computes the selected sites only
 // (pair_selected).  H^K is symmetric, so the block Z = Psi_K(t, i) holds
-// Psi_K(i, t)^T too: its column sums go to this item's last two moments and
-// its row sums to those of the site's atom, all with FP64 atomics onto moments
-// that start at zero (68 % of a bcc cluster's products at 9 moments are in
-// that level).  GMEM as k_moments.
+// Psi_K(i, t)^T too: its column sums go to this item's last two moments; its
+// row sums belong to those of the site's atom and are written out for
+// k_pair_sums (68 % of a bcc cluster's products at 9 moments are in that
+// level).  Every sum has an order of its own: the rows of a level go to the
+// warps there and back in their order, and no atomics, so that moments repeat
+// bit for bit.  GMEM as k_moments.
 template <int NO, bool GMEM>
 __global__ void __launch_bounds__(F64_THREADS, 2)
 k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* __restrict__ onsite, int n, int n_on,
             int n_mom, FwdSmem L, int n_items, double* __restrict__ mu, double* __restrict__ pstore,
-            const long long* __restrict__ psi_off, long long psi_tot, bool pair, double* __restrict__ scratch,
-            size_t slot_elems) {
+            const long long* __restrict__ psi_off, long long psi_tot, bool pair, double2* __restrict__ rowsum, long long nsite,
+            double* __restrict__ scratch, size_t slot_elems) {
   constexpr int NT = F64_THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<double, N>::PS;
@@ -745,7 +746,6 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
   // per-warp partial sums of the two moments of a level, in two buffers
   // (level parity), as k_moments
   __shared__ double red[2][2 * NC][NT / 32];
-  __shared__ int s_next[BOP_MAX_K + 1];  // next sites of a level
   const int K = cv.K;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   ItemExt nx{};
@@ -777,7 +777,6 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
       for (int q = tid; q < PS; q += NT) pitem[q] = q < N && q / NC == q % NC ? 1.0 : 0.0;
     }
     for (int q = tid; q < PS; q += NT) buf[0][q] = q < N && q / NC == q % NC ? 1.0 : 0.0;
-    if (tid <= K) s_next[tid] = 0;
     long long lo_k = 0;
     __syncthreads();
     double* out = mu + (size_t)w * NO * n_mom;
@@ -786,72 +785,73 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
       const bool in_store = GMEM && pstore != nullptr;
       const double* prev = in_store ? pitem + (size_t)lo_k * PS : buf[(k - 1) & 1];
       lo_k += lev[k - 1];
-      const bool half = pair && k == K;
       const int ncol = lev[k - 1], inner = k >= 2 ? lev[k - 2] : 0;
-      const int nrow = half ? ntop : lev[k];
+      const int nrow = pair && k == K ? ntop : lev[k];
       double* next = buf[k & 1];
       double d[2 * NC];
 #pragma unroll
       for (int c = 0; c < 2 * NC; c++) d[c] = 0.0;
-      while (true) {
-        int first = 0;
-        if (lane == 0) first = atomicAdd(&s_next[k], 32);
-        first = __shfl_sync(0xffffffffu, first, 0);
-        if (first >= nrow * NO) break;
-        // (the lanes of a site need not be in one warp: 32 / NO is no whole number)
-        const int q = (first + lane) / NO, r = (first + lane) % NO;
-        if (q >= nrow) continue;  // (the shuffle above reconverges the warp)
-        int u[NO];
+      // two copies of the rows' code: the sums of the half level cost the other
+      // levels registers (2,000 atoms at 17 moments: 22.2 -> 21.7 ms)
+      auto rows = [&](auto last) {
+        constexpr bool half = decltype(last)::value;
+        constexpr int NW = NT / 32;
+        for (int p = 0; 32 * p * NW < nrow * NO; p++) {
+          const int first = 32 * (p * NW + ((p & 1) ? NW - 1 - wid : wid));
+          // (the lanes of a site need not be in one warp: 32 / NO is no whole number)
+          const int q = (first + lane) / NO, r = (first + lane) % NO;
+          if (q >= nrow) continue;
+          int u[NO];
 #pragma unroll
-        for (int g = 0; g < NO; g++) u[g] = UI<NO>(r, g);
-        // rows up to level k-2 are full, shell k-1 has entries up to its own
-        // level, shell k of the one below
-        const int t = half ? (int)(top[q] & 0xffffu)
-                           : (q < inner ? q : (q < ncol ? (int)(order[q] >> 16) : (int)(order[q] & 0xffffu)));
-        const bool in_prev = t < ncol;
-        const int atom_t = satom[t];
-        const double* pt = prev + (size_t)t * PS + r * NC;
-        double acc[NC];
-        if (in_prev) {
-          const double er = E[(size_t)atom_t * NO + r];
+          for (int g = 0; g < NO; g++) u[g] = UI<NO>(r, g);
+          // rows up to level k-2 are full, shell k-1 has entries up to its own
+          // level, shell k of the one below
+          const int t = half ? (int)(top[q] & 0xffffu)
+                             : (q < inner ? q : (q < ncol ? (int)(order[q] >> 16) : (int)(order[q] & 0xffffu)));
+          const bool in_prev = t < ncol;
+          const int atom_t = satom[t];
+          const double* pt = prev + (size_t)t * PS + r * NC;
+          double acc[NC];
+          if (in_prev) {
+            const double er = E[(size_t)atom_t * NO + r];
 #pragma unroll
-          for (int c = 0; c < NC; c++) acc[c] = er * pt[c];
-        } else {
+            for (int c = 0; c < NC; c++) acc[c] = er * pt[c];
+          } else {
 #pragma unroll
-          for (int c = 0; c < NC; c++) acc[c] = 0.0;
-        }
-        const unsigned long long lc = L.stage ? s_lvc[t] : cv.lvcnt[s0 + t];
-        const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
-        const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
-        gather64<NO, PS>(L.stage ? s_adj + q0 : adj + q0, cnt, H, HS, prev, u, acc);
-        const bool other = half && t != 0;
-        double* mt = mu + (((size_t)spin * n + atom_t) * NO + r) * n_mom + 2 * K - 1;  // the last two moments of (atom_t, r)
-        if (in_prev) {
-          double a = 0.0;
-#pragma unroll
-          for (int c = 0; c < NC; c++) {
-            const double p = pt[c];
-            d[c] += p * acc[c];
-            if (half) a += p * acc[c];
+            for (int c = 0; c < NC; c++) acc[c] = 0.0;
           }
-          if (other) atomicAdd(mt, a);
-        }
-        double a = 0.0;
+          const unsigned long long lc = L.stage ? s_lvc[t] : cv.lvcnt[s0 + t];
+          const int cnt = (int)((lc >> (8 * (k - 1))) & 0xff);
+          const int q0 = L.stage ? s_off[t] : (int)(cv.adj_off[s0 + t] - abase);
+          gather64<NO, PS>(L.stage ? s_adj + q0 : adj + q0, cnt, H, HS, prev, u, acc);
+          if (in_prev) {
 #pragma unroll
-        for (int c = 0; c < NC; c++) {
-          d[NC + c] += acc[c] * acc[c];
-          if (half) a += acc[c] * acc[c];
-        }
-        if (other) atomicAdd(mt + 1, a);
-        if (k < K && !in_store) {
+            for (int c = 0; c < NC; c++) d[c] += pt[c] * acc[c];
+          }
 #pragma unroll
-          for (int c = 0; c < NC; c++) next[(size_t)t * PS + r * NC + c] = acc[c];
-        }
-        if (pitem != nullptr) {
+          for (int c = 0; c < NC; c++) d[NC + c] += acc[c] * acc[c];
+          if constexpr (half) {  // the row's sums, for the site's atom
+            double a1 = 0.0, a2 = 0.0;
+            if (in_prev) {
 #pragma unroll
-          for (int c = 0; c < NC; c++) pitem[(size_t)(lo_k + t) * PS + r * NC + c] = acc[c];
+              for (int c = 0; c < NC; c++) a1 += pt[c] * acc[c];
+            }
+#pragma unroll
+            for (int c = 0; c < NC; c++) a2 += acc[c] * acc[c];
+            rowsum[((size_t)spin * nsite + s0 + t) * NO + r] = make_double2(a1, a2);
+          }
+          if (k < K && !in_store) {
+#pragma unroll
+            for (int c = 0; c < NC; c++) next[(size_t)t * PS + r * NC + c] = acc[c];
+          }
+          if (pitem != nullptr) {
+#pragma unroll
+            for (int c = 0; c < NC; c++) pitem[(size_t)(lo_k + t) * PS + r * NC + c] = acc[c];
+          }
         }
-      }
+      };
+      if (pair && k == K) rows(std::true_type{});
+      else rows(std::false_type{});
       int which;
       const double sum = warp_sums<2 * NC>(d, lane, &which);
       if (which >= 0) red[k & 1][which][wid] = sum;
@@ -862,12 +862,52 @@ k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
         double a = 0.0;
         for (int q = 0; q < NT / 32; q++) a += red[k & 1][tid][q];
         const int c = tid % NC;
-        double* m = out + (size_t)c * n_mom + (tid < NC ? 2 * k - 1 : 2 * k);
-        if (half) atomicAdd(m, a);
-        else *m = a;
+        out[(size_t)c * n_mom + (tid < NC ? 2 * k - 1 : 2 * k)] = a;
       }
     }
     if (more) ext_adj(cv, nx);
+  }
+}
+
+// The rest of the last two moments in the pair form: of every site that is not
+// selected, the row sums that its pair left in the cluster of the site's atom
+// (k_pair_mirror).  One block per (spin, atom): a lane per value of a site's row
+// sums and 32 / (2 NO) sites at a time, so that FP64 additions have all lanes;
+// eight warps, since what bounds it is the latency of a place and its row sums
+// (432 atoms with two spins, cold cache: 18 us with one warp, 13 with eight).
+// It is launched while the sweep still runs and waits for it (3 us a pass).  A
+// pass of theirs takes 614 us, 603 with FP64 atomics and sites drawn from a
+// counter, whose moments did not repeat.
+constexpr int PS_THREADS = 256;
+
+template <int NO>
+__global__ void __launch_bounds__(PS_THREADS) k_pair_sums(ClusterView cv, int n, int n_mom,
+                                                          const unsigned* __restrict__ mirror,
+                                                          const double2* __restrict__ rowsum, long long nsite,
+                                                          double* __restrict__ mu) {
+  constexpr int V = 2 * NO, SW = 32 / V, NW = PS_THREADS / 32;
+  __shared__ double sh[NW][V];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int w = blockIdx.x, spin = w / n, atom = w % n, K = cv.K;
+  const int cnt = cv.level_end[(size_t)atom * (K + 1) + K] - (cv.ntop[atom] & 0xffff);
+  const unsigned* list = mirror + cv.site_off[atom];
+  const double* rs = reinterpret_cast<const double*>(rowsum + (size_t)spin * nsite * NO) + lane % V;
+  cudaGridDependencySynchronize();  // the sweep's row sums and moments
+  double a = 0.0;
+  if (lane < V * SW) {
+#pragma unroll 8
+    for (int q = wid * SW + lane / V; q < cnt; q += NW * SW) a += __ldg(rs + (size_t)__ldg(list + q) * V);
+  }
+  double sum = a;
+#pragma unroll
+  for (int p = 1; p < SW; p++) sum += __shfl_sync(0xffffffffu, a, lane + p * V);
+  if (lane < V) sh[wid][lane] = sum;
+  __syncthreads();
+  if (tid < V) {
+    double m = 0.0;
+#pragma unroll
+    for (int q = 0; q < NW; q++) m += sh[q][tid];
+    mu[((size_t)w * NO + tid / 2) * n_mom + 2 * K - 1 + tid % 2] += m;
   }
 }
 
@@ -2361,12 +2401,24 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
   if (most < 1) return n_items == 0 ? 0 : -1;
   const int grid = persistent_grid(fn, NT, smem, n_items, most);
   if (grid < 1) return -1;
-  if (F64 && a.pair && cudaMemsetAsync(a.mu, 0, sizeof(double) * (size_t)a.n_spin * a.n * NO * a.n_mom, s) != cudaSuccess)
-    return -1;
-  if constexpr (F64)
+  if constexpr (F64) {
     fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, a.mu,
-                              (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
-  else
+                              (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, a.rowsum, a.nsite, (T*)a.scratch, slot);
+    if (a.pair) {
+      cudaLaunchAttribute early{};
+      early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      early.val.programmaticStreamSerializationAllowed = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = n_items;
+      cfg.blockDim = PS_THREADS;
+      cfg.stream = s;
+      cfg.attrs = &early;
+      cfg.numAttrs = 1;
+      if (cudaLaunchKernelEx(&cfg, k_pair_sums<NO>, a.cv, a.n, a.n_mom, a.mirror, (const double2*)a.rowsum, a.nsite,
+                             a.mu) != cudaSuccess)
+        return -1;
+    }
+  } else
     fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

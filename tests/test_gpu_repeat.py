@@ -1,0 +1,50 @@
+"""Repeated FP64 calls on the same input give the same bits: moments, energies,
+Fermi level and self-consistent onsite levels (the forces are summed by
+atomics and do not)."""
+import numpy as np
+import pytest
+
+from paper_1803_07491_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MODELS = {"s": I.MODEL_S, "d": I.MODEL_D, "sd": I.MODEL_SD}
+
+
+@pytest.fixture(scope="module")
+def bop():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1803_07491_gb300 import build, bop as b
+    build.build()
+    return b
+
+
+@pytest.mark.parametrize("model,cells,kw", [
+    ("s", (4, 4, 4), {}), ("d", (5, 4, 6), {}), ("d", (2, 2, 3), dict(n_mom=3)), ("sd", (4, 4, 4), {}),
+    ("d", (4, 4, 4), dict(n_mom=13)), ("d", (5, 5, 5), dict(n_mom=9, r_path=5.5)), ("s", (1, 1, 1), dict(n_mom=17)),
+    ("d", (5, 5, 5), dict(scf="lcn", **I.ANDERSON_STEP)),
+    ("d", (4, 4, 4), dict(scf="stoner", n_spin=2, stoner_I=0.8, m_mix=1.0, **I.ANDERSON_STEP))])
+def test_fp64_energy_repeats_bit_for_bit(bop, model, cells, kw):
+    w = I.with_run(I.small_bcc(*cells, 0.035, 41, model=MODELS[model]), **kw)
+    M = w.run.n_spin * w.n_atoms * w.model.norb
+    first = None
+    for _ in range(2):  # contexts
+        ctx = bop.Context(w.model, w.run, "fp64")
+        for forces in (True, False, True):  # the energy after forces stores Psi in its own pass
+            r = ctx.evaluate(w.pos, w.cell, w.pbc, forces=forces)
+            st = bop.bop_get_orbital_state(ctx.h, M, w.run.n_mom)
+            got = [r.e_atom.cpu().numpy(), np.array([r.e_total, r.e_fermi]), st["onsite"].cpu().numpy(),
+                   st["N"].cpu().numpy()]
+            if not forces or w.run.scf == "none":  # the SCF response repeats the last pass in the full form
+                got.append(st["mu"].cpu().numpy())
+            else:
+                got.append(None)
+            first = first or got
+            for q, (a, b) in enumerate(zip(first, got)):
+                if a is None or b is None:
+                    first[q] = a if a is not None else b
+                else:
+                    assert np.array_equal(a, b), q
+        ctx.close()
