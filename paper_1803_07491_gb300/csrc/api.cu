@@ -271,7 +271,7 @@ struct Readback {
         a.at[q] = (int)(off[q] / 4);
         a.words[q] = (int)(len[q] / 4);
       }
-      if (launch_collect(a, s)) return fail(c, BOP_ERR_CUDA, "readback launch: %s", cudaGetErrorString(cudaPeekAtLastError()));
+      if (launch_collect(a, s)) return fail(c, BOP_ERR_CUDA, "readback launch failed");
     }
     sent = true;
     CK(cudaStreamSynchronize(s));
@@ -312,7 +312,8 @@ int check_status(bop_ctx* c, cudaStream_t s) {
 template <class Tin, class Tout>
 int exclusive_scan(bop_ctx* c, const Tin* in, Tout* out, long long n, cudaStream_t s) {
   if (n <= SCAN_SMALL) {  // one launch instead of two
-    if (launch_scan_small<Tin, Tout>(in, out, nullptr, nullptr, (int)n, s)) return fail(c, BOP_ERR_CUDA, "scan launch failed");
+    if (launch_scan_small<Tin, Tout>(in, out, nullptr, nullptr, (int)n, s))
+      return fail(c, BOP_ERR_CUDA, "scan launch failed");
     return BOP_OK;
   }
   size_t tmp = 0;
@@ -1081,7 +1082,7 @@ int compute_weights(bop_ctx* c, double cU, const double* lam, double cN0, double
   wa.onsite = P<double>(c->onsite);
   wa.st = P<FermiState>(c->fstate);
   wa.g = P<double>(c->gjack);
-    wa.g32 = reinterpret_cast<const float*>(P<double>(c->gjack) + c->n_exp + 1);
+  wa.g32 = reinterpret_cast<const float*>(P<double>(c->gjack) + c->n_exp + 1);
   wa.inv = P<double>(c->ginv);
   wa.cU = cU;
   wa.lam = lam;
@@ -1536,7 +1537,8 @@ int bop_create(bop_ctx** out, const bop_model* model) {
   c->bm.rep_p = model->rep_p;
   cudaGetDevice(&c->device);
   memset(&c->st, 0, sizeof(c->st));
-  if ((r = ensure(c, c->status, sizeof(unsigned))) || (r = ensure(c, c->gjack, (sizeof(double) + sizeof(float)) * (c->n_exp + 1))) ||
+  if ((r = ensure(c, c->status, sizeof(unsigned))) ||
+      (r = ensure(c, c->gjack, (sizeof(double) + sizeof(float)) * (c->n_exp + 1))) ||
       (r = ensure(c, c->fstate, sizeof(FermiState))) || (r = ensure(c, c->partials, sizeof(double) * 3 * 4096)) ||
       (r = ensure(c, c->counter, sizeof(unsigned))) || (r = ensure(c, c->result, sizeof(double) * 4)) ||
       (r = ensure(c, c->e_total, sizeof(double))) || (r = ensure(c, c->lam, sizeof(double) * 4)) ||
@@ -1562,11 +1564,13 @@ int bop_create(bop_ctx** out, const bop_model* model) {
 
 int bop_destroy(bop_ctx* c) {
   if (!c) return BOP_OK;
-  DBuf* bufs[] = {&c->pos, &c->cell_of, &c->cell_count, &c->cell_start, &c->cell_fill, &c->cell_atoms, &c->cell_slot, &c->deg,
+  DBuf* bufs[] = {&c->pos, &c->cell_of, &c->cell_count, &c->cell_start, &c->cell_fill, &c->cell_atoms,
+                   &c->cell_slot, &c->deg,
                   &c->row_ptr, &c->col, &c->img, &c->flag, &c->bond_scan, &c->bond_of_edge, &c->bond_atoms,
                   &c->bond_img, &c->bond_d, &c->H64, &c->H32, &c->frac, &c->hkeys, &c->hvals, &c->skeys,
                   &c->sslot, &c->scount, &c->level_end, &c->atom_nsite, &c->atom_nadj, &c->max_level,
-                  &c->site_off, &c->adj_base, &c->site_atom, &c->site_img, &c->adj_off, &c->adj, &c->lvcnt, &c->order, &c->top, &c->ntop, &c->topmask,
+                  &c->site_off, &c->adj_base, &c->site_atom, &c->site_img, &c->adj_off, &c->adj, &c->lvcnt,
+                   &c->order, &c->top, &c->ntop, &c->topmask,
                    &c->mirror, &c->rowsum, &c->onsite,
                   &c->onsite32, &c->delta, &c->mval, &c->delta_new, &c->m_new, &c->mu, &c->a, &c->b, &c->nlev,
                   &c->a_inf, &c->b_inf, &c->gsig, &c->D, &c->gjack, &c->N, &c->U, &c->dos, &c->fstate,
@@ -1574,9 +1578,11 @@ int bop_destroy(bop_ctx* c) {
                   &c->adjscr, &c->Hbar, &c->Ebar, &c->status, &c->cub_tmp, &c->nprod,
                   &c->ginv, &c->hx, &c->hf, &c->gamma, &c->scfred, &c->lbase, &c->lnlev, &c->lflag, &c->lxs,
                   &c->lys, &c->lZ1, &c->lH1, &c->lZ2, &c->lH2, &c->lybar, &c->lcot, &c->lxbar, &c->lcount,
-                  &c->rwN, &c->rwt, &c->rdUE, &c->rvec, &c->rcoef, &c->rjv, &c->rjcnt, &c->rjptr, &c->rjidx, &c->rjrow, &c->vgrad, &c->vq, &c->erep,
+                  &c->rwN, &c->rwt, &c->rdUE, &c->rvec, &c->rcoef, &c->rjv, &c->rjcnt, &c->rjptr, &c->rjidx, &c->rjrow,
+                   &c->vgrad, &c->vq, &c->erep,
                   &c->psi_off, &c->psis, &c->lsum, &c->sdir, &c->vmom, &c->obar, &c->torque,
-                  &c->ncscr, &c->cw_misc, &c->cw_keys, &c->cw_cnt, &c->cw_epack, &c->cw_eoff, &c->cw_rows, &c->fev, &c->gs32};
+                  &c->ncscr, &c->cw_misc, &c->cw_keys, &c->cw_cnt, &c->cw_epack, &c->cw_eoff, &c->cw_rows,
+                   &c->fev, &c->gs32};
   for (DBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   if (c->pin) cudaFreeHost(c->pin);

@@ -237,7 +237,8 @@ __device__ __forceinline__ void chain_polys_reverse(const Chain& ch, int L, int 
 template <int KP, int NS>
 __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double ai, double bi, double E, double ef,
                                         const double* __restrict__ g, const double* __restrict__ inv,
-                                        const float* __restrict__ g32, int ne, int M, int o, const double* cU, const double* cN, double* zs, double* const* zb,
+                                        const float* __restrict__ g32, int ne, int M, int o, const double* cU,
+                                        const double* cN, double* zs, double* const* zb,
                                         double (*abar)[KPMAX + 1], double (*bbar)[KPMAX + 2], double* abar_inf,
                                         double* bbar_inf, double* dE, bool f32 = false) {
   constexpr int NP = 2 * KP + 1;
@@ -455,7 +456,8 @@ __device__ inline void chain_reverse_ns(const Chain& ch, int L, int Kb, double a
 template <int KP>
 __device__ inline double chain_reverse(const Chain& ch, int L, int Kb, double ai, double bi, double E, double ef,
                                        const double* __restrict__ g, const double* __restrict__ inv,
-                                       const float* __restrict__ g32, int ne, int M, int o, double cU, double cN, double* zs, double* zb, double* abar,
+                                       const float* __restrict__ g32, int ne, int M, int o, double cU, double cN,
+                                       double* zs, double* zb, double* abar,
                                        double* bbar, double& abar_inf, double& bbar_inf, bool f32 = false) {
   double* zbs[1] = {zb};
   double ab[1][KPMAX + 1], bb_[1][KPMAX + 2];

@@ -727,8 +727,8 @@ template <int NO, bool GMEM>
 __global__ void __launch_bounds__(F64_THREADS, 2)
 k_moments64(ClusterView cv, const double* __restrict__ H, int HS, const double* __restrict__ onsite, int n, int n_on,
             int n_mom, FwdSmem L, int n_items, double* __restrict__ mu, double* __restrict__ pstore,
-            const long long* __restrict__ psi_off, long long psi_tot, bool pair, double2* __restrict__ rowsum, long long nsite,
-            double* __restrict__ scratch, size_t slot_elems) {
+            const long long* __restrict__ psi_off, long long psi_tot, bool pair, double2* __restrict__ rowsum,
+            long long nsite, double* __restrict__ scratch, size_t slot_elems) {
   constexpr int NT = F64_THREADS, NC = NO;
   constexpr int N = NO * NC;
   constexpr int PS = (N == 1) ? 1 : Row<double, N>::PS;
@@ -1498,11 +1498,12 @@ __device__ __forceinline__ int site_level(const int* lev, int K, int t) {
   return k;
 }
 
-template <typename T, int NO, int NC>
+template <typename T, int NO>
 __global__ void __launch_bounds__(MOM_THREADS)
 k_moments_adj(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite, int n, int n_on, int n_mom,
               int nwork, const double* __restrict__ wts, T* __restrict__ scratch, size_t slot_elems,
               T* __restrict__ Hbar, int HSh, double* __restrict__ Ebar) {
+  constexpr int NC = NO;
   __shared__ T ws[NC][BOP_MAX_NMOM];
   __shared__ int s_lev[BOP_MAX_K + 1];
   __shared__ long long s_off[BOP_MAX_K + 2];
@@ -1510,9 +1511,7 @@ k_moments_adj(ClusterView cv, const T* __restrict__ H, int HS, const T* __restri
   const int tid = threadIdx.x;
   T* psi = scratch + (size_t)blockIdx.x * slot_elems;
   for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
-    const int grp = (NC == NO) ? 0 : (w % NO);
-    const int sa = (NC == NO) ? w : (w / NO);
-    const int spin = sa / n, atom = sa % n;
+    const int spin = w / n, atom = w % n;
     const long long s0 = cv.site_off[atom];
     const int* lev = cv.level_end + (size_t)atom * (K + 1);
     const int* satom = cv.site_atom + s0;
@@ -1529,16 +1528,13 @@ k_moments_adj(ClusterView cv, const T* __restrict__ H, int HS, const T* __restri
     }
     for (int q = tid; q < NC * n_mom; q += blockDim.x) {
       int c = q / n_mom, m = q % n_mom;
-      ws[c][m] = (T)wts[((size_t)sa * NO + grp + c) * n_mom + m];
+      ws[c][m] = (T)wts[((size_t)w * NO + c) * n_mom + m];
     }
     __syncthreads();
     T* P = psi;
     T* Pb = psi + s_off[K + 1] - s_off[1];  // Pb + s_off[k] is Psi-bar_k (k >= 1)
     // forward: all levels
-    for (int q = tid; q < NO * NC; q += blockDim.x) {
-      int r = q / NC, c = q % NC;
-      P[q] = (NC == NO) ? T(r == c ? 1 : 0) : T(r == grp ? 1 : 0);
-    }
+    for (int q = tid; q < NO * NC; q += blockDim.x) P[q] = T(q / NC == q % NC ? 1 : 0);
     __syncthreads();
     for (int k = 1; k <= K; k++) {
       const T* x = P + s_off[k - 1];
@@ -2311,7 +2307,8 @@ int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
   constexpr int NT = NcFwd<T, NO>::THREADS;
   FwdSmem L{a.cap_even, a.cap_odd, a.max_sites, a.max_adj, true};
   const size_t psi = (size_t)(a.cap_even + a.cap_odd) * NO * NCS * sizeof(T);
-  size_t smem = psi + (size_t)a.max_adj * 8 + (size_t)a.max_sites * (sizeof(T) == 8 ? 16 : 12) + (size_t)(a.max_sites + 1) * 4 + 16;
+  size_t smem = psi + (size_t)a.max_adj * 8 + (size_t)a.max_sites * (sizeof(T) == 8 ? 16 : 12) +
+                (size_t)(a.max_sites + 1) * 4 + 16;
   if (smem > 110 * 1024) {
     L.stage = false;
     smem = psi;
@@ -2322,7 +2319,8 @@ int run_nc_fwd(const NcArgs& a, cudaStream_t s) {
   const int n_items = a.n * NO;
   const int grid = persistent_grid(fn, NT, smem, n_items, n_items);
   if (grid < 1) return -1;
-  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, a.mu, a.vmom, (T*)a.pstore, a.psi_off, a.psi_tot);
+  fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items, a.mu,
+                            a.vmom, (T*)a.pstore, a.psi_off, a.psi_tot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2419,7 +2417,8 @@ int run_forward(const MomentsArgs& a, cudaStream_t s) {
         return -1;
     }
   } else
-    fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, a.mu, (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
+    fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items, a.mu,
+                              (T*)a.pstore, a.psi_off, a.psi_tot, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2427,7 +2426,7 @@ template <typename T, int NO>
 int run_adjoint(const AdjointArgs& a, cudaStream_t s) {
   const int nwork = a.n * a.n_spin;
   const int grid = nwork < a.slots ? nwork : a.slots;
-  k_moments_adj<T, NO, NO><<<grid, MOM_THREADS, 0, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on,
+  k_moments_adj<T, NO><<<grid, MOM_THREADS, 0, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on,
                                                        a.n_mom, nwork, a.w, (T*)a.scratch, a.slot_elems,
                                                        (T*)a.Hbar, a.HSh, a.Ebar);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
