@@ -12,7 +12,8 @@ namespace {
 
 constexpr int FT = 256;
 
-template <typename HT>
+// TWO: the cotangents lie in two arrays, `second` elements apart (NcArgs).
+template <typename HT, bool TWO>
 __global__ void __launch_bounds__(FT) k_forces(int nb, BondModel m, const double* __restrict__ bond_d,
                                                const int* __restrict__ bond_atoms, const HT* __restrict__ Hbar,
                                                int HSh, size_t second, double* __restrict__ F,
@@ -36,7 +37,7 @@ __global__ void __launch_bounds__(FT) k_forces(int nb, BondModel m, const double
     ST a0 = ST(0), a1 = ST(0), a2 = ST(0);
     for (int q = 0; q < nu; q++) {
       ST hb = (ST)Hbar[(size_t)b * HSh + q];
-      if (second > 0) hb += (ST)Hbar[second + (size_t)b * HSh + q];
+      if (TWO) hb += (ST)Hbar[second + (size_t)b * HSh + q];
       a0 += hb * u[q].g0;
       a1 += hb * u[q].g1;
       a2 += hb * u[q].g2;
@@ -102,8 +103,10 @@ int launch_forces(int nb, BondModel m, const double* bond_d, const int* bond_ato
   if (g > 4096) g = 4096;
   if (g < 1) g = 1;
   if (fp64)
-    k_forces<double><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const double*)Hbar, HSh, second, forces, virial);
+    k_forces<double, false><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const double*)Hbar, HSh, 0, forces, virial);
+  else if (second > 0)
+    k_forces<float, true><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const float*)Hbar, HSh, second, forces, virial);
   else
-    k_forces<float><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const float*)Hbar, HSh, second, forces, virial);
+    k_forces<float, false><<<g, FT, 0, s>>>(nb, m, bond_d, bond_atoms, (const float*)Hbar, HSh, 0, forces, virial);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

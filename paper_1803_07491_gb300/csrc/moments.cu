@@ -387,11 +387,11 @@ __device__ __forceinline__ void gather_plain(const int2* __restrict__ ent, int c
 // quarters are exchanged between the lanes by 12 shuffles; reductions of
 // scattered records cost the L1 unit one cycle per line).
 template <typename T, int NO>
-__device__ __forceinline__ void add_bond_records(T* __restrict__ Hbar, int bond, const T G[NO][NO], int lane) {
-  constexpr int HV = hbar_stride<T, NO>();
+__device__ __forceinline__ void add_bond_records(T* __restrict__ Hbar, int HSh, int bond, const T G[NO][NO], int lane) {
   if constexpr (NO == 1 || sizeof(T) == 8) {
-    if (bond >= 0) add_bond_cotangent<T, NO>(Hbar + (size_t)bond * HV, G);
+    if (bond >= 0) add_bond_cotangent<T, NO>(Hbar + (size_t)bond * HSh, G);
   } else {
+    constexpr int HV = hbar_stride<T, NO>();
     float v[HV];
 #pragma unroll
     for (int q = 0; q < HV; q++) v[q] = 0.f;
@@ -417,10 +417,10 @@ __device__ __forceinline__ void add_bond_records(T* __restrict__ Hbar, int bond,
         x.w = __shfl_xor_sync(0xffffffffu, x.w, d);
         bd = __shfl_xor_sync(0xffffffffu, bond, d);
       }
-      if (bd >= 0) atomicAdd(reinterpret_cast<float4*>(Hbar + (size_t)bd * HV) + q, x);
+      if (bd >= 0) atomicAdd(reinterpret_cast<float4*>(Hbar + (size_t)bd * HSh) + q, x);
     }
     if (bond >= 0) {
-      float4* dst = reinterpret_cast<float4*>(Hbar + (size_t)bond * HV);
+      float4* dst = reinterpret_cast<float4*>(Hbar + (size_t)bond * HSh);
 #pragma unroll
       for (int w = 4; w < HV / 4; w++)
         atomicAdd(dst + w, make_float4(v[4 * w], v[4 * w + 1], v[4 * w + 2], v[4 * w + 3]));
@@ -438,7 +438,7 @@ template <typename T, int NO, int NC, int PS, bool HBAR>
 __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int first, int step, int cnt, unsigned mask,
                                            bool use_mask, const T* __restrict__ H, int HS, const T* __restrict__ x,
                                            T acc[NO][NC], bool gather, const T pt[NO * NC], T* __restrict__ Hbar,
-                                           int lane) {
+                                           int HSh, int lane) {
   constexpr int HB = hb_count<NO>();
   constexpr int N = NO * NC;
   const int mine = use_mask ? __popc(mask) : (cnt > first ? (cnt - first + step - 1) / step : 0);
@@ -498,7 +498,7 @@ __device__ __forceinline__ void gather_rev(const int2* __restrict__ ent, int fir
 #pragma unroll
         for (int g = 0; g < NO; g++) G[b][g] = T(0);
     }
-    if constexpr (HBAR) add_bond_records<T, NO>(Hbar, bond, G, lane);
+    if constexpr (HBAR) add_bond_records<T, NO>(Hbar, HSh, bond, G, lane);
   }
 }
 
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(F32_THREADS, 2)
 k_adj_rev(ClusterView cv, const float* __restrict__ H, int HS, const float* __restrict__ onsite, int n, int n_on,
           int n_mom, RevSmem L, int n_items, const float* __restrict__ pstore,
           const long long* __restrict__ psi_off, long long psi_tot, const double* __restrict__ wts,
-          float* __restrict__ Hbar, double* __restrict__ Ebar, double* __restrict__ siteval,
+          float* __restrict__ Hbar, int HSh, double* __restrict__ Ebar, double* __restrict__ siteval,
           long long sv_stride, bool pair, float* __restrict__ scratch, size_t slot_elems) {
   using T = float;
   constexpr int NT = F32_THREADS, NC = NO;
@@ -1115,7 +1115,7 @@ k_adj_rev(ClusterView cv, const float* __restrict__ H, int HS, const float* __re
             }
           }
           gather_rev<T, NO, NC, PS, HBAR>(adj + q0, part, 1 << psh, cnt, mask, half, H, HS, xb, acc, k >= 2, pt, Hbar,
-                                          lane);
+                                          HSh, lane);
           for (int o = 1; o < (1 << psh); o <<= 1) {
 #pragma unroll
             for (int r = 0; r < NO; r++)
@@ -2117,7 +2117,7 @@ __global__ void __launch_bounds__(128, 2)
 k_nc_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ onsite,
          const double* __restrict__ sdir, int n, int n_mom, RevSmem L, int n_items,
          const T* __restrict__ pstore, const long long* __restrict__ psi_off, long long psi_tot,
-         const double* __restrict__ wts, T* __restrict__ Hbar0, size_t second, double* __restrict__ obar) {
+         const double* __restrict__ wts, T* __restrict__ Hbar0, int HSh, size_t second, double* __restrict__ obar) {
   constexpr int NT = 128;
   constexpr int PS = NO * NCS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2238,7 +2238,7 @@ k_nc_rev(ClusterView cv, const T* __restrict__ H, int HS, const T* __restrict__ 
           else cnt = L.stage ? s_off[t + 1] - q0 : (int)(cv.adj_off[s0 + t + 1] - abase) - q0;
         }
         gather_rev<T, NO, NCS, PS, true>(adj + q0, part, 1 << psh, cnt, 0u, false, H, HS, xb, acc, k >= 2, pt, Hbar,
-                                         lane);
+                                         HSh, lane);
         if (!live || part != 0 || k < 2) continue;
         T* row = &acc[0][0];
 #pragma unroll
@@ -2343,7 +2343,8 @@ int run_nc_rev(const NcArgs& a, cudaStream_t s) {
   const int grid = persistent_grid(fn, 128, smem, n_items, n_items);
   if (grid < 1) return -1;
   fn<<<grid, 128, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.sdir, a.n, a.n_mom, L, n_items,
-                             (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.second, a.obar);
+                             (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.second,
+                             a.obar);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2468,8 +2469,8 @@ int run_reverse(const AdjointArgs& a, cudaStream_t s) {
                               a.sv_stride, a.pair, (T*)a.scratch, slot);
   else
     fn<<<grid, NT, smem, s>>>(a.cv, (const T*)a.H, a.HS, (const T*)a.onsite, a.n, a.n_on, a.n_mom, L, n_items,
-                              (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.Ebar, a.siteval, a.sv_stride,
-                              a.pair, (T*)a.scratch, slot);
+                              (const T*)a.pstore, a.psi_off, a.psi_tot, a.w, (T*)a.Hbar, a.HSh, a.Ebar, a.siteval,
+                              a.sv_stride, a.pair, (T*)a.scratch, slot);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
