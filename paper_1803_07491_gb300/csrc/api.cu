@@ -21,7 +21,10 @@ constexpr int FERMI_ROUNDS_WARM = 5;  // ... and from the previous SCF iteration
 constexpr int FERMI_ROUNDS_MORE = 64;  // extra rounds if a solve has not converged
 constexpr int FERMI_MAX_ROUNDS = 256;  // hard cap per solve
 constexpr double FERMI_TOL = 1e-13;    // eV
-constexpr int FERMI_F32_START = 65536; // orbitals from which a cold solve starts with FP32 rounds
+// orbitals from which a cold solve starts with FP32 rounds (80,000 orbitals: 0.52
+// against 1.25 ms; drawn for sums on one lane per orbital, whereas they now pay
+// from about 10,000: 0.19 against 0.21 ms)
+constexpr int FERMI_F32_START = 65536;
 
 namespace {
 
@@ -189,6 +192,17 @@ int ensure(bop_ctx* c, DBuf& b, size_t bytes) {
     return fail(c, BOP_ERR_OOM, "cudaMalloc(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
   }
   b.bytes = bytes;
+  return BOP_OK;
+}
+
+// Whether a buffer of `bytes` in the place of `held` takes at most a third of the
+// free memory (the query takes 33 us: not for less than 1 GB).
+int third_of_free(bop_ctx* c, size_t bytes, size_t held, bool* fits) {
+  *fits = true;
+  if (bytes <= (size_t)1 << 30) return BOP_OK;
+  size_t freeb = 0, totalb = 0;
+  if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess) return fail(c, BOP_ERR_CUDA, "memory query failed");
+  *fits = bytes <= (freeb + held) / 3;
   return BOP_OK;
 }
 
@@ -480,11 +494,10 @@ int build_clusters_grid(bop_ctx* c, cudaStream_t s, bool* done) {
     a.qbits = 0;
     while ((1 << a.qbits) < a.newcap) a.qbits++;
     const size_t recs = (size_t)n * a.maxs;
-    if (sizeof(unsigned long long) * recs > c->cw_keys.bytes) {  // a third of the free memory at most
-      size_t freeb = 0, totalb = 0;
-      CK(cudaMemGetInfo(&freeb, &totalb));
-      if ((sizeof(unsigned long long) + 1) * recs > (freeb + c->cw_keys.bytes + c->cw_cnt.bytes) / 3) return BOP_OK;
-    }
+    bool room = true;
+    if (sizeof(unsigned long long) * recs > c->cw_keys.bytes)
+      CKS(third_of_free(c, (sizeof(unsigned long long) + 1) * recs, c->cw_keys.bytes + c->cw_cnt.bytes, &room));
+    if (!room) return BOP_OK;
     CKS(ensure(c, c->cw_keys, sizeof(unsigned long long) * recs));
     CKS(ensure(c, c->cw_cnt, recs));
     a.rows = P<int2>(c->cw_rows);
@@ -771,9 +784,9 @@ int nc_scratch(bop_ctx* c, NcArgs* a) {
 int pair_scratch(bop_ctx* c, MomentsArgs* a, cudaStream_t s) {
   const size_t bytes = sizeof(double2) * (size_t)c->S * c->nsite * c->norb;
   if (bytes > c->rowsum.bytes) {
-    size_t freeb = 0, totalb = 0;
-    CK(cudaMemGetInfo(&freeb, &totalb));
-    if (bytes > (freeb + c->rowsum.bytes) / 3 || c->nsite >= 1ll << 32) {
+    bool room = c->nsite < 1ll << 32;  // places of 32 bits
+    if (room) CKS(third_of_free(c, bytes, c->rowsum.bytes, &room));
+    if (!room) {
       a->pair = false;
       return BOP_OK;
     }

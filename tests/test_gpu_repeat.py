@@ -48,3 +48,18 @@ def test_fp64_energy_repeats_bit_for_bit(bop, model, cells, kw):
                 else:
                     assert np.array_equal(a, b), q
         ctx.close()
+
+
+@pytest.mark.parametrize("model,kw", [("d", {}), ("sd", dict(scf="lcn", **I.ANDERSON_STEP, scf_tol=3e-5)),
+                                      ("d", dict(n_mom=13))])
+def test_fp32_energy_repeats_bit_for_bit(bop, model, kw):
+    w = I.with_run(I.small_bcc(5, 4, 4, 0.05, 42, model=MODELS[model]), **kw)
+    got = []
+    for forces in (True, False):
+        ctx = bop.Context(w.model, w.run, "fp32")
+        for _ in range(2):
+            r = ctx.evaluate(w.pos, w.cell, w.pbc, forces=forces)
+            got.append(np.append(r.e_atom.cpu().numpy(), [r.e_total, r.e_fermi]))
+        ctx.close()
+    for g in got[1:]:
+        assert np.array_equal(g, got[0])
