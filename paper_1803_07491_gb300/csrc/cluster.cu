@@ -332,13 +332,14 @@ k_cluster(int n, int K, const long long* __restrict__ row_ptr, const int* __rest
 // adjacency and keeps the site records; pass 1 fills the table from them and
 // writes sites, adjacency and level counts.
 //
-// What bounds it: issue slots (58 to 68 % used), after the table's 14 to 76
-// KB per cluster has limited the CTAs on an SM, hence several warps per
-// cluster.  The hash-table builder it replaces (one warp per atom, 64-bit
-// keys) took 27.9 k and 34.4 k warp instructions per atom in the two passes,
-// this one 16.3 k and 17.1 k: 131,072 bcc atoms at 9 moments 19.8 -> 5.7 ms,
-// 2,000 atoms at 17 moments (one CTA per atom, hash table in global memory
-// before) 10.6 -> 1.1 ms.
+// What bounds it: issue slots (57 and 63 % used in the two passes), after the
+// table's 14 to 76 KB per cluster has limited the CTAs on an SM, hence several
+// warps per cluster.  The hash-table builder it replaces (one warp per atom,
+// 64-bit keys) took 27.9 k and 34.4 k warp instructions per atom in the two
+// passes, this one 16.5 k and 24.5 k (2,000 bcc atoms at 9 moments, with the
+// pair form's outputs): 131,072 atoms at 9 moments 19.8 -> 6.7 ms, 2,000 atoms
+// at 17 moments (one CTA per atom, hash table in global memory before) 10.6 ->
+// 1.3 ms.
 constexpr unsigned short GRID_CLAIM = 0x8000;  // pass 0: claimed, index not yet assigned; else index + 1
 constexpr int ORDER_KEYS = (BOP_MAX_K + 1) * 33;  // (shell, entries) of a row
 
@@ -1017,11 +1018,13 @@ int launch_cluster_grid(int pass, const GridArgs& a, const PathCut& pc, const Cl
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // Threads per cluster: eight rows a step for many clusters (131,072 atoms of
-  // 14 neighbours: 5.7 / 5.9 / 7.5 ms with 128 / 256 / 512 threads; 1,372 atoms
-  // of 18 neighbours, 32 lanes a row: 0.23 / 0.16 / 0.16 ms), 512 where the
-  // clusters do not fill the SMs (250 atoms: 0.051 / 0.037 / 0.033 ms) or are
-  // large (17 moments, 2,000 atoms: 3.6 / 2.0 / 1.1 ms).
+  // Threads per cluster, both passes with 128 / 256 / 512: eight rows a step for
+  // many clusters (131,072 bcc atoms at 9 moments 6.70 / 7.04 / 9.15 ms, 2,000
+  // atoms 0.123 / 0.126 / 0.159), twice the threads where a row takes 32 lanes,
+  // and 512 where the clusters do not fill the SMs (250 atoms 0.059 / 0.047 /
+  // 0.042 ms) or outgrow the first tier (2,000 atoms at 17 moments 3.18 / 1.93 /
+  // 1.33 ms, 16,000 at 13 moments 4.54 / 3.01 / 2.91; 1,372 fcc atoms at 9
+  // moments, the exception, 0.241 / 0.177 / 0.189).
   if (a.maxs <= 512 && a.n > 4 * sms)
     return a.lpr_shift == 4 ? run_grid_pass<128>(pass, a, pc, out, sms, s) : run_grid_pass<256>(pass, a, pc, out, sms, s);
   return run_grid_pass<512>(pass, a, pc, out, sms, s);

@@ -1388,8 +1388,12 @@ k_adj_rev64(ClusterView cv, const double* __restrict__ H, int HS, const double* 
       const double* xb = buf[k & 1];
       double* yb = buf[(k - 1) & 1];
       const int nrow = s_lev[k - 1];
-      // lanes of few rows: P parts of a row's entries (2 to 14 in bcc) each on
-      // its own lanes, where that shortens the rounds of the CTA's warps
+      // lanes of few rows: P parts of a row's entries each on its own lanes,
+      // where that shortens the rounds of the CTA's warps.  A row is priced at 16
+      // entries, whatever its length (14 in bcc, 18 in fcc, fewer at a surface):
+      // sweeps of 2,000 bcc / 1,372 fcc atoms at 9 moments and 686 bcc at 13 take
+      // 2.89 / 3.33 / 5.56 ms so, 2.89 / 3.32 / 6.03 priced at 14, 2.89 / 3.24 /
+      // 5.42 at 18, 3.59 / 3.33 / 5.95 at 64
       int parts = 1, rows = RPW;  // rows of a warp
       if (!half) {
         int best = 1 << 30;
