@@ -779,21 +779,23 @@ int nc_scratch(bop_ctx* c, NcArgs* a) {
 }
 
 // What the FP64 pair form needs beside the clusters, made by the first pass of a
-// structure.  Row sums that take more than a third of the free memory: the full
-// form instead.
+// structure.  Where the memory is short (row sums of more than a third of what
+// is free, or no room at all) the full form runs instead.
 int pair_scratch(bop_ctx* c, MomentsArgs* a, cudaStream_t s) {
   const size_t bytes = sizeof(double2) * (size_t)c->S * c->nsite * c->norb;
   if (bytes > c->rowsum.bytes) {
     bool room = c->nsite < 1ll << 32;  // places of 32 bits
     if (room) CKS(third_of_free(c, bytes, c->rowsum.bytes, &room));
-    if (!room) {
+    if (!room || ensure(c, c->rowsum, bytes) != BOP_OK) {
       a->pair = false;
       return BOP_OK;
     }
-    CKS(ensure(c, c->rowsum, bytes));
   }
   if (!c->mirror_ok) {
-    CKS(ensure(c, c->mirror, sizeof(unsigned) * (size_t)c->nsite));
+    if (ensure(c, c->mirror, sizeof(unsigned) * (size_t)c->nsite) != BOP_OK) {
+      a->pair = false;
+      return BOP_OK;
+    }
     Region R(c, PK_CLUSTER, 1, s);
     if (launch_pair_mirror(c->nc, c->K, P<long long>(c->site_off), P<int>(c->level_end), P<int>(c->site_atom),
                            P<signed char>(c->site_img), P<unsigned>(c->mirror), P<unsigned>(c->status), s))
