@@ -388,15 +388,16 @@ int bop_set_reduce(bop_ctx* ctx, bop_reduce_fn fn, void* user);
  * Errors: BOP_ERR_ARG for max_iterations < 0 or rtol < 0 or not finite. */
 int bop_set_response_limits(bop_ctx* ctx, int max_iterations, double rtol);
 
-/* Memory for the reverse sweeps of bop_forces.  When several reverse sweeps
- * follow (an SCF with scf_response = 1) and all starting orbitals of an atom
- * share one work item of the moments kernel, bop_forces runs one extra
- * forward pass that stores Psi_k of every atom's cluster (rows of norb x
- * norb values per site and level, FP32 or FP64 as the precision) when it
- * fits in a third of the free device memory, and every reverse sweep then
- * reads Psi instead of recomputing it (the sweep that forms the bond
- * cotangents forms them level by level from the same store).
- * bytes >= 0 caps that store (0 = always recompute, which also frees it);
+/* Memory for the reverse sweeps of bop_forces.  Where it fits in a third of
+ * the free device memory, Psi_k of every atom's cluster (rows of norb x norb
+ * values per site and level, of norb x 8 for spinors, FP32 or FP64 as the
+ * precision) is stored by a forward pass - the energy's own without an SCF
+ * once forces have been asked for, and in every VARIATIONAL iteration, else one
+ * more pass of bop_forces - and the reverse sweeps read it instead of
+ * recomputing it (the sweep that forms the bond cotangents forms them level by
+ * level from the same store).
+ * bytes >= 0 caps that store (0 = always recompute, which also frees it, at
+ * any time: forces after an energy that stored Psi then recompute it);
  * bytes < 0 restores the default. */
 int bop_set_store_budget(bop_ctx* ctx, long long bytes);
 
